@@ -3,7 +3,6 @@
 //       deferred normalisation F_lm a^l                                  (Eq. (multipole))
 //   a4  irregular solid harmonics of the separation vector R0            (Eq. (Formula))
 //   a5  two-center contraction in double                                 (Eq. (Formula))
-//   a6  exact pairwise Coulomb sum in double                             (Eq. (Coulomb))
 #include <cuda_runtime.h>
 
 #include "contract.h"
@@ -17,39 +16,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
-// Fixed-order block sum (deterministic); result valid in thread 0.  blockDim <= 1024.
-__device__ double block_sum(double v, double* sh) {
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  double r = 0.0;
-  if (w == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    r = lane < nw ? sh[lane] : 0.0;
-    r = warp_sum(r);
-  }
-  __syncthreads();
-  return r;
-}
-__device__ __forceinline__ void load_xyz(const void* p, int dtype, long long i, double& x, double& y, double& z,
-                                         double& q) {
-  if (dtype == TCM_F32) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(p) + i);
-    x = v.x;
-    y = v.y;
-    z = v.z;
-    q = v.w;
-  } else {
-    const double2 a = __ldg(reinterpret_cast<const double2*>(p) + 2 * i);
-    const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 2 * i + 1);
-    x = a.x;
-    y = a.y;
-    z = b.x;
-    q = b.y;
-  }
-}
-
 // Degrees l <= kLowLmax of one job from its system's low-degree sums (system pass 2, reduced over
 // the system's tiles by its last tile): the Cartesian sums are rotated by the job's rotation R
 // (P' = R P, T' = R T R^T, p = R d) and turned into the packed Q_lm, l <= 2, with
@@ -607,77 +573,6 @@ __global__ void __launch_bounds__(kContractThreads) k_rotate_moments(const RotDe
   }
 }
 
-// a6: exact pairwise sum.  One thread per atom of A; B staged through shared memory
-// already rotated and translated: b' = R0 + rot (x_b - c_B).  Double precision.
-constexpr int kDirectThreads = 256;
-
-struct alignas(32) Atom4 {  // a staged atom of B: position after rotation and separation, charge
-  double x, y, z, w;
-};
-
-__global__ void __launch_bounds__(kDirectThreads) k_direct(const void* __restrict__ a, long long na, int dta,
-                                                           const void* __restrict__ b, long long nb, int dtb,
-                                                           const SysGeom* __restrict__ geo, const double* __restrict__ xf,
-                                                           double* __restrict__ part) {
-  __shared__ Atom4 sb[kDirectThreads];
-  __shared__ double sh[32];
-  const double* cA = geo[0].c;
-  const double* cB = geo[1].c;
-  const double* rot = xf + 12LL * blockIdx.y;  // this item's rotation of B and separation
-  const double* R0 = rot + 9;
-  part += (long long)blockIdx.y * gridDim.x;
-  const long long i = (long long)blockIdx.x * kDirectThreads + threadIdx.x;
-  double ax = 0.0, ay = 0.0, az = 0.0, qa = 0.0;
-  if (i < na) {
-    load_xyz(a, dta, i, ax, ay, az, qa);
-    ax -= cA[0];
-    ay -= cA[1];
-    az -= cA[2];
-  }
-  double acc = 0.0;
-  for (long long j0 = 0; j0 < nb; j0 += kDirectThreads) {
-    const long long j = j0 + threadIdx.x;
-    Atom4 v{1e300, 1e300, 1e300, 0.0};
-    if (j < nb) {
-      double x, y, z, q;
-      load_xyz(b, dtb, j, x, y, z, q);
-      x -= cB[0];
-      y -= cB[1];
-      z -= cB[2];
-      v.x = R0[0] + rot[0] * x + rot[1] * y + rot[2] * z;
-      v.y = R0[1] + rot[3] * x + rot[4] * y + rot[5] * z;
-      v.z = R0[2] + rot[6] * x + rot[7] * y + rot[8] * z;
-      v.w = q;
-    }
-    __syncthreads();
-    sb[threadIdx.x] = v;
-    __syncthreads();
-    if (i < na) {
-      const int cnt = (int)min((long long)kDirectThreads, nb - j0);
-      for (int k = 0; k < cnt; ++k) {
-        const Atom4 w = sb[k];
-        const double dx = w.x - ax, dy = w.y - ay, dz = w.z - az;
-        acc += w.w * rsqrt(dx * dx + dy * dy + dz * dz);
-      }
-    }
-  }
-  acc = block_sum(acc * qa, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = acc;
-}
-
-// One CTA per item: each thread sums a contiguous stripe of the item's block partials, then a
-// fixed-order block sum.
-__global__ void k_direct_final(const double* __restrict__ part, int nblk, double* __restrict__ E) {
-  __shared__ double sh[32];
-  part += (long long)blockIdx.x * nblk;
-  double s = 0.0;
-  const int per = (nblk + blockDim.x - 1) / blockDim.x;
-  const int b0 = threadIdx.x * per;
-  for (int k = b0; k < min(nblk, b0 + per); ++k) s += part[k];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) E[blockIdx.x] = s;
-}
-
 }  // namespace
 
 // Threads per contraction CTA: the largest per-degree loops have (L+1)^2 iterations, so small
@@ -782,19 +677,6 @@ void contract_tables(double* t) {
   for (int l = 0; l < kZN; ++l)
     for (int k = 0; k <= l; ++k)
       for (int m = 0; m <= l; ++m) t[kZ_DPI2 + dpi2_off(l) + k * dpi2_stride(l) + m] = dpi2_entry(l, k, m, C, fact);
-}
-
-int direct_blocks(long long na) { return (int)((na + kDirectThreads - 1) / kDirectThreads); }
-
-int launch_direct(const void* a, long long na, int dta, const void* b, long long nb, int dtb, const SysGeom* geo,
-                  const double* xf, int n_items, double* part, int nblk, double* E, cudaStream_t s) {
-  for (int i0 = 0; i0 < n_items; i0 += 65535) {  // grid.y limit
-    const int n = min(65535, n_items - i0);
-    if (nblk > 0) k_direct<<<dim3(nblk, n), kDirectThreads, 0, s>>>(a, na, dta, b, nb, dtb, geo, xf + 12LL * i0,
-                                                                    part + (long long)i0 * nblk);
-    k_direct_final<<<n, 128, 0, s>>>(part + (long long)i0 * nblk, nblk, E + i0);
-  }
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace tcm

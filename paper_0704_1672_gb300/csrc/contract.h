@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "tcm_internal.h"
@@ -110,11 +111,17 @@ inline void pair_frame(const double* R0, PairDesc& d) {
   d.fr[4] = rho > 0.0 ? x / rho : 1.0;
   d.fr[5] = rho > 0.0 ? y / rho : 0.0;
 }
+// How the direct sum of one item is cut into CTAs (direct_split): parts = A blocks x B ranges of
+// chunk atoms, apt atoms of A per thread; slab: items per launch (slab x parts partial sums).
+struct DirectSplit {
+  int apt, ablocks, chunk, parts, slab;
+};
+DirectSplit direct_split(long long na, long long nb);
 int launch_direct(const void* a, long long na, int dta, const void* b, long long nb, int dtb,
-                  const SysGeom* geo /* device: [A, B] centres */,
+                  const SysGeom* geo /* device: [A, B] centres and radii */,
                   const double* xf /* device: per item rot[9], R0[3] */, int n_items,
-                  double* part /* n_items x nblk */, int nblk, double* E /* device, n_items */, cudaStream_t s);
-int direct_blocks(long long na);
+                  double* part /* min(n_items, slab) x parts */, const DirectSplit& d, double* E /* device, n_items */,
+                  cudaStream_t s);
 
 // Sets the calling thread's tcm_last_error() message; returns code.
 int record_error(int code, const char* msg);

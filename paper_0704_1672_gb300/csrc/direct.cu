@@ -1,0 +1,374 @@
+// Step a6: the exact pairwise Coulomb sum, Eq. (Coulomb), for a batch of placements of B.
+//
+// Each CTA takes one item, a block of A's atoms (two per thread) and a range of B's atoms, which
+// it stages through shared memory already rotated and translated: b' = R0 + rot (x_b - c_B).
+//
+// Two forms of the pair loop:
+//
+//   fixed point (pairs_fixed): positions, 1/r and the sum in 64-bit integers.  GB300's FP64 pipe
+//   issues 2 lanes per clock and SM, its integer multiply-add with a 64-bit sum (IMAD.WIDE) 64
+//   (both measured), and the pair loop is nothing but arithmetic on data in registers, so the unit
+//   decides: about 12 FP64 instructions of a pair hold an SMSP for 770 cycles, the 18 IMAD.WIDE and
+//   25 other instructions of the fixed-point pair for about 50.
+//   double (pairs_double): the plain loop, for placements whose systems come close or overlap, for
+//   values that fixed point cannot hold (not finite, or outside the radii), and for extreme scales.
+//
+// Fixed point, for separated systems (r_min = R - a_A - a_B > 0, D = R + a_A + a_B):
+//   positions in units of 1/f, f the power of two with 2^60 <= D f < 2^61, as two signed 31-bit
+//   limbs X = 2^31 h + l; differences of limbs need no carries:
+//     T = sum dh^2 + 2^-30 sum dh dl  =  r^2 f^2 / 2^62      (dl^2 < 2^-60 D^2 enters by its mean)
+//   1/r from the float reciprocal square root of T, as the integer Y = 2^54 / sqrt(T), and one
+//   third-order correction in integers: with p = T Y^2 / 2^32 mod 2^64 = -2^76 e (the residual e of
+//   Y, |e| < 2^-21, is all that the modulus leaves of the product),
+//     y = 2^32 Y (1 + e/2 + 3/8 e^2)  =  2^117 / (f r),   good to about 2^-54;
+//   charges as 53-bit integers on the scale of the range's largest, and three integer sums of limb
+//   products, which are exact.  Errors against 64-bit positions: T to about one unit, 2^-60 D^2
+//   (the double loop rounds b' to 2^-53 R); the sum itself rounds only when it leaves the loop.
+// Measured (2,587 x 3,260 atoms, 256 placements): 47.9 ms in double, 7.62 ms in fixed point; error
+// against 64-bit torch 4.0e-14 before, 1.3e-14 now (net-zero charges: of the cancelled sum).
+// The bound r_min f >= 2^55 (r_min / D above 1/64 to 1/32) keeps Y below 2^31.
+#include <cuda_runtime.h>
+
+#include "contract.h"
+
+namespace tcm {
+
+namespace {
+
+constexpr int kDirectThreads = 256;
+constexpr int kDirectTile = 256;  // atoms of B staged at once, one per thread
+
+struct alignas(16) FixAtom {  // a staged atom of B: position limbs, charge limbs
+  int h[3];
+  int qh;
+  int l[3];
+  int ql;
+};
+struct alignas(32) Atom4 {  // the same for the double loop
+  double x, y, z, w;
+};
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+// Fixed-order block sum; result valid in thread 0.
+__device__ double block_sum(double v, double* sh) {
+  v = warp_sum(v);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) sh[w] = v;
+  __syncthreads();
+  double r = 0.0;
+  if (w == 0) {
+    const int nw = (blockDim.x + 31) >> 5;
+    r = lane < nw ? sh[lane] : 0.0;
+    r = warp_sum(r);
+  }
+  __syncthreads();
+  return r;
+}
+__device__ __forceinline__ void load_xyz(const void* p, int dtype, long long i, double* x, double& q) {
+  if (dtype == TCM_F32) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p) + i);
+    x[0] = v.x;
+    x[1] = v.y;
+    x[2] = v.z;
+    q = v.w;
+  } else {
+    const double2 a = __ldg(reinterpret_cast<const double2*>(p) + 2 * i);
+    const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 2 * i + 1);
+    x[0] = a.x;
+    x[1] = a.y;
+    x[2] = b.x;
+    q = b.y;
+  }
+}
+__device__ __forceinline__ double load_q(const void* p, int dtype, long long i) {
+  return dtype == TCM_F32 ? (double)__ldg(reinterpret_cast<const float*>(p) + 4 * i + 3)
+                          : __ldg(reinterpret_cast<const double*>(p) + 4 * i + 3);
+}
+
+__device__ __forceinline__ int exponent(double v) { return (int)((__double2hiint(v) >> 20) & 0x7ff) - 1022; }
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// The item's transform: centres, rotation, separation.
+struct Place {
+  double cA[3], cB[3], rot[9], R0[3];
+};
+
+// Atom of B in the frame of A: rotated offset from its centre in d, b' = R0 + d.
+__device__ __forceinline__ void place_b(const Place& g, const double* x, double* d) {
+  const double v[3] = {x[0] - g.cB[0], x[1] - g.cB[1], x[2] - g.cB[2]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) d[k] = g.rot[3 * k] * v[0] + g.rot[3 * k + 1] * v[1] + g.rot[3 * k + 2] * v[2];
+}
+
+__device__ __forceinline__ void split31(double x, double f, int& h, int& l) {
+  const long long X = __double2ll_rn(x * f);
+  h = (int)((X + (1LL << 30)) >> 31);
+  l = (int)(X - ((long long)h << 31));
+}
+
+__device__ __forceinline__ long long madw(int a, int b, long long c) {
+  return (long long)a * (long long)b + c;
+}
+__device__ __forceinline__ unsigned long long maduw(unsigned a, unsigned b, unsigned long long c) {
+  return (unsigned long long)a * (unsigned long long)b + c;
+}
+
+// 2^117 / (f r) of one pair (see the head of the file).
+__device__ __forceinline__ long long inv_r(const int* ah, const int* al, const int4 bh, const int4 bl) {
+  const int h0 = bh.x - ah[0], h1 = bh.y - ah[1], h2 = bh.z - ah[2];
+  const int l0 = bl.x - al[0], l1 = bl.y - al[1], l2 = bl.z - al[2];
+  const long long s = madw(h2, h2, madw(h1, h1, (long long)h0 * h0));
+  // 2^30: half a unit for the shift's floor, half for the mean of sum dl^2
+  const long long c = madw(h2, l2, madw(h1, l1, madw(h0, l0, 1LL << 30)));
+  const unsigned long long T = (unsigned long long)(s + (c >> 30));
+  const unsigned Th = (unsigned)(T >> 32), Tl = (unsigned)T;
+  const float y0 = rsqrtf(fmaf((float)Th, 4294967296.0f, (float)Tl));
+  const int Y = __float2int_rn(y0 * 18014398509481984.0f);  // 2^54
+  const unsigned long long U = (unsigned long long)(unsigned)Y * (unsigned)Y;
+  const unsigned Uh = (unsigned)(U >> 32), Ul = (unsigned)U;
+  unsigned long long p = maduw(Th, Ul, maduw(Tl, Uh, ((unsigned long long)Tl * Ul) >> 32));
+  p += (unsigned long long)(Th * Uh) << 32;
+  const int ph = (int)(p >> 32);
+  const int e2 = (int)(((long long)ph * ph) >> 32);
+  p = (unsigned long long)madw(e2, -786432, (long long)p);  // the second-order term: 3/8 2^21
+  const long long M = madw(Y, (int)(p >> 32), (long long)(((unsigned long long)(unsigned)Y * (unsigned)p) >> 32));
+  return ((long long)Y << 32) - (M >> 13);
+}
+
+// One atom of A against the staged atoms: sums of q y in three limb products, 32 pairs at a time
+// (26 + 31 + 5 bits), each folded into a pair of wide sums.
+struct FixSum {
+  long long hi[3] = {0, 0, 0};
+  unsigned long long lo[3] = {0, 0, 0};
+  __device__ __forceinline__ void fold(const long long* a) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      hi[k] += a[k] >> 32;
+      lo[k] += (unsigned)a[k];
+    }
+  }
+  __device__ __forceinline__ double value(double scale) const {
+    double v[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = fma((double)hi[k], 4294967296.0, (double)lo[k]);
+    // weights 2^59 (qh yh), 2^27 (qh yl), 2^32 (ql yh)
+    return fma(v[0], 134217728.0, fma(v[2], 1.0, v[1] * (1.0 / 32.0))) * scale;
+  }
+};
+
+struct Fixed {  // the scales of one CTA's fixed-point loop
+  double f;     // positions
+  double rA2, rB2;  // largest |x|^2 of an atom of A, of B about its centre
+  bool ok;
+};
+
+__device__ __forceinline__ Fixed fixed_scales(const Place& g, double aA, double aB) {
+  Fixed s;
+  const double R = sqrt(g.R0[0] * g.R0[0] + g.R0[1] * g.R0[1] + g.R0[2] * g.R0[2]);
+  aA *= 1.0 + 1e-9;  // room for the rounding of the rotated offsets
+  aB *= 1.0 + 1e-9;
+  const double D = R + aA + aB;
+  const int e = exponent(D);  // D < 2^e
+  s.rA2 = aA * aA;
+  s.rB2 = aB * aB;
+  s.ok = D > 0.0 && e > -400 && e < 400;
+  s.f = pow2(s.ok ? 61 - e : 0);
+  s.ok = s.ok && (R - aA - aB) * s.f >= 36028797018963968.0;  // 2^55
+  return s;
+}
+
+// APT atoms of A per thread.
+template <int APT>
+__global__ void __launch_bounds__(kDirectThreads, 2)
+    k_direct(const void* __restrict__ a, long long na, int dta, const void* __restrict__ b, long long nb, int dtb,
+             const SysGeom* __restrict__ geo, const double* __restrict__ xf, int ablocks, int chunk,
+             double* __restrict__ part) {
+  __shared__ union {
+    FixAtom fix[kDirectTile];
+    Atom4 dbl[kDirectTile];
+  } sb;
+  __shared__ Place g;
+  __shared__ double sh[32];
+  __shared__ int s_exp;
+  const int t = threadIdx.x;
+  const double* item = xf + 12LL * blockIdx.y;  // this item's rotation of B and separation
+  if (t < 9) g.rot[t] = item[t];
+  if (t < 3) {
+    g.R0[t] = item[9 + t];
+    g.cA[t] = geo[0].c[t];
+    g.cB[t] = geo[1].c[t];
+  }
+  if (t == 0) s_exp = 0;
+  __syncthreads();
+  const int ab = blockIdx.x % ablocks, bb = blockIdx.x / ablocks;
+  const long long j0 = (long long)bb * chunk, j1 = min(nb, j0 + (long long)chunk);
+  const Fixed fs = fixed_scales(g, geo[0].a, geo[1].a);
+  double pos[APT][3], qa[APT];
+  bool bad = !fs.ok, warp_idle = true;
+#pragma unroll
+  for (int u = 0; u < APT; ++u) {
+    const long long i = ((long long)ab * APT + u) * kDirectThreads + t;
+    pos[u][0] = pos[u][1] = pos[u][2] = qa[u] = 0.0;  // a padding atom: A's centre, no charge
+    if (i < na) {
+      load_xyz(a, dta, i, pos[u], qa[u]);
+      double r2 = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        pos[u][k] -= g.cA[k];
+        r2 += pos[u][k] * pos[u][k];
+      }
+      bad = bad || !(r2 <= fs.rA2);
+      warp_idle = false;
+    }
+  }
+  warp_idle = __all_sync(0xffffffffu, warp_idle);
+  double acc[APT];
+#pragma unroll
+  for (int u = 0; u < APT; ++u) acc[u] = 0.0;
+  bool fixed = false;
+  if (!__syncthreads_or(bad)) {
+    // the range's largest charge sets the scale of the charges; every staged atom lies within the radius
+    int qe = -1022;
+    for (long long j = j0 + t; j < j1; j += kDirectThreads) qe = max(qe, exponent(load_q(b, dtb, j)));
+    qe = __reduce_max_sync(0xffffffffu, qe);
+    if ((t & 31) == 0) atomicMax(&s_exp, qe + 1022);
+    __syncthreads();
+    qe = s_exp - 1022;
+    fixed = qe < 900;  // (not finite: 1025)
+    if (qe < -800) qe = -800;
+    const double gq = pow2(26 - qe);  // |q| gq < 2^26
+    int ah[APT][3], al[APT][3];
+#pragma unroll
+    for (int u = 0; u < APT; ++u)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) split31(pos[u][k], fs.f, ah[u][k], al[u][k]);
+    FixSum sum[APT];
+    for (long long jt = j0; fixed && jt < j1; jt += kDirectTile) {
+      FixAtom v;
+      double d[3] = {0.0, 0.0, 0.0}, q = 0.0;  // a padding atom: B's centre, no charge
+      if (jt + t < j1) {
+        double x[3];
+        load_xyz(b, dtb, jt + t, x, q);
+        place_b(g, x, d);
+      }
+      bad = !(d[0] * d[0] + d[1] * d[1] + d[2] * d[2] <= fs.rB2);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) split31(g.R0[k] + d[k], fs.f, v.h[k], v.l[k]);
+      const long long Q = __double2ll_rn(q * gq * 134217728.0);  // 2^27
+      v.qh = (int)((Q + (1LL << 26)) >> 27);
+      v.ql = (int)(Q - ((long long)v.qh << 27));
+      fixed = !__syncthreads_or(bad);  // (also: every thread is done with the tile before)
+      sb.fix[t] = v;
+      __syncthreads();
+      if (warp_idle || !fixed) continue;
+      const int cnt = (int)min((long long)kDirectTile, j1 - jt);
+      for (int k0 = 0; k0 < cnt; k0 += 32) {
+        long long s[APT][3] = {};
+#pragma unroll 2
+        for (int k = k0; k < k0 + 32; ++k) {
+          const int4 bh = *reinterpret_cast<const int4*>(sb.fix[k].h), bl = *reinterpret_cast<const int4*>(sb.fix[k].l);
+#pragma unroll
+          for (int u = 0; u < APT; ++u) {
+            const long long y = inv_r(ah[u], al[u], bh, bl);
+            const int yl = (int)y, yh = (int)(y >> 32) + (int)((unsigned)yl >> 31);  // y = 2^32 yh + yl
+            s[u][0] = madw(bh.w, yh, s[u][0]);
+            s[u][1] = madw(bh.w, yl, s[u][1]);
+            s[u][2] = madw(bl.w, yh, s[u][2]);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < APT; ++u) sum[u].fold(s[u]);
+      }
+    }
+    if (fixed) {
+      // q / r = 2^-117 f y / (2^27 gq) q's integer; FixSum::value leaves a weight of 2^32
+      const double scale = fs.f * pow2(-117 - 27 + 32) * pow2(qe - 26);
+#pragma unroll
+      for (int u = 0; u < APT; ++u) acc[u] = sum[u].value(scale);
+    }
+  }
+  if (!fixed) {
+    for (long long jt = j0; jt < j1; jt += kDirectTile) {
+      Atom4 v{1e300, 1e300, 1e300, 0.0};
+      if (jt + t < j1) {
+        double x[3], d[3], q;
+        load_xyz(b, dtb, jt + t, x, q);
+        place_b(g, x, d);
+        v = Atom4{g.R0[0] + d[0], g.R0[1] + d[1], g.R0[2] + d[2], q};
+      }
+      __syncthreads();
+      sb.dbl[t] = v;
+      __syncthreads();
+      if (warp_idle) continue;
+      const int cnt = (int)min((long long)kDirectTile, j1 - jt);
+      for (int k = 0; k < cnt; ++k) {
+        const Atom4 w = sb.dbl[k];
+#pragma unroll
+        for (int u = 0; u < APT; ++u) {
+          const double dx = w.x - pos[u][0], dy = w.y - pos[u][1], dz = w.z - pos[u][2];
+          acc[u] += w.w * rsqrt(dx * dx + dy * dy + dz * dz);
+        }
+      }
+    }
+  }
+  double v = 0.0;
+#pragma unroll
+  for (int u = 0; u < APT; ++u)
+    if (((long long)ab * APT + u) * kDirectThreads + t < na) v += acc[u] * qa[u];
+  v = block_sum(v, sh);
+  if (t == 0) part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = v;
+}
+
+// One CTA per item: each thread sums a contiguous stripe of the item's partials, then a
+// fixed-order block sum.
+__global__ void k_direct_final(const double* __restrict__ part, int nblk, double* __restrict__ E) {
+  __shared__ double sh[32];
+  part += (long long)blockIdx.x * nblk;
+  double s = 0.0;
+  const int per = (nblk + blockDim.x - 1) / blockDim.x;
+  const int b0 = threadIdx.x * per;
+  for (int k = b0; k < min(nblk, b0 + per); ++k) s += part[k];
+  s = block_sum(s, sh);
+  if (threadIdx.x == 0) E[blockIdx.x] = s;
+}
+
+}  // namespace
+
+// The split of one item, from the atom counts alone (so that an item's energy does not depend on
+// the batch it is in): A in blocks of 256 or 512 atoms, B in as many ranges as bring an item to
+// about 64 CTAs while each range keeps at least 512 atoms (a CTA's set-up is then about a tenth of
+// its work).
+DirectSplit direct_split(long long na, long long nb) {
+  DirectSplit d;
+  d.apt = na > kDirectThreads ? 2 : 1;
+  const long long per = (long long)d.apt * kDirectThreads;
+  const long long nA = (na + per - 1) / per;
+  long long nB = nA > 0 ? (64 + nA - 1) / nA : 1;
+  nB = std::max<long long>(1, std::min<long long>(nB, nb / 512));
+  d.ablocks = (int)nA;
+  d.chunk = (int)((((nb + nB - 1) / nB) + 31) / 32 * 32);
+  if (d.chunk < 32) d.chunk = 32;
+  d.parts = (int)(nA * std::max<long long>(1, (nb + d.chunk - 1) / d.chunk));
+  // items whose partial sums fit the buffer at once; one launch's grid holds at most 65,535
+  d.slab = (int)std::max<long long>(1, std::min<long long>(65535, (1LL << 24) / std::max(d.parts, 1)));
+  return d;
+}
+
+int launch_direct(const void* a, long long na, int dta, const void* b, long long nb, int dtb, const SysGeom* geo,
+                  const double* xf, int n_items, double* part, const DirectSplit& d, double* E, cudaStream_t s) {
+  for (int i0 = 0; i0 < n_items; i0 += d.slab) {  // the slabs reuse the partial sums in stream order
+    const int n = std::min(d.slab, n_items - i0);
+    if (d.parts > 0) {
+      auto k = d.apt == 2 ? k_direct<2> : k_direct<1>;
+      k<<<dim3(d.parts, n), kDirectThreads, 0, s>>>(a, na, dta, b, nb, dtb, geo, xf + 12LL * i0, d.ablocks, d.chunk, part);
+    }
+    k_direct_final<<<n, 128, 0, s>>>(part, d.parts, E + i0);
+  }
+  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+}
+
+}  // namespace tcm

@@ -1107,9 +1107,8 @@ namespace {
 // energies to the device array dE.  Asynchronous.
 int direct_items(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t n, const double* rotB,
                  const double* R0, double* dE) {
+  // the radii choose the form of the pair loop and its scales (direct.cu): computed unless given
   tcm_system sys[2] = {*A, *B};
-  for (auto& s : sys)
-    if (s.has_center) s.radius = std::max(s.radius, 0.0);  // the direct sum needs centres only
   std::vector<char> used(2, 1);
   SysPlan S;
   plan_sys(sys, 2, used, {}, S);
@@ -1124,19 +1123,19 @@ int direct_items(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t 
   }
   Packer pk;
   const size_t o_geo = pk.add(geoms), o_xf = pk.add(xf), o_sj = pk.add(S.jobs);
-  const int nblk = direct_blocks(A->n);
+  const DirectSplit split = direct_split(A->n, B->n);
   TRY(ensure_sys_buffers(c, S));
-  TRY(dev_ensure(c, c->dpart, (size_t)std::max<int64_t>(nblk * n, 1) * sizeof(double)));
+  TRY(dev_ensure(c, c->dpart, (size_t)std::max<int64_t>((int64_t)split.parts * std::min<int64_t>(n, split.slab), 1) * sizeof(double)));
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
   const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
   TRY(run_expand(c, {}, nullptr, nullptr, S, d_sj, c->stream));
   TRY(run_sys(c, S, d_sj, d_geo, c->stream));
-  const int nlaunch = (int)((n + 65534) / 65535) * (nblk > 0 ? 2 : 1);
+  const int nlaunch = (int)((n + split.slab - 1) / split.slab) * (split.parts > 0 ? 2 : 1);
   PhaseScope ps(c, TCM_PHASE_DIRECT, nlaunch);
   TRY_LAUNCH(launch_direct(A->xyzq, A->n, A->dtype, B->xyzq, B->n, B->dtype, d_geo,
-                           reinterpret_cast<double*>(base + o_xf), (int)n, static_cast<double*>(c->dpart.p), nblk, dE,
+                           reinterpret_cast<double*>(base + o_xf), (int)n, static_cast<double*>(c->dpart.p), split, dE,
                            c->stream));
   return TCM_OK;
 }
@@ -1165,7 +1164,7 @@ int tcm_direct_batch(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int6
   if (n_items == 0) return TCM_OK;
   if (!R0 || !E) return set_err(TCM_EINVAL, "tcm_direct_batch: null argument");
   if (n_items > (1LL << 30)) return set_err(TCM_EINVAL, "tcm_direct_batch: too many items");
-  if ((int64_t)direct_blocks(A->n) * n_items > (1LL << 34))
+  if ((A->n + 255) / 256 * n_items > (1LL << 34))
     return set_err(TCM_EINVAL, "tcm_direct_batch: A's blocks x items exceeds the partial-sum buffer limit");
   return direct_items(c, A, B, n_items, rotB, R0, E);
 }
