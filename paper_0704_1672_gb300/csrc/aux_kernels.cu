@@ -54,12 +54,32 @@ __device__ void low_degrees(const MomJob& job, const double* __restrict__ syspar
   job.out[k] = v;
 }
 
-// a3: one CTA per moment job.  Threads walk the (chunk, slot) entries of the job's partial
-// rows in memory order (coalesced), sum each over the job's tiles in tile order (double) and
-// write F_lm a'^l times the sum to the packed component the slot holds.  The map entry, its
-// factor F_lm and the partial rows do not depend on each other, so their loads overlap; a' is a
-// power of two, so a'^l is formed exactly from its exponent.
+// a3: one CTA per moment job, or gridDim.y CTAs per job with a block of its slots each.  The (chunk,
+// slot) entries of the job's partial rows are summed over the job's tiles in double in one order,
+// whichever the launch: groups of kSumGroup consecutive tiles in tile order, then the groups in
+// order.  F_lm a'^l times the sum goes to the packed component the slot holds; a' is a power of two,
+// so a'^l is formed exactly from its exponent.
+//
+// What bounds it: latency, and for batches of many jobs the read of the partial rows.  A CTA per job
+// has each thread walk the tiles of its slot (coalesced rows, a group's loads in flight together).
+// A few jobs of many tiles would leave all but a few SMs idle at that (one job of 98 tiles x 800
+// slots took 42 us): there kFinSlots slots go to a CTA whose threads take the groups in turn.
 constexpr int kFinalizeThreads = 512;
+constexpr int kSumGroup = 8;
+constexpr int kFinSlots = 64;
+constexpr int kFinLanes = kFinalizeThreads / kFinSlots;  // threads per slot of a split launch
+constexpr int kFinPass = 4 * kFinLanes;                  // groups summed between two barriers
+
+__device__ __forceinline__ double group_sum(const double* base, int row, int t0, int t1) {
+  double s = 0.0;
+  if (t1 - t0 == kSumGroup) {
+#pragma unroll
+    for (int t = 0; t < kSumGroup; ++t) s += __ldcg(base + (long long)(t0 + t) * row);
+  } else {
+    for (int t = t0; t < t1; ++t) s += __ldcg(base + (long long)t * row);
+  }
+  return s;
+}
 __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const MomJob* __restrict__ jobs,
                                                                const double* __restrict__ partials,
                                                                const SysGeom* __restrict__ geoms,
@@ -68,26 +88,47 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const MomJob* __r
                                                                const int* __restrict__ imap_off,
                                                                const double* __restrict__ syspart) {
   __shared__ double s_low[kLowSums];
+  __shared__ double s_grp[kFinPass][kFinSlots];
   pdl_trigger();  // the contraction may be scheduled; it waits for this grid before reading
   pdl_wait();     // the moment kernels' partial rows are complete
   const MomJob& job = jobs[blockIdx.x];
   const int L = job.L;
   const int tpc = job.tiles_per_chunk;
-  const int kmax = plan_kmax(job.plan), row = plan_row(job.plan);
+  const int kmax = plan_slots(job.plan, L), row = plan_row(job.plan);
   const int* off = imap_off + job.plan * (kLmaxMax + 2);
   const int o = off[L];
   const int nq = off[L + 1] - o;  // nch x kmax
   const double a = geoms[job.geom].a;
   int e = 0;  // a' = scale_radius(a) = 2^e
   if (a > 0.0) frexp(a, &e);
-  for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-    const int p = imap[o + q];
-    const double f = fmap[o + q];
+  const bool split = gridDim.y > 1;
+  const int per = split ? kFinSlots : kFinalizeThreads;
+  const int ngroup = (tpc + kSumGroup - 1) / kSumGroup;
+  for (int q0 = split ? blockIdx.y * kFinSlots : 0; q0 < nq; q0 += split ? gridDim.y * kFinSlots : kFinalizeThreads) {
+    const int q = q0 + threadIdx.x % per;
+    const bool in = q < nq;
+    const int p = in ? imap[o + q] : -1;
+    const double f = in ? fmap[o + q] : 0.0;
     const int ch = q / kmax, slot = q - ch * kmax;
     const double* base = partials + (long long)(job.tile_base + ch * tpc) * row + slot;
     double s = 0.0;
-#pragma unroll 8
-    for (int t = 0; t < tpc; ++t) s += __ldcg(base + (long long)t * row);  // loads issued ahead of the adds
+    if (!split) {
+      if (in)
+        for (int g = 0; g < ngroup; ++g) s += group_sum(base, row, g * kSumGroup, min(tpc, (g + 1) * kSumGroup));
+    } else {
+      const int k = threadIdx.x / kFinSlots;
+      for (int g0 = 0; g0 < ngroup; g0 += kFinPass) {
+        const int ng = min(kFinPass, ngroup - g0);
+        for (int g = k; in && g < ng; g += kFinLanes)
+          s_grp[g][threadIdx.x % kFinSlots] =
+              group_sum(base, row, (g0 + g) * kSumGroup, min(tpc, (g0 + g + 1) * kSumGroup));
+        __syncthreads();
+        if (k == 0 && in)
+          for (int g = 0; g < ng; ++g) s += s_grp[g][threadIdx.x];
+        __syncthreads();
+      }
+      if (k != 0) continue;
+    }
     if (p < 0) continue;
     int l = (int)sqrtf((float)p);
     while (l * l > p) --l;
@@ -97,6 +138,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const MomJob* __r
     if (job.low_tiles > 0 && p < kLowComps) continue;  // written from the low-degree sums below
     job.out[p] = f * al * s;
   }
+  if (blockIdx.y > 0) return;
   if (job.low_tiles > 0) low_degrees(job, syspart, s_low);
 }
 
@@ -616,12 +658,17 @@ int launch_rotate_moments(const RotDesc* sets, int n_sets, int Lmax_sets, const 
 }
 
 int launch_finalize(const MomJob* jobs, int n_jobs, const double* partials, const SysGeom* geoms, const int* imap,
-                    const double* fmap, const int* imap_off, const double* syspart, cudaStream_t s) {
+                    const double* fmap, const int* imap_off, const double* syspart, int n_split, cudaStream_t s) {
   if (n_jobs <= 0) return 0;
-  return launch_pdl(k_finalize, dim3(n_jobs), dim3(kFinalizeThreads), 0, s, jobs, partials, geoms, imap, fmap,
+  return launch_pdl(k_finalize, dim3(n_jobs, n_split), dim3(kFinalizeThreads), 0, s, jobs, partials, geoms, imap, fmap,
                     imap_off, syspart) == cudaSuccess
              ? 0
              : -1;
+}
+
+int finalize_split(int n_jobs, int max_tiles, int max_slots) {
+  if (n_jobs > 64 || max_tiles <= 2 * kSumGroup) return 1;  // enough CTAs, or little to sum
+  return (max_slots + kFinSlots - 1) / kFinSlots;
 }
 
 int launch_contract(const PairDesc* items, int n_items, int Lmax_items, const MomJob* jobs, const SysGeom* geoms,

@@ -1,34 +1,20 @@
-// Runtime dispatch from (precision, Lmax) to the explicitly instantiated moment kernels.
+// Runtime dispatch from the chunk plan to the moment kernels, and the tables of the plans.
 #include <cuda_runtime.h>
 
-#include <array>
 #include <cmath>
-#include <utility>
 #include <vector>
 
 #include "tcm_internal.h"
 
 namespace tcm {
 
-// Defined (and explicitly instantiated) in moments_kernel.cuh / moments_*.cu.
+// Defined (and explicitly instantiated) in moments_kernel.cuh / moments_f32_*.cu.
 template <typename T, int L, int KM>
 int launch_moments_t(const MomJob* jobs, const MomTile* tiles, int n_tiles, int* counter, const SysGeom* geoms,
                      double* partials, int grid, cudaStream_t s);
 
 namespace {
 
-using LaunchFn = int (*)(const MomJob*, const MomTile*, int, int*, const SysGeom*, double*, int, cudaStream_t);
-
-template <typename T, int... Ls>
-constexpr auto make_table(std::integer_sequence<int, Ls...>) {
-  return std::array<LaunchFn, sizeof...(Ls)>{{&launch_moments_t<T, Ls, kKmaxF64>...}};
-}
-
-const auto kF64 = make_table<double>(std::make_integer_sequence<int, kLmaxMax + 1>{});
-
-}  // namespace
-
-namespace {
 // The chunk plans, tabulated once (plan_nch and plan_m0 are loops meant for compile time; the
 // host planning of a batch asks for them per job and per group).
 struct ChunkTables {
@@ -90,21 +76,25 @@ void finalize_tables(std::vector<int>& imap_off, std::vector<int>& imap, std::ve
   imap_off.assign(kNumPlans * (N + 1), 0);
   imap.clear();
   for (int pi = 0; pi < kNumPlans; ++pi) {
-    const int kmax = plan_kmax(pi);
     for (int L = 0; L < N; ++L) {
-      const int nch = plan_nch(L, kmax);
+      const int nch = plan_nch(L, plan_kmax(pi));
+      const int slots = plan_slots(pi, L);
       const size_t base = imap.size();
       imap_off[pi * (N + 1) + L] = (int)base;
-      imap.resize(base + (size_t)nch * kmax, -1);
+      imap.resize(base + (size_t)nch * slots, -1);
       for (int ch = 0; ch < nch; ++ch) {
-        const int m0 = plan_m0(L, kmax, nch, ch), m1 = plan_m0(L, kmax, nch, ch + 1);
+        const int m0 = plan_m0(L, plan_kmax(pi), nch, ch), m1 = plan_m0(L, plan_kmax(pi), nch, ch + 1);
+        // slot of component (l, m): the double kernel keeps a column's (Re, Im) side by side
+        auto slot = [&](int l, int m, int part) {
+          return pi == 0 && m > 0 ? chunk_off(L, 0, m) + 2 * (l - m) + part : acc_slot(L, m0, m1, l, m, part);
+        };
         for (int m = m0; m < m1; ++m)
           for (int l = m; l <= L; ++l) {
             if (m == 0) {
-              imap[base + ch * kmax + acc_slot(L, m0, m1, l, 0, 0)] = l * l;
+              imap[base + ch * slots + slot(l, 0, 0)] = l * l;
             } else {
-              imap[base + ch * kmax + acc_slot(L, m0, m1, l, m, 0)] = l * l + 2 * m - 1;
-              imap[base + ch * kmax + acc_slot(L, m0, m1, l, m, 1)] = l * l + 2 * m;
+              imap[base + ch * slots + slot(l, m, 0)] = l * l + 2 * m - 1;
+              imap[base + ch * slots + slot(l, m, 1)] = l * l + 2 * m;
             }
           }
       }
@@ -127,7 +117,7 @@ int launch_moments(int plan, int L, const MomJob* jobs, const MomTile* tiles, in
   switch (plan) {  // the float kernels take tiles of any degree
     case 1: return launch_moments_t<float, -1, kKmaxF32>(jobs, tiles, n_tiles, counter, geoms, partials, grid, s);
     case 2: return launch_moments_t<float, -1, kKmaxF32Small>(jobs, tiles, n_tiles, counter, geoms, partials, grid, s);
-    case 0: return L < 0 || L > kLmaxMax ? -1 : kF64[L](jobs, tiles, n_tiles, counter, geoms, partials, grid, s);
+    case 0: return L < 0 || L > kLmaxMax ? -1 : launch_moments_f64(L, jobs, tiles, n_tiles, counter, geoms, partials, grid, s);
     default: return -1;
   }
 }

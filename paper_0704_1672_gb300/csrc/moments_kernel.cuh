@@ -1,7 +1,7 @@
-// Moment kernels, Eq. (multipole): persistent warps pull warp tiles (job, column chunk,
+// Float moment kernels, Eq. (multipole): persistent warps pull warp tiles (job, column chunk,
 // atom range); every lane keeps the chunk's accumulators in registers while it walks
-// its atoms, then the warp reduces them into one double-precision partial row per tile.  Included by the per-Lmax translation units, which instantiate
-// launch_moments_t<T, L> explicitly.
+// its atoms, then the warp reduces them into one double-precision partial row per tile.  Included by
+// the translation units that instantiate launch_moments_t.  (The double path: moments_f64.cu.)
 //
 // Per atom (after the per-tile transform M = rot / a', a' = scale_radius(a) a power of
 // two, and the split centre c = c_hi + c_lo):
@@ -27,17 +27,9 @@ struct MomTraits<float> {
   static constexpr int row = kKmaxF32;   // partial-row stride of every float plan
   static constexpr int stride = 36;  // row stride (floats) of the transpose buffer: 16-B rows, no LDS.128 conflicts
 };
-template <>
-struct MomTraits<double> {
-  static constexpr int kmax = kKmaxF64;
-  static constexpr int row = kKmaxF64;
-  static constexpr int stride = 34;  // doubles
-};
 
 __device__ __forceinline__ float fmaT(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fmaT(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float rsqrtT(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrtT(double x) { return rsqrt(x); }
 
 template <typename T, int L, int KM = MomTraits<T>::kmax>
 struct Plan {
@@ -56,26 +48,18 @@ struct Plan {
 };
 
 // Pairs: float2 in the float kernels, where the (Re, Im) halves of a complex step go
-// through one packed f32x2 instruction; double2 with scalar arithmetic in the double ones.
+// through one packed f32x2 instruction.
 template <typename T>
 struct Pair;
 template <>
 struct Pair<float> {
   using type = float2;
 };
-template <>
-struct Pair<double> {
-  using type = double2;
-};
 template <typename T>
 using P2 = typename Pair<T>::type;
 
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ double2 mul2(double2 a, double2 b) { return make_double2(a.x * b.x, a.y * b.y); }
-__device__ __forceinline__ double2 fma2(double2 a, double2 b, double2 c) {
-  return make_double2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
-}
 template <typename T>
 __device__ __forceinline__ P2<T> pair(T a, T b) {
   P2<T> r;
@@ -148,13 +132,10 @@ struct KPairs {
 static_assert(KPairs<float>().two[5][1].x != 0.0f && KPairs<float>().two[3][1].y == 1.0f,
               "the coefficient table must be a constant expression");
 static __constant__ KPairs<float> c_kpairs_f = KPairs<float>();
-static __constant__ KPairs<double> c_kpairs_d = KPairs<double>();
 template <typename T>
 __device__ __forceinline__ const KPairs<T>& kpairs();
 template <>
 __device__ __forceinline__ const KPairs<float>& kpairs<float>() { return c_kpairs_f; }
-template <>
-__device__ __forceinline__ const KPairs<double>& kpairs<double>() { return c_kpairs_d; }
 
 // Advance the running diagonal power (dr, di) = u^m to the next column.
 template <typename T, int L, int M0, int M1>
@@ -370,17 +351,6 @@ __device__ __forceinline__ double row_sum32(const float* p) {
       s[k] = t;
     }
   return (double)s[0] + (double)e[0];
-}
-
-__device__ __forceinline__ double row_sum32(const double* p) {
-  const double2* v = reinterpret_cast<const double2*>(p);
-  double s[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const double2 w0 = v[2 * k], w1 = v[2 * k + 1];
-    s[k] = (w0.x + w0.y) + (w1.x + w1.y);
-  }
-  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 }
 
 // Warp reduction of the per-lane accumulators into one double row `out[0..NACC)` (the

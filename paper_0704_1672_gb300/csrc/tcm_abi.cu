@@ -117,6 +117,7 @@ struct tcm_ctx {
   // resident CTAs per SM the persistent grid is sized for
   int atoms_per_thread[2][kLmaxMax + 1];
   int ctas_per_sm[2][kLmaxMax + 1];
+  bool tiling_set[kLmaxMax + 1] = {};  // TCM_FP64: atoms per lane were set (else smaller tiles for small systems)
   int plan_l[kLmaxMax + 1];  // mixed path: the float kernel's chunk plan per degree (1 or 2)
   int64_t cfg_gen = 0;       // bumped by every tiling or chunking change (part of the graph key)
   // phase profiling
@@ -258,7 +259,9 @@ struct Plan {
 void plan_job(tcm_ctx* c, int precision, MomJob& j, int& next_id) {
   j.plan = precision == TCM_FP64 ? 0 : c->plan_l[j.L];
   const int nch = moments_nchunks(j.plan, j.L);
-  const long long per_tile = 32LL * c->atoms_per_thread[precision == TCM_FP64 ? 0 : 1][j.L];  // one warp
+  long long apl = c->atoms_per_thread[precision == TCM_FP64 ? 0 : 1][j.L];
+  if (precision == TCM_FP64 && !c->tiling_set[j.L]) apl = std::min<long long>(apl, f64_rows(j.n));
+  const long long per_tile = 32 * apl;
   long long tpc = (j.n + per_tile - 1) / per_tile;
   if (tpc < 1) tpc = 1;
   j.tiles_per_chunk = (int)tpc;
@@ -338,6 +341,16 @@ int moment_launches(int precision, const Plan& P) {
   return n;
 }
 
+// CTAs per job of the finalisation.
+int split_of(const Plan& P) {
+  int max_tiles = 0, max_slots = 0;
+  for (const MomJob& j : P.jobs) {
+    max_tiles = std::max(max_tiles, j.tiles_per_chunk);
+    max_slots = std::max(max_slots, moments_nchunks(j.plan, j.L) * plan_slots(j.plan, j.L));
+  }
+  return finalize_split((int)P.jobs.size(), max_tiles, max_slots);
+}
+
 // Queue the moment pass (step a2/a3) for every job of the plan.
 // The moment kernels' work counters and exit tickets (counters[L], counters[32 + L]) are zero
 // on entry and left zero by every launch, so they are cleared once, when allocated.
@@ -371,8 +384,7 @@ int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, 
     for (int L = 0; L <= kLmaxMax; ++L) {
       const int b = P.tile_begin[L], e = P.tile_begin[L + 1];
       if (e == b) continue;
-      const int cps = c->ctas_per_sm[0][L];
-      const int grid = std::min((e - b + kThreads / 32 - 1) / (kThreads / 32), cps * c->num_sms);  // warp tiles
+      const int grid = std::min(e - b, c->ctas_per_sm[0][L] * c->num_sms);  // a CTA per tile
       TRY_LAUNCH(launch_moments(0, L, d_jobs, tiles + b, e - b, counters + L, d_geoms, parts, grid, st));
     }
   } else if (P.n_tiles > 0) {
@@ -392,7 +404,7 @@ int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, 
   {
     PhaseScope ps(c, TCM_PHASE_FINALIZE, 1);
     TRY_LAUNCH(launch_finalize(d_jobs, (int)P.jobs.size(), parts, d_geoms, c->d_imap, c->d_fmap, c->d_imap_off,
-                               static_cast<double*>(c->gpart.p), st));
+                               static_cast<double*>(c->gpart.p), split_of(P), st));
   }
   return TCM_OK;
 }
@@ -618,7 +630,10 @@ int tcm_ctx_set_tiling(tcm_ctx_t c, int precision, int atoms_per_lane) {
   if (precision != TCM_FP64 && precision != TCM_MIXED) return set_err(TCM_EINVAL, "tcm_ctx_set_tiling: bad precision");
   if (atoms_per_lane < 1 || atoms_per_lane > 4096)
     return set_err(TCM_EINVAL, "tcm_ctx_set_tiling: atoms_per_lane outside [1, 4096]");
-  for (int L = 0; L <= kLmaxMax; ++L) c->atoms_per_thread[precision == TCM_FP64 ? 0 : 1][L] = atoms_per_lane;
+  for (int L = 0; L <= kLmaxMax; ++L) {
+    c->atoms_per_thread[precision == TCM_FP64 ? 0 : 1][L] = atoms_per_lane;
+    if (precision == TCM_FP64) c->tiling_set[L] = true;
+  }
   ++c->cfg_gen;
   return TCM_OK;
 }
@@ -634,6 +649,7 @@ int tcm_ctx_set_tiling_l(tcm_ctx_t c, int precision, int lmax, int atoms_per_lan
     return set_err(TCM_EINVAL, "tcm_ctx_set_tiling_l: ctas_per_sm outside [1, %d]", cmax);
   c->atoms_per_thread[precision == TCM_FP64 ? 0 : 1][lmax] = atoms_per_lane;
   c->ctas_per_sm[precision == TCM_FP64 ? 0 : 1][lmax] = ctas_per_sm;
+  if (precision == TCM_FP64) c->tiling_set[lmax] = true;
   ++c->cfg_gen;
   return TCM_OK;
 }
@@ -1049,7 +1065,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   if (!c->graphs || c->prof || !c->cap_stream) return enqueue(c->stream);
   // Replay a captured graph of the launch sequence when this call has the same shape and
   // buffers as the captured one (only the uploaded descriptor contents differ).
-  std::vector<long long> key = {precision, G != nullptr, (long long)(uintptr_t)G, (long long)S.jobs.size(),
+  std::vector<long long> key = {precision, split_of(P), G != nullptr, (long long)(uintptr_t)G, (long long)S.jobs.size(),
                                 (long long)S.n1, (long long)S.n2, (long long)P.jobs.size(), P.n_tile_ids,
                                 (long long)n_items, Lmax_items, (long long)o_geo, (long long)o_job, (long long)o_tile,
                                 (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)(uintptr_t)c->systiles.p,

@@ -29,32 +29,31 @@ namespace tcm {
 constexpr int kLmaxMax = TCM_LMAX_MAX;
 constexpr int kThreads = 128;  // threads per moment CTA (4 warps)
 
-// Accumulator budget per thread for the float and double moment kernels, and the CTAs
-// per SM the moment kernels are compiled for (register limit 65536 / (128 x CTAs)).
+// Accumulator budget per thread of the float moment kernel, and the CTAs per SM it is compiled
+// for (register limit 65536 / (128 x CTAs)).
 #ifndef TCM_KMAX_F32
 #define TCM_KMAX_F32 160
-#endif
-#ifndef TCM_KMAX_F64
-#define TCM_KMAX_F64 80
 #endif
 #ifndef TCM_MOMENT_CTAS_PER_SM
 #define TCM_MOMENT_CTAS_PER_SM 2
 #endif
 constexpr int kKmaxF32 = TCM_KMAX_F32;
-constexpr int kKmaxF64 = TCM_KMAX_F64;
+constexpr int kRowF64 = (kLmaxMax + 1) * (kLmaxMax + 1);  // partial row of the double kernel: every component
 
 // Chunk plans ("plans" below): the split of the (L+1)^2 accumulators of degree L into column
-// chunks of at most kmax.  Plan 0 is the double kernels' (kmax = kKmaxF64); the float kernel is
-// built for two budgets, plan 1 (kKmaxF32 accumulators per lane, 2 CTAs per SM) and plan 2
+// chunks of at most kmax.  Plan 0 is the double kernel's (one chunk: it keeps every component of a
+// tile); the float kernel is built for two budgets, plan 1 (kKmaxF32 accumulators per lane, 2 CTAs per SM) and plan 2
 // (kKmaxF32Small, fewer accumulators and registers, 3 CTAs per SM), chosen per degree
 // (tcm_ctx_set_chunking_l, the autotuner).  Partial rows keep the largest budget's stride in
 // every plan.
 constexpr int kKmaxF32Small = 96;
 constexpr int kNumPlans = 3;
 __host__ __device__ constexpr int plan_kmax(int plan) {
-  return plan == 0 ? kKmaxF64 : (plan == 1 ? kKmaxF32 : kKmaxF32Small);
+  return plan == 0 ? kRowF64 : (plan == 1 ? kKmaxF32 : kKmaxF32Small);
 }
-__host__ __device__ constexpr int plan_row(int plan) { return plan == 0 ? kKmaxF64 : kKmaxF32; }
+__host__ __device__ constexpr int plan_row(int plan) { return plan == 0 ? kRowF64 : kKmaxF32; }
+// Slots of one chunk's partial row that degree L uses under a plan (the last chunk's may be fewer).
+__host__ __device__ constexpr int plan_slots(int plan, int L) { return plan == 0 ? (L + 1) * (L + 1) : plan_kmax(plan); }
 // CTAs per SM a float moment kernel of budget kmax is compiled for (its register limit).
 __host__ __device__ constexpr int moment_ctas(int kmax) { return kmax <= kKmaxF32Small ? 3 : TCM_MOMENT_CTAS_PER_SM; }
 
@@ -250,7 +249,7 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 // ---------------------------------------------------------------------------------
 // Launchers (defined in the .cu files).
 
-// Moment kernels: one persistent launch over `n_tiles` tiles.  plan 0 (double kernels): every
+// Moment kernels: one persistent launch over `n_tiles` tiles.  plan 0 (double kernel): every
 // tile has degree L; plans 1 and 2 (float kernels): tiles of any degree whose jobs have that
 // plan (each tile runs the code of its job's degree); the tiles are taken in array order.
 // counter[0] and counter[32] must be zero on entry; the launch leaves them zero.
@@ -262,6 +261,15 @@ int launch_moments(int plan, int L, const MomJob* jobs, const MomTile* tiles, in
 // (job, t), t < sj.n_tiles.  One warp per group or system job.
 int launch_expand_tiles(const MomGroup* groups, int n_groups, const MomJob* jobs, MomTile* tiles, const SysJob* sjobs,
                         int n_sjobs, SysTile* t1, SysTile* t2, cudaStream_t s);
+int launch_moments_f64(int L, const MomJob* jobs, const MomTile* tiles, int n_tiles, int* counter, const SysGeom* geoms,
+                       double* partials, int grid, cudaStream_t s);
+// Rows of 32 atoms in a tile of the double kernel for a system of n atoms (before the tiling
+// setting's limit): about 304 tiles (two per SM), so that one system fills the GPU; at 100,003 atoms
+// and degree 24 285 tiles of 11 rows.
+inline int f64_rows(long long n) {
+  const long long r = (n + 32 * 304 - 1) / (32 * 304);
+  return (int)(r < 1 ? 1 : (r > 4096 ? 4096 : r));
+}
 int moments_nchunks(int plan, int L);
 int moments_chunk_m0(int plan, int L, int chunk);  // first column of a chunk (chunk = nch: L + 1)
 const double* moments_chunk_costs(int plan, int L);  // relative cost per atom of each chunk
@@ -277,15 +285,17 @@ int launch_sys(const SysJob* jobs, const SysTile* t1, int n1, const SysTile* t2,
                SysGeom* geoms, cudaStream_t s);
 int sys_launches(int n1, int n2);
 int sys_tile_atoms(long long n);
-// Step a3: one CTA per job.  imap + imap_off[plan (kLmaxMax + 2) + L] lists, per (chunk, slot) of
-// degree L under the job's plan, the packed component it holds (-1 for none), nch x
-// plan_kmax(plan) entries; fmap beside it holds that component's F_lm with the sign of the
+// Step a3: one CTA per job, or n_split CTAs over the job's slots.  imap + imap_off[plan (kLmaxMax + 2)
+// + L] lists, per (chunk, slot) of degree L under the job's plan, the packed component it holds (-1
+// for none), nch x plan_slots(plan, L) entries; fmap beside it holds that component's F_lm with the sign of the
 // kernels' H variables.  Partial rows are plan_row(plan) doubles apart.
 // Jobs with low_tiles != 0 take their degrees l <= min(kLowLmax, L) from the low-degree sums of
 // their system (row low_base of the system-pass partials syspart) rotated by the job's rotation.
 int launch_finalize(const MomJob* jobs, int n_jobs, const double* partials, const SysGeom* geoms,
-                    const int* imap, const double* fmap, const int* imap_off, const double* syspart,
+                    const int* imap, const double* fmap, const int* imap_off, const double* syspart, int n_split,
                     cudaStream_t s);
+// The split for n_jobs jobs of at most max_tiles tiles per chunk and max_slots (chunk, slot) entries.
+int finalize_split(int n_jobs, int max_tiles, int max_slots);
 
 
 

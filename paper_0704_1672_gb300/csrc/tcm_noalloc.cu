@@ -28,10 +28,12 @@ using namespace tcm;
 namespace {
 
 constexpr long long kNaMaxAtoms = TCM_NOALLOC_MAX_ATOMS;
-constexpr int kNaTileAtoms = 4096;                                   // atoms per tile, both precisions
+constexpr int kNaTileAtoms = 4096;                                   // atoms per tile, mixed path
 constexpr int kNaTilesPerChunk = (int)(kNaMaxAtoms / kNaTileAtoms);  // 64
-constexpr int kNaMaxChunks = 10;                                     // most chunks of any (precision, Lmax)
-constexpr int kNaPartialDoubles = kNaTilesPerChunk * 800;            // max over plans of chunks * kmax = 800
+constexpr int kNaMaxChunks = 10;                                     // rows of the tile list per 4,096 atoms
+constexpr int kNaPartialDoubles = 63840;                             // mixed: 64 tiles x 5 chunks x 160 slots
+constexpr int kNaTilesF64 = kNaPartialDoubles / kRowF64;             // double: 102 tiles of 625 components
+static_assert(kNaTilesPerChunk * 800 <= kNaPartialDoubles, "the mixed path's rows must fit");
 constexpr int kNaMaxTiles = kNaTilesPerChunk * kNaMaxChunks;
 // system-pass rows: sys_tile_atoms gives at most 128 tiles up to 65,536 atoms and 1,024-atom tiles
 // above (256 for the largest request), plus the sum row
@@ -49,7 +51,7 @@ constexpr size_t kOffSTiles1 = align256(kOffSJob + sizeof(SysJob));
 constexpr size_t kOffSTiles2 = align256(kOffSTiles1 + sizeof(SysTile) * kNaSysTiles);
 constexpr size_t kOffSPart = align256(kOffSTiles2 + sizeof(SysTile) * kNaSysTiles);
 constexpr size_t kOffCounters = align256(kOffSPart + sizeof(double) * kSysPart * kNaSysTiles);
-constexpr int kNaImapInts = 4 * kNaCompTotal;  // room for the (chunk, slot) maps of plans 0 and 1
+constexpr int kNaImapInts = kNaCompTotal + 8160;  // the (chunk, slot) maps of plans 0 and 1
 constexpr size_t kOffImapOff = align256(kOffCounters + sizeof(int) * 64);
 constexpr size_t kOffImap = align256(kOffImapOff + sizeof(int) * 2 * (kLmaxMax + 2));
 constexpr size_t kOffFmap = align256(kOffImap + sizeof(int) * kNaImapInts);
@@ -140,10 +142,13 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
   const int plan = precision == TCM_FP64 ? 0 : 1;
-  const int kmax = plan_kmax(plan);
   const int nch = moments_nchunks(plan, lmax);
-  const int tpc = (int)std::max<long long>(1, (s->n + kNaTileAtoms - 1) / kNaTileAtoms);
-  if (nch > kNaMaxChunks || nch * kmax > 800 || tpc > kNaTilesPerChunk)
+  // double: the tiles of tcm_moments, as far as the partial rows go
+  const long long tile_atoms =
+      plan == 0 ? 32LL * std::max<long long>(f64_rows(s->n), (s->n + 32 * kNaTilesF64 - 1) / (32 * kNaTilesF64))
+                : kNaTileAtoms;
+  const int tpc = (int)std::max<long long>(1, (s->n + tile_atoms - 1) / tile_atoms);
+  if (nch * tpc > kNaMaxTiles || (long long)nch * tpc * plan_row(plan) > kNaPartialDoubles)
     return na_err(TCM_EINVAL, "tcm_moments_noalloc: request exceeds the fixed scratch");
   MomJob job{};
   job.xyzq = s->xyzq;
@@ -202,12 +207,13 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   const int n_tiles = nch * tpc;
   if (launch_moments(plan, lmax, d_job, reinterpret_cast<MomTile*>(base + kOffTiles), n_tiles,
                      reinterpret_cast<int*>(base + kOffCounters), d_geom, reinterpret_cast<double*>(base + kOffPartials),
-                     std::min((n_tiles + kThreads / 32 - 1) / (kThreads / 32), 2 * num_sms), st) != 0)
+                     std::min(plan == 0 ? n_tiles : (n_tiles + kThreads / 32 - 1) / (kThreads / 32), 2 * num_sms),
+                     st) != 0)
     return na_err(TCM_ECUDA, "tcm_moments_noalloc: moment launch failed");
   if (launch_finalize(d_job, 1, reinterpret_cast<double*>(base + kOffPartials), d_geom,
                       reinterpret_cast<int*>(base + kOffImap), reinterpret_cast<double*>(base + kOffFmap),
                       reinterpret_cast<int*>(base + kOffImapOff), reinterpret_cast<double*>(base + kOffSPart),
-                      st) != 0)
+                      finalize_split(1, tpc, nch * plan_slots(plan, lmax)), st) != 0)
     return na_err(TCM_ECUDA, "tcm_moments_noalloc: finalisation launch failed");
   if (geom_out && cudaMemcpyAsync(geom_out, d_geom, 4 * sizeof(double), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return na_err(TCM_ECUDA, "tcm_moments_noalloc: copy of the centre and radius failed");
