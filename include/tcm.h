@@ -246,6 +246,9 @@ int tcm_ctx_set_rotate_cached(tcm_ctx_t ctx, int enable);
  *   status: device, n_items int32 (TCM_OK or TCM_ENOTCONV), or NULL
  * Systems that carry a moment cache (tcm_system.moments) reuse it for their unrotated sides
  * (and for rotated sides too under tcm_ctx_set_rotate_cached).
+ * TCM_FP64: a rotated side whose rotB is a rotation to rounding takes B's moments from its
+ * lab-frame set (computed from the atoms once per system and lmax) rotated in the contraction;
+ * any other matrix acts on B's atoms.
  * Returns TCM_ENOTCONV at once if a host-known radius already violates Eq. (mainCond).
  * Asynchronous; results are ready when the context stream reaches this point.
  * Each item's result does not depend on the other items in the batch. */

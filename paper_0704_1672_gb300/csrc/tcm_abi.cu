@@ -512,6 +512,18 @@ void identity(double* r) {
   for (int k = 0; k < 9; ++k) r[k] = (k % 4 == 0) ? 1.0 : 0.0;
 }
 
+// Whether rot is a proper rotation to the rounding of a double: |R^T R - I| <= 3e-15 in every entry
+// (matrices built from unit quaternions in double are within 1.6e-15, products of two within 2e-15)
+// and det R > 0.
+bool is_rotation(const double* R) {
+  for (int i = 0; i < 3; ++i)
+    for (int j = i; j < 3; ++j) {
+      const double d = R[i] * R[j] + R[3 + i] * R[3 + j] + R[6 + i] * R[6 + j] - (i == j ? 1.0 : 0.0);
+      if (!(std::fabs(d) <= 3e-15)) return false;
+    }
+  return R[0] * (R[4] * R[8] - R[5] * R[7]) - R[1] * (R[3] * R[8] - R[5] * R[6]) + R[2] * (R[3] * R[7] - R[4] * R[6]) > 0.0;
+}
+
 // Host tables --------------------------------------------------------------------
 
 int build_tables(tcm_ctx* c) {
@@ -951,8 +963,8 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   std::vector<size_t> job_moff;
   std::vector<MomJob> cached;  // unrotated sides served from a system's moment cache
   std::map<int, int> cached_of;
-  auto get_job = [&](int sys, int L, int rot_item, const double* rot) {
-    if (rot_item < 0 && systems[sys].moments && L <= systems[sys].moments_lmax) {
+  auto get_job = [&](int sys, int L, int rot_item, const double* rot, bool use_cache = true) {
+    if (rot_item < 0 && use_cache && systems[sys].moments && L <= systems[sys].moments_lmax) {
       auto c = cached_of.find(sys);
       if (c != cached_of.end()) return -2 - c->second;
       MomJob j{};
@@ -991,11 +1003,21 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     const tcm_pair_item& it = items[k];
     const int ja = get_job(it.a, it.lmax, -1, nullptr);
     int jb;
-    if (it.has_rot && c->rotate_cached && systems[it.b].moments && it.lmax <= systems[it.b].moments_lmax) {
-      // B's cached lab-frame moments, taken into the frame by W rotB inside the contraction
+    // B's lab-frame moments, taken into the frame by W rotB inside the contraction:
+    //   from_cache  the caller asked for it and B carries its moments;
+    //   from_lab    double path: computed once per (system, degree) from B's atoms and shared by all
+    //               items and by unrotated sides.  The moments of a rotated system are those of the
+    //               system, rotated degree by degree (exact; O(L^3) double operations against
+    //               O(atoms L^2)): 256 orientations of 20,000 atoms at degree 20 take 0.2 ms instead of
+    //               13 ms, at the same error.  Only for matrices that are rotations to rounding; any
+    //               other matrix acts on the atoms, as before.  The mixed path keeps each item's own
+    //               float sums over the rotated atoms, whose rounding errors are independent.
+    const bool from_cache = c->rotate_cached && systems[it.b].moments && it.lmax <= systems[it.b].moments_lmax;
+    const bool from_lab = precision == TCM_FP64 && it.has_rot && is_rotation(it.rotB);
+    if (it.has_rot && (from_cache || from_lab)) {
       double W[9];
       frame_rotation(it.R0, W);
-      jb = get_job(it.b, it.lmax, -1, nullptr);
+      jb = get_job(it.b, it.lmax, -1, nullptr, from_cache);
       pd[k] = PairDesc{ja, jb, it.a, it.b, it.lmax, kBRotate, (long long)rots.size(), {}};
       pair_frame(it.R0, pd[k]);
       double M[9];
