@@ -112,9 +112,9 @@ inline void pair_frame(const double* R0, PairDesc& d) {
   d.fr[5] = rho > 0.0 ? y / rho : 0.0;
 }
 // How the direct sum of one item is cut into CTAs (direct_split): parts = A blocks x B ranges of
-// chunk atoms, apt atoms of A per thread; slab: items per launch (slab x parts partial sums).
+// chunk atoms; slab: items per launch (slab x parts partial sums).
 struct DirectSplit {
-  int apt, ablocks, chunk, parts, slab;
+  int ablocks, chunk, parts, slab;
 };
 DirectSplit direct_split(long long na, long long nb);
 int launch_direct(const void* a, long long na, int dta, const void* b, long long nb, int dtb,

@@ -1,16 +1,15 @@
 // Step a6: the exact pairwise Coulomb sum, Eq. (Coulomb), for a batch of placements of B.
 //
-// Each CTA takes one item, a block of A's atoms (two per thread) and a range of B's atoms, which
+// Each CTA takes one item, a block of A's atoms (one per thread) and a range of B's atoms, which
 // it stages through shared memory already rotated and translated: b' = R0 + rot (x_b - c_B).
 //
 // Two forms of the pair loop:
 //
-//   fixed point (pairs_fixed): positions, 1/r and the sum in 64-bit integers.  GB300's FP64 pipe
-//   issues 2 lanes per clock and SM, its integer multiply-add with a 64-bit sum (IMAD.WIDE) 64
-//   (both measured), and the pair loop is nothing but arithmetic on data in registers, so the unit
-//   decides: about 12 FP64 instructions of a pair hold an SMSP for 770 cycles, the 18 IMAD.WIDE and
-//   25 other instructions of the fixed-point pair for about 50.
-//   double (pairs_double): the plain loop, for placements whose systems come close or overlap, for
+//   fixed point: positions, 1/r and the sum in 64-bit integers.  The FP64 pipe takes 2 lanes per
+//   clock and SM, the integer multiply-add with a 64-bit sum (IMAD.WIDE) 32 to 64, and the pair loop is
+//   nothing but arithmetic on registers: 12 FP64 instructions of a pair held an SMSP for 770 cycles; the
+//   57 instructions of the fixed-point pair (13 IMAD.WIDE) take it 109, the integer multiplier 0.8 busy.
+//   double: the plain loop, for placements whose systems come close or overlap, for
 //   values that fixed point cannot hold (not finite, or outside the radii), and for extreme scales.
 //
 // Fixed point, for separated systems (r_min = R - a_A - a_B > 0, D = R + a_A + a_B):
@@ -18,14 +17,16 @@
 //   limbs X = 2^31 h + l; differences of limbs need no carries:
 //     T = sum dh^2 + 2^-30 sum dh dl  =  r^2 f^2 / 2^62      (dl^2 < 2^-60 D^2 enters by its mean)
 //   1/r from the float reciprocal square root of T, as the integer Y = 2^54 / sqrt(T), and one
-//   third-order correction in integers: with p = T Y^2 / 2^32 mod 2^64 = -2^76 e (the residual e of
-//   Y, |e| < 2^-21, is all that the modulus leaves of the product),
+//   third-order correction: with p = T Y^2 / 2^32 mod 2^64 = -2^76 e (the residual e of
+//   Y, |e| < 2^-21.1 from the bounds of rsqrt.approx and the roundings of its argument and of Y, is all that the modulus leaves of the product),
 //     y = 2^32 Y (1 + e/2 + 3/8 e^2)  =  2^117 / (f r),   good to about 2^-54;
 //   charges as 53-bit integers on the scale of the range's largest, and three integer sums of limb
 //   products, which are exact.  Errors against 64-bit positions: T to about one unit, 2^-60 D^2
 //   (the double loop rounds b' to 2^-53 R); the sum itself rounds only when it leaves the loop.
-// Measured (2,587 x 3,260 atoms, 256 placements): 47.9 ms in double, 7.62 ms in fixed point; error
-// against 64-bit torch 4.0e-14 before, 1.3e-14 now (net-zero charges: of the cancelled sum).
+// Measured (2,587 x 3,260 atoms, 256 placements): 47.9 ms in double, 5.37 ms in fixed point; error
+// against 64-bit torch 4.0e-14 before, 1.3e-14 now (net-zero charges: of the cancelled sum).  Two atoms
+// of A per thread were slower (116 cycles a pair at 128 registers); so were the same steps left to the
+// compiler as 64-bit expressions (125: it spends the multiplier on register moves).
 // The bound r_min f >= 2^55 (r_min / D above 1/64 to 1/32) keeps Y below 2^31.
 #include <cuda_runtime.h>
 
@@ -113,30 +114,42 @@ __device__ __forceinline__ void split31(double x, double f, int& h, int& l) {
 __device__ __forceinline__ long long madw(int a, int b, long long c) {
   return (long long)a * (long long)b + c;
 }
-__device__ __forceinline__ unsigned long long maduw(unsigned a, unsigned b, unsigned long long c) {
-  return (unsigned long long)a * (unsigned long long)b + c;
-}
-
 // 2^117 / (f r) of one pair (see the head of the file).
-__device__ __forceinline__ long long inv_r(const int* ah, const int* al, const int4 bh, const int4 bl) {
+__device__ __forceinline__ int2 inv_r(const int* ah, const int* al, const int4 bh, const int4 bl) {
   const int h0 = bh.x - ah[0], h1 = bh.y - ah[1], h2 = bh.z - ah[2];
   const int l0 = bl.x - al[0], l1 = bl.y - al[1], l2 = bl.z - al[2];
   const long long s = madw(h2, h2, madw(h1, h1, (long long)h0 * h0));
   // 2^30: half a unit for the shift's floor, half for the mean of sum dl^2
   const long long c = madw(h2, l2, madw(h1, l1, madw(h0, l0, 1LL << 30)));
-  const unsigned long long T = (unsigned long long)(s + (c >> 30));
-  const unsigned Th = (unsigned)(T >> 32), Tl = (unsigned)T;
-  const float y0 = rsqrtf(fmaf((float)Th, 4294967296.0f, (float)Tl));
+  unsigned Th, Tl;  // T = s + (c >> 30)
+  asm("{ .reg .u32 a, b, x, y;\n\t"
+      "mov.b64 {a, b}, %2;\n\tmov.b64 {x, y}, %3;\n\t"
+      "shf.r.wrap.b32 x, x, y, 30;\n\tshr.s32 y, y, 30;\n\t"
+      "add.cc.u32 %0, a, x;\n\taddc.u32 %1, b, y; }"
+      : "=r"(Tl), "=r"(Th)
+      : "l"(s), "l"(c));
+  float y0;  // within 2^-22.9
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(fmaf((float)Th, 4294967296.0f, (float)Tl)));
   const int Y = __float2int_rn(y0 * 18014398509481984.0f);  // 2^54
   const unsigned long long U = (unsigned long long)(unsigned)Y * (unsigned)Y;
   const unsigned Uh = (unsigned)(U >> 32), Ul = (unsigned)U;
-  unsigned long long p = maduw(Th, Ul, maduw(Tl, Uh, ((unsigned long long)Tl * Ul) >> 32));
-  p += (unsigned long long)(Th * Uh) << 32;
-  const int ph = (int)(p >> 32);
-  const int e2 = (int)(((long long)ph * ph) >> 32);
-  p = (unsigned long long)madw(e2, -786432, (long long)p);  // the second-order term: 3/8 2^21
-  const long long M = madw(Y, (int)(p >> 32), (long long)(((unsigned long long)(unsigned)Y * (unsigned)p) >> 32));
-  return ((long long)Y << 32) - (M >> 13);
+  // p = T U / 2^32 mod 2^64 (its multiple of 2^76 drops out), |p| < 2^55; the product of the low
+  // words by their upper halves
+  const unsigned long long w = (unsigned long long)Tl * Uh + (unsigned long long)Th * Ul;
+  unsigned pl, ph;
+  asm("{ .reg .u32 a, b;\n\t"
+      "mov.b64 {a, b}, %2;\n\tadd.cc.u32 %0, a, %3;\n\taddc.u32 b, b, 0;\n\tmad.lo.u32 %1, %4, %5, b; }"
+      : "=r"(pl), "=r"(ph)
+      : "l"(w), "r"((Tl >> 16) * (Ul >> 16)), "r"(Th), "r"(Uh));
+  const float t = (float)(int)ph;
+  // p / 2^24 with the second-order term, 3/8 e^2 2^53
+  const int q = (int)__funnelshift_r(pl, ph, 24) - __float2int_rn(t * t * (0.375f / 34359738368.0f));
+  const long long M = (long long)Y * q;
+  int lo, hi;
+  asm("sub.cc.u32 %0, 0, %2;\n\tsubc.u32 %1, %3, %4;"  // 2^32 Y - (M >> 21)
+      : "=r"(lo), "=r"(hi)
+      : "r"(__funnelshift_r((unsigned)M, (unsigned)(M >> 32), 21)), "r"(Y), "r"((int)(M >> 32) >> 21));
+  return make_int2(lo, hi);
 }
 
 // One atom of A against the staged atoms: sums of q y in three limb products, 32 pairs at a time
@@ -181,9 +194,7 @@ __device__ __forceinline__ Fixed fixed_scales(const Place& g, double aA, double 
   return s;
 }
 
-// APT atoms of A per thread.
-template <int APT>
-__global__ void __launch_bounds__(kDirectThreads, 2)
+__global__ void __launch_bounds__(kDirectThreads, 4)
     k_direct(const void* __restrict__ a, long long na, int dta, const void* __restrict__ b, long long nb, int dtb,
              const SysGeom* __restrict__ geo, const double* __restrict__ xf, int ablocks, int chunk,
              double* __restrict__ part) {
@@ -207,28 +218,21 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
   const int ab = blockIdx.x % ablocks, bb = blockIdx.x / ablocks;
   const long long j0 = (long long)bb * chunk, j1 = min(nb, j0 + (long long)chunk);
   const Fixed fs = fixed_scales(g, geo[0].a, geo[1].a);
-  double pos[APT][3], qa[APT];
-  bool bad = !fs.ok, warp_idle = true;
+  const long long i = (long long)ab * kDirectThreads + t;
+  double pos[3] = {0.0, 0.0, 0.0}, qa = 0.0;  // a padding atom: A's centre, no charge
+  bool bad = !fs.ok;
+  if (i < na) {
+    load_xyz(a, dta, i, pos, qa);
+    double r2 = 0.0;
 #pragma unroll
-  for (int u = 0; u < APT; ++u) {
-    const long long i = ((long long)ab * APT + u) * kDirectThreads + t;
-    pos[u][0] = pos[u][1] = pos[u][2] = qa[u] = 0.0;  // a padding atom: A's centre, no charge
-    if (i < na) {
-      load_xyz(a, dta, i, pos[u], qa[u]);
-      double r2 = 0.0;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        pos[u][k] -= g.cA[k];
-        r2 += pos[u][k] * pos[u][k];
-      }
-      bad = bad || !(r2 <= fs.rA2);
-      warp_idle = false;
+    for (int k = 0; k < 3; ++k) {
+      pos[k] -= g.cA[k];
+      r2 += pos[k] * pos[k];
     }
+    bad = bad || !(r2 <= fs.rA2);
   }
-  warp_idle = __all_sync(0xffffffffu, warp_idle);
-  double acc[APT];
-#pragma unroll
-  for (int u = 0; u < APT; ++u) acc[u] = 0.0;
+  const bool warp_idle = __all_sync(0xffffffffu, i >= na);
+  double acc = 0.0;
   bool fixed = false;
   if (!__syncthreads_or(bad)) {
     // the range's largest charge sets the scale of the charges; every staged atom lies within the radius
@@ -241,12 +245,10 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
     fixed = qe < 900;  // (not finite: 1025)
     if (qe < -800) qe = -800;
     const double gq = pow2(26 - qe);  // |q| gq < 2^26
-    int ah[APT][3], al[APT][3];
+    int ah[3], al[3];
 #pragma unroll
-    for (int u = 0; u < APT; ++u)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) split31(pos[u][k], fs.f, ah[u][k], al[u][k]);
-    FixSum sum[APT];
+    for (int k = 0; k < 3; ++k) split31(pos[k], fs.f, ah[k], al[k]);
+    FixSum sum;
     for (long long jt = j0; fixed && jt < j1; jt += kDirectTile) {
       FixAtom v;
       double d[3] = {0.0, 0.0, 0.0}, q = 0.0;  // a padding atom: B's centre, no charge
@@ -267,28 +269,23 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
       if (warp_idle || !fixed) continue;
       const int cnt = (int)min((long long)kDirectTile, j1 - jt);
       for (int k0 = 0; k0 < cnt; k0 += 32) {
-        long long s[APT][3] = {};
+        long long s[3] = {};
 #pragma unroll 2
         for (int k = k0; k < k0 + 32; ++k) {
           const int4 bh = *reinterpret_cast<const int4*>(sb.fix[k].h), bl = *reinterpret_cast<const int4*>(sb.fix[k].l);
-#pragma unroll
-          for (int u = 0; u < APT; ++u) {
-            const long long y = inv_r(ah[u], al[u], bh, bl);
-            const int yl = (int)y, yh = (int)(y >> 32) + (int)((unsigned)yl >> 31);  // y = 2^32 yh + yl
-            s[u][0] = madw(bh.w, yh, s[u][0]);
-            s[u][1] = madw(bh.w, yl, s[u][1]);
-            s[u][2] = madw(bl.w, yh, s[u][2]);
-          }
+          const int2 y = inv_r(ah, al, bh, bl);
+          const int yh = y.y + (int)((unsigned)y.x >> 31);  // y = 2^32 yh + yl, yl signed
+          s[0] = madw(bh.w, yh, s[0]);
+          s[1] = madw(bh.w, y.x, s[1]);
+          s[2] = madw(bl.w, yh, s[2]);
         }
-#pragma unroll
-        for (int u = 0; u < APT; ++u) sum[u].fold(s[u]);
+        sum.fold(s);
       }
     }
     if (fixed) {
       // q / r = 2^-117 f y / (2^27 gq) q's integer; FixSum::value leaves a weight of 2^32
       const double scale = fs.f * pow2(-117 - 27 + 32) * pow2(qe - 26);
-#pragma unroll
-      for (int u = 0; u < APT; ++u) acc[u] = sum[u].value(scale);
+      acc = sum.value(scale);
     }
   }
   if (!fixed) {
@@ -307,19 +304,12 @@ __global__ void __launch_bounds__(kDirectThreads, 2)
       const int cnt = (int)min((long long)kDirectTile, j1 - jt);
       for (int k = 0; k < cnt; ++k) {
         const Atom4 w = sb.dbl[k];
-#pragma unroll
-        for (int u = 0; u < APT; ++u) {
-          const double dx = w.x - pos[u][0], dy = w.y - pos[u][1], dz = w.z - pos[u][2];
-          acc[u] += w.w * rsqrt(dx * dx + dy * dy + dz * dz);
-        }
+        const double dx = w.x - pos[0], dy = w.y - pos[1], dz = w.z - pos[2];
+        acc += w.w * rsqrt(dx * dx + dy * dy + dz * dz);
       }
     }
   }
-  double v = 0.0;
-#pragma unroll
-  for (int u = 0; u < APT; ++u)
-    if (((long long)ab * APT + u) * kDirectThreads + t < na) v += acc[u] * qa[u];
-  v = block_sum(v, sh);
+  const double v = block_sum(i < na ? acc * qa : 0.0, sh);
   if (t == 0) part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = v;
 }
 
@@ -339,19 +329,16 @@ __global__ void k_direct_final(const double* __restrict__ part, int nblk, double
 }  // namespace
 
 // The split of one item, from the atom counts alone (so that an item's energy does not depend on
-// the batch it is in): A in blocks of 256 or 512 atoms, B in as many ranges as bring an item to
+// the batch it is in): A in blocks of 256 atoms, B in as many ranges as bring an item to
 // about 64 CTAs while each range keeps at least 512 atoms (a CTA's set-up is then about a tenth of
 // its work).
 DirectSplit direct_split(long long na, long long nb) {
   DirectSplit d;
-  d.apt = na > kDirectThreads ? 2 : 1;
-  const long long per = (long long)d.apt * kDirectThreads;
-  const long long nA = (na + per - 1) / per;
+  const long long nA = (na + kDirectThreads - 1) / kDirectThreads;
   long long nB = nA > 0 ? (64 + nA - 1) / nA : 1;
   nB = std::max<long long>(1, std::min<long long>(nB, nb / 512));
   d.ablocks = (int)nA;
-  d.chunk = (int)((((nb + nB - 1) / nB) + 31) / 32 * 32);
-  if (d.chunk < 32) d.chunk = 32;
+  d.chunk = (int)std::max<long long>(32, ((nb + nB - 1) / nB + 31) / 32 * 32);
   d.parts = (int)(nA * std::max<long long>(1, (nb + d.chunk - 1) / d.chunk));
   // items whose partial sums fit the buffer at once; one launch's grid holds at most 65,535
   d.slab = (int)std::max<long long>(1, std::min<long long>(65535, (1LL << 24) / std::max(d.parts, 1)));
@@ -362,10 +349,8 @@ int launch_direct(const void* a, long long na, int dta, const void* b, long long
                   const double* xf, int n_items, double* part, const DirectSplit& d, double* E, cudaStream_t s) {
   for (int i0 = 0; i0 < n_items; i0 += d.slab) {  // the slabs reuse the partial sums in stream order
     const int n = std::min(d.slab, n_items - i0);
-    if (d.parts > 0) {
-      auto k = d.apt == 2 ? k_direct<2> : k_direct<1>;
-      k<<<dim3(d.parts, n), kDirectThreads, 0, s>>>(a, na, dta, b, nb, dtb, geo, xf + 12LL * i0, d.ablocks, d.chunk, part);
-    }
+    if (d.parts > 0)
+      k_direct<<<dim3(d.parts, n), kDirectThreads, 0, s>>>(a, na, dta, b, nb, dtb, geo, xf + 12LL * i0, d.ablocks, d.chunk, part);
     k_direct_final<<<n, 128, 0, s>>>(part, d.parts, E + i0);
   }
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
