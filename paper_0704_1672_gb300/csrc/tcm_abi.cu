@@ -351,6 +351,14 @@ int split_of(const Plan& P) {
   return finalize_split((int)P.jobs.size(), max_tiles, max_slots);
 }
 
+// Most columns in a chunk of the jobs under one float plan (the column kernel's grid).
+int max_cols_of(const Plan& P, int plan) {
+  int mx = 0;
+  for (const MomJob& j : P.jobs)
+    if (j.plan == plan) mx = std::max(mx, moments_max_cols(plan, j.L));
+  return mx;
+}
+
 // Queue the moment pass (step a2/a3) for every job of the plan.
 // The moment kernels' work counters and exit tickets (counters[L], counters[32 + L]) are zero
 // on entry and left zero by every launch, so they are cleared once, when allocated.
@@ -392,6 +400,10 @@ int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, 
     for (int p = 1; p < kNumPlans; ++p) {
       const int b = P.tile_begin[p - 1], e = P.tile_begin[p];
       if (e == b) continue;
+      if (moments_use_cols(P.n_tiles, c->num_sms)) {
+        TRY_LAUNCH(launch_moments_cols(d_jobs, tiles + b, e - b, max_cols_of(P, p), d_geoms, parts, st));
+        continue;
+      }
       int cps = 1;  // the grid: the largest CTAs per SM of the plan's degrees, within its kernel's limit
       for (const MomJob& j : P.jobs)
         if (j.plan == p) cps = std::max(cps, c->ctas_per_sm[1][j.L]);
@@ -1087,7 +1099,8 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   if (!c->graphs || c->prof || !c->cap_stream) return enqueue(c->stream);
   // Replay a captured graph of the launch sequence when this call has the same shape and
   // buffers as the captured one (only the uploaded descriptor contents differ).
-  std::vector<long long> key = {precision, split_of(P), G != nullptr, (long long)(uintptr_t)G, (long long)S.jobs.size(),
+  const bool cols = precision == TCM_MIXED && moments_use_cols(P.n_tiles, c->num_sms);
+  std::vector<long long> key = {precision, split_of(P), cols ? max_cols_of(P, 1) : 0, cols ? max_cols_of(P, 2) : 0, G != nullptr, (long long)(uintptr_t)G, (long long)S.jobs.size(),
                                 (long long)S.n1, (long long)S.n2, (long long)P.jobs.size(), P.n_tile_ids,
                                 (long long)n_items, Lmax_items, (long long)o_geo, (long long)o_job, (long long)o_tile,
                                 (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)(uintptr_t)c->systiles.p,

@@ -270,6 +270,12 @@ inline int f64_rows(long long n) {
   const long long r = (n + 32 * 304 - 1) / (32 * 304);
   return (int)(r < 1 ? 1 : (r > 4096 ? 4096 : r));
 }
+// The same tiles (float plans) by columns, for calls with few of them (moments_cols.cu): jobs whose
+// low degrees come from the system pass.  max_cols: over the degrees of the tiles' jobs.
+int launch_moments_cols(const MomJob* jobs, const MomTile* tiles, int n_tiles, int max_cols, const SysGeom* geoms,
+                        double* partials, cudaStream_t s);
+bool moments_use_cols(int n_tiles, int num_sms);
+int moments_max_cols(int plan, int L);
 int moments_nchunks(int plan, int L);
 int moments_chunk_m0(int plan, int L, int chunk);  // first column of a chunk (chunk = nch: L + 1)
 const double* moments_chunk_costs(int plan, int L);  // relative cost per atom of each chunk
