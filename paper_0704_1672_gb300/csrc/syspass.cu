@@ -1,22 +1,33 @@
 // The pass over each system's atoms before the moment pass (step a1 and the mixed path's
-// low-degree sums), for any mix of system sizes, in two launches:
+// low-degree sums):
+//   - the centroid, for systems without a given centre (Section II: the centres may be any point; the
+//     centroid of the positions by default);
+//   - the radius a = max |x - c| (exact in double) and, for the mixed path, the low-degree sums
+//     S = sum q, P_k = sum q d_k, T_kl = sum q d_k d_l (d = x - c) from which k_finalize forms
+//     Q_lm, l <= 2, of every moment job of the system (Eq. (multipole) in Cartesian form).
 //
-//   pass 1 (systems without a given centre): the centroid (Section II: the centres may be any
-//           point; the centroid of the positions by default);
-//   pass 2: the radius a = max |x - c| (exact in double) and, for the mixed path, the
-//           low-degree sums S = sum q, P_k = sum q d_k, T_kl = sum q d_k d_l (d = x - c) from
-//           which k_finalize forms Q_lm, l <= 2, of every moment job of the system
-//           (Eq. (multipole) in Cartesian form).
+// Which kernel a system takes depends on its own atom count only, so its results do not depend on
+// the batch it is in:
+//   up to 8,192 atoms     one CTA per system (k_sys_one<1>), centroid and second pass in one kernel
+//                         (double records, whose FP64 instructions one SM issues at 2 lanes per clock:
+//                         up to 1,024);
+//   up to 65,536 atoms    one cluster of 8 CTAs per system (k_sys_one<8>), which exchange their sums
+//                         through distributed shared memory;
+//   above                 warp tiles of 1,024 atoms, all systems' tiles in one launch per pass
+//                         (k_sys_centroid, k_sys_radius_low); the last tile of a system to finish (a
+//                         ticket) reduces its tile rows in tile order.
+// What bounds it: for small calls the chain of dependent steps: a tile list, and a launch, a ticket and
+// a last tile per pass, took 28 us for one system of 20,000 atoms and 27 for two of 200; one kernel takes
+// 17 and 13.  For batches the instructions, about 140 float ones an atom for the float-float sums, and the
+// reads of the coordinates: 2,048 uneven systems 405 us before, 416 now.  The limits: at 2,048 atoms for
+// one CTA the batch paid for clusters with an atom or two per thread (462 us); double records of 3,260
+// atoms take 21 us on one CTA, 15 on a cluster.
 //
-// Each system is cut into warp tiles whose size depends on its own atom count only (so a
-// system's results do not depend on the batch it is in); one warp per tile, all systems' tiles
-// in one launch, so small and large systems alike spread over the GPU.  A lane issues the loads
-// of several atoms before their arithmetic.  Per-atom arithmetic is
-// float for float records: error-free two-sums for the centroid, float-float (two-sum and
-// fma-based two-product) for the low-degree sums, and a float filter for the radius: a second
-// scan of the tile (from cache) recomputes in double only the atoms within a relative 4e-6 of
-// the tile's float maximum.  Tile partials are doubles; the last tile of a system to finish (a ticket)
-// reduces them in tile order, so every result is deterministic.
+// Per-atom arithmetic is float for float records: error-free two-sums for the centroid, float-float
+// (two-sum and fma-based two-product) for the low-degree sums, and a float filter for the radius: a
+// second scan (from cache) recomputes in double only the atoms within a relative 4e-6 of the float
+// maximum.  Every reduction runs in a fixed order.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "tcm_internal.h"
@@ -305,9 +316,10 @@ __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __re
 __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob* __restrict__ jobs,
                                                                 const SysTile* __restrict__ tiles, int n_tiles,
                                                                 double* __restrict__ part, int* __restrict__ tickets,
-                                                                SysGeom* __restrict__ geoms) {
+                                                                SysGeom* __restrict__ geoms, bool trigger) {
   const int w = blockIdx.x * kSysWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  if (trigger) pdl_trigger();
   if (w >= n_tiles) return;
   const SysTile tl = tiles[w];
   const SysJob j = jobs[tl.job];
@@ -418,30 +430,273 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   }
 }
 
-}  // namespace
-
-int sys_tile_atoms(long long n) {
-  // 256-atom tiles (8 per lane) up to 32,768 atoms, 512 up to 65,536, 1,024 above: enough warps
-  // for the GPU even for a single system, few enough partial rows for the largest (128-atom
-  // tiles were tried: their per-tile reductions cost more on a batch of many systems than the
-  // extra warps gained on a pair of 20,000-atom systems)
-  long long t = 256;
-  while (t < 1024 && t * 128 < n) t *= 2;
-  return (int)t;
+// Sums of one low-degree accumulator set over atoms i, i + step, ... and the largest |x - c|^2: in
+// float (mf, float records) or exact (rmax, double records).
+template <bool kLow>
+__device__ __forceinline__ void scan_atoms(const SysJob& j, const double* c, const float* chi, const float* clo,
+                                           long long i0, long long step, float* s, float* e, float& mf, double& rmax) {
+  if (j.dtype == TCM_F32) {
+    const float4* X = reinterpret_cast<const float4*>(j.xyzq);
+    for (long long i = i0; i < j.n; i += step * kSysBatch) {
+      float4 v[kSysBatch];
+#pragma unroll
+      for (int u = 0; u < kSysBatch; ++u)
+        v[u] = i + step * u < j.n ? __ldg(X + i + step * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < kSysBatch; ++u) {
+        const FF d[3] = {ff_sub_split(v[u].x, chi[0], clo[0]), ff_sub_split(v[u].y, chi[1], clo[1]),
+                         ff_sub_split(v[u].z, chi[2], clo[2])};
+        if (i + step * u < j.n) mf = fmaxf(mf, r2_float(d));
+        if (kLow) low_accumulate(s, e, v[u].w, d);  // padding atoms carry q = 0
+      }
+    }
+  } else {
+    const double2* X = reinterpret_cast<const double2*>(j.xyzq);
+    for (long long i = i0; i < j.n; i += step * kSysBatch) {
+      double2 a[kSysBatch], b[kSysBatch];
+#pragma unroll
+      for (int u = 0; u < kSysBatch; ++u) {
+        const bool ok = i + step * u < j.n;
+        a[u] = ok ? __ldg(X + 2 * (i + step * u)) : make_double2(c[0], c[1]);
+        b[u] = ok ? __ldg(X + 2 * (i + step * u) + 1) : make_double2(c[2], 0.0);  // padding: d = 0, q = 0
+      }
+#pragma unroll
+      for (int u = 0; u < kSysBatch; ++u) {
+        const double dd[4] = {a[u].x - c[0], a[u].y - c[1], b[u].x - c[2], b[u].y};
+        rmax = fmax(rmax, dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
+        if (kLow) {
+          FF t[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float h = (float)dd[k];
+            t[k] = FF{h, (float)(dd[k] - (double)h)};
+          }
+          low_accumulate(s, e, t[3], t);
+        }
+      }
+    }
+  }
 }
 
-int launch_sys(const SysJob* jobs, const SysTile* t1, int n1, const SysTile* t2, int n2, double* part, int* tickets,
+// One system per cluster of CL CTAs; atom i belongs to thread i mod (CL kSysThreads).
+template <int CL>
+struct OneShared {
+  float2 wlow[kSysWarps][kLowSums];  // each warp's sums
+  double wcen[kSysWarps][3], wr2[kSysWarps];
+  float wmf[kSysWarps];
+  double cen[CL][3];                 // each CTA's centroid sums (in every CTA)
+  float2 low[CL][kLowSums];          // each CTA's low-degree sums and maximum (in CTA 0)
+  double r2[CL];
+  double c[3];
+  float chi[3], clo[3];
+};
+
+template <int CL>
+__global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __restrict__ jobs, double* __restrict__ part,
+                                                            SysGeom* __restrict__ geoms, bool trigger) {
+  namespace cg = cooperative_groups;
+  __shared__ OneShared<CL> sh;
+  if (trigger) pdl_trigger();
+  const SysJob j = jobs[blockIdx.x / CL];
+  const int rank = blockIdx.x % CL;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  constexpr long long step = (long long)CL * kSysThreads;
+  const long long i0 = (long long)rank * kSysThreads + t;
+  auto sync = [] {
+    if constexpr (CL > 1)
+      cg::this_cluster().sync();
+    else
+      __syncthreads();
+  };
+  auto of_rank = [&](auto* p, int r) {  // the same variable in CTA r of the cluster
+    if constexpr (CL > 1) return cg::this_cluster().map_shared_rank(p, r);
+    else return p;
+  };
+  if (j.need_center) {
+    double cs[3] = {0.0, 0.0, 0.0};
+    if (j.dtype == TCM_F32) {
+      const float4* X = reinterpret_cast<const float4*>(j.xyzq);
+      float s[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
+      for (long long i = i0; i < j.n; i += step * kSysBatch) {
+        float4 v[kSysBatch];
+#pragma unroll
+        for (int u = 0; u < kSysBatch; ++u)  // padding atoms add exact zeros
+          v[u] = i + step * u < j.n ? __ldg(X + i + step * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < kSysBatch; ++u) {
+          ff_acc(s[0], e[0], FF{v[u].x, 0.f});
+          ff_acc(s[1], e[1], FF{v[u].y, 0.f});
+          ff_acc(s[2], e[2], FF{v[u].z, 0.f});
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        ff_warp_sum(s[k], e[k]);
+        cs[k] = (double)s[k] + (double)e[k];
+      }
+    } else {
+      const double2* X = reinterpret_cast<const double2*>(j.xyzq);
+      for (long long i = i0; i < j.n; i += step) {
+        const double2 a = __ldg(X + 2 * i), b = __ldg(X + 2 * i + 1);
+        cs[0] += a.x;
+        cs[1] += a.y;
+        cs[2] += b.x;
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) cs[k] = warp_sum_d(cs[k]);
+    }
+    if (lane < 3) sh.wcen[w][lane] = lane == 0 ? cs[0] : (lane == 1 ? cs[1] : cs[2]);
+    __syncthreads();
+    if (t < 3) {
+      double v = 0.0;
+#pragma unroll
+      for (int k = 0; k < kSysWarps; ++k) v += sh.wcen[k][t];
+#pragma unroll
+      for (int r = 0; r < CL; ++r) of_rank(&sh.cen[0][0], r)[3 * rank + t] = v;
+    }
+    sync();
+    if (t < 3) {  // the centre and its split into float parts
+      double v = 0.0;
+#pragma unroll
+      for (int r = 0; r < CL; ++r) v += sh.cen[r][t];
+      const double c = v * (j.n > 0 ? 1.0 / (double)j.n : 0.0);
+      const float hi = (float)c;
+      const float lo = (float)(c - (double)hi);
+      sh.c[t] = c;
+      sh.chi[t] = hi;
+      sh.clo[t] = lo;
+      if (rank == 0) {
+        geoms[j.geom].c[t] = c;
+        geoms[j.geom].chi[t] = hi;
+        geoms[j.geom].clo[t] = lo;
+      }
+    }
+  } else if (t < 3) {
+    sh.c[t] = geoms[j.geom].c[t];
+    sh.chi[t] = geoms[j.geom].chi[t];
+    sh.clo[t] = geoms[j.geom].clo[t];
+  }
+  __syncthreads();
+  if (!j.need_radius && !j.need_low) {  // the whole cluster
+    pdl_wait();
+    return;
+  }
+  const double c[3] = {sh.c[0], sh.c[1], sh.c[2]};
+  const float chi[3] = {sh.chi[0], sh.chi[1], sh.chi[2]}, clo[3] = {sh.clo[0], sh.clo[1], sh.clo[2]};
+  float s[kLowSums], e[kLowSums], mf = 0.f;
+  double rmax = 0.0;
+#pragma unroll
+  for (int k = 0; k < kLowSums; ++k) s[k] = e[k] = 0.f;
+  if (j.need_low) {
+    scan_atoms<true>(j, c, chi, clo, i0, step, s, e, mf, rmax);
+    ff_reduce_scatter<kLowSums, 16>(s, e, lane);
+    if ((kRs10Lanes >> lane) & 1u)
+      sh.wlow[w][5 * ((lane >> 4) & 1) + 3 * ((lane >> 3) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1)] =
+          make_float2(s[0], e[0]);
+  } else {
+    scan_atoms<false>(j, c, chi, clo, i0, step, s, e, mf, rmax);
+  }
+  if (j.need_radius && j.dtype == TCM_F32) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+    if (lane == 0) sh.wmf[w] = mf;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSysWarps; ++k) mf = fmaxf(mf, sh.wmf[k]);
+    const float thr = mf * (1.0f - 4e-6f);
+    const float4* X = reinterpret_cast<const float4*>(j.xyzq);
+    for (long long iw = i0 - lane; iw < j.n; iw += step) {  // warp-uniform trip count
+      const bool cand = iw + lane < j.n && r2_plain(__ldg(X + iw + lane), chi, clo) >= thr;
+      unsigned m = __ballot_sync(0xffffffffu, cand);  // the candidates one at a time: see k_sys_radius_low
+      while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        const float4 v = __ldg(X + iw + src);
+        const double ex = (double)v.x - c[0], ey = (double)v.y - c[1], ez = (double)v.z - c[2];
+        rmax = fmax(rmax, ex * ex + ey * ey + ez * ez);
+      }
+    }
+  }
+  rmax = warp_max_d(rmax);
+  if (lane == 0) sh.wr2[w] = rmax;
+  __syncthreads();
+  if (t < kLowSums && j.need_low) {
+    FF v{0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < kSysWarps; ++k) ff_acc(v.h, v.l, FF{sh.wlow[k][t].x, sh.wlow[k][t].y});
+    of_rank(&sh.low[0][0], 0)[rank * kLowSums + t] = make_float2(v.h, v.l);
+  }
+  if (t == 32) {
+    double m = 0.0;
+#pragma unroll
+    for (int k = 0; k < kSysWarps; ++k) m = fmax(m, sh.wr2[k]);
+    of_rank(&sh.r2[0], 0)[rank] = m;
+  }
+  sync();
+  pdl_wait();  // this grid's completion implies that of the kernels it overlaps
+  if (rank != 0) return;
+  if (t < kLowSums && j.need_low) {
+    FF v{0.f, 0.f};
+#pragma unroll
+    for (int r = 0; r < CL; ++r) ff_acc(v.h, v.l, FF{sh.low[r][t].x, sh.low[r][t].y});
+    part[(long long)j.sum_row * kSysPart + kSysPartLow + t] = (double)v.h + (double)v.l;
+  }
+  if (t == 32 && j.need_radius) {
+    double m = 0.0;
+#pragma unroll
+    for (int r = 0; r < CL; ++r) m = fmax(m, sh.r2[r]);
+    geoms[j.geom].a = sqrt(m);
+  }
+}
+
+}  // namespace
+
+int sys_class(long long n, int dtype) {
+  return n <= (dtype == TCM_F32 ? kSysOneMaxF32 : kSysOneMaxF64) ? 0 : (n <= kSysClusterMax ? 1 : 2);
+}
+
+int sys_tile_atoms(long long) { return 1024; }
+
+// Largest systems first.  The kernels of different classes do not depend on each other: all but the
+// last trigger their successor on entry, and each of those waits for its predecessors before it ends
+// (in sequence, each with its own tail, they took 462 us for 2,048 uneven systems).
+int launch_sys(const SysJob* jobs, const SysCount& n, const SysTile* t1, const SysTile* t2, double* part, int* tickets,
                SysGeom* geoms, cudaStream_t s) {
-  if (n1 > 0) {
-    k_sys_centroid<<<(n1 + kSysWarps - 1) / kSysWarps, kSysThreads, 0, s>>>(jobs, t1, n1, part, tickets, geoms);
+  if (n.tiles1 > 0) {
+    k_sys_centroid<<<(n.tiles1 + kSysWarps - 1) / kSysWarps, kSysThreads, 0, s>>>(jobs, t1, n.tiles1, part, tickets, geoms);
     if (cudaPeekAtLastError() != cudaSuccess) return -1;
   }
-  if (n2 > 0 && launch_pdl(k_sys_radius_low, dim3((n2 + kSysWarps - 1) / kSysWarps), dim3(kSysThreads), 0, s, jobs,
-                           t2, n2, part, tickets, geoms) != cudaSuccess)
+  if (n.tiles2 > 0 && launch_pdl(k_sys_radius_low, dim3((n.tiles2 + kSysWarps - 1) / kSysWarps), dim3(kSysThreads), 0, s,
+                                 jobs, t2, n.tiles2, part, tickets, geoms, n.cluster + n.one > 0) != cudaSuccess)
     return -1;
+  const bool overlap = n.tiles2 > 0;  // (a centroid always comes with its radius)
+  if (n.cluster > 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n.cluster * kSysClusterSize);
+    cfg.blockDim = dim3(kSysThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kSysClusterSize;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 2 : 1;
+    if (cudaLaunchKernelEx(&cfg, k_sys_one<kSysClusterSize>, jobs + n.one, part, geoms, n.one > 0) != cudaSuccess)
+      return -1;
+  }
+  if (n.one > 0) {
+    if (n.cluster > 0 || overlap) {
+      if (launch_pdl(k_sys_one<1>, dim3(n.one), dim3(kSysThreads), 0, s, jobs, part, geoms, false) != cudaSuccess) return -1;
+    } else {
+      k_sys_one<1><<<n.one, kSysThreads, 0, s>>>(jobs, part, geoms, false);
+      if (cudaPeekAtLastError() != cudaSuccess) return -1;
+    }
+  }
   return 0;
 }
 
-int sys_launches(int n1, int n2) { return (n1 > 0 ? 1 : 0) + (n2 > 0 ? 1 : 0); }
+int sys_launches(const SysCount& n) { return (n.one > 0) + (n.cluster > 0) + (n.tiles1 > 0) + (n.tiles2 > 0); }
 
 }  // namespace tcm

@@ -379,12 +379,11 @@ int ensure_moment_buffers(tcm_ctx* c, int precision, const Plan& P) {
 // chunk plan p over all degrees.
 constexpr int kAnyCounter = kLmaxMax;  // + plan (1 or 2)
 
-int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, const SysGeom* d_geoms,
-                cudaStream_t st) {
+int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, const MomTile* tiles,
+                const SysGeom* d_geoms, cudaStream_t st) {
   TRY(ensure_moment_buffers(c, precision, P));
   int* counters = static_cast<int*>(c->counters.p);
   double* parts = static_cast<double*>(c->partials.p);
-  MomTile* tiles = static_cast<MomTile*>(c->tiles.p);
   if (precision == TCM_FP64) {
     int ngroups = 0;
     for (int L = 0; L <= kLmaxMax; ++L) ngroups += P.tile_begin[L + 1] > P.tile_begin[L];
@@ -425,8 +424,8 @@ int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, 
 // whose centre or radius is not given, and the low-degree sums of the mixed path for every
 // system with a computed moment job.
 struct SysPlan {
-  std::vector<SysJob> jobs;
-  int n1 = 0, n2 = 0;            // tiles of pass 1 (centroid) and pass 2 (radius, low-degree sums)
+  std::vector<SysJob> jobs;     // by class
+  SysCount n;
   std::vector<int> of_system;   // system -> index of its SysJob, or -1
   int rows = 0;
 };
@@ -435,6 +434,7 @@ struct SysPlan {
 void plan_sys(const tcm_system* systems, int n_systems, const std::vector<char>& used, const std::vector<char>& low,
               SysPlan& S) {
   S.of_system.assign(std::max(n_systems, 0), -1);
+  std::vector<SysJob> of_class[3];
   for (int s = 0; s < n_systems; ++s) {
     if (!used[s]) continue;
     const tcm_system& sy = systems[s];
@@ -450,21 +450,32 @@ void plan_sys(const tcm_system* systems, int n_systems, const std::vector<char>&
     j.need_center = nc;
     j.need_radius = nr;
     j.need_low = nl;
-    j.atoms_per_tile = sys_tile_atoms(sy.n);
-    j.n_tiles = (int)std::max<long long>(1, (sy.n + j.atoms_per_tile - 1) / j.atoms_per_tile);
-    j.tile_base = S.rows;
-    S.rows += j.n_tiles;
-    j.sum_row = -1;
-    const int ji = (int)S.jobs.size();
-    j.first1 = nc ? S.n1 : -1;
-    j.first2 = (nr || nl) ? S.n2 : -1;
-    if (nc) S.n1 += j.n_tiles;
-    if (nr || nl) S.n2 += j.n_tiles;
-    S.of_system[s] = ji;
-    S.jobs.push_back(j);
+    j.sum_row = j.first1 = j.first2 = -1;
+    const int cl = sys_class(sy.n, sy.dtype);
+    if (cl == 2) {
+      j.atoms_per_tile = sys_tile_atoms(sy.n);
+      j.n_tiles = (int)((sy.n + j.atoms_per_tile - 1) / j.atoms_per_tile);
+      j.tile_base = S.rows;
+      S.rows += j.n_tiles;
+      if (nc) {
+        j.first1 = S.n.tiles1;
+        S.n.tiles1 += j.n_tiles;
+      }
+      if (nr || nl) {
+        j.first2 = S.n.tiles2;
+        S.n.tiles2 += j.n_tiles;
+      }
+    }
+    of_class[cl].push_back(j);
   }
-  for (SysJob& j : S.jobs)  // one sum row per system after the tile rows
-    if (j.need_low) j.sum_row = S.rows++;
+  S.n.one = (int)of_class[0].size();
+  S.n.cluster = (int)of_class[1].size();
+  for (auto& v : of_class)
+    for (SysJob& j : v) {
+      if (j.need_low) j.sum_row = S.rows++;  // one sum row per system after the tile rows
+      S.of_system[j.geom] = (int)S.jobs.size();
+      S.jobs.push_back(j);
+    }
 }
 
 // Mixed path: every computed moment job takes its degrees l <= 2 from its system's low sums.
@@ -484,28 +495,66 @@ int ensure_sys_buffers(tcm_ctx* c, const SysPlan& S) {
   void* before = c->systk.p;
   TRY(dev_ensure(c, c->systk, std::max<size_t>(2 * S.jobs.size(), 64) * sizeof(int)));
   if (c->systk.p != before) TRY_CUDA(cudaMemsetAsync(c->systk.p, 0, c->systk.cap, c->stream));
-  TRY(dev_ensure(c, c->systiles, (size_t)std::max(S.n1 + S.n2, 1) * sizeof(SysTile)));
+  TRY(dev_ensure(c, c->systiles, (size_t)std::max(S.n.tiles1 + S.n.tiles2, 1) * sizeof(SysTile)));
   return TCM_OK;
 }
 
-int run_sys(tcm_ctx* c, const SysPlan& S, const SysJob* d_sj, SysGeom* d_geo, cudaStream_t st) {
+// The tile lists of a call: written by the host into the descriptor block when they are short (a
+// launch saved: about 4 us of a small call), else on the device from the groups and system jobs (long
+// lists cost more to build and upload than the launch).
+constexpr int kHostTiles = 2048;
+struct Lists {
+  bool on_host = false;
+  std::vector<MomTile> mom;
+  std::vector<SysTile> sys;  // pass 1, then pass 2
+  size_t o_mom = 0, o_sys = 0;
+  MomTile* d_mom = nullptr;
+  SysTile* d_sys = nullptr;
+
+  void plan(const Plan* P, const SysPlan& S, Packer& pk) {
+    const int nm = P ? P->n_tiles : 0, ns = S.n.tiles1 + S.n.tiles2;
+    on_host = nm + ns <= kHostTiles;
+    if (!on_host) return;
+    mom.resize(nm);
+    sys.resize(ns);
+    if (P)
+      for (const MomGroup& g : P->groups) {
+        const MomJob& j = P->jobs[g.job];
+        for (int t = 0; t < g.n; ++t)
+          mom[g.first + t] = MomTile{g.job, g.chunk, t, j.tile_base + g.chunk * j.tiles_per_chunk + t};
+      }
+    for (int ji = 0; ji < (int)S.jobs.size(); ++ji) {
+      const SysJob& j = S.jobs[ji];
+      for (int t = 0; t < j.n_tiles; ++t) {
+        if (j.first1 >= 0) sys[j.first1 + t] = SysTile{ji, t};
+        if (j.first2 >= 0) sys[S.n.tiles1 + j.first2 + t] = SysTile{ji, t};
+      }
+    }
+    o_mom = pk.add(mom);
+    o_sys = pk.add(sys);
+  }
+  void place(tcm_ctx* c, char* base) {
+    d_mom = on_host ? reinterpret_cast<MomTile*>(base + o_mom) : static_cast<MomTile*>(c->tiles.p);
+    d_sys = on_host ? reinterpret_cast<SysTile*>(base + o_sys) : static_cast<SysTile*>(c->systiles.p);
+  }
+};
+
+int run_sys(tcm_ctx* c, const SysPlan& S, const Lists& T, const SysJob* d_sj, SysGeom* d_geo, cudaStream_t st) {
   if (S.jobs.empty()) return TCM_OK;
-  PhaseScope ps(c, TCM_PHASE_GEOM, sys_launches(S.n1, S.n2));
-  SysTile* t1 = static_cast<SysTile*>(c->systiles.p);
-  TRY_LAUNCH(launch_sys(d_sj, t1, S.n1, t1 + S.n1, S.n2, static_cast<double*>(c->gpart.p),
+  PhaseScope ps(c, TCM_PHASE_GEOM, sys_launches(S.n));
+  TRY_LAUNCH(launch_sys(d_sj, S.n, T.d_sys, T.d_sys + S.n.tiles1, static_cast<double*>(c->gpart.p),
                         static_cast<int*>(c->systk.p), d_geo, st));
   return TCM_OK;
 }
 
-// The tile lists of the call (moment pass and system pass), written on the device from the
-// groups and system jobs: the first launch of a call (it depends on nothing queued before it).
+// Long tile lists, written on the device: the first launch of a call (it depends on nothing queued
+// before it).
 int run_expand(tcm_ctx* c, const std::vector<MomGroup>& groups, const MomJob* d_jobs, const MomGroup* d_groups,
-               const SysPlan& S, const SysJob* d_sj, cudaStream_t st) {
-  if (groups.empty() && S.jobs.empty()) return TCM_OK;
+               const SysPlan& S, const Lists& T, const SysJob* d_sj, cudaStream_t st) {
+  if (T.on_host) return TCM_OK;
   PhaseScope ps(c, TCM_PHASE_GEOM, 1);
-  SysTile* t1 = static_cast<SysTile*>(c->systiles.p);
-  TRY_LAUNCH(launch_expand_tiles(d_groups, (int)groups.size(), d_jobs, static_cast<MomTile*>(c->tiles.p), d_sj,
-                                 (int)S.jobs.size(), t1, t1 + S.n1, st));
+  TRY_LAUNCH(launch_expand_tiles(d_groups, (int)groups.size(), d_jobs, T.d_mom, d_sj, (int)S.jobs.size(), T.d_sys,
+                                 T.d_sys + S.n.tiles1, st));
   return TCM_OK;
 }
 
@@ -756,13 +805,16 @@ int tcm_prepare(tcm_ctx_t c, tcm_system* s) {
   std::vector<SysGeom> geoms{host_geom(*s)};
   Packer pk;
   const size_t o_geo = pk.add(geoms), o_sj = pk.add(S.jobs);
+  Lists T;
+  T.plan(nullptr, S, pk);
   TRY(ensure_sys_buffers(c, S));
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
   const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
-  TRY(run_expand(c, {}, nullptr, nullptr, S, d_sj, c->stream));
-  TRY(run_sys(c, S, d_sj, d_geo, c->stream));
+  T.place(c, base);
+  TRY(run_expand(c, {}, nullptr, nullptr, S, T, d_sj, c->stream));
+  TRY(run_sys(c, S, T, d_sj, d_geo, c->stream));
   TRY_CUDA(cudaMemcpyAsync(c->pinned_small, d_geo, sizeof(SysGeom), cudaMemcpyDeviceToHost, c->stream));
   TRY_CUDA(cudaStreamSynchronize(c->stream));
   const SysGeom* g = static_cast<const SysGeom*>(c->pinned_small);
@@ -804,16 +856,19 @@ int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, i
   std::vector<SysGeom> geoms{host_geom(*s)};
   Packer pk;
   const size_t o_geo = pk.add(geoms), o_job = pk.add(P.jobs), o_tile = pk.add(P.groups), o_sj = pk.add(S.jobs);
+  Lists T;
+  T.plan(&P, S, pk);
   TRY(ensure_moment_buffers(c, precision, P));
   TRY(ensure_sys_buffers(c, S));
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
   const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
-  TRY(run_expand(c, P.groups, reinterpret_cast<MomJob*>(base + o_job), reinterpret_cast<MomGroup*>(base + o_tile), S,
+  T.place(c, base);
+  TRY(run_expand(c, P.groups, reinterpret_cast<MomJob*>(base + o_job), reinterpret_cast<MomGroup*>(base + o_tile), S, T,
                  d_sj, c->stream));
-  TRY(run_sys(c, S, d_sj, d_geo, c->stream));
-  TRY(run_moments(c, precision, P, reinterpret_cast<MomJob*>(base + o_job), d_geo, c->stream));
+  TRY(run_sys(c, S, T, d_sj, d_geo, c->stream));
+  TRY(run_moments(c, precision, P, reinterpret_cast<MomJob*>(base + o_job), T.d_mom, d_geo, c->stream));
   out->lmax = lmax;
   if (!geom_known(*s)) {
     TRY_CUDA(cudaMemcpyAsync(c->pinned_small, d_geo, sizeof(SysGeom), cudaMemcpyDeviceToHost, c->stream));
@@ -1077,6 +1132,8 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   Packer pk;
   const size_t o_geo = pk.add(geoms), o_job = pk.add2(P.jobs, cached), o_tile = pk.add(P.groups), o_sj = pk.add(S.jobs),
                o_it = pk.add(pd), o_rot = pk.add(rots);
+  Lists T;
+  T.plan(&P, S, pk);
   // every buffer the launches touch is sized before anything is queued (no reallocation
   // may happen while a graph is being captured)
   TRY(ensure_sys_buffers(c, S));
@@ -1085,11 +1142,12 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
   const MomJob* d_jobs = reinterpret_cast<MomJob*>(base + o_job);
+  T.place(c, base);
   auto enqueue = [&](cudaStream_t st) -> int {
     const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
-    TRY(run_expand(c, P.groups, d_jobs, reinterpret_cast<MomGroup*>(base + o_tile), S, d_sj, st));
-    TRY(run_sys(c, S, d_sj, d_geo, st));
-    TRY(run_moments(c, precision, P, d_jobs, d_geo, st));
+    TRY(run_expand(c, P.groups, d_jobs, reinterpret_cast<MomGroup*>(base + o_tile), S, T, d_sj, st));
+    TRY(run_sys(c, S, T, d_sj, d_geo, st));
+    TRY(run_moments(c, precision, P, d_jobs, T.d_mom, d_geo, st));
     PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
     TRY_LAUNCH(launch_contract(reinterpret_cast<PairDesc*>(base + o_it), (int)n_items, Lmax_items, d_jobs, d_geo,
                                c->d_ztab, rots.empty() ? nullptr : reinterpret_cast<double*>(base + o_rot), E,
@@ -1101,7 +1159,8 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   // buffers as the captured one (only the uploaded descriptor contents differ).
   const bool cols = precision == TCM_MIXED && moments_use_cols(P.n_tiles, c->num_sms);
   std::vector<long long> key = {precision, split_of(P), cols ? max_cols_of(P, 1) : 0, cols ? max_cols_of(P, 2) : 0, G != nullptr, (long long)(uintptr_t)G, (long long)S.jobs.size(),
-                                (long long)S.n1, (long long)S.n2, (long long)P.jobs.size(), P.n_tile_ids,
+                                S.n.one, S.n.cluster, S.n.tiles1, S.n.tiles2, (long long)T.o_mom, (long long)T.o_sys,
+                                T.on_host, (long long)P.jobs.size(), P.n_tile_ids,
                                 (long long)n_items, Lmax_items, (long long)o_geo, (long long)o_job, (long long)o_tile,
                                 (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)(uintptr_t)c->systiles.p,
                                 (long long)rots.empty(), (long long)(uintptr_t)base, (long long)(uintptr_t)c->gpart.p,
@@ -1144,8 +1203,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   }
   TRY_CUDA(cudaGraphLaunch(c->gexec, c->stream));
   ++c->graph_launches;
-  c->launches[TCM_PHASE_GEOM] += (S.jobs.empty() ? 0 : sys_launches(S.n1, S.n2)) +
-                                  ((P.groups.empty() && S.jobs.empty()) ? 0 : 1);
+  c->launches[TCM_PHASE_GEOM] += sys_launches(S.n) + !T.on_host;
   c->launches[TCM_PHASE_MOMENTS] += moment_launches(precision, P);
   c->launches[TCM_PHASE_FINALIZE] += 1;
   c->launches[TCM_PHASE_CONTRACT] += 1;
@@ -1174,6 +1232,8 @@ int direct_items(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t 
   }
   Packer pk;
   const size_t o_geo = pk.add(geoms), o_xf = pk.add(xf), o_sj = pk.add(S.jobs);
+  Lists T;
+  T.plan(nullptr, S, pk);
   const DirectSplit split = direct_split(A->n, B->n);
   TRY(ensure_sys_buffers(c, S));
   TRY(dev_ensure(c, c->dpart, (size_t)std::max<int64_t>((int64_t)split.parts * std::min<int64_t>(n, split.slab), 1) * sizeof(double)));
@@ -1181,8 +1241,9 @@ int direct_items(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t 
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
   const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
-  TRY(run_expand(c, {}, nullptr, nullptr, S, d_sj, c->stream));
-  TRY(run_sys(c, S, d_sj, d_geo, c->stream));
+  T.place(c, base);
+  TRY(run_expand(c, {}, nullptr, nullptr, S, T, d_sj, c->stream));
+  TRY(run_sys(c, S, T, d_sj, d_geo, c->stream));
   const int nlaunch = (int)((n + split.slab - 1) / split.slab) * (split.parts > 0 ? 2 : 1);
   PhaseScope ps(c, TCM_PHASE_DIRECT, nlaunch);
   TRY_LAUNCH(launch_direct(A->xyzq, A->n, A->dtype, B->xyzq, B->n, B->dtype, d_geo,

@@ -183,9 +183,9 @@ struct MomGroup {  // the tiles of one (job, chunk), written to the tile list on
   int first;       // position of its first tile in the tile list
 };
 
-// The pass over a system's atoms before the moment pass (syspass.cu): pass 1 its centroid
-// (need_center), pass 2 its radius (need_radius) and, for the mixed path, its low-degree sums
-// (need_low).  A system's warp tiles depend on its atom count only (sys_tile_atoms).
+// The pass over a system's atoms before the moment pass (syspass.cu): its centroid (need_center),
+// radius (need_radius) and, for the mixed path, its low-degree sums (need_low).  The kernel depends on
+// the atom count (sys_class): 0 one CTA, 1 one cluster, 2 warp tiles in two passes (the tile fields).
 struct SysJob {
   const void* xyzq;
   long long n;
@@ -215,6 +215,12 @@ constexpr int kLowSums = 10;            // S, P_x, P_y, P_z, T_xx, T_xy, T_xz, T
 constexpr int kLowLmax = 2;             // degrees replaced by the low-degree sums
 
 constexpr int kSysThreads = 256;
+constexpr int kSysClusterSize = 8;
+// atoms of class 0 (float and double records: the latter's arithmetic needs more SMs) and of class 1
+constexpr long long kSysOneMaxF32 = 8192, kSysOneMaxF64 = 1024, kSysClusterMax = 65536;
+struct SysCount {  // one call's system pass: systems of class 0 and 1, tiles of the two passes of class 2
+  int one = 0, cluster = 0, tiles1 = 0, tiles2 = 0;
+};
 constexpr int kSysPartR2 = 3;    // partial row: the centroid sums [0, 3), the tile's max |x - c|^2,
 constexpr int kSysPartLow = 4;   // and the low-degree sums [4, 4 + kLowSums)
 constexpr int kSysPart = kSysPartLow + kLowSums;
@@ -283,13 +289,13 @@ const double* moments_chunk_costs(int plan, int L);  // relative cost per atom o
 // kNumPlans (kLmaxMax + 2) entries, plan by plan, each block ending with its total).
 void finalize_tables(std::vector<int>& imap_off, std::vector<int>& imap, std::vector<double>& fmap);
 
-// Step a1 and the low-degree sums: pass 1 over the n1 tiles of the systems that need a centroid,
-// then pass 2 over the n2 tiles of those that need a radius or low-degree sums (programmatic
-// serialization).  part: kSysPart doubles per tile row; tickets: two ints per job, zero on entry
-// and left zero.
-int launch_sys(const SysJob* jobs, const SysTile* t1, int n1, const SysTile* t2, int n2, double* part, int* tickets,
+// Step a1 and the low-degree sums: the jobs of class 0, then those of class 1, then the tiles of the
+// others (centroid, then radius and sums).  part: kSysPart doubles per row; tickets: two ints per job,
+// zero on entry and left zero.
+int launch_sys(const SysJob* jobs, const SysCount& n, const SysTile* t1, const SysTile* t2, double* part, int* tickets,
                SysGeom* geoms, cudaStream_t s);
-int sys_launches(int n1, int n2);
+int sys_launches(const SysCount& n);
+int sys_class(long long n, int dtype);
 int sys_tile_atoms(long long n);
 // Step a3: one CTA per job, or n_split CTAs over the job's slots.  imap + imap_off[plan (kLmaxMax + 2)
 // + L] lists, per (chunk, slot) of degree L under the job's plan, the packed component it holds (-1

@@ -35,8 +35,7 @@ constexpr int kNaPartialDoubles = 63840;                             // mixed: 6
 constexpr int kNaTilesF64 = kNaPartialDoubles / kRowF64;             // double: 102 tiles of 625 components
 static_assert(kNaTilesPerChunk * 800 <= kNaPartialDoubles, "the mixed path's rows must fit");
 constexpr int kNaMaxTiles = kNaTilesPerChunk * kNaMaxChunks;
-// system-pass rows: sys_tile_atoms gives at most 128 tiles up to 65,536 atoms and 1,024-atom tiles
-// above (256 for the largest request), plus the sum row
+// system-pass rows: 1,024-atom tiles above 65,536 atoms (256 for the largest request), plus the sum row
 constexpr int kNaSysTiles = (int)((kNaMaxAtoms + 1023) / 1024) + 1;
 constexpr int kNaCompTotal = 5525;  // sum over L = 0..24 of (L+1)^2
 
@@ -180,8 +179,9 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   sj.need_center = s->has_center ? 0 : 1;
   sj.need_radius = (sj.need_center || s->radius < 0.0) ? 1 : 0;
   sj.need_low = precision == TCM_MIXED ? 1 : 0;
+  const int cl = sys_class(s->n, s->dtype);
   sj.atoms_per_tile = sys_tile_atoms(s->n);
-  sj.n_tiles = (int)std::max<long long>(1, (s->n + sj.atoms_per_tile - 1) / sj.atoms_per_tile);
+  sj.n_tiles = cl == 2 ? (int)((s->n + sj.atoms_per_tile - 1) / sj.atoms_per_tile) : 0;
   sj.tile_base = 0;
   sj.first1 = sj.need_center ? 0 : -1;  // the tile lists are written by k_noalloc_prepare
   sj.first2 = 0;
@@ -189,16 +189,20 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   if (sj.n_tiles + 1 > kNaSysTiles) return na_err(TCM_EINVAL, "tcm_moments_noalloc: request exceeds the fixed scratch");
   job.low_base = sj.sum_row;
   job.low_tiles = sj.need_low ? 1 : 0;
-  const int n1 = sj.need_center ? sj.n_tiles : 0;
-  const int n2 = (sj.need_radius || sj.need_low) ? sj.n_tiles : 0;
+  SysCount ns;
+  if (sj.need_center || sj.need_radius || sj.need_low) {
+    ns.one = cl == 0;
+    ns.cluster = cl == 1;
+  }
+  ns.tiles1 = sj.need_center ? sj.n_tiles : 0;
+  ns.tiles2 = (sj.need_radius || sj.need_low) ? sj.n_tiles : 0;
 
   MomJob* d_job = reinterpret_cast<MomJob*>(base + kOffJob);
   SysGeom* d_geom = reinterpret_cast<SysGeom*>(base + kOffGeom);
   k_noalloc_prepare<<<1, 256, 0, st>>>(base, job, geom, sj, nch, tpc);
   if (cudaPeekAtLastError() != cudaSuccess) return na_err(TCM_ECUDA, "tcm_moments_noalloc: launch failed");
-  if ((n1 > 0 || n2 > 0) &&
-      launch_sys(reinterpret_cast<SysJob*>(base + kOffSJob), reinterpret_cast<SysTile*>(base + kOffSTiles1), n1,
-                 reinterpret_cast<SysTile*>(base + kOffSTiles2), n2, reinterpret_cast<double*>(base + kOffSPart),
+  if (launch_sys(reinterpret_cast<SysJob*>(base + kOffSJob), ns, reinterpret_cast<SysTile*>(base + kOffSTiles1),
+                 reinterpret_cast<SysTile*>(base + kOffSTiles2), reinterpret_cast<double*>(base + kOffSPart),
                  reinterpret_cast<int*>(base + kOffCounters) + 40, d_geom, st) != 0)
     return na_err(TCM_ECUDA, "tcm_moments_noalloc: centre/radius launch failed");
   int num_sms = 0;
