@@ -323,9 +323,8 @@ __global__ void __launch_bounds__(kContractThreads, kGrad ? 1 : 2) k_contract(co
                                                                const MomJob* __restrict__ jobs,
                                                                const SysGeom* __restrict__ geoms,
                                                                const double* __restrict__ ztab,
-                                                               const double* __restrict__ rots,
-                                                               double* __restrict__ E, int32_t* __restrict__ status,
-                                                               double* __restrict__ G) {
+                                                               const EulerZYZ* __restrict__ rots,
+                                                               const PairOut* __restrict__ out) {
   extern __shared__ double2 sm2[];
   constexpr int kVWarps = kContractThreads / 32;
   __shared__ double she[kContractThreads];           // the virtual lanes' energy sums
@@ -352,6 +351,9 @@ __global__ void __launch_bounds__(kContractThreads, kGrad ? 1 : 2) k_contract(co
   // host uploaded ahead of the kernels (the d^l(pi/2) rows, the phase and power tables of the
   // frame, the moment sets' addresses), so it overlaps the tail of the kernel before.
   load_dpi2(Ds, ztab, L);
+  double* E = out->E;
+  int32_t* status = out->status;
+  double* G = out->G;
   const int bmode = d.b_mode;
   const double* pa = jobs[d.jobA].out;
   const double* pb = jobs[d.jobB].out;
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(kContractThreads, kGrad ? 1 : 2) k_contract(co
     const int lane = threadIdx.x & 31;
     const int ntask = bmode == kBRotate ? 7 : 4;
     for (int tt = threadIdx.x >> 5; tt < ntask; tt += blockDim.x >> 5) {
-      const EulerZYZ* e = reinterpret_cast<const EulerZYZ*>(rots) + d.rot;
+      const EulerZYZ* e = rots + d.rot;
       switch (tt) {
         case 0: in_phases(ph, make_double2(d.fr[4], d.fr[5]), L, lane); break;
         case 1: beta_phases(eb, d.fr[2], d.fr[3], L, lane); break;
@@ -672,21 +674,38 @@ int finalize_split(int n_jobs, int max_tiles, int max_slots) {
 }
 
 int launch_contract(const PairDesc* items, int n_items, int Lmax_items, const MomJob* jobs, const SysGeom* geoms,
-                    const double* ztab, const double* rots, double* E, int32_t* status, double* G, cudaStream_t s) {
+                    const double* ztab, const EulerZYZ* rots, const PairOut* out, bool grad, bool pdl, cudaStream_t s) {
   if (n_items <= 0) return 0;
   const int smem = contract_smem_bytes(Lmax_items);
   const int nt = contract_threads(Lmax_items, n_items);
-  if (G) {
-    if (raise_smem_limit(k_contract<true>, smem) != 0) return -1;
-    if (launch_pdl(k_contract<true>, dim3(n_items), dim3(nt), smem, s, items, jobs, geoms, ztab, rots, E, status, G) !=
-        cudaSuccess)
-      return -1;
-  } else {
-    if (raise_smem_limit(k_contract<false>, smem) != 0) return -1;
-    if (launch_pdl(k_contract<false>, dim3(n_items), dim3(nt), smem, s, items, jobs, geoms, ztab, rots, E, status,
-                   (double*)nullptr) != cudaSuccess)
-      return -1;
-  }
+  auto k = grad ? k_contract<true> : k_contract<false>;
+  if (raise_smem_limit(k, smem) != 0) return -1;
+  if (!pdl)
+    k<<<n_items, nt, smem, s>>>(items, jobs, geoms, ztab, rots, out);
+  else if (launch_pdl(k, dim3(n_items), dim3(nt), smem, s, items, jobs, geoms, ztab, rots, out) != cudaSuccess)
+    return -1;
+  return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
+}
+
+namespace {
+// One thread per item: about 15 double square roots and divisions for a rotated one, which cost the
+// host 100 to 150 ns an item (108,360 items of a surface scan: 2.6 ms of planning) and this kernel about
+// 20 us for all of them.
+__global__ void __launch_bounds__(128) k_frames(const PairSrc* __restrict__ src, int n_items, int n_computed,
+                                                const double* __restrict__ rotB, PairDesc* __restrict__ items,
+                                                EulerZYZ* __restrict__ rots) {
+  pdl_trigger();
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n_items) return;
+  PairDesc d;
+  make_pair(src[k], n_computed, rotB, d, rots);
+  items[k] = d;
+}
+}  // namespace
+
+int launch_frames(const PairSrc* src, int n_items, int n_computed, const double* rotB, PairDesc* items, EulerZYZ* rots,
+                  cudaStream_t s) {
+  k_frames<<<(n_items + 127) / 128, 128, 0, s>>>(src, n_items, n_computed, rotB, items, rots);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -23,8 +23,56 @@ struct PairDesc {  // one energy: moments of jobA and jobB at lmax L, separation
   int b_mode;      // kBLab, kBInFrame or kBRotate
   long long rot;   // kBRotate: index of the Euler record (EulerZYZ) of Mb = W rotB, which takes
                    // B's lab-frame moments into the frame, in the call's rotation array
-  double fr[6];    // R0 by its frame W = R_y(-b) R_z(-a) (pair_frame): 1/R, R, cos b, sin b, cos a, sin a
+  double fr[6];    // R0 by its frame W = R_y(-b) R_z(-a) (r0_frame): 1/R, R, cos b, sin b, cos a, sin a
 };
+
+// What the host writes for an item of a batch; the PairDesc (and Euler record) is made from it on the
+// host for small batches, by k_frames for large ones, with the same roundings (frame arithmetic below).
+struct PairSrc {
+  int jobA, jobB;  // computed jobs; ~k: the k-th cached set, which follow the computed ones
+  int geomA, geomB;
+  short L, b_mode;
+  int rot;
+  double R0[3];
+};
+
+// Where a batched call's results go (device; status and G may be null).
+struct PairOut {
+  double* E;
+  int32_t* status;
+  double* G;
+};
+
+// Frame arithmetic: every operation rounded by itself, on the device as on the host (where the build
+// does not contract either), so that an item's frame does not depend on where it is made.
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ double xmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double xadd(double a, double b) { return __dadd_rn(a, b); }
+#else
+inline double xmul(double a, double b) { return a * b; }
+inline double xadd(double a, double b) { return a + b; }
+#endif
+
+// The frame record of R0: 1/R, R, cos b = z/R, sin b = rho/R, e^{ia} = (x + iy)/rho (1 on the z axis).
+__host__ __device__ inline void r0_frame(const double* R0, double* fr) {
+  const double x = R0[0], y = R0[1], z = R0[2];
+  const double rho2 = xadd(xmul(x, x), xmul(y, y));
+  const double rho = sqrt(rho2), R = sqrt(xadd(rho2, xmul(z, z)));
+  fr[0] = 1.0 / R;
+  fr[1] = R;
+  fr[2] = z / R;
+  fr[3] = rho / R;
+  fr[4] = rho > 0.0 ? x / rho : 1.0;
+  fr[5] = rho > 0.0 ? y / rho : 0.0;
+}
+// W rot of a frame record: W = R_y(-b) R_z(-a) takes R0hat to the z axis (row-major).
+__host__ __device__ inline void frame_times(const double* fr, const double* rot, double* M) {
+  const double cb = fr[2], sb = fr[3], ca = fr[4], sa = fr[5];
+  const double W[9] = {xmul(cb, ca), xmul(cb, sa), -sb, -sa, ca, 0.0, xmul(sb, ca), xmul(sb, sa), cb};
+  for (int i = 0; i < 3; ++i)
+    for (int j = 0; j < 3; ++j)
+      M[3 * i + j] = xadd(xadd(xmul(W[3 * i], rot[j]), xmul(W[3 * i + 1], rot[3 + j])), xmul(W[3 * i + 2], rot[6 + j]));
+}
 
 // A rotation M = R_z(-gamma) R_y(-beta) R_z(-alpha), beta in [0, pi], as (cos beta, sin beta,
 // e^{i alpha}, e^{i gamma}).
@@ -39,34 +87,52 @@ struct EulerZYZ {
 //   e^{i(alpha+gamma)/2} = (w - i z) / cos(beta/2),  e^{i(alpha-gamma)/2} = (-y + i x) / sin(beta/2),
 // which stays accurate near beta = 0 and pi (where only alpha+gamma, resp. alpha-gamma, matters).
 __host__ __device__ inline EulerZYZ euler_zyz(const double* M) {
-  const double t = M[0] + M[4] + M[8];
+  const double t = xadd(xadd(M[0], M[4]), M[8]);
   double w, x, y, z;
   if (t > 0.0) {
-    const double s = 2.0 * sqrt(t + 1.0);
-    w = 0.25 * s; x = (M[7] - M[5]) / s; y = (M[2] - M[6]) / s; z = (M[3] - M[1]) / s;
+    const double s = xmul(2.0, sqrt(xadd(t, 1.0)));
+    w = xmul(0.25, s); x = xadd(M[7], -M[5]) / s; y = xadd(M[2], -M[6]) / s; z = xadd(M[3], -M[1]) / s;
   } else if (M[0] > M[4] && M[0] > M[8]) {
-    const double s = 2.0 * sqrt(1.0 + M[0] - M[4] - M[8]);
-    w = (M[7] - M[5]) / s; x = 0.25 * s; y = (M[1] + M[3]) / s; z = (M[2] + M[6]) / s;
+    const double s = xmul(2.0, sqrt(xadd(xadd(xadd(1.0, M[0]), -M[4]), -M[8])));
+    w = xadd(M[7], -M[5]) / s; x = xmul(0.25, s); y = xadd(M[1], M[3]) / s; z = xadd(M[2], M[6]) / s;
   } else if (M[4] > M[8]) {
-    const double s = 2.0 * sqrt(1.0 + M[4] - M[0] - M[8]);
-    w = (M[2] - M[6]) / s; x = (M[1] + M[3]) / s; y = 0.25 * s; z = (M[5] + M[7]) / s;
+    const double s = xmul(2.0, sqrt(xadd(xadd(xadd(1.0, M[4]), -M[0]), -M[8])));
+    w = xadd(M[2], -M[6]) / s; x = xadd(M[1], M[3]) / s; y = xmul(0.25, s); z = xadd(M[5], M[7]) / s;
   } else {
-    const double s = 2.0 * sqrt(1.0 + M[8] - M[0] - M[4]);
-    w = (M[3] - M[1]) / s; x = (M[2] + M[6]) / s; y = (M[5] + M[7]) / s; z = 0.25 * s;
+    const double s = xmul(2.0, sqrt(xadd(xadd(xadd(1.0, M[8]), -M[0]), -M[4])));
+    w = xadd(M[3], -M[1]) / s; x = xadd(M[2], M[6]) / s; y = xadd(M[5], M[7]) / s; z = xmul(0.25, s);
   }
-  const double n = 1.0 / sqrt(w * w + x * x + y * y + z * z);
-  w *= n; x *= n; y *= n; z *= n;
-  const double ch = sqrt(w * w + z * z), sh = sqrt(x * x + y * y);
+  const double c2 = xadd(xmul(w, w), xmul(z, z)), s2 = xadd(xmul(x, x), xmul(y, y));
+  const double n = 1.0 / sqrt(xadd(c2, s2));
+  w = xmul(w, n); x = xmul(x, n); y = xmul(y, n); z = xmul(z, n);
+  const double ch = sqrt(xadd(xmul(w, w), xmul(z, z))), sh = sqrt(xadd(xmul(x, x), xmul(y, y)));
   const double pr = ch > 0.0 ? w / ch : 1.0, pi = ch > 0.0 ? -z / ch : 0.0;   // p = e^{i(alpha+gamma)/2}
   const double qr = sh > 0.0 ? -y / sh : 1.0, qi = sh > 0.0 ? x / sh : 0.0;   // q = e^{i(alpha-gamma)/2}
   EulerZYZ e;
-  e.cb = (ch - sh) * (ch + sh);
-  e.sb = 2.0 * ch * sh;
-  e.ea[0] = pr * qr - pi * qi;  // p q
-  e.ea[1] = pr * qi + pi * qr;
-  e.eg[0] = pr * qr + pi * qi;  // p conj(q)
-  e.eg[1] = pi * qr - pr * qi;
+  e.cb = xmul(xadd(ch, -sh), xadd(ch, sh));
+  e.sb = xmul(xmul(2.0, ch), sh);
+  e.ea[0] = xadd(xmul(pr, qr), -xmul(pi, qi));  // p q
+  e.ea[1] = xadd(xmul(pr, qi), xmul(pi, qr));
+  e.eg[0] = xadd(xmul(pr, qr), xmul(pi, qi));  // p conj(q)
+  e.eg[1] = xadd(xmul(pi, qr), -xmul(pr, qi));
   return e;
+}
+
+// The descriptor of one item; rotB: the rotations of the kBRotate items.
+__host__ __device__ inline void make_pair(const PairSrc& s, int n_computed, const double* rotB, PairDesc& d, EulerZYZ* e) {
+  d.jobA = s.jobA >= 0 ? s.jobA : n_computed + ~s.jobA;
+  d.jobB = s.jobB >= 0 ? s.jobB : n_computed + ~s.jobB;
+  d.geomA = s.geomA;
+  d.geomB = s.geomB;
+  d.L = s.L;
+  d.b_mode = s.b_mode;
+  d.rot = s.rot;
+  r0_frame(s.R0, d.fr);
+  if (s.b_mode == kBRotate) {
+    double M[9];
+    frame_times(d.fr, rotB + 9LL * s.rot, M);
+    e[s.rot] = euler_zyz(M);
+  }
 }
 
 struct RotDesc {  // one moment set rotated about its centre: out = moments of (M x) from in
@@ -76,41 +142,22 @@ struct RotDesc {  // one moment set rotated about its centre: out = moments of (
   double M[9];
 };
 
-// G (optional, device, 9 doubles per item): force on B, torque on A, torque on B (lab frame).
-// rots: device, one EulerZYZ per kBRotate item (PairDesc.rot), or null when there is none.
+// out (device): where the results go; grad: also G, 9 doubles per item: force on B, torque on A, torque
+// on B (lab frame).  rots: device, one EulerZYZ per kBRotate item (PairDesc.rot), or null when there is
+// none.  pdl: the descriptors are complete before the kernel before this one.
 int launch_contract(const PairDesc* items, int n_items, int Lmax_items, const MomJob* jobs,
-                    const SysGeom* geoms, const double* ztab, const double* rots, double* E, int32_t* status,
-                    double* G, cudaStream_t s);
+                    const SysGeom* geoms, const double* ztab, const EulerZYZ* rots, const PairOut* out, bool grad,
+                    bool pdl, cudaStream_t s);
+// Descriptors of a large batch (n_items PairSrc -> PairDesc, Euler records).  Its successor on the stream
+// may start at once (and waits for it before it ends).
+int launch_frames(const PairSrc* src, int n_items, int n_computed, const double* rotB, PairDesc* items, EulerZYZ* rots,
+                  cudaStream_t s);
 int contract_smem_bytes(int L);
 int rotate_smem_bytes(int L);
 int launch_rotate_moments(const RotDesc* sets, int n_sets, int Lmax_sets, const double* ztab, cudaStream_t s);
 int contract_table_size();
 void contract_tables(double* t);  // host: fills contract_table_size() doubles
 
-// Rotation W = R_y(-beta) R_z(-alpha) taking R0hat to the z axis (row-major).
-__host__ __device__ inline void frame_rotation(const double* R0, double* W) {
-  const double x = R0[0], y = R0[1], z = R0[2];
-  const double R = sqrt(x * x + y * y + z * z);
-  const double rho = sqrt(x * x + y * y);
-  const double cb = z / R, sb = rho / R;
-  const double ca = rho > 0.0 ? x / rho : 1.0, sa = rho > 0.0 ? y / rho : 0.0;
-  W[0] = cb * ca; W[1] = cb * sa; W[2] = -sb;
-  W[3] = -sa;     W[4] = ca;      W[5] = 0.0;
-  W[6] = sb * ca; W[7] = sb * sa; W[8] = cb;
-}
-// Host: the frame record PairDesc.fr of R0 (cos b = z/R, sin b = rho/R, e^{ia} = (x + iy)/rho,
-// e^{ia} = 1 on the z axis).
-inline void pair_frame(const double* R0, PairDesc& d) {
-  const double x = R0[0], y = R0[1], z = R0[2];
-  const double rho = sqrt(x * x + y * y);
-  const double R = sqrt(x * x + y * y + z * z);
-  d.fr[0] = 1.0 / R;
-  d.fr[1] = R;
-  d.fr[2] = z / R;
-  d.fr[3] = rho / R;
-  d.fr[4] = rho > 0.0 ? x / rho : 1.0;
-  d.fr[5] = rho > 0.0 ? y / rho : 0.0;
-}
 // How the direct sum of one item is cut into CTAs (direct_split): parts = A blocks x B ranges of
 // chunk atoms; slab: items per launch (slab x parts partial sums).
 struct DirectSplit {

@@ -661,7 +661,7 @@ int sys_tile_atoms(long long) { return 1024; }
 // last trigger their successor on entry, and each of those waits for its predecessors before it ends
 // (in sequence, each with its own tail, they took 462 us for 2,048 uneven systems).
 int launch_sys(const SysJob* jobs, const SysCount& n, const SysTile* t1, const SysTile* t2, double* part, int* tickets,
-               SysGeom* geoms, cudaStream_t s) {
+               SysGeom* geoms, bool pdl, cudaStream_t s) {
   if (n.tiles1 > 0) {
     k_sys_centroid<<<(n.tiles1 + kSysWarps - 1) / kSysWarps, kSysThreads, 0, s>>>(jobs, t1, n.tiles1, part, tickets, geoms);
     if (cudaPeekAtLastError() != cudaSuccess) return -1;
@@ -669,7 +669,7 @@ int launch_sys(const SysJob* jobs, const SysCount& n, const SysTile* t1, const S
   if (n.tiles2 > 0 && launch_pdl(k_sys_radius_low, dim3((n.tiles2 + kSysWarps - 1) / kSysWarps), dim3(kSysThreads), 0, s,
                                  jobs, t2, n.tiles2, part, tickets, geoms, n.cluster + n.one > 0) != cudaSuccess)
     return -1;
-  const bool overlap = n.tiles2 > 0;  // (a centroid always comes with its radius)
+  const bool overlap = pdl || n.tiles2 > 0;  // (a centroid always comes with its radius)
   if (n.cluster > 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n.cluster * kSysClusterSize);

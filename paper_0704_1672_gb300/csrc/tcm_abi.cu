@@ -8,10 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <map>
-#include <unordered_map>
 #include <new>
-#include <tuple>
 #include <vector>
 
 #include "contract.h"
@@ -98,7 +95,13 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 }  // namespace
 
+namespace {
+struct BatchScratch;
+}
+
 struct tcm_ctx {
+  BatchScratch* scratch = nullptr;  // host arrays of the batched calls, kept for their capacity
+  void (*free_scratch)(BatchScratch*) = nullptr;
   int device = 0;
   int num_sms = 0;
   int lmax_cap = 0;
@@ -191,33 +194,46 @@ int dev_ensure(tcm_ctx* c, DevBuf& b, size_t bytes) {
   return TCM_OK;
 }
 
-// Copy the packed descriptors to the device through a pinned slot; returns the
-// device base address in *dbase.
-int upload(tcm_ctx* c, const Packer& pk, char** dbase) {
-  const size_t bytes = std::max<size_t>(pk.size, 1);
-  TRY(dev_ensure(c, c->desc, bytes));
+// The next pinned staging slot, free to write and at least `bytes` large; the first `keep` bytes of the
+// slot survive its growth.
+int stage_slot(tcm_ctx* c, size_t bytes, size_t keep, Stage** out) {
   Stage& st = c->stage[c->stage_next];
-  c->stage_next = (c->stage_next + 1) % kStages;
   if (st.pending) {
     TRY_CUDA(cudaEventSynchronize(st.ev));
     st.pending = false;
   }
   if (st.cap < bytes) {
-    if (st.host) TRY_CUDA(cudaFreeHost(st.host));
-    st.host = nullptr;
-    st.cap = 0;
-    const size_t nc = align_up(std::max<size_t>(bytes * 2, 4096));
-    if (cudaHostAlloc(&st.host, nc, cudaHostAllocDefault) != cudaSuccess) {
+    const size_t nc = align_up(std::max<size_t>(bytes + bytes / 2, 4096));
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, nc, cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
       return set_err(TCM_ENOMEM, "cudaHostAlloc of %zu bytes failed", nc);
     }
+    if (st.host) {
+      if (keep) std::memcpy(p, st.host, std::min(keep, st.cap));
+      cudaFreeHost(st.host);
+    }
+    st.host = p;
     st.cap = nc;
   }
+  *out = &st;
+  return TCM_OK;
+}
+
+// Copy the packed descriptors to the device through a pinned slot (its first `in_place` bytes were
+// written there by the caller, Packer's size began with them); returns the device base address in *dbase.
+// `behind` more bytes of the device buffer follow the block (at align_up(pk.size)) for the call's kernels.
+int upload(tcm_ctx* c, const Packer& pk, char** dbase, size_t in_place = 0, size_t behind = 0) {
+  const size_t bytes = std::max<size_t>(pk.size, 1);
+  TRY(dev_ensure(c, c->desc, align_up(bytes) + behind));
+  Stage* st = nullptr;
+  TRY(stage_slot(c, bytes, in_place, &st));
+  c->stage_next = (c->stage_next + 1) % kStages;
   for (const Packer::Span& sp : pk.spans)
-    if (sp.bytes) std::memcpy(static_cast<char*>(st.host) + sp.off, sp.p, sp.bytes);
-  TRY_CUDA(cudaMemcpyAsync(c->desc.p, st.host, bytes, cudaMemcpyHostToDevice, c->stream));
-  TRY_CUDA(cudaEventRecord(st.ev, c->stream));
-  st.pending = true;
+    if (sp.bytes) std::memcpy(static_cast<char*>(st->host) + sp.off, sp.p, sp.bytes);
+  TRY_CUDA(cudaMemcpyAsync(c->desc.p, st->host, bytes, cudaMemcpyHostToDevice, c->stream));
+  TRY_CUDA(cudaEventRecord(st->ev, c->stream));
+  st->pending = true;
   *dbase = static_cast<char*>(c->desc.p);
   return TCM_OK;
 }
@@ -253,7 +269,11 @@ struct Plan {
   // [tile_begin[p - 1], tile_begin[p])
   int tile_begin[kLmaxMax + 2] = {};
   int n_tile_ids = 0;
-  size_t moms_doubles = 0;
+  struct Group {
+    int job, chunk;
+  };
+  std::vector<Group> sort_groups;  // working arrays of build_tiles
+  std::vector<uint32_t> sort_key, sort_key2, sort_order, sort_order2;
 };
 
 void plan_job(tcm_ctx* c, int precision, MomJob& j, int& next_id) {
@@ -280,13 +300,11 @@ void build_tiles(int precision, Plan& P) {
   // 27 bits]; a stable sort keeps ties in their planning order, so the order is deterministic.
   // The sort is a least-significant-digit radix sort (three passes of 11 bits): for the tens of
   // thousands of groups of a large batch it takes a fraction of a comparison sort's time.
-  struct Group {
-    int job, chunk;
-  };
-  std::vector<Group> g;
-  std::vector<uint32_t> key;
-  g.reserve(P.jobs.size() * 2);
-  key.reserve(P.jobs.size() * 2);
+  using Group = Plan::Group;
+  std::vector<Group>& g = P.sort_groups;
+  std::vector<uint32_t>& key = P.sort_key;
+  g.clear();
+  key.clear();
   const bool by_degree = precision == TCM_FP64;
   for (int ji = 0; ji < (int)P.jobs.size(); ++ji) {
     const MomJob& j = P.jobs[ji];
@@ -300,7 +318,10 @@ void build_tiles(int precision, Plan& P) {
     }
   }
   const size_t n = key.size();
-  std::vector<uint32_t> order(n), k2(n), o2(n);
+  std::vector<uint32_t>&order = P.sort_order, &k2 = P.sort_key2, &o2 = P.sort_order2;
+  order.resize(n);
+  k2.resize(n);
+  o2.resize(n);
   for (size_t i = 0; i < n; ++i) order[i] = (uint32_t)i;
   for (int shift = 0; shift < 32; shift += 11) {
     uint32_t count[2049] = {};
@@ -362,10 +383,11 @@ int max_cols_of(const Plan& P, int plan) {
 // Queue the moment pass (step a2/a3) for every job of the plan.
 // The moment kernels' work counters and exit tickets (counters[L], counters[32 + L]) are zero
 // on entry and left zero by every launch, so they are cleared once, when allocated.
-int ensure_moment_buffers(tcm_ctx* c, int precision, const Plan& P) {
+int ensure_moment_buffers(tcm_ctx* c, int precision, const Plan& P, bool tiles_on_host) {
+  if (P.jobs.empty()) return TCM_OK;
   TRY(dev_ensure(c, c->partials, (size_t)std::max(P.n_tile_ids, 1) * plan_row(precision == TCM_FP64 ? 0 : 1) *
                                      sizeof(double)));
-  TRY(dev_ensure(c, c->tiles, (size_t)std::max(P.n_tiles, 1) * sizeof(MomTile)));
+  if (!tiles_on_host) TRY(dev_ensure(c, c->tiles, (size_t)std::max(P.n_tiles, 1) * sizeof(MomTile)));
   void* before = c->counters.p;
   TRY(dev_ensure(c, c->counters, 64 * sizeof(int)));
   if (c->counters.p != before) {
@@ -381,7 +403,7 @@ constexpr int kAnyCounter = kLmaxMax;  // + plan (1 or 2)
 
 int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, const MomTile* tiles,
                 const SysGeom* d_geoms, cudaStream_t st) {
-  TRY(ensure_moment_buffers(c, precision, P));
+  if (P.jobs.empty()) return TCM_OK;
   int* counters = static_cast<int*>(c->counters.p);
   double* parts = static_cast<double*>(c->partials.p);
   if (precision == TCM_FP64) {
@@ -428,13 +450,18 @@ struct SysPlan {
   SysCount n;
   std::vector<int> of_system;   // system -> index of its SysJob, or -1
   int rows = 0;
+  std::vector<SysJob> of_class[3];  // working arrays of plan_sys
 };
 
 // used[s]: system s takes part in the call; low[s]: its low-degree sums are needed.
 void plan_sys(const tcm_system* systems, int n_systems, const std::vector<char>& used, const std::vector<char>& low,
               SysPlan& S) {
   S.of_system.assign(std::max(n_systems, 0), -1);
-  std::vector<SysJob> of_class[3];
+  S.jobs.clear();
+  S.n = SysCount{};
+  S.rows = 0;
+  std::vector<SysJob>* of_class = S.of_class;
+  for (int k = 0; k < 3; ++k) of_class[k].clear();
   for (int s = 0; s < n_systems; ++s) {
     if (!used[s]) continue;
     const tcm_system& sy = systems[s];
@@ -470,8 +497,8 @@ void plan_sys(const tcm_system* systems, int n_systems, const std::vector<char>&
   }
   S.n.one = (int)of_class[0].size();
   S.n.cluster = (int)of_class[1].size();
-  for (auto& v : of_class)
-    for (SysJob& j : v) {
+  for (int k = 0; k < 3; ++k)
+    for (SysJob& j : of_class[k]) {
       if (j.need_low) j.sum_row = S.rows++;  // one sum row per system after the tile rows
       S.of_system[j.geom] = (int)S.jobs.size();
       S.jobs.push_back(j);
@@ -490,12 +517,14 @@ void link_low(const SysPlan& S, Plan& P) {
 
 // Partial rows and tickets of the system pass; the tickets are zeroed when allocated and every
 // launch leaves them zero.
-int ensure_sys_buffers(tcm_ctx* c, const SysPlan& S) {
+int ensure_sys_buffers(tcm_ctx* c, const SysPlan& S, bool tiles_on_host) {
+  if (S.jobs.empty()) return TCM_OK;
   TRY(dev_ensure(c, c->gpart, (size_t)std::max(S.rows, 1) * kSysPart * sizeof(double)));
+  if (S.n.tiles1 + S.n.tiles2 == 0) return TCM_OK;
   void* before = c->systk.p;
   TRY(dev_ensure(c, c->systk, std::max<size_t>(2 * S.jobs.size(), 64) * sizeof(int)));
   if (c->systk.p != before) TRY_CUDA(cudaMemsetAsync(c->systk.p, 0, c->systk.cap, c->stream));
-  TRY(dev_ensure(c, c->systiles, (size_t)std::max(S.n.tiles1 + S.n.tiles2, 1) * sizeof(SysTile)));
+  if (!tiles_on_host) TRY(dev_ensure(c, c->systiles, (size_t)std::max(S.n.tiles1 + S.n.tiles2, 1) * sizeof(SysTile)));
   return TCM_OK;
 }
 
@@ -514,6 +543,7 @@ struct Lists {
   void plan(const Plan* P, const SysPlan& S, Packer& pk) {
     const int nm = P ? P->n_tiles : 0, ns = S.n.tiles1 + S.n.tiles2;
     on_host = nm + ns <= kHostTiles;
+    o_mom = o_sys = 0;
     if (!on_host) return;
     mom.resize(nm);
     sys.resize(ns);
@@ -543,7 +573,7 @@ int run_sys(tcm_ctx* c, const SysPlan& S, const Lists& T, const SysJob* d_sj, Sy
   if (S.jobs.empty()) return TCM_OK;
   PhaseScope ps(c, TCM_PHASE_GEOM, sys_launches(S.n));
   TRY_LAUNCH(launch_sys(d_sj, S.n, T.d_sys, T.d_sys + S.n.tiles1, static_cast<double*>(c->gpart.p),
-                        static_cast<int*>(c->systk.p), d_geo, st));
+                        static_cast<int*>(c->systk.p), d_geo, true, st));
   return TCM_OK;
 }
 
@@ -606,6 +636,7 @@ int build_tables(tcm_ctx* c) {
 
 void free_ctx(tcm_ctx* c) {
   if (!c) return;
+  if (c->scratch) c->free_scratch(c->scratch);
   cudaStreamSynchronize(c->stream);
   cudaFree(c->d_fmap);
   cudaFree(c->d_ztab);
@@ -807,7 +838,7 @@ int tcm_prepare(tcm_ctx_t c, tcm_system* s) {
   const size_t o_geo = pk.add(geoms), o_sj = pk.add(S.jobs);
   Lists T;
   T.plan(nullptr, S, pk);
-  TRY(ensure_sys_buffers(c, S));
+  TRY(ensure_sys_buffers(c, S, T.on_host));
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
@@ -858,8 +889,8 @@ int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, i
   const size_t o_geo = pk.add(geoms), o_job = pk.add(P.jobs), o_tile = pk.add(P.groups), o_sj = pk.add(S.jobs);
   Lists T;
   T.plan(&P, S, pk);
-  TRY(ensure_moment_buffers(c, precision, P));
-  TRY(ensure_sys_buffers(c, S));
+  TRY(ensure_moment_buffers(c, precision, P, T.on_host));
+  TRY(ensure_sys_buffers(c, S, T.on_host));
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
@@ -903,19 +934,20 @@ int tcm_energy(tcm_ctx_t c, const tcm_moments_t* A, const tcm_moments_t* B, cons
   geoms[0].a = A->radius;
   geoms[1].a = B->radius;
   std::vector<PairDesc> items(1);
-  items[0] = PairDesc{0, 1, 0, 1, lmax, kBLab, 0, {}};
-  pair_frame(R0, items[0]);
-  Packer pk;
-  const size_t o_job = pk.add(jobs), o_geo = pk.add(geoms), o_it = pk.add(items);
-  char* base = nullptr;
-  TRY(upload(c, pk, &base));
+  PairSrc src{0, 1, 0, 1, (short)lmax, kBLab, 0, {R0[0], R0[1], R0[2]}};
+  make_pair(src, 2, nullptr, items[0], nullptr);
   TRY(dev_ensure(c, c->escr, 64));
   double* dE = static_cast<double*>(c->escr.p);
+  std::vector<PairOut> out{PairOut{dE, nullptr, nullptr}};
+  Packer pk;
+  const size_t o_job = pk.add(jobs), o_geo = pk.add(geoms), o_it = pk.add(items), o_out = pk.add(out);
+  char* base = nullptr;
+  TRY(upload(c, pk, &base));
   {
     PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
     TRY_LAUNCH(launch_contract(reinterpret_cast<PairDesc*>(base + o_it), 1, lmax,
                                reinterpret_cast<MomJob*>(base + o_job), reinterpret_cast<SysGeom*>(base + o_geo),
-                               c->d_ztab, nullptr, dE, nullptr, nullptr, c->stream));
+                               c->d_ztab, nullptr, reinterpret_cast<PairOut*>(base + o_out), false, true, c->stream));
   }
   TRY_CUDA(cudaMemcpyAsync(c->pinned_small, dE, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   TRY_CUDA(cudaStreamSynchronize(c->stream));
@@ -971,7 +1003,12 @@ namespace {
 int timed_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t n_items, const tcm_pair_item* items,
                 int precision, double* E, int32_t* status, double* G) {
   const auto t0 = std::chrono::steady_clock::now();
-  const int rc = energy_batch(c, n_systems, systems, n_items, items, precision, E, status, G);
+  int rc;
+  try {
+    rc = energy_batch(c, n_systems, systems, n_items, items, precision, E, status, G);
+  } catch (const std::bad_alloc&) {
+    rc = set_err(TCM_ENOMEM, "tcm_energy_batch: host allocation failed");
+  }
   if (c && c->prof) c->host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   return rc;
 }
@@ -989,6 +1026,45 @@ int tcm_gradients_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, i
 }
 
 namespace {
+// Items from which their descriptors are made on the device.
+constexpr int64_t kDeviceFrames = 128;
+
+// Host arrays of the batched calls (one context, one thread at a time): cleared, not freed, between calls,
+// and lookups stamped with the call's epoch instead of being cleared.
+struct BatchScratch {
+  Plan P;
+  SysPlan S;
+  Lists T;
+  std::vector<PairSrc> src;
+  std::vector<PairDesc> pd;
+  std::vector<EulerZYZ> rots;
+  std::vector<double> rotB;
+  std::vector<MomJob> cached;
+  std::vector<size_t> job_moff;
+  std::vector<SysGeom> geoms;
+  std::vector<PairOut> out;
+  std::vector<char> used, low;
+  std::vector<uint64_t> job_of, cached_of;  // epoch << 32 | index, by (system, degree) and by system
+  uint32_t epoch = 0;
+  std::vector<long long> key;
+
+  void begin(int n_systems) {
+    if (++epoch == 0) {  // wrapped: no stamp of the past may match
+      std::fill(job_of.begin(), job_of.end(), 0);
+      std::fill(cached_of.begin(), cached_of.end(), 0);
+      epoch = 1;
+    }
+    if (job_of.size() < (size_t)n_systems * (kLmaxMax + 1)) job_of.resize((size_t)n_systems * (kLmaxMax + 1), 0);
+    if (cached_of.size() < (size_t)n_systems) cached_of.resize(n_systems, 0);
+    used.assign(n_systems, 0);
+    low.assign(n_systems, 0);
+    P.jobs.clear();
+    rotB.clear();
+    cached.clear();
+    job_moff.clear();
+  }
+};
+
 int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t n_items, const tcm_pair_item* items,
                  int precision, double* E, int32_t* status, double* G) {
   TRY(check_ctx(c));
@@ -997,57 +1073,34 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   if (!systems || !items || !E) return set_err(TCM_EINVAL, "tcm_energy_batch: null argument");
   if (n_items > (1LL << 30)) return set_err(TCM_EINVAL, "tcm_energy_batch: too many items");
   if (precision != TCM_FP64 && precision != TCM_MIXED) return set_err(TCM_EINVAL, "tcm_energy_batch: bad precision");
-  std::vector<char> used(n_systems, 0);
-  for (int64_t k = 0; k < n_items; ++k) {
-    const tcm_pair_item& it = items[k];
-    if (it.a < 0 || it.a >= n_systems || it.b < 0 || it.b >= n_systems)
-      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld refers to a system outside [0, %d)", (long long)k, n_systems);
-    if (it.lmax < 0 || it.lmax > c->lmax_cap)
-      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld lmax %d outside [0, %d]", (long long)k, it.lmax, c->lmax_cap);
-    used[it.a] = used[it.b] = 1;
+  if (!c->scratch) {
+    c->scratch = new BatchScratch;
+    c->free_scratch = [](BatchScratch* s) { delete s; };
   }
-  for (int s = 0; s < n_systems; ++s)
-    if (used[s]) TRY(check_system(&systems[s], "tcm_energy_batch"));
-  // host-known radii: reject non-convergent items before any work is queued
-  for (int64_t k = 0; k < n_items; ++k) {
-    const tcm_pair_item& it = items[k];
-    if (geom_known(systems[it.a]) && geom_known(systems[it.b])) {
-      const double R = std::sqrt(it.R0[0] * it.R0[0] + it.R0[1] * it.R0[1] + it.R0[2] * it.R0[2]);
-      const double aa = systems[it.a].radius + systems[it.b].radius;
-      if (!(R > aa))
-        return set_err(TCM_ENOTCONV, "tcm_energy_batch: item %lld: |R0| = %.17g <= a_A + a_B = %.17g (Eq. (mainCond))",
-                       (long long)k, R, aa);
-    }
+  BatchScratch& B = *c->scratch;
+  B.begin(n_systems);
+  Plan& P = B.P;
+  // Large batches: the items' descriptors are made on the device (k_frames) from records written straight
+  // into the staging slot; small ones on the host (a launch costs more than their square roots).
+  const bool on_device = n_items >= kDeviceFrames;
+  PairSrc* src = nullptr;
+  size_t in_place = 0;
+  if (on_device) {
+    in_place = (size_t)n_items * sizeof(PairSrc);
+    Stage* st = nullptr;
+    TRY(stage_slot(c, in_place + in_place / 4 + 65536, 0, &st));
+    src = static_cast<PairSrc*>(st->host);
+  } else {
+    B.src.resize(n_items);
+    src = B.src.data();
   }
-  // moment jobs (A sides and unrotated B sides shared)
-  Plan P;
-  std::unordered_map<long long, int> job_of;  // unrotated jobs by (system, Lmax)
-  job_of.reserve((size_t)std::min<int64_t>(n_items, 1 << 20) * 2);
-  P.jobs.reserve((size_t)std::min<int64_t>(n_items, 1 << 20) * 2);
-  std::vector<PairDesc> pd(n_items);
-  int next_id = 0;
+  // One pass over the items: checks, moment jobs (A sides and unrotated B sides shared), records.
+  int next_id = 0, Lmax_items = 0;
   size_t moff = 0;
-  std::vector<size_t> job_moff;
-  std::vector<MomJob> cached;  // unrotated sides served from a system's moment cache
-  std::map<int, int> cached_of;
-  auto get_job = [&](int sys, int L, int rot_item, const double* rot, bool use_cache = true) {
-    if (rot_item < 0 && use_cache && systems[sys].moments && L <= systems[sys].moments_lmax) {
-      auto c = cached_of.find(sys);
-      if (c != cached_of.end()) return -2 - c->second;
-      MomJob j{};
-      j.L = systems[sys].moments_lmax;
-      j.geom = sys;
-      j.out = const_cast<double*>(systems[sys].moments);
-      cached.push_back(j);
-      cached_of[sys] = (int)cached.size() - 1;
-      return -2 - ((int)cached.size() - 1);
-    }
-    const long long key = (long long)sys * (kLmaxMax + 1) + L;
-    if (rot_item < 0) {  // rotated jobs are unique to their item: no lookup
-      auto itr = job_of.find(key);
-      if (itr != job_of.end()) return itr->second;
-    }
-    MomJob j{};
+  auto new_job = [&](int sys, int L, const double* rot) {
+    P.jobs.emplace_back();
+    MomJob& j = P.jobs.back();
+    j = MomJob{};
     j.xyzq = systems[sys].xyzq;
     j.n = systems[sys].n;
     j.dtype = systems[sys].dtype;
@@ -1058,18 +1111,64 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     else
       identity(j.rot);
     plan_job(c, precision, j, next_id);
-    job_moff.push_back(moff);
+    B.job_moff.push_back(moff);
     moff += (size_t)(L + 1) * (L + 1);
-    const int id = (int)P.jobs.size();
-    P.jobs.push_back(j);
-    if (rot_item < 0) job_of[key] = id;
-    return id;
+    return (int)P.jobs.size() - 1;
   };
-  std::vector<EulerZYZ> rots;  // Euler record of W rotB per rotate-from-cache item
+  // the unrotated set of (system, L): from the system's moment cache (~index) or computed (index)
+  auto unrotated = [&](int sys, int L, bool use_cache) {
+    const tcm_system& sy = systems[sys];
+    if (use_cache && sy.moments && L <= sy.moments_lmax) {
+      uint64_t& e = B.cached_of[sys];
+      if ((e >> 32) != B.epoch) {
+        MomJob j{};
+        j.L = sy.moments_lmax;
+        j.geom = sys;
+        j.out = const_cast<double*>(sy.moments);
+        e = (uint64_t)B.epoch << 32 | (uint32_t)B.cached.size();
+        B.cached.push_back(j);
+      }
+      return ~(int)(uint32_t)e;
+    }
+    uint64_t& e = B.job_of[(size_t)sys * (kLmaxMax + 1) + L];
+    if ((e >> 32) != B.epoch) e = (uint64_t)B.epoch << 32 | (uint32_t)new_job(sys, L, nullptr);
+    return (int)(uint32_t)e;
+  };
+  int64_t nc_item = -1;  // first item that a host-known radius shows not to converge
+  double nc_R = 0.0, nc_a = 0.0;
   for (int64_t k = 0; k < n_items; ++k) {
     const tcm_pair_item& it = items[k];
-    const int ja = get_job(it.a, it.lmax, -1, nullptr);
-    int jb;
+    if (it.a < 0 || it.a >= n_systems || it.b < 0 || it.b >= n_systems)
+      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld refers to a system outside [0, %d)", (long long)k, n_systems);
+    if (it.lmax < 0 || it.lmax > c->lmax_cap)
+      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld lmax %d outside [0, %d]", (long long)k, it.lmax, c->lmax_cap);
+    B.used[it.a] = B.used[it.b] = 1;
+    const tcm_system &sa = systems[it.a], &sb = systems[it.b];
+    if (geom_known(sa) && geom_known(sb) && nc_item < 0) {
+      const double R2 = it.R0[0] * it.R0[0] + it.R0[1] * it.R0[1] + it.R0[2] * it.R0[2];
+      const double aa = sa.radius + sb.radius;
+      if (!(R2 > aa * aa * (1.0 + 1e-12))) {  // (the square root only near the limit)
+        const double R = std::sqrt(R2);
+        if (!(R > aa)) {
+          nc_item = k;
+          nc_R = R;
+          nc_a = aa;
+        }
+      }
+    }
+    Lmax_items = std::max(Lmax_items, (int)it.lmax);
+    PairSrc& p = src[k];
+    p.geomA = it.a;
+    p.geomB = it.b;
+    p.L = (short)it.lmax;
+    p.rot = 0;
+    for (int d = 0; d < 3; ++d) p.R0[d] = it.R0[d];
+    p.jobA = unrotated(it.a, it.lmax, true);
+    if (!it.has_rot) {
+      p.b_mode = kBLab;
+      p.jobB = unrotated(it.b, it.lmax, true);
+      continue;
+    }
     // B's lab-frame moments, taken into the frame by W rotB inside the contraction:
     //   from_cache  the caller asked for it and B carries its moments;
     //   from_lab    double path: computed once per (system, degree) from B's atoms and shared by all
@@ -1079,95 +1178,99 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     //               13 ms, at the same error.  Only for matrices that are rotations to rounding; any
     //               other matrix acts on the atoms, as before.  The mixed path keeps each item's own
     //               float sums over the rotated atoms, whose rounding errors are independent.
-    const bool from_cache = c->rotate_cached && systems[it.b].moments && it.lmax <= systems[it.b].moments_lmax;
-    const bool from_lab = precision == TCM_FP64 && it.has_rot && is_rotation(it.rotB);
-    if (it.has_rot && (from_cache || from_lab)) {
-      double W[9];
-      frame_rotation(it.R0, W);
-      jb = get_job(it.b, it.lmax, -1, nullptr, from_cache);
-      pd[k] = PairDesc{ja, jb, it.a, it.b, it.lmax, kBRotate, (long long)rots.size(), {}};
-      pair_frame(it.R0, pd[k]);
-      double M[9];
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j)
-          M[3 * i + j] = W[3 * i + 0] * it.rotB[0 + j] + W[3 * i + 1] * it.rotB[3 + j] + W[3 * i + 2] * it.rotB[6 + j];
-      rots.push_back(euler_zyz(M));
-      continue;
-    }
-    if (it.has_rot) {
+    const bool from_cache = c->rotate_cached && sb.moments && it.lmax <= sb.moments_lmax;
+    if (from_cache || (precision == TCM_FP64 && is_rotation(it.rotB))) {
+      p.b_mode = kBRotate;
+      p.rot = (int)(B.rotB.size() / 9);
+      B.rotB.insert(B.rotB.end(), it.rotB, it.rotB + 9);
+      p.jobB = unrotated(it.b, it.lmax, from_cache);
+    } else {
       // B is moved per item anyway: fold the rotation W that takes R0hat to z into its
       // atom transform, so the contraction receives B's moments already in that frame.
-      double W[9], M[9];
-      frame_rotation(it.R0, W);
-      for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j)
-          M[3 * i + j] = W[3 * i + 0] * it.rotB[0 + j] + W[3 * i + 1] * it.rotB[3 + j] + W[3 * i + 2] * it.rotB[6 + j];
-      jb = get_job(it.b, it.lmax, (int)k, M);
-    } else {
-      jb = get_job(it.b, it.lmax, -1, nullptr);
+      double fr[6], M[9];
+      r0_frame(it.R0, fr);
+      frame_times(fr, it.rotB, M);
+      p.b_mode = kBInFrame;
+      p.jobB = new_job(it.b, it.lmax, M);
     }
-    pd[k] = PairDesc{ja, jb, it.a, it.b, it.lmax, it.has_rot ? kBInFrame : kBLab, 0, {}};
-    pair_frame(it.R0, pd[k]);
   }
+  for (int s = 0; s < n_systems; ++s)
+    if (B.used[s]) TRY(check_system(&systems[s], "tcm_energy_batch"));
+  if (nc_item >= 0)  // rejected before any work is queued
+    return set_err(TCM_ENOTCONV, "tcm_energy_batch: item %lld: |R0| = %.17g <= a_A + a_B = %.17g (Eq. (mainCond))",
+                   (long long)nc_item, nc_R, nc_a);
   P.n_tile_ids = next_id;
   TRY(dev_ensure(c, c->moms, std::max<size_t>(moff, 1) * sizeof(double)));
-  for (size_t ji = 0; ji < P.jobs.size(); ++ji) P.jobs[ji].out = static_cast<double*>(c->moms.p) + job_moff[ji];
+  for (size_t ji = 0; ji < P.jobs.size(); ++ji) P.jobs[ji].out = static_cast<double*>(c->moms.p) + B.job_moff[ji];
   build_tiles(precision, P);
-  std::vector<char> low(n_systems, 0);
   if (precision == TCM_MIXED)
-    for (const MomJob& j : P.jobs) low[j.geom] = 1;
-  SysPlan S;
-  plan_sys(systems, n_systems, used, low, S);
+    for (const MomJob& j : P.jobs) B.low[j.geom] = 1;
+  SysPlan& S = B.S;
+  plan_sys(systems, n_systems, B.used, B.low, S);
   link_low(S, P);
-  // cached sides follow the computed jobs in the descriptor array (not finalised)
-  const int n_computed = (int)P.jobs.size();
-  for (auto& d : pd) {
-    if (d.jobA <= -2) d.jobA = n_computed + (-2 - d.jobA);
-    if (d.jobB <= -2) d.jobB = n_computed + (-2 - d.jobB);
-  }
-  int Lmax_items = 0;
-  for (int64_t k = 0; k < n_items; ++k) Lmax_items = std::max(Lmax_items, (int)items[k].lmax);
-  std::vector<SysGeom> geoms(std::max(n_systems, 1));
-  for (int s = 0; s < n_systems; ++s) geoms[s] = host_geom(systems[s]);
+  const int n_computed = (int)P.jobs.size();  // cached sides follow them in the descriptor array (not finalised)
+  const int n_rot = (int)(B.rotB.size() / 9);
+  B.geoms.resize(std::max(n_systems, 1));
+  for (int s = 0; s < n_systems; ++s) B.geoms[s] = host_geom(systems[s]);
+  B.out.assign(1, PairOut{E, status, G});
   Packer pk;
-  const size_t o_geo = pk.add(geoms), o_job = pk.add2(P.jobs, cached), o_tile = pk.add(P.groups), o_sj = pk.add(S.jobs),
-               o_it = pk.add(pd), o_rot = pk.add(rots);
-  Lists T;
+  pk.size = in_place;
+  const size_t o_geo = pk.add(B.geoms), o_job = pk.add2(P.jobs, B.cached), o_tile = pk.add(P.groups),
+               o_sj = pk.add(S.jobs), o_out = pk.add(B.out);
+  size_t o_it = 0, o_rot = 0;
+  if (on_device) {
+    o_rot = pk.add(B.rotB);
+  } else {
+    B.pd.resize(n_items);
+    B.rots.resize(n_rot);
+    for (int64_t k = 0; k < n_items; ++k) make_pair(src[k], n_computed, B.rotB.data(), B.pd[k], B.rots.data());
+    o_it = pk.add(B.pd);
+    o_rot = pk.add(B.rots);
+  }
+  Lists& T = B.T;
   T.plan(&P, S, pk);
   // every buffer the launches touch is sized before anything is queued (no reallocation
   // may happen while a graph is being captured)
-  TRY(ensure_sys_buffers(c, S));
-  TRY(ensure_moment_buffers(c, precision, P));
+  TRY(ensure_sys_buffers(c, S, T.on_host));
+  TRY(ensure_moment_buffers(c, precision, P, T.on_host));
   char* base = nullptr;
-  TRY(upload(c, pk, &base));
+  TRY(upload(c, pk, &base, in_place,
+             on_device ? (size_t)n_items * sizeof(PairDesc) + (size_t)n_rot * sizeof(EulerZYZ) : 0));
   SysGeom* d_geo = reinterpret_cast<SysGeom*>(base + o_geo);
   const MomJob* d_jobs = reinterpret_cast<MomJob*>(base + o_job);
   T.place(c, base);
+  PairDesc* d_items = reinterpret_cast<PairDesc*>(base + (on_device ? align_up(pk.size) : o_it));
+  EulerZYZ* d_rots = on_device ? reinterpret_cast<EulerZYZ*>(d_items + n_items) : reinterpret_cast<EulerZYZ*>(base + o_rot);
+  const bool no_moments = P.jobs.empty() && S.jobs.empty();
   auto enqueue = [&](cudaStream_t st) -> int {
     const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
     TRY(run_expand(c, P.groups, d_jobs, reinterpret_cast<MomGroup*>(base + o_tile), S, T, d_sj, st));
+    if (on_device) {
+      PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
+      TRY_LAUNCH(launch_frames(reinterpret_cast<PairSrc*>(base), (int)n_items, n_computed,
+                               reinterpret_cast<double*>(base + o_rot), d_items, d_rots, st));
+    }
     TRY(run_sys(c, S, T, d_sj, d_geo, st));
     TRY(run_moments(c, precision, P, d_jobs, T.d_mom, d_geo, st));
     PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
-    TRY_LAUNCH(launch_contract(reinterpret_cast<PairDesc*>(base + o_it), (int)n_items, Lmax_items, d_jobs, d_geo,
-                               c->d_ztab, rots.empty() ? nullptr : reinterpret_cast<double*>(base + o_rot), E,
-                               status, G, st));
+    // (directly behind k_frames the contraction must not read the descriptors ahead of its end)
+    TRY_LAUNCH(launch_contract(d_items, (int)n_items, Lmax_items, d_jobs, d_geo, c->d_ztab, n_rot ? d_rots : nullptr,
+                               reinterpret_cast<PairOut*>(base + o_out), G != nullptr, !(on_device && no_moments), st));
     return TCM_OK;
   };
   if (!c->graphs || c->prof || !c->cap_stream) return enqueue(c->stream);
   // Replay a captured graph of the launch sequence when this call has the same shape and
   // buffers as the captured one (only the uploaded descriptor contents differ).
   const bool cols = precision == TCM_MIXED && moments_use_cols(P.n_tiles, c->num_sms);
-  std::vector<long long> key = {precision, split_of(P), cols ? max_cols_of(P, 1) : 0, cols ? max_cols_of(P, 2) : 0, G != nullptr, (long long)(uintptr_t)G, (long long)S.jobs.size(),
-                                S.n.one, S.n.cluster, S.n.tiles1, S.n.tiles2, (long long)T.o_mom, (long long)T.o_sys,
-                                T.on_host, (long long)P.jobs.size(), P.n_tile_ids,
-                                (long long)n_items, Lmax_items, (long long)o_geo, (long long)o_job, (long long)o_tile,
-                                (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)(uintptr_t)c->systiles.p,
-                                (long long)rots.empty(), (long long)(uintptr_t)base, (long long)(uintptr_t)c->gpart.p,
-                                (long long)(uintptr_t)c->systk.p, (long long)(uintptr_t)c->partials.p,
-                                (long long)(uintptr_t)c->counters.p, (long long)(uintptr_t)E, (long long)(uintptr_t)status,
-                                (long long)P.groups.size(), (long long)P.n_tiles, (long long)(uintptr_t)c->tiles.p,
-                                (long long)c->cfg_gen};
+  std::vector<long long>& key = B.key;
+  key = {precision, split_of(P), cols ? max_cols_of(P, 1) : 0, cols ? max_cols_of(P, 2) : 0, G != nullptr, S.n.one,
+         S.n.cluster, S.n.tiles1, S.n.tiles2, (long long)S.jobs.size(), (long long)T.o_mom, (long long)T.o_sys, T.on_host,
+         (long long)P.jobs.size(), P.n_tile_ids, (long long)n_items, n_rot, Lmax_items, (long long)o_geo, (long long)o_job,
+         (long long)o_tile, (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)o_out,
+         (long long)pk.size, (long long)(uintptr_t)c->systiles.p, (long long)(uintptr_t)base,
+         (long long)(uintptr_t)c->gpart.p, (long long)(uintptr_t)c->systk.p, (long long)(uintptr_t)c->partials.p,
+         (long long)(uintptr_t)c->counters.p, (long long)P.groups.size(), (long long)P.n_tiles,
+         (long long)(uintptr_t)c->tiles.p, (long long)c->cfg_gen};
   for (int L = 0; L <= kLmaxMax + 1; ++L) key.push_back(P.tile_begin[L]);
   if (!c->gexec || key != c->gkey) {
     // by default capture only a shape seen twice in a row: a stream of changing shapes
@@ -1204,8 +1307,9 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   TRY_CUDA(cudaGraphLaunch(c->gexec, c->stream));
   ++c->graph_launches;
   c->launches[TCM_PHASE_GEOM] += sys_launches(S.n) + !T.on_host;
+  c->launches[TCM_PHASE_CONTRACT] += on_device;
   c->launches[TCM_PHASE_MOMENTS] += moment_launches(precision, P);
-  c->launches[TCM_PHASE_FINALIZE] += 1;
+  c->launches[TCM_PHASE_FINALIZE] += !P.jobs.empty();
   c->launches[TCM_PHASE_CONTRACT] += 1;
   return TCM_OK;
 }
@@ -1235,7 +1339,7 @@ int direct_items(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t 
   Lists T;
   T.plan(nullptr, S, pk);
   const DirectSplit split = direct_split(A->n, B->n);
-  TRY(ensure_sys_buffers(c, S));
+  TRY(ensure_sys_buffers(c, S, T.on_host));
   TRY(dev_ensure(c, c->dpart, (size_t)std::max<int64_t>((int64_t)split.parts * std::min<int64_t>(n, split.slab), 1) * sizeof(double)));
   char* base = nullptr;
   TRY(upload(c, pk, &base));

@@ -291,9 +291,10 @@ void finalize_tables(std::vector<int>& imap_off, std::vector<int>& imap, std::ve
 
 // Step a1 and the low-degree sums: the jobs of class 0, then those of class 1, then the tiles of the
 // others (centroid, then radius and sums).  part: kSysPart doubles per row; tickets: two ints per job,
-// zero on entry and left zero.
+// zero on entry and left zero.  pdl: a kernel before on the stream wrote none of the jobs and geoms, so
+// the systems' kernels may start while it drains (they wait for it before they end).
 int launch_sys(const SysJob* jobs, const SysCount& n, const SysTile* t1, const SysTile* t2, double* part, int* tickets,
-               SysGeom* geoms, cudaStream_t s);
+               SysGeom* geoms, bool pdl, cudaStream_t s);
 int sys_launches(const SysCount& n);
 int sys_class(long long n, int dtype);
 int sys_tile_atoms(long long n);

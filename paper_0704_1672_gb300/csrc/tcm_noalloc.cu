@@ -203,7 +203,7 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   if (cudaPeekAtLastError() != cudaSuccess) return na_err(TCM_ECUDA, "tcm_moments_noalloc: launch failed");
   if (launch_sys(reinterpret_cast<SysJob*>(base + kOffSJob), ns, reinterpret_cast<SysTile*>(base + kOffSTiles1),
                  reinterpret_cast<SysTile*>(base + kOffSTiles2), reinterpret_cast<double*>(base + kOffSPart),
-                 reinterpret_cast<int*>(base + kOffCounters) + 40, d_geom, st) != 0)
+                 reinterpret_cast<int*>(base + kOffCounters) + 40, d_geom, false, st) != 0)
     return na_err(TCM_ECUDA, "tcm_moments_noalloc: centre/radius launch failed");
   int num_sms = 0;
   if (cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)

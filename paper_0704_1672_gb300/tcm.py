@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 
 import numpy as np
@@ -106,9 +107,12 @@ def _check(rc):
 
 def _dptr(arr):
     """Host pointer of a contiguous float64 numpy array (or None)."""
-    if arr is None:
-        return None
-    return arr.ctypes.data_as(ctypes.c_void_p)
+    return None if arr is None else arr.ctypes.data
+
+
+# the fields of tcm_system in order, packed at once: setting them one by one costs several times as much
+_SYSTEM = struct.Struct("@Pqii4dPii")
+assert _SYSTEM.size == ctypes.sizeof(tcm_system)
 
 
 def make_system(xyzq: torch.Tensor, center=None, radius=None, moments: "MomentSet | None" = None) -> tcm_system:
@@ -126,19 +130,12 @@ def make_system(xyzq: torch.Tensor, center=None, radius=None, moments: "MomentSe
         dt = TCM_F64
     else:
         raise TcmError(TCM_EINVAL, "coordinates must be float32 or float64")
-    s = tcm_system()
-    s.xyzq = xyzq.data_ptr() if xyzq.numel() else None
-    s.n = xyzq.shape[0]
-    s.dtype = dt
-    if center is not None:
-        s.has_center = 1
-        for k in range(3):
-            s.center[k] = float(center[k])
-    s.radius = -1.0 if radius is None else float(radius)
-    if moments is not None:
-        s.moments = moments.q.data_ptr()
-        s.moments_lmax = moments.lmax
-    return s
+    n = xyzq.shape[0]
+    x, y, z = (0.0, 0.0, 0.0) if center is None else (float(center[0]), float(center[1]), float(center[2]))
+    return tcm_system.from_buffer_copy(_SYSTEM.pack(
+        xyzq.data_ptr() if n else 0, n, dt, 0 if center is None else 1, x, y, z,
+        -1.0 if radius is None else float(radius), 0 if moments is None else moments.q.data_ptr(),
+        0 if moments is None else moments.lmax, 0))
 
 
 @dataclass
@@ -303,14 +300,12 @@ class Context:
     def tcm_energy_batch_packed(self, pb: "PackedBatch", precision=TCM_MIXED, E=None, status=None):
         """tcm_energy_batch on arguments already marshalled by ``pack_batch``."""
         k = len(pb.items)
-        dev = torch.device("cuda", torch.cuda.current_device())
         if E is None:
-            E = torch.empty(k, dtype=torch.float64, device=dev)
+            E = torch.empty(k, dtype=torch.float64, device="cuda")
         if status is None:
-            status = torch.empty(k, dtype=torch.int32, device=dev)
-        _check(lib().tcm_energy_batch(self._h, pb.n_systems, ctypes.cast(pb.sys_arr, ctypes.c_void_p), k,
-                                      pb.items.ctypes.data_as(ctypes.c_void_p), int(precision),
-                                      ctypes.c_void_p(E.data_ptr()), ctypes.c_void_p(status.data_ptr())))
+            status = torch.empty(k, dtype=torch.int32, device="cuda")
+        _check(lib().tcm_energy_batch(self._h, pb.n_systems, ctypes.addressof(pb.sys_arr), k, pb.items.ctypes.data,
+                                      int(precision), E.data_ptr(), status.data_ptr()))
         return E, status
 
     def tcm_gradients_batch(self, systems, a, b, lmax, R0, rotB=None, precision=TCM_MIXED, E=None, G=None,
@@ -320,17 +315,14 @@ class Context:
         Returns (E, G, status): G is a (k, 9) device tensor [F_B, tau_A, tau_B] per item."""
         pb = pack_batch(systems, a, b, lmax, R0, rotB)
         k = len(pb.items)
-        dev = torch.device("cuda", torch.cuda.current_device())
         if E is None:
-            E = torch.empty(k, dtype=torch.float64, device=dev)
+            E = torch.empty(k, dtype=torch.float64, device="cuda")
         if G is None:
-            G = torch.empty((k, 9), dtype=torch.float64, device=dev)
+            G = torch.empty((k, 9), dtype=torch.float64, device="cuda")
         if status is None:
-            status = torch.empty(k, dtype=torch.int32, device=dev)
-        _check(lib().tcm_gradients_batch(self._h, pb.n_systems, ctypes.cast(pb.sys_arr, ctypes.c_void_p), k,
-                                         pb.items.ctypes.data_as(ctypes.c_void_p), int(precision),
-                                         ctypes.c_void_p(E.data_ptr()), ctypes.c_void_p(G.data_ptr()),
-                                         ctypes.c_void_p(status.data_ptr())))
+            status = torch.empty(k, dtype=torch.int32, device="cuda")
+        _check(lib().tcm_gradients_batch(self._h, pb.n_systems, ctypes.addressof(pb.sys_arr), k, pb.items.ctypes.data,
+                                         int(precision), E.data_ptr(), G.data_ptr(), status.data_ptr()))
         return E, G, status
 
     # ---------------------------------------------------------------- Eq. (Coulomb)
@@ -404,24 +396,26 @@ class PackedBatch:
 
 
 def pack_batch(systems, a, b, lmax, R0, rotB=None) -> PackedBatch:
-    sys_arr = (tcm_system * max(len(systems), 1))()
-    keep = []
-    for i, s in enumerate(systems):
+    keep, descr = [], []
+    for s in systems:
         if not isinstance(s, tcm_system):
-            t, c, r = s
-            s = make_system(t, center=c, radius=r)
-            keep.append(t)
-        sys_arr[i] = s
+            x, c, r = s
+            keep.append(x)
+            s = make_system(x, center=c, radius=r)
+        descr.append(s)
+    sys_arr = (tcm_system * max(len(descr), 1))(*descr)
     k = len(R0)
     items = np.zeros(k, dtype=PAIR_ITEM_DTYPE)
-    items["a"] = a
-    items["b"] = b
-    items["lmax"] = lmax
-    items["R0"] = np.asarray(R0, dtype=np.float64).reshape(k, 3)
+    f = items.view(np.float64).reshape(k, 14)  # the same records by 8-byte words: [a b | lmax has_rot | rotB | R0]
+    i = items.view(np.int32).reshape(k, 28)
+    i[:, 0] = a
+    i[:, 1] = b
+    i[:, 2] = lmax
+    f[:, 11:14] = np.asarray(R0, dtype=np.float64).reshape(k, 3)
     if rotB is not None:
-        items["has_rot"] = 1
-        items["rotB"] = np.asarray(rotB, dtype=np.float64).reshape(k, 9)
-    return PackedBatch(sys_arr, len(systems), items, keep)
+        i[:, 3] = 1
+        f[:, 2:11] = np.asarray(rotB, dtype=np.float64).reshape(k, 9)
+    return PackedBatch(sys_arr, len(descr), items, keep)
 
 
 def unpack(q, lmax=None):
