@@ -142,21 +142,48 @@ struct RotDesc {  // one moment set rotated about its centre: out = moments of (
   double M[9];
 };
 
+// Tables of the contraction and of the rotation, built once per process.
+constexpr int kZN = kLmaxMax + 1;
+__host__ __device__ constexpr int dpi2_stride(int l) { return (l + 1) | 1; }
+__host__ __device__ constexpr int dpi2_off(int l) {  // sum over l' < l of (l'+1) dpi2_stride(l')
+  return l * (l + 1) * (2 * l + 1) / 6 + (l / 2) * (l / 2 + 1);
+}
+struct Fx {  // fixed point: 2^30 h + l, |l| <= 2^29
+  int h, l;
+};
+struct ContractTables {
+  double dpi2[dpi2_off(kZN)];  // rows of d^l(pi/2)
+  Fx row[dpi2_off(kZN)];       // the same times 2^59, columns m >= 1 doubled
+  Fx hat[kZN][kZN];            // [l][m]: 2^60 l!/sqrt((l+m)!(l-m)!)
+  double binom[kZN][kZN];      // [l1][l2]: C(l1 + l2, l1)
+};
+const ContractTables& contract_tables();
+// The order in which a call's items are contracted: by degree, so that a CTA takes contract_group(L)
+// items of one degree L at a time.  Items of degree L are order[first[L]] .. order[first[L + 1] - 1]
+// (order null: in place), groups gfirst[L] .. gfirst[L + 1] - 1.
+struct ContractPlan {
+  int first[kLmaxMax + 2], gfirst[kLmaxMax + 2];
+};
+int contract_group(int L);
 // out (device): where the results go; grad: also G, 9 doubles per item: force on B, torque on A, torque
 // on B (lab frame).  rots: device, one EulerZYZ per kBRotate item (PairDesc.rot), or null when there is
 // none.  pdl: the descriptors are complete before the kernel before this one.
-int launch_contract(const PairDesc* items, int n_items, int Lmax_items, const MomJob* jobs,
-                    const SysGeom* geoms, const double* ztab, const EulerZYZ* rots, const PairOut* out, bool grad,
-                    bool pdl, cudaStream_t s);
+int launch_contract(const PairDesc* items, const int* order, const ContractPlan* plan, int n_groups, int Lmax_items,
+                    const MomJob* jobs, const SysGeom* geoms, const ContractTables* tab, const EulerZYZ* rots,
+                    const PairOut* out, bool grad, bool pdl, int num_sms, cudaStream_t s);
 // Descriptors of a large batch (n_items PairSrc -> PairDesc, Euler records).  Its successor on the stream
 // may start at once (and waits for it before it ends).
 int launch_frames(const PairSrc* src, int n_items, int n_computed, const double* rotB, PairDesc* items, EulerZYZ* rots,
                   cudaStream_t s);
-int contract_smem_bytes(int L);
 int rotate_smem_bytes(int L);
 int launch_rotate_moments(const RotDesc* sets, int n_sets, int Lmax_sets, const double* ztab, cudaStream_t s);
-int contract_table_size();
-void contract_tables(double* t);  // host: fills contract_table_size() doubles
+
+__device__ __forceinline__ int tri_l(int k) {  // l with l(l+1)/2 <= k < (l+1)(l+2)/2
+  int l = (int)((sqrtf(8.0f * k + 1.0f) - 1.0f) * 0.5f);
+  while (l * (l + 1) / 2 > k) --l;
+  while ((l + 1) * (l + 2) / 2 <= k) ++l;
+  return l;
+}
 
 // How the direct sum of one item is cut into CTAs (direct_split): parts = A blocks x B ranges of
 // chunk atoms; slab: items per launch (slab x parts partial sums).

@@ -108,7 +108,7 @@ struct tcm_ctx {
   cudaStream_t stream = nullptr;
   // tables
   double* d_fmap = nullptr;  // F_lm of the component each (chunk, slot) holds
-  double* d_ztab = nullptr;  // contraction tables (factorials, 1/sqrt((l+m)!(l-m)!), the rows of d^l(pi/2))
+  ContractTables* d_ctab = nullptr;  // tables of the contraction and of the rotation of moments
   int* d_imap = nullptr;      // (chunk, slot) -> packed component, both precisions
   int* d_imap_off = nullptr;  // [precision][L] offsets into d_imap
   // scratch
@@ -627,10 +627,9 @@ int build_tables(tcm_ctx* c) {
   TRY_CUDA(cudaMemcpy(c->d_fmap, fmap.data(), fmap.size() * sizeof(double), cudaMemcpyHostToDevice));
   TRY_CUDA(cudaMemcpy(c->d_imap, imap.data(), imap.size() * sizeof(int), cudaMemcpyHostToDevice));
   TRY_CUDA(cudaMemcpy(c->d_imap_off, imap_off.data(), imap_off.size() * sizeof(int), cudaMemcpyHostToDevice));
-  std::vector<double> zt(contract_table_size());
-  contract_tables(zt.data());
-  TRY_CUDA(cudaMalloc(&c->d_ztab, zt.size() * sizeof(double)));
-  TRY_CUDA(cudaMemcpy(c->d_ztab, zt.data(), zt.size() * sizeof(double), cudaMemcpyHostToDevice));
+  const ContractTables& t = contract_tables();
+  TRY_CUDA(cudaMalloc(&c->d_ctab, sizeof t));
+  TRY_CUDA(cudaMemcpy(c->d_ctab, &t, sizeof t, cudaMemcpyHostToDevice));
   return TCM_OK;
 }
 
@@ -639,7 +638,7 @@ void free_ctx(tcm_ctx* c) {
   if (c->scratch) c->free_scratch(c->scratch);
   cudaStreamSynchronize(c->stream);
   cudaFree(c->d_fmap);
-  cudaFree(c->d_ztab);
+  cudaFree(c->d_ctab);
   cudaFree(c->d_imap);
   cudaFree(c->d_imap_off);
   for (DevBuf* b : {&c->desc, &c->partials, &c->gpart, &c->systk, &c->systiles, &c->counters, &c->moms, &c->escr,
@@ -939,15 +938,19 @@ int tcm_energy(tcm_ctx_t c, const tcm_moments_t* A, const tcm_moments_t* B, cons
   TRY(dev_ensure(c, c->escr, 64));
   double* dE = static_cast<double*>(c->escr.p);
   std::vector<PairOut> out{PairOut{dE, nullptr, nullptr}};
+  std::vector<ContractPlan> plan(1);
+  for (int L = 0; L <= kLmaxMax + 1; ++L) plan[0].first[L] = plan[0].gfirst[L] = L > lmax;
   Packer pk;
-  const size_t o_job = pk.add(jobs), o_geo = pk.add(geoms), o_it = pk.add(items), o_out = pk.add(out);
+  const size_t o_job = pk.add(jobs), o_geo = pk.add(geoms), o_it = pk.add(items), o_out = pk.add(out), o_plan = pk.add(plan);
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   {
     PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
-    TRY_LAUNCH(launch_contract(reinterpret_cast<PairDesc*>(base + o_it), 1, lmax,
+    TRY_LAUNCH(launch_contract(reinterpret_cast<PairDesc*>(base + o_it), nullptr,
+                               reinterpret_cast<ContractPlan*>(base + o_plan), 1, lmax,
                                reinterpret_cast<MomJob*>(base + o_job), reinterpret_cast<SysGeom*>(base + o_geo),
-                               c->d_ztab, nullptr, reinterpret_cast<PairOut*>(base + o_out), false, true, c->stream));
+                               c->d_ctab, nullptr, reinterpret_cast<PairOut*>(base + o_out), false, true, c->num_sms,
+                               c->stream));
   }
   TRY_CUDA(cudaMemcpyAsync(c->pinned_small, dE, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   TRY_CUDA(cudaStreamSynchronize(c->stream));
@@ -983,7 +986,7 @@ int tcm_rotate_moments(tcm_ctx_t c, int64_t n, const tcm_moments_t* in, const do
   char* base = nullptr;
   TRY(upload(c, pk, &base));
   PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
-  TRY_LAUNCH(launch_rotate_moments(reinterpret_cast<RotDesc*>(base + o_set), (int)n, Lmax, c->d_ztab, c->stream));
+  TRY_LAUNCH(launch_rotate_moments(reinterpret_cast<RotDesc*>(base + o_set), (int)n, Lmax, c->d_ctab->dpi2, c->stream));
   return TCM_OK;
 }
 
@@ -1043,6 +1046,10 @@ struct BatchScratch {
   std::vector<size_t> job_moff;
   std::vector<SysGeom> geoms;
   std::vector<PairOut> out;
+  std::vector<ContractPlan> plan;
+  std::vector<int> order;
+  std::vector<uint8_t> degree;
+  int count[kLmaxMax + 1];  // items per degree
   std::vector<char> used, low;
   std::vector<uint64_t> job_of, cached_of;  // epoch << 32 | index, by (system, degree) and by system
   uint32_t epoch = 0;
@@ -1096,6 +1103,8 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   }
   // One pass over the items: checks, moment jobs (A sides and unrotated B sides shared), records.
   int next_id = 0, Lmax_items = 0;
+  std::fill(B.count, B.count + kLmaxMax + 1, 0);
+  B.degree.resize(n_items);
   size_t moff = 0;
   auto new_job = [&](int sys, int L, const double* rot) {
     P.jobs.emplace_back();
@@ -1136,34 +1145,50 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   };
   int64_t nc_item = -1;  // first item that a host-known radius shows not to converge
   double nc_R = 0.0, nc_a = 0.0;
+  // a scan's items repeat their pair and degree: what depends on those alone is kept from item to item
+  struct {
+    int a = -1, b = -1, lmax = -1, jobA = 0;
+    bool known = false;  // both radii known on the host
+    double aa = 0.0, near2 = 0.0;
+  } last;
   for (int64_t k = 0; k < n_items; ++k) {
     const tcm_pair_item& it = items[k];
-    if (it.a < 0 || it.a >= n_systems || it.b < 0 || it.b >= n_systems)
-      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld refers to a system outside [0, %d)", (long long)k, n_systems);
-    if (it.lmax < 0 || it.lmax > c->lmax_cap)
-      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld lmax %d outside [0, %d]", (long long)k, it.lmax, c->lmax_cap);
-    B.used[it.a] = B.used[it.b] = 1;
-    const tcm_system &sa = systems[it.a], &sb = systems[it.b];
-    if (geom_known(sa) && geom_known(sb) && nc_item < 0) {
+    if (it.a != last.a || it.b != last.b || it.lmax != last.lmax) {
+      if (it.a < 0 || it.a >= n_systems || it.b < 0 || it.b >= n_systems)
+        return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld refers to a system outside [0, %d)", (long long)k, n_systems);
+      if (it.lmax < 0 || it.lmax > c->lmax_cap)
+        return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld lmax %d outside [0, %d]", (long long)k, it.lmax, c->lmax_cap);
+      last.a = it.a;
+      last.b = it.b;
+      last.lmax = it.lmax;
+      B.used[it.a] = B.used[it.b] = 1;
+      last.known = geom_known(systems[it.a]) && geom_known(systems[it.b]);
+      last.aa = systems[it.a].radius + systems[it.b].radius;
+      last.near2 = last.aa * last.aa * (1.0 + 1e-12);
+      last.jobA = unrotated(it.a, it.lmax, true);
+      Lmax_items = std::max(Lmax_items, (int)it.lmax);
+    }
+    const tcm_system& sb = systems[it.b];
+    if (last.known && nc_item < 0) {
       const double R2 = it.R0[0] * it.R0[0] + it.R0[1] * it.R0[1] + it.R0[2] * it.R0[2];
-      const double aa = sa.radius + sb.radius;
-      if (!(R2 > aa * aa * (1.0 + 1e-12))) {  // (the square root only near the limit)
+      if (!(R2 > last.near2)) {  // (the square root only near the limit)
         const double R = std::sqrt(R2);
-        if (!(R > aa)) {
+        if (!(R > last.aa)) {
           nc_item = k;
           nc_R = R;
-          nc_a = aa;
+          nc_a = last.aa;
         }
       }
     }
-    Lmax_items = std::max(Lmax_items, (int)it.lmax);
+    ++B.count[it.lmax];
+    B.degree[k] = (uint8_t)it.lmax;
     PairSrc& p = src[k];
+    p.jobA = last.jobA;
     p.geomA = it.a;
     p.geomB = it.b;
     p.L = (short)it.lmax;
     p.rot = 0;
     for (int d = 0; d < 3; ++d) p.R0[d] = it.R0[d];
-    p.jobA = unrotated(it.a, it.lmax, true);
     if (!it.has_rot) {
       p.b_mode = kBLab;
       p.jobB = unrotated(it.b, it.lmax, true);
@@ -1213,10 +1238,30 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   B.geoms.resize(std::max(n_systems, 1));
   for (int s = 0; s < n_systems; ++s) B.geoms[s] = host_geom(systems[s]);
   B.out.assign(1, PairOut{E, status, G});
+  // the contraction's order: items by degree, in place when there is one degree only
+  B.plan.resize(1);
+  ContractPlan& cp = B.plan[0];
+  int n_groups = 0, at = 0;
+  for (int L = 0; L <= kLmaxMax + 1; ++L) {
+    cp.first[L] = at;
+    cp.gfirst[L] = n_groups;
+    if (L > kLmaxMax) break;
+    at += B.count[L];
+    n_groups += (B.count[L] + contract_group(L) - 1) / contract_group(L);
+  }
+  const bool ordered = B.count[Lmax_items] != n_items;
+  if (ordered) {
+    int next[kLmaxMax + 1];
+    std::copy(cp.first, cp.first + kLmaxMax + 1, next);
+    B.order.resize(n_items);
+    for (int64_t k = 0; k < n_items; ++k) B.order[next[B.degree[k]]++] = (int)k;
+  } else {
+    B.order.clear();
+  }
   Packer pk;
   pk.size = in_place;
   const size_t o_geo = pk.add(B.geoms), o_job = pk.add2(P.jobs, B.cached), o_tile = pk.add(P.groups),
-               o_sj = pk.add(S.jobs), o_out = pk.add(B.out);
+               o_sj = pk.add(S.jobs), o_out = pk.add(B.out), o_plan = pk.add(B.plan), o_ord = pk.add(B.order);
   size_t o_it = 0, o_rot = 0;
   if (on_device) {
     o_rot = pk.add(B.rotB);
@@ -1254,8 +1299,10 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     TRY(run_moments(c, precision, P, d_jobs, T.d_mom, d_geo, st));
     PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
     // (directly behind k_frames the contraction must not read the descriptors ahead of its end)
-    TRY_LAUNCH(launch_contract(d_items, (int)n_items, Lmax_items, d_jobs, d_geo, c->d_ztab, n_rot ? d_rots : nullptr,
-                               reinterpret_cast<PairOut*>(base + o_out), G != nullptr, !(on_device && no_moments), st));
+    TRY_LAUNCH(launch_contract(d_items, ordered ? reinterpret_cast<int*>(base + o_ord) : nullptr,
+                               reinterpret_cast<ContractPlan*>(base + o_plan), n_groups, Lmax_items, d_jobs, d_geo,
+                               c->d_ctab, n_rot ? d_rots : nullptr, reinterpret_cast<PairOut*>(base + o_out),
+                               G != nullptr, !(on_device && no_moments), c->num_sms, st));
     return TCM_OK;
   };
   if (!c->graphs || c->prof || !c->cap_stream) return enqueue(c->stream);
@@ -1267,6 +1314,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
          S.n.cluster, S.n.tiles1, S.n.tiles2, (long long)S.jobs.size(), (long long)T.o_mom, (long long)T.o_sys, T.on_host,
          (long long)P.jobs.size(), P.n_tile_ids, (long long)n_items, n_rot, Lmax_items, (long long)o_geo, (long long)o_job,
          (long long)o_tile, (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)o_out,
+         n_groups, ordered, (long long)o_ord,
          (long long)pk.size, (long long)(uintptr_t)c->systiles.p, (long long)(uintptr_t)base,
          (long long)(uintptr_t)c->gpart.p, (long long)(uintptr_t)c->systk.p, (long long)(uintptr_t)c->partials.p,
          (long long)(uintptr_t)c->counters.p, (long long)P.groups.size(), (long long)P.n_tiles,
