@@ -332,22 +332,33 @@ int finalize_split(int n_jobs, int max_tiles, int max_slots) {
 namespace {
 // One thread per item: about 15 double square roots and divisions for a rotated one, which cost the
 // host 100 to 150 ns an item (108,360 items of a surface scan: 2.6 ms of planning) and this kernel about
-// 20 us for all of them.
-__global__ void __launch_bounds__(128) k_frames(const PairSrc* __restrict__ src, int n_items, int n_computed,
+// 20 us for all of them.  A thread finds its item's run by bisection.
+__global__ void __launch_bounds__(128) k_frames(const PairRun* __restrict__ runs, int n_runs,
+                                                const double* __restrict__ R0, int n_items, int n_computed,
                                                 const double* __restrict__ rotB, PairDesc* __restrict__ items,
                                                 EulerZYZ* __restrict__ rots) {
   pdl_trigger();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n_items) return;
+  int lo = 0, hi = n_runs;  // runs[lo].first <= k < runs[hi].first
+  if (n_runs == n_items) {
+    lo = k;
+  } else {
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (runs[mid].first <= k) lo = mid;
+      else hi = mid;
+    }
+  }
   PairDesc d;
-  make_pair(src[k], n_computed, rotB, d, rots);
+  make_pair(runs[lo], k, R0 + 3LL * k, n_computed, rotB, d, rots);
   items[k] = d;
 }
 }  // namespace
 
-int launch_frames(const PairSrc* src, int n_items, int n_computed, const double* rotB, PairDesc* items, EulerZYZ* rots,
-                  cudaStream_t s) {
-  k_frames<<<(n_items + 127) / 128, 128, 0, s>>>(src, n_items, n_computed, rotB, items, rots);
+int launch_frames(const PairRun* runs, int n_runs, const double* R0, int n_items, int n_computed, const double* rotB,
+                  PairDesc* items, EulerZYZ* rots, cudaStream_t s) {
+  k_frames<<<(n_items + 127) / 128, 128, 0, s>>>(runs, n_runs, R0, n_items, n_computed, rotB, items, rots);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
 }
 

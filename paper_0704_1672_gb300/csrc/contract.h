@@ -26,15 +26,16 @@ struct PairDesc {  // one energy: moments of jobA and jobB at lmax L, separation
   double fr[6];    // R0 by its frame W = R_y(-b) R_z(-a) (r0_frame): 1/R, R, cos b, sin b, cos a, sin a
 };
 
-// What the host writes for an item of a batch; the PairDesc (and Euler record) is made from it on the
-// host for small batches, by k_frames for large ones, with the same roundings (frame arithmetic below).
-struct PairSrc {
-  int jobA, jobB;  // computed jobs; ~k: the k-th cached set, which follow the computed ones
+// What the host writes for the items of a batch: runs of consecutive items of one pair, degree and mode
+// (a scan is one run), and each item's R0.  The descriptors are made from them on the host for small
+// batches, by k_frames for large ones, with the same roundings (frame arithmetic below).
+struct PairRun {
+  int first;         // its first item
+  int jobA, jobB;    // computed sets; ~k: the k-th cached set, which follow the computed ones
   int geomA, geomB;
   short L, b_mode;
-  int rot;
-  double R0[3];
-};
+  int rot;           // kBRotate: rotation of the first item; the others follow
+};                   // kBInFrame: jobB of the first item; the others follow
 
 // Where a batched call's results go (device; status and G may be null).
 struct PairOut {
@@ -118,20 +119,23 @@ __host__ __device__ inline EulerZYZ euler_zyz(const double* M) {
   return e;
 }
 
-// The descriptor of one item; rotB: the rotations of the kBRotate items.
-__host__ __device__ inline void make_pair(const PairSrc& s, int n_computed, const double* rotB, PairDesc& d, EulerZYZ* e) {
-  d.jobA = s.jobA >= 0 ? s.jobA : n_computed + ~s.jobA;
-  d.jobB = s.jobB >= 0 ? s.jobB : n_computed + ~s.jobB;
-  d.geomA = s.geomA;
-  d.geomB = s.geomB;
-  d.L = s.L;
-  d.b_mode = s.b_mode;
-  d.rot = s.rot;
-  r0_frame(s.R0, d.fr);
-  if (s.b_mode == kBRotate) {
+// The descriptor of item k of run r at separation R0; rotB: the rotations of the kBRotate items.
+__host__ __device__ inline void make_pair(const PairRun& r, int k, const double* R0, int n_computed, const double* rotB,
+                                          PairDesc& d, EulerZYZ* e) {
+  const int i = k - r.first;
+  const int jobB = r.b_mode == kBInFrame ? r.jobB + i : r.jobB;
+  d.jobA = r.jobA >= 0 ? r.jobA : n_computed + ~r.jobA;
+  d.jobB = jobB >= 0 ? jobB : n_computed + ~jobB;
+  d.geomA = r.geomA;
+  d.geomB = r.geomB;
+  d.L = r.L;
+  d.b_mode = r.b_mode;
+  d.rot = r.b_mode == kBRotate ? r.rot + i : 0;
+  r0_frame(R0, d.fr);
+  if (r.b_mode == kBRotate) {
     double M[9];
-    frame_times(d.fr, rotB + 9LL * s.rot, M);
-    e[s.rot] = euler_zyz(M);
+    frame_times(d.fr, rotB + 9 * d.rot, M);
+    e[d.rot] = euler_zyz(M);
   }
 }
 
@@ -171,10 +175,10 @@ int contract_group(int L);
 int launch_contract(const PairDesc* items, const int* order, const ContractPlan* plan, int n_groups, int Lmax_items,
                     const MomJob* jobs, const SysGeom* geoms, const ContractTables* tab, const EulerZYZ* rots,
                     const PairOut* out, bool grad, bool pdl, int num_sms, cudaStream_t s);
-// Descriptors of a large batch (n_items PairSrc -> PairDesc, Euler records).  Its successor on the stream
-// may start at once (and waits for it before it ends).
-int launch_frames(const PairSrc* src, int n_items, int n_computed, const double* rotB, PairDesc* items, EulerZYZ* rots,
-                  cudaStream_t s);
+// Descriptors of a large batch from its runs and separations.  Its successor on the stream may start at
+// once (and waits for it before it ends).
+int launch_frames(const PairRun* runs, int n_runs, const double* R0, int n_items, int n_computed, const double* rotB,
+                  PairDesc* items, EulerZYZ* rots, cudaStream_t s);
 int rotate_smem_bytes(int L);
 int launch_rotate_moments(const RotDesc* sets, int n_sets, int Lmax_sets, const double* ztab, cudaStream_t s);
 

@@ -318,12 +318,19 @@ void build_tiles(int precision, Plan& P) {
     }
   }
   const size_t n = key.size();
+  const bool few = n <= 64;  // an insertion sort beats the radix sort's histograms
   std::vector<uint32_t>&order = P.sort_order, &k2 = P.sort_key2, &o2 = P.sort_order2;
   order.resize(n);
   k2.resize(n);
   o2.resize(n);
   for (size_t i = 0; i < n; ++i) order[i] = (uint32_t)i;
-  for (int shift = 0; shift < 32; shift += 11) {
+  for (size_t i = 1; few && i < n; ++i) {
+    const uint32_t o = order[i];
+    size_t j = i;
+    for (; j > 0 && key[order[j - 1]] > key[o]; --j) order[j] = order[j - 1];
+    order[j] = o;
+  }
+  for (int shift = 0; !few && shift < 32; shift += 11) {
     uint32_t count[2049] = {};
     for (size_t i = 0; i < n; ++i) ++count[((key[i] >> shift) & 2047u) + 1];
     for (int b = 0; b < 2048; ++b) count[b + 1] += count[b];
@@ -933,8 +940,7 @@ int tcm_energy(tcm_ctx_t c, const tcm_moments_t* A, const tcm_moments_t* B, cons
   geoms[0].a = A->radius;
   geoms[1].a = B->radius;
   std::vector<PairDesc> items(1);
-  PairSrc src{0, 1, 0, 1, (short)lmax, kBLab, 0, {R0[0], R0[1], R0[2]}};
-  make_pair(src, 2, nullptr, items[0], nullptr);
+  make_pair(PairRun{0, 0, 1, 0, 1, (short)lmax, kBLab, 0}, 0, R0, 2, nullptr, items[0], nullptr);
   TRY(dev_ensure(c, c->escr, 64));
   double* dE = static_cast<double*>(c->escr.p);
   std::vector<PairOut> out{PairOut{dE, nullptr, nullptr}};
@@ -1038,7 +1044,8 @@ struct BatchScratch {
   Plan P;
   SysPlan S;
   Lists T;
-  std::vector<PairSrc> src;
+  std::vector<PairRun> runs;
+  std::vector<double> R0;
   std::vector<PairDesc> pd;
   std::vector<EulerZYZ> rots;
   std::vector<double> rotB;
@@ -1048,7 +1055,6 @@ struct BatchScratch {
   std::vector<PairOut> out;
   std::vector<ContractPlan> plan;
   std::vector<int> order;
-  std::vector<uint8_t> degree;
   int count[kLmaxMax + 1];  // items per degree
   std::vector<char> used, low;
   std::vector<uint64_t> job_of, cached_of;  // epoch << 32 | index, by (system, degree) and by system
@@ -1067,6 +1073,7 @@ struct BatchScratch {
     low.assign(n_systems, 0);
     P.jobs.clear();
     rotB.clear();
+    runs.clear();
     cached.clear();
     job_moff.clear();
   }
@@ -1087,24 +1094,25 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   BatchScratch& B = *c->scratch;
   B.begin(n_systems);
   Plan& P = B.P;
-  // Large batches: the items' descriptors are made on the device (k_frames) from records written straight
-  // into the staging slot; small ones on the host (a launch costs more than their square roots).
+  // Large batches: the items' descriptors are made on the device (k_frames) from runs of items and the
+  // separations, which are written straight into the staging slot; small ones on the host (a launch costs
+  // more than their square roots).
   const bool on_device = n_items >= kDeviceFrames;
-  PairSrc* src = nullptr;
+  double* R0s = nullptr;
   size_t in_place = 0;
   if (on_device) {
-    in_place = (size_t)n_items * sizeof(PairSrc);
+    in_place = (size_t)n_items * 3 * sizeof(double);
     Stage* st = nullptr;
     TRY(stage_slot(c, in_place + in_place / 4 + 65536, 0, &st));
-    src = static_cast<PairSrc*>(st->host);
+    R0s = static_cast<double*>(st->host);
   } else {
-    B.src.resize(n_items);
-    src = B.src.data();
+    B.R0.resize(3 * n_items);
+    R0s = B.R0.data();
   }
   // One pass over the items: checks, moment jobs (A sides and unrotated B sides shared), records.
   int next_id = 0, Lmax_items = 0;
   std::fill(B.count, B.count + kLmaxMax + 1, 0);
-  B.degree.resize(n_items);
+  bool sorted = true;  // degrees never fall from item to item
   size_t moff = 0;
   auto new_job = [&](int sys, int L, const double* rot) {
     P.jobs.emplace_back();
@@ -1145,79 +1153,72 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   };
   int64_t nc_item = -1;  // first item that a host-known radius shows not to converge
   double nc_R = 0.0, nc_a = 0.0;
-  // a scan's items repeat their pair and degree: what depends on those alone is kept from item to item
-  struct {
-    int a = -1, b = -1, lmax = -1, jobA = 0;
-    bool known = false;  // both radii known on the host
-    double aa = 0.0, near2 = 0.0;
-  } last;
-  for (int64_t k = 0; k < n_items; ++k) {
+  // B's moments of a rotated item, in its frame, in the contraction:
+  //   from_cache  the caller asked for it and B carries its moments: the cached set, rotated by W rotB;
+  //   from_lab    double path: B's lab-frame set, computed once per (system, degree) from B's atoms and
+  //               shared by all items and by unrotated sides, rotated by W rotB.  The moments of a rotated
+  //               system are those of the system, rotated degree by degree (exact; O(L^3) operations
+  //               against O(atoms L^2)): 256 orientations of 20,000 atoms at degree 20 take 0.16 ms
+  //               instead of 13 ms, at the same error.  Only for matrices that are rotations to rounding;
+  //   else        a set of the item's own, the frame rotation W folded into its atom transform: any other
+  //               matrix of the double path, and the mixed path, which keeps each item's own float sums
+  //               over the rotated atoms, whose rounding errors are independent.
+  int last_L = 0;
+  for (int64_t k = 0; k < n_items;) {
     const tcm_pair_item& it = items[k];
-    if (it.a != last.a || it.b != last.b || it.lmax != last.lmax) {
-      if (it.a < 0 || it.a >= n_systems || it.b < 0 || it.b >= n_systems)
-        return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld refers to a system outside [0, %d)", (long long)k, n_systems);
-      if (it.lmax < 0 || it.lmax > c->lmax_cap)
-        return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld lmax %d outside [0, %d]", (long long)k, it.lmax, c->lmax_cap);
-      last.a = it.a;
-      last.b = it.b;
-      last.lmax = it.lmax;
-      B.used[it.a] = B.used[it.b] = 1;
-      last.known = geom_known(systems[it.a]) && geom_known(systems[it.b]);
-      last.aa = systems[it.a].radius + systems[it.b].radius;
-      last.near2 = last.aa * last.aa * (1.0 + 1e-12);
-      last.jobA = unrotated(it.a, it.lmax, true);
-      Lmax_items = std::max(Lmax_items, (int)it.lmax);
-    }
-    const tcm_system& sb = systems[it.b];
-    if (last.known && nc_item < 0) {
-      const double R2 = it.R0[0] * it.R0[0] + it.R0[1] * it.R0[1] + it.R0[2] * it.R0[2];
-      if (!(R2 > last.near2)) {  // (the square root only near the limit)
-        const double R = std::sqrt(R2);
-        if (!(R > last.aa)) {
-          nc_item = k;
-          nc_R = R;
-          nc_a = last.aa;
+    if (it.a < 0 || it.a >= n_systems || it.b < 0 || it.b >= n_systems)
+      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld refers to a system outside [0, %d)", (long long)k, n_systems);
+    if (it.lmax < 0 || it.lmax > c->lmax_cap)
+      return set_err(TCM_EINVAL, "tcm_energy_batch: item %lld lmax %d outside [0, %d]", (long long)k, it.lmax, c->lmax_cap);
+    const int ia = it.a, ib = it.b, L = it.lmax, has_rot = it.has_rot != 0;
+    const tcm_system &sa = systems[ia], &sb = systems[ib];
+    B.used[ia] = B.used[ib] = 1;
+    const bool known = geom_known(sa) && geom_known(sb);  // both radii known on the host
+    const double aa = sa.radius + sb.radius, near2 = aa * aa * (1.0 + 1e-12);
+    const bool from_cache = has_rot && c->rotate_cached && sb.moments && L <= sb.moments_lmax;
+    const bool lab = has_rot && !from_cache && precision == TCM_FP64;
+    auto mode_of = [&](const tcm_pair_item& x) {
+      return !has_rot ? kBLab : (from_cache || (lab && is_rotation(x.rotB)) ? kBRotate : kBInFrame);
+    };
+    const int mode = mode_of(it);
+    PairRun r{(int)k, unrotated(ia, L, true), 0, ia, ib, (short)L, (short)mode, (int)(B.rotB.size() / 9)};
+    if (mode != kBInFrame) r.jobB = unrotated(ib, L, mode == kBLab || from_cache);
+    else r.jobB = (int)P.jobs.size();
+    int64_t e = k;
+    for (; e < n_items; ++e) {
+      const tcm_pair_item& x = items[e];
+      if (x.a != ia || x.b != ib || x.lmax != L || (x.has_rot != 0) != (has_rot != 0)) break;
+      if (lab && e > k && mode_of(x) != mode) break;
+      const double x0 = x.R0[0], x1 = x.R0[1], x2 = x.R0[2];
+      R0s[3 * e] = x0;
+      R0s[3 * e + 1] = x1;
+      R0s[3 * e + 2] = x2;
+      if (known) {
+        const double R2 = x0 * x0 + x1 * x1 + x2 * x2;
+        if (!(R2 > near2) && nc_item < 0) {  // (the square root only near the limit)
+          const double R = std::sqrt(R2);
+          if (!(R > aa)) {
+            nc_item = e;
+            nc_R = R;
+            nc_a = aa;
+          }
         }
       }
+      if (mode == kBRotate) {
+        B.rotB.insert(B.rotB.end(), x.rotB, x.rotB + 9);
+      } else if (mode == kBInFrame) {
+        double fr[6], M[9];
+        r0_frame(x.R0, fr);
+        frame_times(fr, x.rotB, M);
+        new_job(ib, L, M);
+      }
     }
-    ++B.count[it.lmax];
-    B.degree[k] = (uint8_t)it.lmax;
-    PairSrc& p = src[k];
-    p.jobA = last.jobA;
-    p.geomA = it.a;
-    p.geomB = it.b;
-    p.L = (short)it.lmax;
-    p.rot = 0;
-    for (int d = 0; d < 3; ++d) p.R0[d] = it.R0[d];
-    if (!it.has_rot) {
-      p.b_mode = kBLab;
-      p.jobB = unrotated(it.b, it.lmax, true);
-      continue;
-    }
-    // B's lab-frame moments, taken into the frame by W rotB inside the contraction:
-    //   from_cache  the caller asked for it and B carries its moments;
-    //   from_lab    double path: computed once per (system, degree) from B's atoms and shared by all
-    //               items and by unrotated sides.  The moments of a rotated system are those of the
-    //               system, rotated degree by degree (exact; O(L^3) double operations against
-    //               O(atoms L^2)): 256 orientations of 20,000 atoms at degree 20 take 0.2 ms instead of
-    //               13 ms, at the same error.  Only for matrices that are rotations to rounding; any
-    //               other matrix acts on the atoms, as before.  The mixed path keeps each item's own
-    //               float sums over the rotated atoms, whose rounding errors are independent.
-    const bool from_cache = c->rotate_cached && sb.moments && it.lmax <= sb.moments_lmax;
-    if (from_cache || (precision == TCM_FP64 && is_rotation(it.rotB))) {
-      p.b_mode = kBRotate;
-      p.rot = (int)(B.rotB.size() / 9);
-      B.rotB.insert(B.rotB.end(), it.rotB, it.rotB + 9);
-      p.jobB = unrotated(it.b, it.lmax, from_cache);
-    } else {
-      // B is moved per item anyway: fold the rotation W that takes R0hat to z into its
-      // atom transform, so the contraction receives B's moments already in that frame.
-      double fr[6], M[9];
-      r0_frame(it.R0, fr);
-      frame_times(fr, it.rotB, M);
-      p.b_mode = kBInFrame;
-      p.jobB = new_job(it.b, it.lmax, M);
-    }
+    B.runs.push_back(r);
+    B.count[L] += (int)(e - k);
+    sorted = sorted && L >= last_L;
+    last_L = L;
+    Lmax_items = std::max(Lmax_items, L);
+    k = e;
   }
   for (int s = 0; s < n_systems; ++s)
     if (B.used[s]) TRY(check_system(&systems[s], "tcm_energy_batch"));
@@ -1249,26 +1250,34 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     at += B.count[L];
     n_groups += (B.count[L] + contract_group(L) - 1) / contract_group(L);
   }
-  const bool ordered = B.count[Lmax_items] != n_items;
+  const bool ordered = !sorted;
+  B.order.clear();
   if (ordered) {
     int next[kLmaxMax + 1];
     std::copy(cp.first, cp.first + kLmaxMax + 1, next);
     B.order.resize(n_items);
-    for (int64_t k = 0; k < n_items; ++k) B.order[next[B.degree[k]]++] = (int)k;
-  } else {
-    B.order.clear();
+    for (size_t r = 0; r < B.runs.size(); ++r) {
+      const int end = r + 1 < B.runs.size() ? B.runs[r + 1].first : (int)n_items;
+      for (int k = B.runs[r].first; k < end; ++k) B.order[next[B.runs[r].L]++] = k;
+    }
   }
   Packer pk;
   pk.size = in_place;
   const size_t o_geo = pk.add(B.geoms), o_job = pk.add2(P.jobs, B.cached), o_tile = pk.add(P.groups),
                o_sj = pk.add(S.jobs), o_out = pk.add(B.out), o_plan = pk.add(B.plan), o_ord = pk.add(B.order);
-  size_t o_it = 0, o_rot = 0;
+  size_t o_it = 0, o_rot = 0, o_run = 0;
+  const int n_runs = (int)B.runs.size();
   if (on_device) {
+    o_run = pk.add(B.runs);
     o_rot = pk.add(B.rotB);
   } else {
     B.pd.resize(n_items);
     B.rots.resize(n_rot);
-    for (int64_t k = 0; k < n_items; ++k) make_pair(src[k], n_computed, B.rotB.data(), B.pd[k], B.rots.data());
+    for (int r = 0; r < n_runs; ++r) {
+      const int end = r + 1 < n_runs ? B.runs[r + 1].first : (int)n_items;
+      for (int k = B.runs[r].first; k < end; ++k)
+        make_pair(B.runs[r], k, R0s + 3 * k, n_computed, B.rotB.data(), B.pd[k], B.rots.data());
+    }
     o_it = pk.add(B.pd);
     o_rot = pk.add(B.rots);
   }
@@ -1292,8 +1301,8 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     TRY(run_expand(c, P.groups, d_jobs, reinterpret_cast<MomGroup*>(base + o_tile), S, T, d_sj, st));
     if (on_device) {
       PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
-      TRY_LAUNCH(launch_frames(reinterpret_cast<PairSrc*>(base), (int)n_items, n_computed,
-                               reinterpret_cast<double*>(base + o_rot), d_items, d_rots, st));
+      TRY_LAUNCH(launch_frames(reinterpret_cast<PairRun*>(base + o_run), n_runs, reinterpret_cast<double*>(base),
+                               (int)n_items, n_computed, reinterpret_cast<double*>(base + o_rot), d_items, d_rots, st));
     }
     TRY(run_sys(c, S, T, d_sj, d_geo, st));
     TRY(run_moments(c, precision, P, d_jobs, T.d_mom, d_geo, st));
@@ -1314,7 +1323,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
          S.n.cluster, S.n.tiles1, S.n.tiles2, (long long)S.jobs.size(), (long long)T.o_mom, (long long)T.o_sys, T.on_host,
          (long long)P.jobs.size(), P.n_tile_ids, (long long)n_items, n_rot, Lmax_items, (long long)o_geo, (long long)o_job,
          (long long)o_tile, (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)o_out,
-         n_groups, ordered, (long long)o_ord,
+         n_groups, ordered, (long long)o_ord, (long long)o_run, n_runs,
          (long long)pk.size, (long long)(uintptr_t)c->systiles.p, (long long)(uintptr_t)base,
          (long long)(uintptr_t)c->gpart.p, (long long)(uintptr_t)c->systk.p, (long long)(uintptr_t)c->partials.p,
          (long long)(uintptr_t)c->counters.p, (long long)P.groups.size(), (long long)P.n_tiles,

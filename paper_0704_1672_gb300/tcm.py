@@ -396,14 +396,18 @@ class PackedBatch:
 
 
 def pack_batch(systems, a, b, lmax, R0, rotB=None) -> PackedBatch:
-    keep, descr = [], []
-    for s in systems:
-        if not isinstance(s, tcm_system):
-            x, c, r = s
-            keep.append(x)
-            s = make_system(x, center=c, radius=r)
-        descr.append(s)
-    sys_arr = (tcm_system * max(len(descr), 1))(*descr)
+    keep, descr = [], systems
+    if any(type(s) is not tcm_system for s in systems):
+        descr = []
+        for s in systems:
+            if not isinstance(s, tcm_system):
+                x, c, r = s
+                keep.append(x)
+                s = make_system(x, center=c, radius=r)
+            descr.append(s)
+    n = len(descr)
+    # (joined as bytes: the array's constructor copies the records one attribute access at a time)
+    sys_arr = (tcm_system * n).from_buffer_copy(b"".join(descr)) if n else (tcm_system * 1)()
     k = len(R0)
     items = np.zeros(k, dtype=PAIR_ITEM_DTYPE)
     f = items.view(np.float64).reshape(k, 14)  # the same records by 8-byte words: [a b | lmax has_rot | rotB | R0]
@@ -415,7 +419,7 @@ def pack_batch(systems, a, b, lmax, R0, rotB=None) -> PackedBatch:
     if rotB is not None:
         i[:, 3] = 1
         f[:, 2:11] = np.asarray(rotB, dtype=np.float64).reshape(k, 9)
-    return PackedBatch(sys_arr, len(descr), items, keep)
+    return PackedBatch(sys_arr, n, items, keep)
 
 
 def unpack(q, lmax=None):
