@@ -89,11 +89,7 @@ __global__ void __launch_bounds__(kColThreads)
   const bool active = m < m1;
   const int n = L - m;
   const SysGeom& g = geoms[job.geom];
-  if (threadIdx.x < 9) xf.M[threadIdx.x] = (float)(job.rot[threadIdx.x] * (1.0 / scale_radius(g.a)));
-  if (threadIdx.x < 3) {
-    xf.chi[threadIdx.x] = g.chi[threadIdx.x];
-    xf.clo[threadIdx.x] = g.clo[threadIdx.x];
-  }
+  if (w == 0) make_xform<float>(job, g, lane, &xf);
   const double cd[3] = {g.c[0], g.c[1], g.c[2]};
   const long long i0 = (long long)tile.t * job.atoms_per_tile;
   const long long i1 = min(job.n, i0 + (long long)job.atoms_per_tile);

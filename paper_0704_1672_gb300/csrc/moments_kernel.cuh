@@ -86,19 +86,10 @@ struct Regs {
   T g0, p0;             // column 0: H_j, H_j-1
   P2<T> g[NC], p[NC];   // columns m >= 1
   T dr, di;             // running diagonal power u^m
-  T q00, q00e;          // float kernels: Q_00 = sum q as an error-free (sum, error) pair
 };
 
-// Q_00 is the total charge: for a neutral system it is a tiny difference of large partial
-// sums, and a charged partner multiplies its error by its own charge.  The float kernels
-// therefore accumulate it with Knuth's two-sum (the rounding error of every addition goes
-// to q00e) and reduce it across the warp in double.
-__device__ __forceinline__ void two_sum_acc(float& s, float& e, float x) {
-  const float t = s + x;
-  const float bb = t - s;
-  e += (s - (t - bb)) + (x - bb);
-  s = t;
-}
+// The degrees l <= kLowLmax of every job come from the system pass's float-float sums (k_finalize), so the
+// kernels neither accumulate nor reduce them: their slots of the partial rows stay zero.
 
 // The signed recurrence coefficient of step jj (>= 2) along column m at degree l.
 template <typename T, int l, int m>
@@ -160,10 +151,7 @@ __device__ __forceinline__ void col0_step(Regs<T, L, M0, M1>& s, P2<T> cc, P2<T>
     s.p0 = s.g0;
     s.g0 = n;
   }
-  if constexpr (l == 0 && sizeof(T) == 4)
-    two_sum_acc(s.q00, s.q00e, qq.x);  // G_00 = 1
-  else
-    s.acc0[l] = fmaT(qq.x, s.g0, s.acc0[l]);
+  if constexpr (l > kLowLmax) s.acc0[l] = fmaT(qq.x, s.g0, s.acc0[l]);
 }
 
 // A single complex column m at degree l: (Re, Im) in one pair register.
@@ -184,7 +172,7 @@ __device__ __forceinline__ void single_step(Regs<T, L, M0, M1>& s, T ux, T uy, P
       s.g[j] = n;
     }
     constexpr int a = (acc_slot(L, M0, M1, l, m, 0) - Regs<T, L, M0, M1>::N0) / 2;
-    s.accp[a] = fma2(qq, s.g[j], s.accp[a]);
+    if constexpr (l > kLowLmax) s.accp[a] = fma2(qq, s.g[j], s.accp[a]);
   }
 }
 
@@ -202,8 +190,10 @@ __device__ __forceinline__ void pair_step(Regs<T, L, M0, M1>& s, T ux, T uy, P2<
       s.g[ja].x = s.dr;
       s.g[jb].x = s.di;
       constexpr int a = (acc_slot(L, M0, M1, l, ma, 0) - R::N0) / 2;
-      s.accp[a].x = fmaT(qq.x, s.dr, s.accp[a].x);
-      s.accp[a].y = fmaT(qq.x, s.di, s.accp[a].y);
+      if constexpr (l > kLowLmax) {
+        s.accp[a].x = fmaT(qq.x, s.dr, s.accp[a].x);
+        s.accp[a].y = fmaT(qq.x, s.di, s.accp[a].y);
+      }
     } else {
       if constexpr (l == mb) {  // column a: G = c G; column b: seed
         s.p[ja].x = s.g[ja].x;
@@ -226,8 +216,10 @@ __device__ __forceinline__ void pair_step(Regs<T, L, M0, M1>& s, T ux, T uy, P2<
       }
       constexpr int ar = (acc_slot(L, M0, M1, l, ma, 0) - R::N0) / 2;  // (Re_a, Re_b)
       constexpr int ai = (acc_slot(L, M0, M1, l, ma, 1) - R::N0) / 2;  // (Im_a, Im_b)
-      s.accp[ar] = fma2(qq, s.g[ja], s.accp[ar]);
-      s.accp[ai] = fma2(qq, s.g[jb], s.accp[ai]);
+      if constexpr (l > kLowLmax) {
+        s.accp[ar] = fma2(qq, s.g[ja], s.accp[ar]);
+        s.accp[ai] = fma2(qq, s.g[jb], s.accp[ai]);
+      }
     }
   }
 }
@@ -261,18 +253,28 @@ struct Xform {
   T M[9];
 };
 
+// 1 / scale_radius(a): the exponent's bits for any radius but 0, denormals and the largest.
+__device__ __forceinline__ double inv_scale_radius(double a) {
+  const int be = (__double2hiint(a) >> 20) & 0x7ff;
+  if (be > 0 && be < 2045 && a > 0.0) return __longlong_as_double((long long)(2045 - be) << 52);
+  return 1.0 / scale_radius(a);
+}
+
+// Written by the lanes of one warp, an entry each, from loads that are issued together: rot / a' is one
+// exact scaling (a' a power of two) and one rounding.  (One lane forming all of it, with a division, held
+// its warp for about 2,000 cycles of every tile.)
 template <typename T>
-__device__ __forceinline__ Xform<T> make_xform(const MomJob& job, const SysGeom& g) {
-  Xform<T> x;
-  const double ia = 1.0 / scale_radius(g.a);  // exact: a power of two
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {  // float: the centre's split from the geometry record
-    x.chi[k] = sizeof(T) == 4 ? (T)g.chi[k] : (T)g.c[k];
-    x.clo[k] = sizeof(T) == 4 ? (T)g.clo[k] : (T)0;
+__device__ __forceinline__ void make_xform(const MomJob& job, const SysGeom& g, int lane, Xform<T>* x) {
+  const double a = g.a;
+  const double rot = job.rot[lane < 9 ? lane : 0];
+  const int k = lane >= 9 && lane < 12 ? lane - 9 : 0;
+  const float chi = g.chi[k], clo = g.clo[k];  // the centre's split from the geometry record
+  if (lane < 9) {
+    x->M[lane] = (T)(rot * inv_scale_radius(a));
+  } else if (lane < 12) {
+    x->chi[k] = chi;
+    x->clo[k] = clo;
   }
-#pragma unroll
-  for (int k = 0; k < 9; ++k) x.M[k] = (T)(job.rot[k] * ia);
-  return x;
 }
 
 // Centred coordinates of one atom record.  The input type is a template parameter so that
@@ -324,10 +326,13 @@ __device__ __forceinline__ void setup(T d0, T d1, T d2, const Xform<T>& xf, T& u
 // sum keeps about 48 bits (a plain float tree would add about 2 x 2^-24 of the row's
 // magnitude).  Float instructions only: on GB300 the FP64 pipe runs at 1/64 of the FP32 rate,
 // and a double tree (with its conversions) held the warps at the end of every tile.
+// (The error from the larger of the two operands, 3 additions and a comparison on the other pipe,
+// instead of Knuth's 6 additions: the same value.)
 __device__ __forceinline__ void two_sum_ff(float a, float b, float& s, float& e) {
   s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
+  const bool first = fabsf(a) >= fabsf(b);
+  const float hi = first ? a : b, lo = first ? b : a;
+  e = lo - (s - hi);
 }
 __device__ __forceinline__ double row_sum32(const float* p) {
   const float4* v = reinterpret_cast<const float4*>(p);
@@ -376,12 +381,6 @@ __device__ __forceinline__ void warp_reduce_store(const Regs<T, L, M0, M1>& s, T
     const int r = lane + 32 * rr;
     if (r < NACC) out[r] = row_sum32(wb + r * S);
   }
-  if constexpr (M0 == 0 && sizeof(T) == 4) {  // slot 0 is Q_00: exact lane pairs summed in double
-    double v = (double)s.q00 + (double)s.q00e;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) out[0] = v;
-  }
   __syncwarp();
 }
 
@@ -417,8 +416,6 @@ __device__ __forceinline__ void atom_loop(Regs<T, L, M0, M1>& s, const Rec* __re
     if (i + 32 < i1) nxt = load_rec(xyzq, i + 32);
     T d0, d1, d2, q, ux, uy, cz, rho;
     centre<T>(cur, xf, cd, d0, d1, d2, q);
-    if constexpr (M0 == 0 && sizeof(T) == 4 && sizeof(Rec) == 32)
-      s.q00e += (T)(cur.b.y - (double)q);  // double input: keep the charge's rounding remainder in Q_00
     setup<T>(d0, d1, d2, xf, ux, uy, cz, rho);
     const P2<T> cc = pair<T>(cz, cz), rr = pair<T>(rho, rho), qq = pair<T>(q, q);
     if constexpr (M0 == 0) {
@@ -438,7 +435,7 @@ __device__ __forceinline__ void run_chunk(const MomTile& tile, const MomJob* __r
   using R = Regs<T, L, M0, M1>;
   const MomJob& job = jobs[tile.job];
   const SysGeom g = geoms[job.geom];
-  if ((threadIdx.x & 31) == 0) *xf_w = make_xform<T>(job, g);  // double math once per tile
+  make_xform<T>(job, geoms[job.geom], threadIdx.x & 31, xf_w);
   __syncwarp();
   const Xform<T> xf = *xf_w;
   const long long n = job.n;
@@ -447,7 +444,6 @@ __device__ __forceinline__ void run_chunk(const MomTile& tile, const MomJob* __r
   const void* xyzq = job.xyzq;
   const int dtype = job.dtype;
   R s;
-  s.q00 = s.q00e = (T)0;
 #pragma unroll
   for (int k = 0; k < R::N0; ++k) s.acc0[k] = (T)0;
 #pragma unroll
@@ -500,16 +496,20 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? moment_ctas(KM) : T
   constexpr int kRow = LK >= 0 ? Plan<T, (LK >= 0 ? LK : 0), KM>::max_nacc() : KM;
   T* wb = reinterpret_cast<T*>(smem) + warp * (kRow * MomTraits<T>::stride);
   pdl_wait();  // the centres and radii of the launch before are complete
+  int nx = lane == 0 ? atomicAdd(counter, 1) : 0;
   for (;;) {
-    int ti = 0;
-    if (lane == 0) ti = atomicAdd(counter, 1);
-    ti = __shfl_sync(0xffffffffu, ti, 0);
+    const int ti = __shfl_sync(0xffffffffu, nx, 0);
     if (ti >= n_tiles) break;
     const MomTile tile = tiles[ti];
+    // the next tile's number is fetched while this one is worked on, but for the last rounds, in which a
+    // warp must not hold a tile that an idle one could take
+    const bool ahead = ti < n_tiles - 2 * (int)(gridDim.x * (kThreads / 32));
+    if (ahead && lane == 0) nx = atomicAdd(counter, 1);
     if constexpr (LK >= 0)
       run_tile<T, LK, 0, KM>(tile, jobs, geoms, partials, wb, &s_xf[warp]);
     else
       run_tile_any<T, 0, KM>(jobs[tile.job].L, tile, jobs, geoms, partials, wb, &s_xf[warp]);
+    if (!ahead && lane == 0) nx = atomicAdd(counter, 1);
   }
   // the last warp out leaves the work counter and its own ticket at zero for the next launch
   if (lane == 0 && atomicAdd(counter + 32, 1) == (int)(gridDim.x * (kThreads / 32)) - 1) {
