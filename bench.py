@@ -36,7 +36,8 @@ METRIC = "atom-moments/s and TCM energies/s vs plain FP64 GPU path at stated err
 UNIT = "atom-moments/s"
 FP32_LANES_PER_SM = 128
 FP64_PER_SM_CLK = 2          # FP64 pipe results per SM per clock (GB300)
-DIRECT_FP64_PER_PAIR = 10    # algorithmic FP64 operations per pair of Eq. (Coulomb), besides the rsqrt
+IMAD_PER_SM_CLK = 64         # 32 x 32 + 64 bit multiply-adds per SM per clock (two shared operands; 32 without)
+DIRECT_IMADS_PER_PAIR = 13   # of them, algorithmic ones per pair of Eq. (Coulomb) in the fixed-point loop
 
 
 def parse():
@@ -71,16 +72,17 @@ def moment_instr_per_atom(L):
     return 3 * (L + 1) ** 2 + 12
 
 
-def contract_fp64_ops(L):
-    """Algorithmic FP64 operations of one energy in k_contract when B's moments arrive in the
-    frame of R0 and A's are rotated in the kernel: the input and beta phases and the scalings of
-    the (l, m >= 0) entries (12 per entry), the two products through d^l(pi/2)
-    (2 sum_l (l+1)^2), the z-axis contraction (sum over (l1, l2) of 2 min(l1, l2), plus 3 per
-    pair) and the power tables (about 250)."""
+def contract_imads(L, rotated_b=False):
+    """Algorithmic 32 x 32 + 64 bit multiply-adds (IMAD.WIDE, three per fixed-point product) of one
+    energy in k_contract: per (l, m >= 0) entry of A the input and beta phases (4 products each) and
+    the hat factor (2), of B the hat factor, or the same as A when its moments are rotated in the
+    kernel (and 4 more for the output phase); the two products through d^l(pi/2) (2 sum_l (l+1)^2 per
+    rotated side); the z-axis contraction (sum over (l1, l2) of 1 + 2 min(l1, l2))."""
     T = (L + 1) * (L + 2) // 2
     S2 = (L + 1) * (L + 2) * (2 * L + 3) // 6
-    Z = sum(2 * min(a, b) for a in range(L + 1) for b in range(L + 1))
-    return 12 * T + 2 * S2 + Z + 3 * (L + 1) ** 2 + 250
+    Z = sum(1 + 2 * min(a, b) for a in range(L + 1) for b in range(L + 1))
+    side = 10 * T + 2 * S2
+    return 3 * (side + (side + 4 * T if rotated_b else 2 * T) + Z)
 
 
 def measured_peaks():
@@ -392,6 +394,7 @@ def run_ours(args, rank, world, dist):
     smx = sm_max_mhz()
     peak_fp32 = n_sm * FP32_LANES_PER_SM * smx * 1e6 / 1e12      # T lane-instr/s
     peak_fp64 = n_sm * FP64_PER_SM_CLK * smx * 1e6 / 1e9         # G FP64 op/s
+    peak_imad = n_sm * IMAD_PER_SM_CLK * smx * 1e6 / 1e9         # G IMAD.WIDE lane-op/s
     prec = tcm.TCM_MIXED if args.precision == "mixed" else tcm.TCM_FP64
     stream = torch.cuda.current_stream()
     timer = Timer(torch, stream)
@@ -402,6 +405,8 @@ def run_ours(args, rank, world, dist):
     L = s.L
     cfg = config4_cfg(s)
     atoms_per_step = cfg["atom_moments_per_step"]
+    if prec == tcm.TCM_FP64:  # the double path computes B's moments once and rotates them per orientation
+        atoms_per_step = len(s.A) + len(s.B)
     A = torch.tensor(s.A, dtype=torch.float32, device="cuda")
     B = torch.tensor(s.B, dtype=torch.float32, device="cuda")
     ctx = tcm.Context(lmax_cap=24, stream=stream)
@@ -462,12 +467,12 @@ def run_ours(args, rank, world, dist):
                 "peak_source": f"{n_sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x {smx:.0f} MHz (max SM clock of measured)",
                 "algorithmic_instr_per_atom": moment_instr_per_atom(L), "launch_ms": mom_launch_ms}
     con_launch_ms = phase_ms["contract"] / max(1, launches["contract"])
-    con_ops = k * contract_fp64_ops(L)
-    contract_roofline = {"bound": "fp64", "kernel": "k_contract<false>", "achieved": con_ops / (con_launch_ms * 1e-3) / 1e9,
-                         "peak": peak_fp64, "unit": "G FP64 op/s",
-                         "frac": con_ops / (con_launch_ms * 1e-3) / 1e9 / peak_fp64,
-                         "algorithmic_fp64_per_energy": contract_fp64_ops(L), "launch_ms": con_launch_ms,
-                         "peak_source": f"{n_sm} SMs x {FP64_PER_SM_CLK} FP64/clk x {smx:.0f} MHz"}
+    con_ops = k * contract_imads(L)
+    con_rate = con_ops / (con_launch_ms * 1e-3) / 1e9
+    contract_roofline = {"bound": "int", "kernel": "k_contract<false>", "achieved": con_rate, "peak": peak_imad,
+                         "unit": "G IMAD.WIDE lane-op/s", "frac": con_rate / peak_imad,
+                         "algorithmic_imads_per_energy": contract_imads(L), "launch_ms": con_launch_ms,
+                         "peak_source": f"{n_sm} SMs x {IMAD_PER_SM_CLK} per clk x {smx:.0f} MHz"}
 
     # the same steps with the library's default launch mode (phase events off: a replayed CUDA graph)
     g_ms = timer.run(step, min(args.steps, 10), 3)
@@ -621,7 +626,8 @@ def bench_config2(torch, tcm, synth, autotune, timer, stream, prec, peak_fp32, p
     instr = atoms * moment_instr_per_atom(L) / max(1.0, la["moments"] / n)
     ach = instr / (mom_launch_ms * 1e-3) / 1e12
     con_launch_ms = ph["contract"] / max(1, la["contract"])
-    con = k * contract_fp64_ops(L) / (con_launch_ms * 1e-3) / 1e9
+    con = k * contract_imads(L) / (con_launch_ms * 1e-3) / 1e9
+    peak_imad = n_sm * IMAD_PER_SM_CLK * smx * 1e6 / 1e9
     g_ms = timer.run(step, steps, 3)
     out = {"workload": "protein-like PES scan: 2 x 20000 random-walk atoms (r=30 A, N(0,0.3) net-zero), 256 "
                        "orientations of B, |R0| in [70,150] A, Lmax=20",
@@ -633,9 +639,9 @@ def bench_config2(torch, tcm, synth, autotune, timer, stream, prec, peak_fp32, p
            "roofline": {"bound": "alu", "kernel": f"k_moments<float,{L}>", "achieved": ach, "peak": peak_fp32,
                         "unit": "T FP32-pipe lane-instr/s", "frac": ach / peak_fp32, "launch_ms": mom_launch_ms,
                         "traffic": captured_traffic("k_moments_pes_scan_L20.md", ["moments_kernel.cuh", "tcm_internal.h"])},
-           "contract_roofline": {"bound": "fp64", "achieved": con, "peak": peak_fp64, "unit": "G FP64 op/s",
-                                 "frac": con / peak_fp64, "launch_ms": con_launch_ms,
-                                 "algorithmic_fp64_per_energy": contract_fp64_ops(L)},
+           "contract_roofline": {"bound": "int", "achieved": con, "peak": peak_imad, "unit": "G IMAD.WIDE lane-op/s",
+                                 "frac": con / peak_imad, "launch_ms": con_launch_ms,
+                                 "algorithmic_imads_per_energy": contract_imads(L)},
            "tiling": ({"atoms_per_lane": tuned.best[L][0], "ctas_per_sm": tuned.best[L][1], "kmax": tuned.best[L][2],
                        "chunks": ctx.tcm_ctx_get_chunking_l(L)[1]} if tuned else (fixed or "default"))}
     # B's moments rotated from a cache (Wigner rotation in the contraction kernel) instead of
@@ -657,8 +663,10 @@ def bench_config2(torch, tcm, synth, autotune, timer, stream, prec, peak_fp32, p
     ph, la = ctx.tcm_ctx_read_profile()
     ctx.tcm_ctx_set_profiling(False)
     d_mom = ph["moments"] / max(1, la["moments"])
-    d_ach = atoms * moment_instr_per_atom(L) / (d_mom * 1e-3) / 1e9
-    out["fp64_batched_gpu"] = {"ms_per_step": float(np.mean(d_ms)), "value": atoms / (np.mean(d_ms) * 1e-3),
+    # B's moments are computed once, in the lab frame, and rotated per orientation in the contraction
+    d_ach = (len(s.A) + len(s.B)) * moment_instr_per_atom(L) / (d_mom * 1e-3) / 1e9
+    out["fp64_batched_gpu"] = {"ms_per_step": float(np.mean(d_ms)),
+                               "how": "moments of A and B once each, B's rotated per orientation (O(L^3))",
                                "energies_per_s": k / (np.mean(d_ms) * 1e-3),
                                "moments_roofline": {"bound": "fp64", "achieved": d_ach, "peak": peak_fp64,
                                                     "unit": "G FP64 instr/s", "frac": d_ach / peak_fp64}}
@@ -798,17 +806,17 @@ def run_pes_grid(torch, tcm, prec, n_sm, sm_mhz, stream):
     n = len(R0)
     t = res.timings_ms
     pairs = n * len(g.A) * len(g.B)
-    achieved = pairs * DIRECT_FP64_PER_PAIR / (t["direct"] * 1e-3) / 1e9
-    peak = n_sm * FP64_PER_SM_CLK * sm_mhz * 1e6 / 1e9
+    achieved = pairs * DIRECT_IMADS_PER_PAIR / (t["direct"] * 1e-3) / 1e9
+    peak = n_sm * IMAD_PER_SM_CLK * sm_mhz * 1e6 / 1e9
     return {"workload": g.name, "points": n, "lmax": list(g.lmax),
             "tcm_energies": n * len(g.lmax), "tcm_ms": t["tcm_energies"], "moments_ms": t["moments"],
             "item_packing_host_ms": t["item_packing_host"],
             "tcm_energies_per_s": n * len(g.lmax) / (t["tcm_energies"] * 1e-3),
             "direct_ms": t["direct"], "direct_pairs_per_s": pairs / (t["direct"] * 1e-3),
-            "direct_roofline": {"bound": "fp64", "kernel": "k_direct", "achieved": achieved, "peak": peak,
-                                "unit": "G FP64 op/s", "frac": achieved / peak,
-                                "algorithmic_fp64_per_pair": DIRECT_FP64_PER_PAIR,
-                                "peak_source": f"{n_sm} SMs x {FP64_PER_SM_CLK} FP64/clk x {sm_mhz:.0f} MHz"},
+            "direct_roofline": {"bound": "int", "kernel": "k_direct", "achieved": achieved, "peak": peak,
+                                "unit": "G IMAD.WIDE lane-op/s", "frac": achieved / peak,
+                                "algorithmic_imads_per_pair": DIRECT_IMADS_PER_PAIR,
+                                "peak_source": f"{n_sm} SMs x {IMAD_PER_SM_CLK} per clk x {sm_mhz:.0f} MHz"},
             "eq_error_percent_median": {str(L): float(np.median(res.eta(L))) for L in g.lmax},
             "eq_error_percent_max": {str(L): float(np.max(res.eta(L))) for L in g.lmax}}
 

@@ -1300,7 +1300,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     const SysJob* d_sj = reinterpret_cast<SysJob*>(base + o_sj);
     TRY(run_expand(c, P.groups, d_jobs, reinterpret_cast<MomGroup*>(base + o_tile), S, T, d_sj, st));
     if (on_device) {
-      PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
+      PhaseScope ps(c, TCM_PHASE_GEOM, 1);
       TRY_LAUNCH(launch_frames(reinterpret_cast<PairRun*>(base + o_run), n_runs, reinterpret_cast<double*>(base),
                                (int)n_items, n_computed, reinterpret_cast<double*>(base + o_rot), d_items, d_rots, st));
     }
@@ -1363,8 +1363,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   }
   TRY_CUDA(cudaGraphLaunch(c->gexec, c->stream));
   ++c->graph_launches;
-  c->launches[TCM_PHASE_GEOM] += sys_launches(S.n) + !T.on_host;
-  c->launches[TCM_PHASE_CONTRACT] += on_device;
+  c->launches[TCM_PHASE_GEOM] += sys_launches(S.n) + !T.on_host + on_device;
   c->launches[TCM_PHASE_MOMENTS] += moment_launches(precision, P);
   c->launches[TCM_PHASE_FINALIZE] += !P.jobs.empty();
   c->launches[TCM_PHASE_CONTRACT] += 1;

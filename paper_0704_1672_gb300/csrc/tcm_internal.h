@@ -270,11 +270,15 @@ int launch_expand_tiles(const MomGroup* groups, int n_groups, const MomJob* jobs
 int launch_moments_f64(int L, const MomJob* jobs, const MomTile* tiles, int n_tiles, int* counter, const SysGeom* geoms,
                        double* partials, int grid, cudaStream_t s);
 // Rows of 32 atoms in a tile of the double kernel for a system of n atoms (before the tiling
-// setting's limit): about 304 tiles (two per SM), so that one system fills the GPU; at 100,003 atoms
-// and degree 24 285 tiles of 11 rows.
+// setting's limit): whole rounds of one tile per SM, as few as tiles of 32 rows allow, but two for
+// systems under 38,912 atoms, whose tiles would have fewer than 8 rows (several such systems share a launch).
+// 100,003 atoms at degree 24: 149 tiles of 21 rows in one round; as 285 tiles of 11 rows the second
+// round was not full (353 us a call; now 320).
 inline int f64_rows(long long n) {
-  const long long r = (n + 32 * 304 - 1) / (32 * 304);
-  return (int)(r < 1 ? 1 : (r > 4096 ? 4096 : r));
+  const long long per = 32 * 152;
+  const long long rounds = n < 8 * per ? 2 : (n + 32 * per - 1) / (32 * per);
+  const long long r = (n + per * rounds - 1) / (per * rounds);
+  return (int)(r < 1 ? 1 : r);
 }
 // The same tiles (float plans) by columns, for calls with few of them (moments_cols.cu): jobs whose
 // low degrees come from the system pass.  max_cols: over the degrees of the tiles' jobs.
