@@ -33,8 +33,10 @@
 // largest component of its degree (double: 2^-53 of each), sums of products are exact to the last limb.  Only
 // the factor C(l1+l2, l1) / R^(l1+l2+1), the sum over (l1, l2) and the gradient's combinations stay in
 // double: 3 FP64 instructions per (l1, l2).
-// Measured, before and now: 108,360 energies at degrees 1 to 10 1,340 and 345 us, 2,048 at degrees 8 to
-// 24 (B rotated) 140 and 65, 256 at degree 20 24 and 13, forces and torques of 512 at degree 12 92 and 24.
+// Measured, in double and now: 108,360 energies at degrees 1 to 10 1,340 and 298 us, 2,048 at degrees 8 to
+// 24 (B rotated) 140 and 64, 256 at degree 20 24 and 16, forces and torques of 512 at degree 12 92 and 25.
+// What bounds it now: the phases between barriers (a third of the stalls) with the multiplier 0.45 busy and
+// the FP64 pipe 0.27; 80 registers and 3 CTAs per SM instead of 64 and 4 took 342 us of the first.
 // A CTA takes a group of items of one degree side by side (contract_group), so that its lanes are full
 // at low degrees too, one lane column per item.  The group size, and with it the order of every sum,
 // depends on the degree alone: an item's result does not depend on its batch.
@@ -196,7 +198,7 @@ __device__ __forceinline__ void row_split(const Fx* row, const int4* x, int G, i
 // A's moments are kept as a_m = (-1)^m Qa_m, so that T0 = Re sum a_m conj(b_m) and so on without signs;
 // the sums weighted by m take (m/32) a_m.
 template <bool kGrad>
-__global__ void __launch_bounds__(kCT, kGrad ? 2 : 3)
+__global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
     k_contract(const PairDesc* __restrict__ items, const int* __restrict__ order, const ContractPlan* __restrict__ plan,
                int n_groups, int Lmax, const MomJob* __restrict__ jobs, const SysGeom* __restrict__ geoms,
                const ContractTables* __restrict__ tab, const EulerZYZ* __restrict__ rots,
@@ -247,10 +249,15 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 3)
     const int bmode = d.b_mode;
     if (in) {
       // the phase tables, one entry per step: (-i)^m e^{-i m alpha}, e^{i k beta} of W; in mode kBRotate
-      // those of W rotB and i^m e^{-i m gamma}
+      // those of W rotB and i^m e^{-i m gamma}; then the powers of 1/R (other threads', so side by side)
       const int ntab = bmode == kBRotate ? kTabs : 2;
-      for (int q = q0; q < ntab * n1; q += Q) {
+      for (int q = q0; q < ntab * n1 + 2 * L + 2; q += Q) {
         const int t = q / n1, m = q - t * n1;
+        if (t >= ntab) {
+          const int k = q - ntab * n1;
+          rp[k * G + it] = rpow(d.fr[0], k + 1);
+          continue;
+        }
         double zx, zy;
         if (t < 2) {
           zx = t == 0 ? d.fr[4] : d.fr[2];
@@ -263,7 +270,6 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 3)
         const int4 z = zpow(unit(zx, zy), m);
         ph[q * G + it] = (t == 0 || t == 2) ? ipow(z, -m) : (t == 4 ? ipow(z, m) : z);
       }
-      for (int q = q0; q < 2 * L + 2; q += Q) rp[q * G + it] = rpow(d.fr[0], q + 1);
     }
     if (!waited) {
       pdl_wait();  // the moments (and centres and radii) of the launches before are complete
@@ -475,7 +481,7 @@ int launch_contract(const PairDesc* items, const int* order, const ContractPlan*
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(kLmaxMax, grad)) != cudaSuccess)
     return -1;
   // CTAs stay resident and walk the groups (the tables are loaded once per CTA)
-  const int per_sm = std::max(1, std::min(grad ? 2 : 3, 227 * 1024 / (smem + (grad ? 23 : 6) * 1024)));
+  const int per_sm = std::max(1, std::min(grad ? 2 : 4, 227 * 1024 / (smem + (grad ? 23 : 6) * 1024)));
   const int grid = std::min(n_groups, per_sm * num_sms);
   if (!pdl)
     k<<<grid, kCT, smem, s>>>(items, order, plan, n_groups, Lmax_items, jobs, geoms, tab, rots, out);
