@@ -18,10 +18,11 @@
 //                         ticket) reduces its tile rows in tile order.
 // What bounds it: for small calls the chain of dependent steps: a tile list, and a launch, a ticket and
 // a last tile per pass, took 28 us for one system of 20,000 atoms and 27 for two of 200; one kernel takes
-// 17 and 13.  For batches the instructions, about 140 float ones an atom for the float-float sums, and the
-// reads of the coordinates: 2,048 uneven systems 405 us before, 416 now.  The limits: at 2,048 atoms for
-// one CTA the batch paid for clusters with an atom or two per thread (462 us); double records of 3,260
-// atoms take 21 us on one CTA, 15 on a cluster.
+// 17 and 13.  For batches the instructions, 141 float operations an atom for the float-float sums (two to a
+// packed f32x2 instruction), and the reads of the coordinates: 2,048 uneven systems took 423 us with single
+// instructions and loads in fours, 397 packed and in pairs (fewer registers spilled; three CTAs per SM
+// without spills: 439).  The limits: at 2,048 atoms for one CTA the batch paid for clusters with an atom or
+// two per thread (462 us; at 4,096 419); double records of 3,260 atoms take 21 us on one CTA, 15 on a cluster.
 //
 // Per-atom arithmetic is float for float records: error-free two-sums for the centroid, float-float
 // (two-sum and fma-based two-product) for the low-degree sums, and a float filter for the radius: a
@@ -66,12 +67,39 @@ __device__ __forceinline__ FF ff_sub_split(float x, float hi, float lo) {
   return FF{s, e - lo};
 }
 
+// The same operations on two independent values at once, packed f32x2 instructions with the roundings of
+// the single ones (a - b as b (-1) + a, rounded once).
+struct FF2 {
+  float2 h, l;
+};
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ void ff_acc2(float2& s, float2& e, FF2 x) {
+  const float2 t = __fadd2_rn(s, x.h);
+  const float2 bb = sub2(t, s);
+  e = __fadd2_rn(e, __fadd2_rn(__fadd2_rn(sub2(s, sub2(t, bb)), sub2(x.h, bb)), x.l));
+  s = t;
+}
+__device__ __forceinline__ FF2 ff_mul2(FF2 a, FF2 b) {
+  const float2 p = __fmul2_rn(a.h, b.h);
+  float2 e = __ffma2_rn(a.h, b.h, make_float2(-p.x, -p.y));
+  e = __ffma2_rn(a.h, b.l, e);
+  e = __ffma2_rn(a.l, b.h, e);
+  return FF2{p, e};
+}
+__device__ __forceinline__ FF2 ff_sub_split2(float2 x, float2 hi, float2 lo) {
+  const float2 s = sub2(x, hi);
+  const float2 bb = sub2(s, x);
+  const float2 e = __fadd2_rn(sub2(x, sub2(s, bb)), sub2(make_float2(-hi.x, -hi.y), bb));
+  return FF2{s, sub2(e, lo)};
+}
+
 // |x - c|^2 in float from the exact difference d (each coordinate rounded once): within about
 // 3 x 2^-24 of the exact value.  The first scan of the radius filter takes this from the
 // differences it forms for the low-degree sums anyway.
-__device__ __forceinline__ float r2_float(const FF* d) {
-  const float x = d[0].h + d[0].l, y = d[1].h + d[1].l, z = d[2].h + d[2].l;
-  return __fmaf_rn(x, x, __fmaf_rn(y, y, z * z));
+__device__ __forceinline__ float r2_float(FF2 d01, FF d2) {
+  const float2 xy = __fadd2_rn(d01.h, d01.l);
+  const float z = d2.h + d2.l;
+  return __fmaf_rn(xy.x, xy.x, __fmaf_rn(xy.y, xy.y, z * z));
 }
 
 // |x - c|^2 in plain float, d_k = (x_k - c_hi,k) - c_lo,k: each difference within 2^-23 of its
@@ -213,32 +241,49 @@ __device__ __forceinline__ bool last_tile(int* ticket, int n_tiles, int lane) {
 
 // Atoms per lane whose loads are issued together before any of their arithmetic (the per-atom
 // work is short, so a lane must keep several loads in flight to cover the memory latency).
-constexpr int kSysBatch = 4;
+constexpr int kSysBatch = 4;  // centroid
+constexpr int kLowBatch = 2;  // radius and low-degree sums: more arithmetic per load, more registers
 
-template <typename Q>
-__device__ __forceinline__ FF q_times(Q q, FF d);
-template <>
-__device__ __forceinline__ FF q_times<FF>(FF q, FF d) { return ff_mul(q, d); }
-template <>
-__device__ __forceinline__ FF q_times<float>(float q, FF d) { return ff_mul_f(q, d); }
+__device__ __forceinline__ FF2 q_times2(FF q, FF2 d) { return ff_mul2(FF2{make_float2(q.h, q.h), make_float2(q.l, q.l)}, d); }
+__device__ __forceinline__ FF q_times(FF q, FF d) { return ff_mul(q, d); }
+__device__ __forceinline__ FF2 q_times2(float q, FF2 d) {
+  const float2 q2 = make_float2(q, q), p = __fmul2_rn(q2, d.h);
+  return FF2{p, __ffma2_rn(q2, d.l, __ffma2_rn(q2, d.h, make_float2(-p.x, -p.y)))};
+}
+__device__ __forceinline__ FF q_times(float q, FF d) { return ff_mul_f(q, d); }
 __device__ __forceinline__ FF as_ff(FF q) { return q; }
 __device__ __forceinline__ FF as_ff(float q) { return FF{q, 0.f}; }
 
-// q is a float (float records: the charge is exact) or an FF pair (double records).
-template <typename Q>
-__device__ __forceinline__ void low_accumulate(float* s, float* e, Q q, const FF* d) {
-  ff_acc(s[0], e[0], as_ff(q));
-  const FF qd0 = q_times(q, d[0]), qd1 = q_times(q, d[1]), qd2 = q_times(q, d[2]);
-  ff_acc(s[1], e[1], qd0);
-  ff_acc(s[2], e[2], qd1);
-  ff_acc(s[3], e[3], qd2);
-  ff_acc(s[4], e[4], ff_mul(qd0, d[0]));
-  ff_acc(s[5], e[5], ff_mul(qd0, d[1]));
-  ff_acc(s[6], e[6], ff_mul(qd0, d[2]));
-  ff_acc(s[7], e[7], ff_mul(qd1, d[1]));
-  ff_acc(s[8], e[8], ff_mul(qd1, d[2]));
-  ff_acc(s[9], e[9], ff_mul(qd2, d[2]));
-}
+// The ten low-degree sums of a lane, two to a packed accumulator: (S, P_z), (P_x, P_y), (T_xx, T_yy),
+// (T_xz, T_yz), (T_xy, T_zz).  Packed, an atom takes about 90 issue slots instead of 141.
+struct LowAcc {
+  float2 s[5], e[5];
+  __device__ __forceinline__ LowAcc() {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) s[k] = e[k] = make_float2(0.f, 0.f);
+  }
+  // q is a float (float records: the charge is exact) or an FF pair (double records).
+  template <typename Q>
+  __device__ __forceinline__ void add(Q q, FF2 d01, FF d2) {
+    const FF2 qd01 = q_times2(q, d01);
+    const FF qd2 = q_times(q, d2), qq = as_ff(q);
+    ff_acc2(s[0], e[0], FF2{make_float2(qq.h, qd2.h), make_float2(qq.l, qd2.l)});
+    ff_acc2(s[1], e[1], qd01);
+    ff_acc2(s[2], e[2], ff_mul2(qd01, d01));
+    ff_acc2(s[3], e[3], ff_mul2(qd01, FF2{make_float2(d2.h, d2.h), make_float2(d2.l, d2.l)}));
+    ff_acc2(s[4], e[4], ff_mul2(FF2{make_float2(qd01.h.x, qd2.h), make_float2(qd01.l.x, qd2.l)},
+                                FF2{make_float2(d01.h.y, d2.h), make_float2(d01.l.y, d2.l)}));
+  }
+  // in the order S, P_x, P_y, P_z, T_xx, T_xy, T_xz, T_yy, T_yz, T_zz
+  __device__ __forceinline__ void get(float* so, float* eo) const {
+    auto put = [&](const float2* v, float* o) {
+      o[0] = v[0].x; o[1] = v[1].x; o[2] = v[1].y; o[3] = v[0].y; o[4] = v[2].x;
+      o[5] = v[4].x; o[6] = v[3].x; o[7] = v[2].y; o[8] = v[3].y; o[9] = v[4].y;
+    };
+    put(s, so);
+    put(e, eo);
+  }
+};
 
 __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __restrict__ jobs,
                                                               const SysTile* __restrict__ tiles, int n_tiles,
@@ -255,6 +300,7 @@ __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __re
   if (j.dtype == TCM_F32) {
     const float4* X = reinterpret_cast<const float4*>(j.xyzq);
     float s[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
+    float2 s2 = make_float2(0.f, 0.f), e2 = make_float2(0.f, 0.f);
     for (long long i = i0 + lane; i < i1; i += 32 * kSysBatch) {
       float4 v[kSysBatch];
 #pragma unroll
@@ -262,11 +308,11 @@ __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __re
         v[u] = i + 32 * u < i1 ? __ldg(X + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < kSysBatch; ++u) {
-        ff_acc(s[0], e[0], FF{v[u].x, 0.f});
-        ff_acc(s[1], e[1], FF{v[u].y, 0.f});
+        ff_acc2(s2, e2, FF2{make_float2(v[u].x, v[u].y), make_float2(0.f, 0.f)});
         ff_acc(s[2], e[2], FF{v[u].z, 0.f});
       }
     }
+    s[0] = s2.x, s[1] = s2.y, e[0] = e2.x, e[1] = e2.y;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       ff_warp_sum(s[k], e[k]);
@@ -328,25 +374,23 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   const long long i0 = (long long)tl.t * j.atoms_per_tile;
   const long long i1 = min(j.n, i0 + (long long)j.atoms_per_tile);
   double rmax = 0.0;  // exact max |x - c|^2 of the tile's atoms
-  float s[kLowSums], e[kLowSums];
-#pragma unroll
-  for (int k = 0; k < kLowSums; ++k) s[k] = e[k] = 0.f;
+  LowAcc acc;
   if (j.dtype == TCM_F32) {
     const float4* X = reinterpret_cast<const float4*>(j.xyzq);
     const float* chi = g.chi;
     const float* clo = g.clo;
     float mf = 0.f;  // lane's largest |x - c|^2 in float (within about 4e-7 of the exact value)
-    for (long long i = i0 + lane; i < i1; i += 32 * kSysBatch) {
-      float4 v[kSysBatch];
+    for (long long i = i0 + lane; i < i1; i += 32 * kLowBatch) {
+      float4 v[kLowBatch];
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u)
+      for (int u = 0; u < kLowBatch; ++u)
         v[u] = i + 32 * u < i1 ? __ldg(X + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
-        const FF d[3] = {ff_sub_split(v[u].x, chi[0], clo[0]), ff_sub_split(v[u].y, chi[1], clo[1]),
-                         ff_sub_split(v[u].z, chi[2], clo[2])};
-        if (i + 32 * u < i1) mf = fmaxf(mf, r2_float(d));
-        if (j.need_low) low_accumulate(s, e, v[u].w, d);  // padding atoms carry q = 0
+      for (int u = 0; u < kLowBatch; ++u) {
+        const FF2 d01 = ff_sub_split2(make_float2(v[u].x, v[u].y), make_float2(chi[0], chi[1]), make_float2(clo[0], clo[1]));
+        const FF d2 = ff_sub_split(v[u].z, chi[2], clo[2]);
+        if (i + 32 * u < i1) mf = fmaxf(mf, r2_float(d01, d2));
+        if (j.need_low) acc.add(v[u].w, d01, d2);  // padding atoms carry q = 0
       }
     }
     // the exact radius: only atoms within a relative 4e-6 of the tile's float maximum can hold
@@ -373,16 +417,16 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
     }
   } else {
     const double2* X = reinterpret_cast<const double2*>(j.xyzq);
-    for (long long i = i0 + lane; i < i1; i += 32 * kSysBatch) {
-      double2 a[kSysBatch], b[kSysBatch];
+    for (long long i = i0 + lane; i < i1; i += 32 * kLowBatch) {
+      double2 a[kLowBatch], b[kLowBatch];
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
+      for (int u = 0; u < kLowBatch; ++u) {
         const bool ok = i + 32 * u < i1;
         a[u] = ok ? __ldg(X + 2 * (i + 32 * u)) : make_double2(g.c[0], g.c[1]);
         b[u] = ok ? __ldg(X + 2 * (i + 32 * u) + 1) : make_double2(g.c[2], 0.0);  // padding: d = 0, q = 0
       }
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
+      for (int u = 0; u < kLowBatch; ++u) {
         const double dd[4] = {a[u].x - g.c[0], a[u].y - g.c[1], b[u].x - g.c[2], b[u].y};
         rmax = fmax(rmax, dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
         if (j.need_low) {
@@ -392,7 +436,7 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
             const float h = (float)dd[k];
             t[k] = FF{h, (float)(dd[k] - (double)h)};
           }
-          low_accumulate(s, e, t[3], t);
+          acc.add(t[3], FF2{make_float2(t[0].h, t[1].h), make_float2(t[0].l, t[1].l)}, t[2]);
         }
       }
     }
@@ -401,6 +445,8 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   double* row = part + (long long)(j.tile_base + tl.t) * kSysPart;
   if (j.need_low) {
     static_assert(kLowSums == 10, "the lane map of the reduce-scatter is for ten sums");
+    float s[kLowSums], e[kLowSums];
+    acc.get(s, e);
     ff_reduce_scatter<kLowSums, 16>(s, e, lane);
     if ((kRs10Lanes >> lane) & 1u) {  // the lane holding sum k writes its (hi, lo) pair
       const int k = 5 * ((lane >> 4) & 1) + 3 * ((lane >> 3) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1);
@@ -434,34 +480,34 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
 // float (mf, float records) or exact (rmax, double records).
 template <bool kLow>
 __device__ __forceinline__ void scan_atoms(const SysJob& j, const double* c, const float* chi, const float* clo,
-                                           long long i0, long long step, float* s, float* e, float& mf, double& rmax) {
+                                           long long i0, long long step, LowAcc& acc, float& mf, double& rmax) {
   if (j.dtype == TCM_F32) {
     const float4* X = reinterpret_cast<const float4*>(j.xyzq);
-    for (long long i = i0; i < j.n; i += step * kSysBatch) {
-      float4 v[kSysBatch];
+    for (long long i = i0; i < j.n; i += step * kLowBatch) {
+      float4 v[kLowBatch];
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u)
+      for (int u = 0; u < kLowBatch; ++u)
         v[u] = i + step * u < j.n ? __ldg(X + i + step * u) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
-        const FF d[3] = {ff_sub_split(v[u].x, chi[0], clo[0]), ff_sub_split(v[u].y, chi[1], clo[1]),
-                         ff_sub_split(v[u].z, chi[2], clo[2])};
-        if (i + step * u < j.n) mf = fmaxf(mf, r2_float(d));
-        if (kLow) low_accumulate(s, e, v[u].w, d);  // padding atoms carry q = 0
+      for (int u = 0; u < kLowBatch; ++u) {
+        const FF2 d01 = ff_sub_split2(make_float2(v[u].x, v[u].y), make_float2(chi[0], chi[1]), make_float2(clo[0], clo[1]));
+        const FF d2 = ff_sub_split(v[u].z, chi[2], clo[2]);
+        if (i + step * u < j.n) mf = fmaxf(mf, r2_float(d01, d2));
+        if (kLow) acc.add(v[u].w, d01, d2);  // padding atoms carry q = 0
       }
     }
   } else {
     const double2* X = reinterpret_cast<const double2*>(j.xyzq);
-    for (long long i = i0; i < j.n; i += step * kSysBatch) {
-      double2 a[kSysBatch], b[kSysBatch];
+    for (long long i = i0; i < j.n; i += step * kLowBatch) {
+      double2 a[kLowBatch], b[kLowBatch];
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
+      for (int u = 0; u < kLowBatch; ++u) {
         const bool ok = i + step * u < j.n;
         a[u] = ok ? __ldg(X + 2 * (i + step * u)) : make_double2(c[0], c[1]);
         b[u] = ok ? __ldg(X + 2 * (i + step * u) + 1) : make_double2(c[2], 0.0);  // padding: d = 0, q = 0
       }
 #pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
+      for (int u = 0; u < kLowBatch; ++u) {
         const double dd[4] = {a[u].x - c[0], a[u].y - c[1], b[u].x - c[2], b[u].y};
         rmax = fmax(rmax, dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
         if (kLow) {
@@ -471,7 +517,7 @@ __device__ __forceinline__ void scan_atoms(const SysJob& j, const double* c, con
             const float h = (float)dd[k];
             t[k] = FF{h, (float)(dd[k] - (double)h)};
           }
-          low_accumulate(s, e, t[3], t);
+          acc.add(t[3], FF2{make_float2(t[0].h, t[1].h), make_float2(t[0].l, t[1].l)}, t[2]);
         }
       }
     }
@@ -517,6 +563,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
     if (j.dtype == TCM_F32) {
       const float4* X = reinterpret_cast<const float4*>(j.xyzq);
       float s[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
+      float2 s2 = make_float2(0.f, 0.f), e2 = make_float2(0.f, 0.f);
       for (long long i = i0; i < j.n; i += step * kSysBatch) {
         float4 v[kSysBatch];
 #pragma unroll
@@ -524,11 +571,11 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
           v[u] = i + step * u < j.n ? __ldg(X + i + step * u) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < kSysBatch; ++u) {
-          ff_acc(s[0], e[0], FF{v[u].x, 0.f});
-          ff_acc(s[1], e[1], FF{v[u].y, 0.f});
+          ff_acc2(s2, e2, FF2{make_float2(v[u].x, v[u].y), make_float2(0.f, 0.f)});
           ff_acc(s[2], e[2], FF{v[u].z, 0.f});
         }
       }
+      s[0] = s2.x, s[1] = s2.y, e[0] = e2.x, e[1] = e2.y;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         ff_warp_sum(s[k], e[k]);
@@ -583,18 +630,19 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
   }
   const double c[3] = {sh.c[0], sh.c[1], sh.c[2]};
   const float chi[3] = {sh.chi[0], sh.chi[1], sh.chi[2]}, clo[3] = {sh.clo[0], sh.clo[1], sh.clo[2]};
-  float s[kLowSums], e[kLowSums], mf = 0.f;
+  LowAcc acc;
+  float mf = 0.f;
   double rmax = 0.0;
-#pragma unroll
-  for (int k = 0; k < kLowSums; ++k) s[k] = e[k] = 0.f;
   if (j.need_low) {
-    scan_atoms<true>(j, c, chi, clo, i0, step, s, e, mf, rmax);
+    scan_atoms<true>(j, c, chi, clo, i0, step, acc, mf, rmax);
+    float s[kLowSums], e[kLowSums];
+    acc.get(s, e);
     ff_reduce_scatter<kLowSums, 16>(s, e, lane);
     if ((kRs10Lanes >> lane) & 1u)
       sh.wlow[w][5 * ((lane >> 4) & 1) + 3 * ((lane >> 3) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1)] =
           make_float2(s[0], e[0]);
   } else {
-    scan_atoms<false>(j, c, chi, clo, i0, step, s, e, mf, rmax);
+    scan_atoms<false>(j, c, chi, clo, i0, step, acc, mf, rmax);
   }
   if (j.need_radius && j.dtype == TCM_F32) {
 #pragma unroll
