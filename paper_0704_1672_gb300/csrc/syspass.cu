@@ -20,14 +20,16 @@
 // a last tile per pass, took 28 us for one system of 20,000 atoms and 27 for two of 200; one kernel takes
 // 17 and 13.  For batches the instructions, 141 float operations an atom for the float-float sums (two to a
 // packed f32x2 instruction), and the reads of the coordinates: 2,048 uneven systems took 423 us with single
-// instructions and loads in fours, 397 packed and in pairs (fewer registers spilled; three CTAs per SM
-// without spills: 439).  The limits: at 2,048 atoms for one CTA the batch paid for clusters with an atom or
-// two per thread (462 us; at 4,096 419); double records of 3,260 atoms take 21 us on one CTA, 15 on a cluster.
+// instructions, 397 packed, 348 with 32-bit indices, full batches without predicates and the radius's
+// candidates kept from the one scan instead of found by another.  The limits: at 2,048 atoms for one CTA
+// the batch paid for clusters with an atom or two per thread (462 us before; at 4,096 419 against 406);
+// double records of 3,260 atoms take 21 us on one CTA, 15 on a cluster.
 //
 // Per-atom arithmetic is float for float records: error-free two-sums for the centroid, float-float
-// (two-sum and fma-based two-product) for the low-degree sums, and a float filter for the radius: a
-// second scan (from cache) recomputes in double only the atoms within a relative 4e-6 of the float
-// maximum.  Every reduction runs in a fixed order.
+// (two-sum and fma-based two-product) for the low-degree sums, and a float filter for the radius: each
+// thread keeps its farthest atom, and only those within a relative 4e-6 of the float maximum are
+// recomputed in double (if a thread's second farthest is as near, the atoms are scanned again).  Every
+// reduction runs in a fixed order.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -93,19 +95,9 @@ __device__ __forceinline__ FF2 ff_sub_split2(float2 x, float2 hi, float2 lo) {
   return FF2{s, sub2(e, lo)};
 }
 
-// |x - c|^2 in float from the exact difference d (each coordinate rounded once): within about
-// 3 x 2^-24 of the exact value.  The first scan of the radius filter takes this from the
-// differences it forms for the low-degree sums anyway.
-__device__ __forceinline__ float r2_float(FF2 d01, FF d2) {
-  const float2 xy = __fadd2_rn(d01.h, d01.l);
-  const float z = d2.h + d2.l;
-  return __fmaf_rn(xy.x, xy.x, __fmaf_rn(xy.y, xy.y, z * z));
-}
-
 // |x - c|^2 in plain float, d_k = (x_k - c_hi,k) - c_lo,k: each difference within 2^-23 of its
-// value, the square within about 7 x 2^-24 (4.2e-7).  The second scan of the radius filter uses
-// this cheaper form; with the first scan's 1.8e-7 the two stay far inside the filter's 4e-6
-// margin, so the atom of the exact maximum is always among the candidates.
+// value, the square within about 7 x 2^-24 (4.2e-7), far inside the radius filter's margin of 4e-6:
+// the atom of the exact maximum is always among the candidates.
 __device__ __forceinline__ float r2_plain(const float4& v, const float* chi, const float* clo) {
   const float x = (v.x - chi[0]) - clo[0], y = (v.y - chi[1]) - clo[1], z = (v.z - chi[2]) - clo[2];
   return __fmaf_rn(x, x, __fmaf_rn(y, y, z * z));
@@ -285,6 +277,23 @@ struct LowAcc {
   }
 };
 
+// Float-float sums of the positions of atoms i, i + step, ... < n (float records).
+__device__ __forceinline__ void sum_f32(const float4* X, int n, int i, int step, float2& s2, float2& e2, float& sz, float& ez) {
+  auto one = [&](const float4& v) {
+    ff_acc2(s2, e2, FF2{make_float2(v.x, v.y), make_float2(0.f, 0.f)});
+    ff_acc(sz, ez, FF{v.z, 0.f});
+  };
+  for (; i + (kSysBatch - 1) * step < n; i += kSysBatch * step) {
+    float4 v[kSysBatch];
+#pragma unroll
+    for (int u = 0; u < kSysBatch; ++u) v[u] = __ldg(X + i + u * step);
+#pragma unroll
+    for (int u = 0; u < kSysBatch; ++u) one(v[u]);
+  }
+#pragma unroll 1
+  for (; i < n; i += step) one(__ldg(X + i));
+}
+
 __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __restrict__ jobs,
                                                               const SysTile* __restrict__ tiles, int n_tiles,
                                                               double* __restrict__ part, int* __restrict__ tickets,
@@ -301,17 +310,7 @@ __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __re
     const float4* X = reinterpret_cast<const float4*>(j.xyzq);
     float s[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
     float2 s2 = make_float2(0.f, 0.f), e2 = make_float2(0.f, 0.f);
-    for (long long i = i0 + lane; i < i1; i += 32 * kSysBatch) {
-      float4 v[kSysBatch];
-#pragma unroll
-      for (int u = 0; u < kSysBatch; ++u)  // padding atoms add exact zeros
-        v[u] = i + 32 * u < i1 ? __ldg(X + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < kSysBatch; ++u) {
-        ff_acc2(s2, e2, FF2{make_float2(v[u].x, v[u].y), make_float2(0.f, 0.f)});
-        ff_acc(s[2], e[2], FF{v[u].z, 0.f});
-      }
-    }
+    sum_f32(X + i0, (int)(i1 - i0), lane, 32, s2, e2, s[2], e[2]);
     s[0] = s2.x, s[1] = s2.y, e[0] = e2.x, e[1] = e2.y;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -359,6 +358,95 @@ __global__ void __launch_bounds__(kSysThreads) k_sys_centroid(const SysJob* __re
   }
 }
 
+// A thread's two largest |x - c|^2 in float and the atom of the largest: what the radius filter needs
+// to name its candidates without a second scan of the atoms.
+struct Farthest {
+  float m1 = -1.f, m2 = -1.f;
+  int at = 0;
+  __device__ __forceinline__ void add(float r, int i) {
+    if (r > m1) at = i;
+    m2 = fmaxf(m2, fminf(m1, r));
+    m1 = fmaxf(m1, r);
+  }
+};
+
+// Float records: low-degree sums over atoms i, i + step, ... < n of X and the farthest of them.
+template <bool kLow>
+__device__ __forceinline__ void scan_f32(const float4* X, int n, int i, int step, const float* chi, const float* clo,
+                                         LowAcc& acc, Farthest& far) {
+  const float2 hi2 = make_float2(chi[0], chi[1]), lo2 = make_float2(clo[0], clo[1]);
+  auto one = [&](const float4& v, int at) {
+    const FF2 d01 = ff_sub_split2(make_float2(v.x, v.y), hi2, lo2);
+    const FF d2 = ff_sub_split(v.z, chi[2], clo[2]);
+    const float2 xy = sub2(sub2(make_float2(v.x, v.y), hi2), lo2);  // r2_plain
+    const float z = (v.z - chi[2]) - clo[2];
+    far.add(__fmaf_rn(xy.x, xy.x, __fmaf_rn(xy.y, xy.y, z * z)), at);
+    if (kLow) acc.add(v.w, d01, d2);
+  };
+  for (; i + (kLowBatch - 1) * step < n; i += kLowBatch * step) {
+    float4 v[kLowBatch];
+#pragma unroll
+    for (int u = 0; u < kLowBatch; ++u) v[u] = __ldg(X + i + u * step);
+#pragma unroll
+    for (int u = 0; u < kLowBatch; ++u) one(v[u], i + u * step);
+  }
+  for (; i < n; i += step) one(__ldg(X + i), i);
+}
+
+// The same of double records; rmax: the exact largest |x - c|^2.
+template <bool kLow>
+__device__ __forceinline__ void scan_f64(const double2* X, int n, int i0, int step, const double* c, LowAcc& acc, double& rmax) {
+  for (int i = i0; i < n; i += step * kLowBatch) {
+    double2 a[kLowBatch], b[kLowBatch];
+#pragma unroll
+    for (int u = 0; u < kLowBatch; ++u) {
+      const bool ok = i + step * u < n;
+      a[u] = ok ? __ldg(X + 2 * (i + step * u)) : make_double2(c[0], c[1]);
+      b[u] = ok ? __ldg(X + 2 * (i + step * u) + 1) : make_double2(c[2], 0.0);  // padding: d = 0, q = 0
+    }
+#pragma unroll
+    for (int u = 0; u < kLowBatch; ++u) {
+      const double dd[4] = {a[u].x - c[0], a[u].y - c[1], b[u].x - c[2], b[u].y};
+      rmax = fmax(rmax, dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
+      if (kLow) {
+        FF t[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float h = (float)dd[k];
+          t[k] = FF{h, (float)(dd[k] - (double)h)};
+        }
+        acc.add(t[3], FF2{make_float2(t[0].h, t[1].h), make_float2(t[0].l, t[1].l)}, t[2]);
+      }
+    }
+  }
+}
+
+// The exact largest |x - c|^2 of a warp's atoms (float records) among those within a relative 4e-6 of
+// the float maximum mf: each lane's farthest; if a lane's second is within it too, every atom in
+// question is looked at.  The candidates are taken one at a time, in a loop whose trip count is the
+// warp's candidate count: a predicated double block would occupy the 1/64-rate FP64 pipe every time.
+// Lane l's atoms are i0 + l, i0 + l + step, ... < n.
+__device__ __forceinline__ double exact_r2(const float4* X, int n, int i0, int step, int lane, const double* c,
+                                           const float* chi, const float* clo, const Farthest& far, float mf) {
+  const float thr = mf * (1.0f - 4e-6f);
+  double rmax = 0.0;
+  auto exact = [&](int i) {
+    const float4 v = __ldg(X + i);
+    const double ex = (double)v.x - c[0], ey = (double)v.y - c[1], ez = (double)v.z - c[2];
+    rmax = fmax(rmax, ex * ex + ey * ey + ez * ez);  // the same value in every lane
+  };
+  if (!__any_sync(0xffffffffu, far.m2 >= thr)) {
+    for (unsigned m = __ballot_sync(0xffffffffu, far.m1 >= thr); m; m &= m - 1)
+      exact(__shfl_sync(0xffffffffu, far.at, __ffs(m) - 1));
+    return rmax;
+  }
+  for (int iw = i0; iw < n; iw += step) {  // warp-uniform trip count
+    const bool cand = iw + lane < n && r2_plain(__ldg(X + iw + lane), chi, clo) >= thr;
+    for (unsigned m = __ballot_sync(0xffffffffu, cand); m; m &= m - 1) exact(iw + __ffs(m) - 1);
+  }
+  return rmax;
+}
+
 __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob* __restrict__ jobs,
                                                                 const SysTile* __restrict__ tiles, int n_tiles,
                                                                 double* __restrict__ part, int* __restrict__ tickets,
@@ -375,71 +463,26 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   const long long i1 = min(j.n, i0 + (long long)j.atoms_per_tile);
   double rmax = 0.0;  // exact max |x - c|^2 of the tile's atoms
   LowAcc acc;
+  const int cnt = (int)(i1 - i0);
   if (j.dtype == TCM_F32) {
-    const float4* X = reinterpret_cast<const float4*>(j.xyzq);
-    const float* chi = g.chi;
-    const float* clo = g.clo;
-    float mf = 0.f;  // lane's largest |x - c|^2 in float (within about 4e-7 of the exact value)
-    for (long long i = i0 + lane; i < i1; i += 32 * kLowBatch) {
-      float4 v[kLowBatch];
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u)
-        v[u] = i + 32 * u < i1 ? __ldg(X + i + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u) {
-        const FF2 d01 = ff_sub_split2(make_float2(v[u].x, v[u].y), make_float2(chi[0], chi[1]), make_float2(clo[0], clo[1]));
-        const FF d2 = ff_sub_split(v[u].z, chi[2], clo[2]);
-        if (i + 32 * u < i1) mf = fmaxf(mf, r2_float(d01, d2));
-        if (j.need_low) acc.add(v[u].w, d01, d2);  // padding atoms carry q = 0
-      }
-    }
-    // the exact radius: only atoms within a relative 4e-6 of the tile's float maximum can hold
-    // the exact maximum; a second scan of the tile (from cache) recomputes just those in double
+    const float4* X = reinterpret_cast<const float4*>(j.xyzq) + i0;
+    Farthest far;
+    if (j.need_low)
+      scan_f32<true>(X, cnt, lane, 32, g.chi, g.clo, acc, far);
+    else
+      scan_f32<false>(X, cnt, lane, 32, g.chi, g.clo, acc, far);
     if (j.need_radius) {
+      float mf = far.m1;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
-      const float thr = mf * (1.0f - 4e-6f);
-      for (long long i0w = i0; i0w < i1; i0w += 32) {  // warp-uniform trip count
-        const long long i = i0w + lane;
-        bool cand = false;
-        if (i < i1) cand = r2_plain(__ldg(X + i), chi, clo) >= thr;
-        // the candidates one at a time, in a loop whose trip count is the warp's candidate count:
-        // a predicated double block would occupy GB300's 1/64-rate FP64 pipe for every atom
-        unsigned m = __ballot_sync(0xffffffffu, cand);
-        while (m) {
-          const int src = __ffs(m) - 1;
-          m &= m - 1;
-          const float4 w = __ldcg(X + i0w + src);
-          const double ex = (double)w.x - g.c[0], ey = (double)w.y - g.c[1], ez = (double)w.z - g.c[2];
-          rmax = fmax(rmax, ex * ex + ey * ey + ez * ez);  // the same value in every lane
-        }
-      }
+      rmax = exact_r2(X, cnt, 0, 32, lane, g.c, g.chi, g.clo, far, mf);
     }
   } else {
-    const double2* X = reinterpret_cast<const double2*>(j.xyzq);
-    for (long long i = i0 + lane; i < i1; i += 32 * kLowBatch) {
-      double2 a[kLowBatch], b[kLowBatch];
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u) {
-        const bool ok = i + 32 * u < i1;
-        a[u] = ok ? __ldg(X + 2 * (i + 32 * u)) : make_double2(g.c[0], g.c[1]);
-        b[u] = ok ? __ldg(X + 2 * (i + 32 * u) + 1) : make_double2(g.c[2], 0.0);  // padding: d = 0, q = 0
-      }
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u) {
-        const double dd[4] = {a[u].x - g.c[0], a[u].y - g.c[1], b[u].x - g.c[2], b[u].y};
-        rmax = fmax(rmax, dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
-        if (j.need_low) {
-          FF t[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float h = (float)dd[k];
-            t[k] = FF{h, (float)(dd[k] - (double)h)};
-          }
-          acc.add(t[3], FF2{make_float2(t[0].h, t[1].h), make_float2(t[0].l, t[1].l)}, t[2]);
-        }
-      }
-    }
+    const double2* X = reinterpret_cast<const double2*>(j.xyzq) + 2 * i0;
+    if (j.need_low)
+      scan_f64<true>(X, cnt, lane, 32, g.c, acc, rmax);
+    else
+      scan_f64<false>(X, cnt, lane, 32, g.c, acc, rmax);
   }
   rmax = warp_max_d(rmax);
   double* row = part + (long long)(j.tile_base + tl.t) * kSysPart;
@@ -476,54 +519,6 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   }
 }
 
-// Sums of one low-degree accumulator set over atoms i, i + step, ... and the largest |x - c|^2: in
-// float (mf, float records) or exact (rmax, double records).
-template <bool kLow>
-__device__ __forceinline__ void scan_atoms(const SysJob& j, const double* c, const float* chi, const float* clo,
-                                           long long i0, long long step, LowAcc& acc, float& mf, double& rmax) {
-  if (j.dtype == TCM_F32) {
-    const float4* X = reinterpret_cast<const float4*>(j.xyzq);
-    for (long long i = i0; i < j.n; i += step * kLowBatch) {
-      float4 v[kLowBatch];
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u)
-        v[u] = i + step * u < j.n ? __ldg(X + i + step * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u) {
-        const FF2 d01 = ff_sub_split2(make_float2(v[u].x, v[u].y), make_float2(chi[0], chi[1]), make_float2(clo[0], clo[1]));
-        const FF d2 = ff_sub_split(v[u].z, chi[2], clo[2]);
-        if (i + step * u < j.n) mf = fmaxf(mf, r2_float(d01, d2));
-        if (kLow) acc.add(v[u].w, d01, d2);  // padding atoms carry q = 0
-      }
-    }
-  } else {
-    const double2* X = reinterpret_cast<const double2*>(j.xyzq);
-    for (long long i = i0; i < j.n; i += step * kLowBatch) {
-      double2 a[kLowBatch], b[kLowBatch];
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u) {
-        const bool ok = i + step * u < j.n;
-        a[u] = ok ? __ldg(X + 2 * (i + step * u)) : make_double2(c[0], c[1]);
-        b[u] = ok ? __ldg(X + 2 * (i + step * u) + 1) : make_double2(c[2], 0.0);  // padding: d = 0, q = 0
-      }
-#pragma unroll
-      for (int u = 0; u < kLowBatch; ++u) {
-        const double dd[4] = {a[u].x - c[0], a[u].y - c[1], b[u].x - c[2], b[u].y};
-        rmax = fmax(rmax, dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2]);
-        if (kLow) {
-          FF t[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float h = (float)dd[k];
-            t[k] = FF{h, (float)(dd[k] - (double)h)};
-          }
-          acc.add(t[3], FF2{make_float2(t[0].h, t[1].h), make_float2(t[0].l, t[1].l)}, t[2]);
-        }
-      }
-    }
-  }
-}
-
 // One system per cluster of CL CTAs; atom i belongs to thread i mod (CL kSysThreads).
 template <int CL>
 struct OneShared {
@@ -546,8 +541,9 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
   const SysJob j = jobs[blockIdx.x / CL];
   const int rank = blockIdx.x % CL;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  constexpr long long step = (long long)CL * kSysThreads;
-  const long long i0 = (long long)rank * kSysThreads + t;
+  const int n = (int)j.n;  // at most kSysClusterMax
+  constexpr int step = CL * kSysThreads;
+  const int i0 = rank * kSysThreads + t;
   auto sync = [] {
     if constexpr (CL > 1)
       cg::this_cluster().sync();
@@ -564,17 +560,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
       const float4* X = reinterpret_cast<const float4*>(j.xyzq);
       float s[3] = {0.f, 0.f, 0.f}, e[3] = {0.f, 0.f, 0.f};
       float2 s2 = make_float2(0.f, 0.f), e2 = make_float2(0.f, 0.f);
-      for (long long i = i0; i < j.n; i += step * kSysBatch) {
-        float4 v[kSysBatch];
-#pragma unroll
-        for (int u = 0; u < kSysBatch; ++u)  // padding atoms add exact zeros
-          v[u] = i + step * u < j.n ? __ldg(X + i + step * u) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int u = 0; u < kSysBatch; ++u) {
-          ff_acc2(s2, e2, FF2{make_float2(v[u].x, v[u].y), make_float2(0.f, 0.f)});
-          ff_acc(s[2], e[2], FF{v[u].z, 0.f});
-        }
-      }
+      sum_f32(X, n, i0, step, s2, e2, s[2], e[2]);
       s[0] = s2.x, s[1] = s2.y, e[0] = e2.x, e[1] = e2.y;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
@@ -583,7 +569,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
       }
     } else {
       const double2* X = reinterpret_cast<const double2*>(j.xyzq);
-      for (long long i = i0; i < j.n; i += step) {
+      for (int i = i0; i < n; i += step) {
         const double2 a = __ldg(X + 2 * i), b = __ldg(X + 2 * i + 1);
         cs[0] += a.x;
         cs[1] += a.y;
@@ -631,39 +617,35 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
   const double c[3] = {sh.c[0], sh.c[1], sh.c[2]};
   const float chi[3] = {sh.chi[0], sh.chi[1], sh.chi[2]}, clo[3] = {sh.clo[0], sh.clo[1], sh.clo[2]};
   LowAcc acc;
-  float mf = 0.f;
+  Farthest far;
   double rmax = 0.0;
+  const float4* X4 = reinterpret_cast<const float4*>(j.xyzq);
+  const double2* X8 = reinterpret_cast<const double2*>(j.xyzq);
   if (j.need_low) {
-    scan_atoms<true>(j, c, chi, clo, i0, step, acc, mf, rmax);
+    if (j.dtype == TCM_F32)
+      scan_f32<true>(X4, n, i0, step, chi, clo, acc, far);
+    else
+      scan_f64<true>(X8, n, i0, step, c, acc, rmax);
     float s[kLowSums], e[kLowSums];
     acc.get(s, e);
     ff_reduce_scatter<kLowSums, 16>(s, e, lane);
     if ((kRs10Lanes >> lane) & 1u)
       sh.wlow[w][5 * ((lane >> 4) & 1) + 3 * ((lane >> 3) & 1) + 2 * ((lane >> 2) & 1) + ((lane >> 1) & 1)] =
           make_float2(s[0], e[0]);
+  } else if (j.dtype == TCM_F32) {
+    scan_f32<false>(X4, n, i0, step, chi, clo, acc, far);
   } else {
-    scan_atoms<false>(j, c, chi, clo, i0, step, acc, mf, rmax);
+    scan_f64<false>(X8, n, i0, step, c, acc, rmax);
   }
   if (j.need_radius && j.dtype == TCM_F32) {
+    float mf = far.m1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
     if (lane == 0) sh.wmf[w] = mf;
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kSysWarps; ++k) mf = fmaxf(mf, sh.wmf[k]);
-    const float thr = mf * (1.0f - 4e-6f);
-    const float4* X = reinterpret_cast<const float4*>(j.xyzq);
-    for (long long iw = i0 - lane; iw < j.n; iw += step) {  // warp-uniform trip count
-      const bool cand = iw + lane < j.n && r2_plain(__ldg(X + iw + lane), chi, clo) >= thr;
-      unsigned m = __ballot_sync(0xffffffffu, cand);  // the candidates one at a time: see k_sys_radius_low
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        const float4 v = __ldg(X + iw + src);
-        const double ex = (double)v.x - c[0], ey = (double)v.y - c[1], ez = (double)v.z - c[2];
-        rmax = fmax(rmax, ex * ex + ey * ey + ez * ez);
-      }
-    }
+    rmax = exact_r2(X4, n, i0 - lane, step, lane, c, chi, clo, far, mf);
   }
   rmax = warp_max_d(rmax);
   if (lane == 0) sh.wr2[w] = rmax;
