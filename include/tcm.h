@@ -73,8 +73,9 @@ typedef enum { TCM_F32 = 0, TCM_F64 = 1 } tcm_dtype;
 typedef enum {
   TCM_FP64 = 0,  /* every step in double precision */
   TCM_MIXED = 1  /* moment recurrence and per-atom products in float on radius-scaled
-                    coordinates; block partials, cross-block reduction, tables and the
-                    contraction in double */
+                    coordinates; block partials and the cross-block reduction in double.
+                    The contraction is the same for both: products in 60-bit fixed
+                    point, sums over (l1, l2) in double */
 } tcm_precision;
 
 typedef struct tcm_ctx* tcm_ctx_t;
@@ -131,7 +132,8 @@ const char* tcm_last_error(void);
 
 /* Phases of the path, for tracing and benchmarks. */
 typedef enum {
-  TCM_PHASE_GEOM = 0,     /* a1: centre and radius; set-up of the moment pass (tile list, low-degree sums) */
+  TCM_PHASE_GEOM = 0,     /* a1: centre and radius; set-up of the moment pass (tile list, low-degree sums,
+                             the contraction's pair items) */
   TCM_PHASE_MOMENTS = 1,  /* a2: per-atom moment accumulation and per-tile CTA reduction */
   TCM_PHASE_FINALIZE = 2, /* a3: cross-tile reduction in double and normalisation */
   TCM_PHASE_CONTRACT = 3, /* a4 + a5: irregular harmonics at R0 and the two-center contraction */
@@ -141,9 +143,10 @@ typedef enum {
   TCM_NPHASES = 6
 } tcm_phase;
 
-/* Tiling of the moment pass for one precision, every degree: each warp of the moment kernels
- * takes tiles of 32 x atoms_per_lane atoms (1..4096; defaults 64 for TCM_MIXED, 32 for
- * TCM_FP64).  A system's tiles, and so the rounding of its moments, depend only on its
+/* Tiling of the moment pass for one precision, every degree: a tile (a warp's in TCM_MIXED, a
+ * CTA's in TCM_FP64) has at most 32 x atoms_per_lane atoms (1..4096; defaults 64 for TCM_MIXED, 32
+ * for TCM_FP64, where the default gives small systems smaller tiles and a setting made here is taken
+ * as it is).  A system's tiles, and so the rounding of its moments, depend only on its
  * atom count, its Lmax and this setting.  Used by the autotuner. */
 int tcm_ctx_set_tiling(tcm_ctx_t ctx, int precision, int atoms_per_lane);
 
@@ -268,16 +271,17 @@ int tcm_gradients_batch(tcm_ctx_t ctx, int n_systems, const tcm_system* systems,
                         const tcm_pair_item* items, int precision, double* E, double* G, int32_t* status);
 
 /* Eq. (Coulomb): exact pairwise energy of A and B (B rotated by rotB about its centre,
- * NULL = identity) with the centre of B at the centre of A plus R0, in double
- * precision.  Writes the host double *E.  Synchronous. */
+ * NULL = identity) with the centre of B at the centre of A plus R0, as
+ * tcm_direct_batch.  Writes the host double *E.  Synchronous. */
 int tcm_direct(tcm_ctx_t ctx, const tcm_system* A, const tcm_system* B, const double* rotB,
                const double* R0, double* E);
 
 /* Eq. (Coulomb) for many placements of B against A (a potential-energy-surface scan, Section
  * IV): for item k, B rotated by rotB + 9 k (host row-major 3x3 array per item, or NULL for
  * none) about its centre, with its centre at A's centre plus R0 + 3 k (host).  E: device,
- * n_items doubles.  Double precision, one CTA per (item, 256 atoms of A), fixed-order sums.
- * Asynchronous on the context stream. */
+ * n_items doubles.  Fixed-order sums, split by the atom counts alone; for
+ * separated systems the pairs are summed in 64-bit fixed point (error against double below that of
+ * double arithmetic), otherwise in double.  Asynchronous on the context stream. */
 int tcm_direct_batch(tcm_ctx_t ctx, const tcm_system* A, const tcm_system* B, int64_t n_items,
                      const double* rotB, const double* R0, double* E);
 

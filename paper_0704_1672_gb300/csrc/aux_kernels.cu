@@ -1,8 +1,8 @@
 // Kernels around the moment pass:
 //   a3  cross-tile reduction of the moment partials in double, fixed order, plus the
 //       deferred normalisation F_lm a^l                                  (Eq. (multipole))
-//   a4  irregular solid harmonics of the separation vector R0            (Eq. (Formula))
-//   a5  two-center contraction in double                                 (Eq. (Formula))
+//   the contraction's pair items (frame of R0, Euler record) from runs of items
+//   the rotation of moment sets (tcm_rotate_moments)
 #include <cuda_runtime.h>
 
 #include "contract.h"

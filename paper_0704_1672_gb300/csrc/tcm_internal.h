@@ -227,10 +227,11 @@ constexpr int kSysPart = kSysPartLow + kLowSums;
 
 // Programmatic dependent launch: a kernel launched with programmatic stream serialization
 // is set up while its predecessor drains; pdl_wait() blocks until the predecessor grid has
-// completed and its memory is visible (a no-op for an ordinary launch).  Only the finalisation
-// issues griddepcontrol.launch_dependents (pdl_trigger), so that the contraction's CTAs set up
-// their tables while the last finalisation CTAs run; dependent CTAs made resident before the
-// moment kernel's tail had drained slowed the replayed step down (0.372 ms against 0.325 ms).
+// completed and its memory is visible (a no-op for an ordinary launch).  Who
+// issues griddepcontrol.launch_dependents (pdl_trigger): the finalisation, so that the contraction's
+// CTAs set up their tables while the last finalisation CTAs run, the kernels of the system pass
+// but the last, so that those of different sizes overlap, and k_frames.  Not the moment kernels: dependent CTAs
+// resident before their tail had drained slowed the replayed step down (0.372 ms against 0.325 ms).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -1,5 +1,5 @@
 """The system pass (centroid, radius, low-degree sums) at the limits of its three kernels: one CTA up
-to 2,048 atoms, a cluster up to 65,536, warp tiles above; float and double records, centre computed or
+to 8,192 atoms (1,024 double records), a cluster up to 65,536, warp tiles above; float and double records, centre computed or
 given.  Centre and radius to double rounding; the mixed path's degrees l <= 2, which come from the
 float-float sums (about 2^-44 of their terms), to 1e-11 of the terms' magnitude."""
 import numpy as np
