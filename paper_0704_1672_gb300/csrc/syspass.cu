@@ -519,6 +519,10 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   }
 }
 
+// The two halves of a cluster barrier: every thread of the cluster arrives, and waits for all.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
 // One system per cluster of CL CTAs; atom i belongs to thread i mod (CL kSysThreads).
 template <int CL>
 struct OneShared {
@@ -538,6 +542,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
   namespace cg = cooperative_groups;
   __shared__ OneShared<CL> sh;
   if (trigger) pdl_trigger();
+  if constexpr (CL > 1) cluster_arrive();  // (its wait: others_started)
   const SysJob j = jobs[blockIdx.x / CL];
   const int rank = blockIdx.x % CL;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -549,6 +554,12 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
       cg::this_cluster().sync();
     else
       __syncthreads();
+  };
+  // Ahead of a CTA's first access to another's shared memory: every CTA of the cluster has started (one
+  // that owns no atoms would store within a microsecond of its own start).  The barrier was entered at the
+  // top, so the wait is over by the time the scan of the atoms is.
+  auto others_started = [] {
+    if constexpr (CL > 1) cluster_wait();
   };
   auto of_rank = [&](auto* p, int r) {  // the same variable in CTA r of the cluster
     if constexpr (CL > 1) return cg::this_cluster().map_shared_rank(p, r);
@@ -579,6 +590,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
       for (int k = 0; k < 3; ++k) cs[k] = warp_sum_d(cs[k]);
     }
     if (lane < 3) sh.wcen[w][lane] = lane == 0 ? cs[0] : (lane == 1 ? cs[1] : cs[2]);
+    others_started();
     __syncthreads();
     if (t < 3) {
       double v = 0.0;
@@ -611,6 +623,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
   }
   __syncthreads();
   if (!j.need_radius && !j.need_low) {  // the whole cluster
+    if (!j.need_center) others_started();
     pdl_wait();
     return;
   }
@@ -649,6 +662,7 @@ __global__ void __launch_bounds__(kSysThreads, 4) k_sys_one(const SysJob* __rest
   }
   rmax = warp_max_d(rmax);
   if (lane == 0) sh.wr2[w] = rmax;
+  if (!j.need_center) others_started();
   __syncthreads();
   if (t < kLowSums && j.need_low) {
     FF v{0.f, 0.f};
