@@ -455,9 +455,11 @@ __global__ void __launch_bounds__(kSysThreads, 3) k_sys_radius_low(const SysJob*
   const int lane = threadIdx.x & 31;
   if (trigger) pdl_trigger();
   if (w >= n_tiles) return;
+  // the centroids of pass 1 are complete; with given centres there is no pass 1, and the kernel before is
+  // the one that wrote the tiles and jobs (a long tile list, the fixed scratch's descriptors)
+  pdl_wait();
   const SysTile tl = tiles[w];
   const SysJob j = jobs[tl.job];
-  pdl_wait();  // the centroids of pass 1 are complete
   const SysGeom g = geoms[j.geom];
   const long long i0 = (long long)tl.t * j.atoms_per_tile;
   const long long i1 = min(j.n, i0 + (long long)j.atoms_per_tile);
@@ -713,7 +715,8 @@ int launch_sys(const SysJob* jobs, const SysCount& n, const SysTile* t1, const S
   if (n.tiles2 > 0 && launch_pdl(k_sys_radius_low, dim3((n.tiles2 + kSysWarps - 1) / kSysWarps), dim3(kSysThreads), 0, s,
                                  jobs, t2, n.tiles2, part, tickets, geoms, n.cluster + n.one > 0) != cudaSuccess)
     return -1;
-  const bool overlap = pdl || n.tiles2 > 0;  // (a centroid always comes with its radius)
+  // (a centroid always comes with its radius, and k_sys_radius_low waits before it reads anything)
+  const bool overlap = pdl || n.tiles2 > 0;
   if (n.cluster > 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n.cluster * kSysClusterSize);
