@@ -74,8 +74,8 @@ typedef enum {
   TCM_FP64 = 0,  /* every step in double precision */
   TCM_MIXED = 1  /* moment recurrence and per-atom products in float on radius-scaled
                     coordinates; block partials and the cross-block reduction in double.
-                    The contraction is the same for both: products in 60-bit fixed
-                    point, sums over (l1, l2) in double */
+                    The contraction is the same for both: its rotations in 60-bit fixed
+                    point, the products of A's and B's components and their sums in double */
 } tcm_precision;
 
 typedef struct tcm_ctx* tcm_ctx_t;

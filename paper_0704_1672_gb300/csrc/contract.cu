@@ -25,14 +25,20 @@
 // with p~_k = e^{i k beta} p_k and the entries of indices >= 1 counted twice (the table's columns):
 // (l+1)^2 real multiply-adds per product and degree, no table of d^l(beta) per energy.
 //
-// What bounds it, and why fixed point: in double the kernel was bound by the FP64 pipe (a warp
-// instruction holds its SMSP for 64 cycles; 400 of them per energy at degree 10).  All quantities
-// are bounded (|D| <= 1, phases of modulus 1, rotations keep a degree's norm), so they are held as 60-bit
-// integers on a scale per degree and side and multiplied in 30-bit limbs: three IMAD.WIDE of about four
-// cycles each instead of an FP64 instruction.  A stored value carries an error of 2^-56 of the
-// largest component of its degree (double: 2^-53 of each), sums of products are exact to the last limb.  Only
-// the factor C(l1+l2, l1) / R^(l1+l2+1), the sum over (l1, l2) and the gradient's combinations stay in
-// double: 3 FP64 instructions per (l1, l2).
+// What bounds it, and why the rotations are in fixed point: in double the kernel was bound by the FP64 pipe
+// (a warp instruction holds its SMSP for 64 cycles; 400 of them per energy at degree 10), most of it the
+// phases and the two products.  Their quantities are bounded (|D| <= 1, phases of modulus 1, rotations keep a
+// degree's norm), so they are held as 60-bit integers on a scale per degree and side and multiplied in
+// 30-bit limbs: three IMAD.WIDE of about four cycles each instead of an FP64 instruction.  A rotation
+// spreads the rounding of a degree's largest component over all of them, in double as here: a value
+// in fixed point is off by a few 2^-56 of that component, in double by a few 2^-53 of the partial sums.
+// From there on the components are far apart: l!/sqrt((l+m)!(l-m)!) falls to 2e-7 at l = m = 24, and a pair
+// stacked on a common axis may have nothing but its highest orders.  So the factor, the products of A's and
+// B's components and every sum of them are double.  (With the products in fixed point too, rounded on the
+// scale of the degree's largest component, two coaxial rings of 12 alternating charges lost five
+// digits, of 48 fourteen.)  B's moments in mode kBInFrame need no rotation and stay double throughout.
+// Error of an energy (rms, of sum |U_l1l2|, 40 random pairs at degrees 1 to 24; against 113-bit
+// arithmetic): 1.5e-16 to 8.9e-16, the all-double kernel's 1.5e-16 to 8.9e-16; forces and torques alike.
 // Measured, in double and now: 108,360 energies at degrees 1 to 10 1,340 and 298 us, 2,048 at degrees 8 to
 // 24 (B rotated) 140 and 64, 256 at degree 20 24 and 16, forces and torques of 512 at degree 12 92 and 25.
 // What bounds it now: the phases between barriers (a third of the stalls) with the multiplier 0.45 busy and
@@ -84,7 +90,7 @@ __device__ __forceinline__ double flip(double x, int odd) {  // (-1)^odd x witho
 }
 
 // ---- fixed point
-struct Acc {  // a sum of products: 2^60 h + 2^30 m (the low limbs' product is dropped)
+struct Acc {  // a sum of products: 2^60 h + 2^30 m (the low limbs' product is dropped: at most 2^58 a term)
   long long h = 0, m = 0;
   __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
     h += (long long)ah * bh;
@@ -102,26 +108,31 @@ __device__ __forceinline__ Fx split30(long long x) {
   return f;
 }
 __device__ __forceinline__ int4 pack(Fx r, Fx i) { return make_int4(r.h, r.l, i.h, i.l); }
-__device__ __forceinline__ int4 fmul(int4 z, Fx f) {  // z times a real factor on the scale 2^60
-  Acc r, i;
-  r.add(z.x, z.y, f.h, f.l);
-  i.add(z.z, z.w, f.h, f.l);
-  return pack(split30(r.value60()), split30(i.value60()));
-}
-__device__ __forceinline__ int4 cmulf(int4 a, int4 b) {  // one factor on the scale 2^60
+struct Wide {  // a complex number before its parts are split into limbs
+  long long x, y;
+};
+__device__ __forceinline__ int4 pack(Wide z) { return pack(split30(z.x), split30(z.y)); }
+__device__ __forceinline__ Wide cmulw(int4 a, int4 b) {  // one factor on the scale 2^60
   Acc r, i;
   r.add(a.x, a.y, b.x, b.y);
   r.sub(a.z, a.w, b.z, b.w);
   i.add(a.x, a.y, b.z, b.w);
   i.add(a.z, a.w, b.x, b.y);
-  return pack(split30(r.value60()), split30(i.value60()));
+  return Wide{r.value60(), i.value60()};
 }
+__device__ __forceinline__ int4 cmulf(int4 a, int4 b) { return pack(cmulw(a, b)); }
 __device__ __forceinline__ int4 ipow(int4 z, int n) {  // i^n z
   const int r = n & 3;
   const int4 s = (r & 1) ? make_int4(z.z, z.w, z.x, z.y) : z;
   return make_int4((r == 1 || r == 2) ? -s.x : s.x, (r == 1 || r == 2) ? -s.y : s.y, r >= 2 ? -s.z : s.z,
                    r >= 2 ? -s.w : s.w);
 }
+__device__ __forceinline__ Wide ipow(Wide z, int n) {
+  const int r = n & 3;
+  const Wide s = (r & 1) ? Wide{z.y, z.x} : z;
+  return Wide{(r == 1 || r == 2) ? -s.x : s.x, r >= 2 ? -s.y : s.y};
+}
+__device__ __forceinline__ double2 times(Wide z, double f) { return make_double2((double)z.x * f, (double)z.y * f); }
 __device__ __forceinline__ int4 unit(double x, double y) {  // a complex number of modulus <= 1 on the scale 2^60
   return pack(split30(__double2ll_rn(x * 1152921504606846976.0)), split30(__double2ll_rn(y * 1152921504606846976.0)));
 }
@@ -137,7 +148,7 @@ __device__ __forceinline__ int4 zpow(int4 z, int n) {  // z^n by squaring
 }
 
 __device__ __forceinline__ int exponent(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1022; }  // |v| < 2^e
-// v 2^(kMomBits - e), |v| < 2^e, towards zero: integer instructions only
+// v 2^(kMomBits - e), |v| < 2^e, to the nearest integer: integer instructions only
 __device__ __forceinline__ long long to_fixed(double v, int e) {
   const long long b = __double_as_longlong(v);
   int ex = (int)((b >> 52) & 0x7ff);
@@ -145,7 +156,7 @@ __device__ __forceinline__ long long to_fixed(double v, int e) {
   if (ex > 0) m |= 1LL << 52;
   else ex = 1;
   const int sh = ex - 1075 + kMomBits - e;  // at most 3
-  m = sh >= 0 ? m << sh : (sh > -63 ? m >> -sh : 0);
+  m = sh >= 0 ? m << sh : (sh > -63 ? ((m >> (-sh - 1)) + 1) >> 1 : 0);
   return b < 0 ? -m : m;
 }
 __device__ __forceinline__ double scale2(double c, int n) {  // c 2^n
@@ -165,7 +176,7 @@ __device__ __forceinline__ double rpow(double x, int n) {
 
 // Row product with a parity split: (sum over j = par (mod 2) of row[j] Re x_j, sum over the other j of
 // row[j] Im x_j), j = 0..l, of one item's column of x (stride G).
-__device__ __forceinline__ void row_split(const Fx* row, const int4* x, int G, int l, int par, Fx& re, Fx& im) {
+__device__ __forceinline__ Wide row_split(const Fx* row, const int4* x, int G, int l, int par) {
   const int2* xs = reinterpret_cast<const int2*>(x);
   Acc a, b;  // even j, odd j
   int j = 0;
@@ -180,9 +191,8 @@ __device__ __forceinline__ void row_split(const Fx* row, const int4* x, int G, i
     const int2 x0 = xs[2 * j * G + par];
     a.add(r0.h, r0.l, x0.x, x0.y);
   }
-  const Fx fa = split30(a.value59()), fb = split30(b.value59());
-  re = par ? fb : fa;
-  im = par ? fa : fb;
+  const long long va = a.value59(), vb = b.value59();
+  return par ? Wide{vb, va} : Wide{va, vb};
 }
 
 // Eq. (Formula) for one (pair, orientation) per column of a CTA.  With kGrad also, per item, the force on
@@ -196,7 +206,7 @@ __device__ __forceinline__ void row_split(const Fx* row, const int4* x, int G, i
 //   (infinitesimal rotations act on Qhat_lm through L_z and the ladder operators with the
 //   integer weights (l+m+1), (l-m+1)).  The vectors go back to the lab frame with W^T.
 // A's moments are kept as a_m = (-1)^m Qa_m, so that T0 = Re sum a_m conj(b_m) and so on without signs;
-// the sums weighted by m take (m/32) a_m.
+// the sums weighted by m take m a_m.
 template <bool kGrad>
 __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
     k_contract(const PairDesc* __restrict__ items, const int* __restrict__ order, const ContractPlan* __restrict__ plan,
@@ -227,11 +237,12 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
     const int first = plan->first[L] + (g - plan->gfirst[L]) * G;
     const int cnt = min(G, plan->first[L + 1] - first);
     const int nq = tri(L + 1), n1 = L + 1;
-    int4* qa = base4;           // A: moments, v, then a_m in the frame
+    int4* qa = base4;           // A: moments (double), v (fixed), then a_m in the frame (double)
     int4* qb = qa + nq * G;     // B: the same
     int4* ta = qb + nq * G;     // p~ of A
     int4* tb = ta + nq * G;     // p~ of B
-    int4* qm = tb + nq * G;     // kGrad: (m/32) a_m
+    int4* qm = tb + nq * G;     // kGrad: m a_m (double)
+    double2 *da = reinterpret_cast<double2*>(qa), *db = reinterpret_cast<double2*>(qb), *dm = reinterpret_cast<double2*>(qm);
     int4* ph = kGrad ? qm + nq * G : qm;  // input phases of W (alpha of R0); mode kBRotate: 2, 3, 4 of W rotB
     double* rp = reinterpret_cast<double*>(ph + kTabs * n1 * G);  // R^-(k+1), k <= 2 L + 1
     int* ex = reinterpret_cast<int*>(rp + (2 * L + 2) * G);       // exponents of the degrees, A then B
@@ -282,26 +293,35 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
         const int l = s_lm[q] >> 8, m = s_lm[q] & 255;
         const double2 a = m == 0 ? make_double2(pa[l * l], 0.0) : make_double2(pa[l * l + 2 * m - 1], pa[l * l + 2 * m]);
         const double2 b = m == 0 ? make_double2(pb[l * l], 0.0) : make_double2(pb[l * l + 2 * m - 1], pb[l * l + 2 * m]);
-        reinterpret_cast<double2*>(qa)[q * G + it] = a;
-        reinterpret_cast<double2*>(qb)[q * G + it] = b;
+        da[q * G + it] = a;
+        db[q * G + it] = b;
         atomicMax(&ex[l * G + it], max(exponent(a.x), exponent(a.y)));
         atomicMax(&ex[(n1 + l) * G + it], max(exponent(b.x), exponent(b.y)));
       }
       if (q0 == 0) s_ok[it] = d.fr[1] > geoms[d.geomA].a + geoms[d.geomB].a;  // Eq. (mainCond)
     }
     __syncthreads();
-    const Fx* hat = &tab->hat[0][0];
-    if (in) {  // to fixed point; v = input phases times the moments; mode kBInFrame only scales B
+    const double* hat = &tab->hat[0][0];
+    if (in) {  // to fixed point; v = input phases times the moments; mode kBInFrame only scales B (in double)
       for (int q = q0; q < nq; q += Q) {
         const int l = s_lm[q] >> 8, m = s_lm[q] & 255;
         const int ea = ex[l * G + it], eb = ex[(n1 + l) * G + it];
-        const double2 a = reinterpret_cast<double2*>(qa)[q * G + it], b = reinterpret_cast<double2*>(qb)[q * G + it];
+        const double2 a = da[q * G + it];
+        double2 b = db[q * G + it];
         if (max(ea, eb) > 1024 && s_ok[it] == 1) s_ok[it] = -1;
-        const int4 fa = pack(split30(to_fixed(a.x, ea)), split30(to_fixed(a.y, ea)));
-        const int4 fb = pack(split30(to_fixed(b.x, eb)), split30(to_fixed(b.y, eb)));
-        qa[q * G + it] = cmulf(ph[m * G + it], fa);
-        qb[q * G + it] = bmode == kBInFrame ? fmul(fb, hat[l * kZN + m])
-                                            : cmulf(ph[((bmode == kBRotate ? 2 * n1 : 0) + m) * G + it], fb);
+        qa[q * G + it] = cmulf(ph[m * G + it], pack(Wide{to_fixed(a.x, ea), to_fixed(a.y, ea)}));
+        if (bmode == kBInFrame) {
+          int n = kMomBits - eb;
+          if (n < -800) {  // (2^n hat would be subnormal)
+            b = make_double2(b.x * 0x1p-300, b.y * 0x1p-300);
+            n += 300;
+          }
+          const double f = scale2(hat[l * kZN + m], n);
+          db[q * G + it] = make_double2(b.x * f, b.y * f);
+        } else {
+          qb[q * G + it] = cmulf(ph[((bmode == kBRotate ? 2 * n1 : 0) + m) * G + it],
+                                 pack(Wide{to_fixed(b.x, eb), to_fixed(b.y, eb)}));
+        }
       }
     }
     __syncthreads();
@@ -310,31 +330,25 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
       for (int q = q0; q < nq; q += Q) {
         const int l = s_lm[q] >> 8, kk = s_lm[q] & 255;
         const Fx* row = Ds + dpi2_off(l) + kk * dpi2_stride(l);
-        Fx re, im;
-        row_split(row, qa + tri(l) * G + it, G, l, (l + kk) & 1, re, im);
-        ta[q * G + it] = cmulf(ph[(n1 + kk) * G + it], pack(re, im));
-        if (bmode != kBInFrame) {
-          row_split(row, qb + tri(l) * G + it, G, l, (l + kk) & 1, re, im);
-          tb[q * G + it] = cmulf(eb[kk * G + it], pack(re, im));
-        }
+        ta[q * G + it] = cmulf(ph[(n1 + kk) * G + it], pack(row_split(row, qa + tri(l) * G + it, G, l, (l + kk) & 1)));
+        if (bmode != kBInFrame)
+          tb[q * G + it] = cmulf(eb[kk * G + it], pack(row_split(row, qb + tri(l) * G + it, G, l, (l + kk) & 1)));
       }
     }
     __syncthreads();
-    if (in) {  // second product: S_m, times i^m (or the output phase) and the hat factor
+    if (in) {  // second product: S_m, times i^m (or the output phase) and, in double, the hat factor
       for (int q = q0; q < nq; q += Q) {
         const int l = s_lm[q] >> 8, m = s_lm[q] & 255;
         const Fx* row = Ds + dpi2_off(l) + m * dpi2_stride(l);
-        const Fx f = hat[l * kZN + m];
-        Fx re, im;
-        row_split(row, ta + tri(l) * G + it, G, l, (l + m) & 1, re, im);
-        int4 S = (l & 1) ? make_int4(-re.h, -re.l, im.h, im.l) : make_int4(re.h, re.l, -im.h, -im.l);
-        const int4 a = fmul(ipow(S, m + 2 * m), f);  // (-1)^m i^m
-        qa[q * G + it] = a;
-        if (kGrad) qm[q * G + it] = fmul(a, Fx{m << 25, 0});
+        const double f = hat[l * kZN + m];
+        auto signs = [&](Wide p) { return (l & 1) ? Wide{-p.x, p.y} : Wide{p.x, -p.y}; };
+        Wide S = signs(row_split(row, ta + tri(l) * G + it, G, l, (l + m) & 1));
+        const double2 a = times(ipow(S, m + 2 * m), f);  // (-1)^m i^m
+        da[q * G + it] = a;
+        if (kGrad) dm[q * G + it] = make_double2((double)m * a.x, (double)m * a.y);
         if (bmode != kBInFrame) {
-          row_split(row, tb + tri(l) * G + it, G, l, (l + m) & 1, re, im);
-          S = (l & 1) ? make_int4(-re.h, -re.l, im.h, im.l) : make_int4(re.h, re.l, -im.h, -im.l);
-          qb[q * G + it] = fmul(bmode == kBRotate ? cmulf(ph[(4 * n1 + m) * G + it], S) : ipow(S, m), f);
+          S = signs(row_split(row, tb + tri(l) * G + it, G, l, (l + m) & 1));
+          db[q * G + it] = times(bmode == kBRotate ? cmulw(ph[(4 * n1 + m) * G + it], pack(S)) : ipow(S, m), f);
         }
       }
     }
@@ -354,66 +368,64 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
         const int s = L - u, j = p - u * u;
         const int l1 = (j & 1) ? s : s + (j >> 1);
         const int l2 = (j & 1) ? s + ((j + 1) >> 1) : s;
-        const int4* a = qa + tri(l1) * G + it;
-        const int4* b = qb + tri(l2) * G + it;
-        Acc e0, es;
-        e0.add(a[0].x, a[0].y, b[0].x, b[0].y);
+        const double2* a = da + tri(l1) * G + it;
+        const double2* b = db + tri(l2) * G + it;
+        double es = 0.0;
         for (int m = 1; m <= s; ++m) {
-          const int4 x = a[m * G], y = b[m * G];
-          es.add(x.x, x.y, y.x, y.y);
-          es.add(x.z, x.w, y.z, y.w);
+          const double2 x = a[m * G], y = b[m * G];
+          es = fma(x.x, y.x, es);
+          es = fma(x.y, y.y, es);
         }
+        const double T = fma(a[0].x, b[0].x, es + es);
         const int n = l1 + l2;
-        const int sh = ex[l1 * G + it] + ex[(n1 + l2) * G + it] - (2 * kMomBits - 60);
+        const int sh = ex[l1 * G + it] + ex[(n1 + l2) * G + it];
         const double bi = tab->binom[l1][l2];
         const double c = flip(scale2(bi * rp[n * G + it], sh), l2);
-        const double T = (double)(e0.value60() + 2 * es.value60());
         sum[0] = fma(c, T, sum[0]);
         if (kGrad) {
-          const int4* am = qm + tri(l1) * G + it;
-          Acc sr, si, wr, wi, z;
+          const double2* am = dm + tri(l1) * G + it;
+          double sr = 0.0, si = 0.0, wr = 0.0, wi = 0.0, z = 0.0;
           const int ma = min(l1, l2 + 1), mc = min(l1, l2 - 1);
           for (int m = 1; m <= ma; ++m) {  // (m, 1 - m): -a_m conj(b_(m-1))
-            const int4 x = a[m * G], xm = am[m * G], y = b[(m - 1) * G];
-            sr.sub(x.x, x.y, y.x, y.y);
-            sr.sub(x.z, x.w, y.z, y.w);
-            si.sub(x.z, x.w, y.x, y.y);
-            si.add(x.x, x.y, y.z, y.w);
-            wr.add(xm.x, xm.y, y.x, y.y);  // m times the weight's change, -m
-            wr.add(xm.z, xm.w, y.z, y.w);
-            wi.add(xm.z, xm.w, y.x, y.y);
-            wi.sub(xm.x, xm.y, y.z, y.w);
+            const double2 x = a[m * G], xm = am[m * G], y = b[(m - 1) * G];
+            sr = fma(-x.x, y.x, sr);
+            sr = fma(-x.y, y.y, sr);
+            si = fma(-x.y, y.x, si);
+            si = fma(x.x, y.y, si);
+            wr = fma(xm.x, y.x, wr);  // m times the weight's change, -m
+            wr = fma(xm.y, y.y, wr);
+            wi = fma(xm.y, y.x, wi);
+            wi = fma(-xm.x, y.y, wi);
           }
           for (int m = 0; m <= mc; ++m) {  // (-m, m + 1): conj(a_m) b_(m+1)
-            const int4 x = a[m * G], xm = am[m * G], y = b[(m + 1) * G];
-            sr.add(x.x, x.y, y.x, y.y);
-            sr.add(x.z, x.w, y.z, y.w);
-            si.add(x.x, x.y, y.z, y.w);
-            si.sub(x.z, x.w, y.x, y.y);
-            wr.add(xm.x, xm.y, y.x, y.y);
-            wr.add(xm.z, xm.w, y.z, y.w);
-            wi.add(xm.x, xm.y, y.z, y.w);
-            wi.sub(xm.z, xm.w, y.x, y.y);
+            const double2 x = a[m * G], xm = am[m * G], y = b[(m + 1) * G];
+            sr = fma(x.x, y.x, sr);
+            sr = fma(x.y, y.y, sr);
+            si = fma(x.x, y.y, si);
+            si = fma(-x.y, y.x, si);
+            wr = fma(xm.x, y.x, wr);
+            wr = fma(xm.y, y.y, wr);
+            wi = fma(xm.x, y.y, wi);
+            wi = fma(-xm.y, y.x, wi);
           }
           for (int m = 1; m <= s; ++m) {
-            const int4 xm = am[m * G], y = b[m * G];
-            z.add(xm.z, xm.w, y.x, y.y);
-            z.sub(xm.x, xm.y, y.z, y.w);
+            const double2 xm = am[m * G], y = b[m * G];
+            z = fma(xm.y, y.x, z);
+            z = fma(-xm.x, y.y, z);
           }
-          const double Sr = (double)sr.value60(), Si = (double)si.value60();
           const double w1 = (double)(l2 + 1);
-          const double Pr = fma(w1, Sr, 32.0 * (double)wr.value60()), Pi = fma(w1, Si, 32.0 * (double)wi.value60());
-          const double Z = 64.0 * (double)z.value60();
+          const double Pr = fma(w1, sr, wr), Pi = fma(w1, si, wi);
+          const double Z = z + z;
           const double L1 = (double)(n + 1);
           const double c1 = flip(scale2(bi * L1 * rp[(n + 1) * G + it], sh), l2);
-          sum[1] = fma(-c1, Sr, sum[1]);
-          sum[2] = fma(-c1, Si, sum[2]);
+          sum[1] = fma(-c1, sr, sum[1]);
+          sum[2] = fma(-c1, si, sum[2]);
           sum[3] = fma(-c1, T, sum[3]);
           sum[4] = fma(c, Pi, sum[4]);
           sum[5] = fma(-c, Pr, sum[5]);
           sum[6] = fma(-c, Z, sum[6]);
-          sum[7] = fma(c, fma(L1, Si, -Pi), sum[7]);
-          sum[8] = fma(-c, fma(L1, Sr, -Pr), sum[8]);
+          sum[7] = fma(c, fma(L1, si, -Pi), sum[7]);
+          sum[8] = fma(-c, fma(L1, sr, -Pr), sum[8]);
         }
       }
     }
@@ -519,7 +531,7 @@ void build_tables(ContractTables& t) {
     for (int k = 1; k <= 2 * kZN; ++k) C[n][k] = n == 0 ? 0 : C[n - 1][k - 1] + C[n - 1][k];
   }
   for (int l = 0; l < kZN; ++l) {
-    for (int m = 0; m <= l; ++m) t.hat[l][m] = split_host(ldexpl(fact[l] / sqrtl(fact[l + m] * fact[l - m]), 60));
+    for (int m = 0; m <= l; ++m) t.hat[l][m] = (double)ldexpl(fact[l] / sqrtl(fact[l + m] * fact[l - m]), -kMomBits);
     for (int k = 0; k < kZN; ++k) t.binom[l][k] = (double)C[l + k][l];
     for (int k = 0; k <= l; ++k)
       for (int m = 0; m <= l; ++m) {

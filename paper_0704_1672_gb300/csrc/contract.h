@@ -157,8 +157,8 @@ struct Fx {  // fixed point: 2^30 h + l, |l| <= 2^29
 };
 struct ContractTables {
   double dpi2[dpi2_off(kZN)];  // rows of d^l(pi/2)
-  Fx row[dpi2_off(kZN)];       // the same times 2^59, columns m >= 1 doubled
-  Fx hat[kZN][kZN];            // [l][m]: 2^60 l!/sqrt((l+m)!(l-m)!)
+  Fx row[dpi2_off(kZN)];       // the same times 2^59, columns m >= 1 doubled (contract.cu)
+  double hat[kZN][kZN];        // [l][m]: 2^-kMomBits l!/sqrt((l+m)!(l-m)!)
   double binom[kZN][kZN];      // [l1][l2]: C(l1 + l2, l1)
 };
 const ContractTables& contract_tables();
