@@ -31,7 +31,7 @@
 // degree's norm), so they are held as 60-bit integers on a scale per degree and side and multiplied in
 // 30-bit limbs: three IMAD.WIDE of about four cycles each instead of an FP64 instruction.  A rotation
 // spreads the rounding of a degree's largest component over all of them, in double as here: a value
-// in fixed point is off by a few 2^-56 of that component, in double by a few 2^-53 of the partial sums.
+// in fixed point is off by a few 2^-57 of that component, in double by a few 2^-53 of the partial sums.
 // From there on the components are far apart: l!/sqrt((l+m)!(l-m)!) falls to 2e-7 at l = m = 24, and a pair
 // stacked on a common axis may have nothing but its highest orders.  So the factor, the products of A's and
 // B's components and every sum of them are double.  (With the products in fixed point too, rounded on the
@@ -59,9 +59,10 @@ namespace {
 
 constexpr int kCT = 256;  // threads of a contraction CTA
 constexpr int kMaxGroup = 16;
-// X = Q 2^(kMomBits - e), |Q_lm| < 2^e: the norm of a degree, below 2^(e + 3.3), stays below 2^58.3, so
-// that the high-limb sums of up to 25 products stay below 2^60 and the cross sums below 2^62.
-constexpr int kMomBits = 55;
+// X = Q 2^(kMomBits - e), parts of Q_lm below 2^e: the norm of a degree, at most sqrt(97) 2^e, and with it
+// every value on the way is below 2^60.3, so that a high limb stays below 2^30.3, the high-limb sums (a table
+// row has norm 1, the orders m and -m share it) below 2^61.3 and the cross sums of 13 products below 2^61.5.
+constexpr int kMomBits = 57;
 
 __host__ __device__ constexpr int group_of(int L) {
   const int g = 512 / ((L + 1) * (L + 2));
@@ -90,7 +91,7 @@ __device__ __forceinline__ double flip(double x, int odd) {  // (-1)^odd x witho
 }
 
 // ---- fixed point
-struct Acc {  // a sum of products: 2^60 h + 2^30 m (the low limbs' product is dropped: at most 2^58 a term)
+struct Acc {  // a sum of products: 2^60 h + 2^30 m (the low limbs' product, at most 2^58, is dropped)
   long long h = 0, m = 0;
   __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
     h += (long long)ah * bh;
@@ -155,7 +156,7 @@ __device__ __forceinline__ long long to_fixed(double v, int e) {
   long long m = b & 0xfffffffffffffLL;
   if (ex > 0) m |= 1LL << 52;
   else ex = 1;
-  const int sh = ex - 1075 + kMomBits - e;  // at most 3
+  const int sh = ex - 1075 + kMomBits - e;  // at most 4
   m = sh >= 0 ? m << sh : (sh > -63 ? ((m >> (-sh - 1)) + 1) >> 1 : 0);
   return b < 0 ? -m : m;
 }
