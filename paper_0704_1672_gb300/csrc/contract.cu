@@ -148,6 +148,7 @@ __device__ __forceinline__ int4 zpow(int4 z, int n) {  // z^n by squaring
   return r;
 }
 
+__device__ __forceinline__ bool finite(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) != 0x7ff; }
 __device__ __forceinline__ int exponent(double v) { return ((__double2hiint(v) >> 20) & 0x7ff) - 1022; }  // |v| < 2^e
 // v 2^(kMomBits - e), |v| < 2^e, to the nearest integer: integer instructions only
 __device__ __forceinline__ long long to_fixed(double v, int e) {
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
                const PairOut* __restrict__ out) {
   extern __shared__ __align__(16) int4 sm4[];
   __shared__ PairDesc s_d[kMaxGroup];
-  __shared__ int s_item[kMaxGroup], s_ok[kMaxGroup];  // s_ok: 1 converges, 0 not, -1 moments that are not finite
+  __shared__ int s_item[kMaxGroup], s_ok[kMaxGroup];  // s_ok: 1 converges, 0 not, -1 moments or phases that are not finite
   __shared__ unsigned short s_lm[(kLmaxMax + 1) * (kLmaxMax + 2) / 2];
   __shared__ double s_sum[kGrad ? 9 : 1][kCT];
   constexpr int kTabs = 5;
@@ -299,7 +300,17 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
         atomicMax(&ex[l * G + it], max(exponent(a.x), exponent(a.y)));
         atomicMax(&ex[(n1 + l) * G + it], max(exponent(b.x), exponent(b.y)));
       }
-      if (q0 == 0) s_ok[it] = d.fr[1] > geoms[d.geomA].a + geoms[d.geomB].a;  // Eq. (mainCond)
+      if (q0 == 0) {
+        s_ok[it] = d.fr[1] > geoms[d.geomA].a + geoms[d.geomB].a;  // Eq. (mainCond)
+        // phases that are not finite have no fixed-point form (degree 0 has no phase)
+        bool ok = L == 0 || (finite(d.fr[2]) && finite(d.fr[3]) && finite(d.fr[4]) && finite(d.fr[5]));
+        if (L > 0 && bmode == kBRotate) {
+          const EulerZYZ* e = rots + d.rot;
+          ok = ok && finite(e->cb) && finite(e->sb) && finite(e->ea[0]) && finite(e->ea[1]) && finite(e->eg[0]) &&
+               finite(e->eg[1]);
+        }
+        if (s_ok[it] && !ok) s_ok[it] = -1;
+      }
     }
     __syncthreads();
     const double* hat = &tab->hat[0][0];
@@ -450,7 +461,7 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
         o.E[item] = v[0];
       } else if (s_ok[i] == 0) {  // the expansion does not converge
         o.E[item] = nan;
-      } else {  // moments that are not finite: only Lmax = 0 has a product of its own
+      } else {  // moments or phases that are not finite: only Lmax = 0 has a product of its own
         const PairDesc& e = s_d[i];
         o.E[item] = L == 0 ? jobs[e.jobA].out[0] * jobs[e.jobB].out[0] * e.fr[0] : nan;
       }
