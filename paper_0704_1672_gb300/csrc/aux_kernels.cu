@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const MomJob* __r
   const MomJob& job = jobs[blockIdx.x];
   const int L = job.L;
   const int tpc = job.tiles_per_chunk;
-  const int kmax = plan_slots(job.plan, L), row = plan_row(job.plan);
+  const int kmax = plan_slots(job.plan, L), row = plan_row(job.plan, L);
   const int* off = imap_off + job.plan * (kLmaxMax + 2);
   const int o = off[L];
   const int nq = off[L + 1] - o;  // nch x kmax
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const MomJob* __r
     const int p = in ? imap[o + q] : -1;
     const double f = in ? fmap[o + q] : 0.0;
     const int ch = q / kmax, slot = q - ch * kmax;
-    const double* base = partials + (long long)(job.tile_base + ch * tpc) * row + slot;
+    const double* base = partials + job.part + (long long)ch * tpc * row + slot;
     double s = 0.0;
     if (!split) {
       if (in)

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(512, 2)
       }
     }
     __syncthreads();
-    double* row = partials + (long long)tile.id * kRowF64;
+    double* row = partials + job.part + (long long)tile.t * ncomp;
     for (int k = threadIdx.x; k < ncomp; k += blockDim.x) {
       double v = 0.0;
       for (int gr = 0; gr < ng; ++gr) {

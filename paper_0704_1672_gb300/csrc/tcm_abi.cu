@@ -260,14 +260,25 @@ bool geom_known(const tcm_system& s) { return s.has_center && s.radius >= 0.0; }
 // Moment-job planning -------------------------------------------------------------
 
 
+// Doubles of partial rows a pass of the double path may take (1 GiB).  Its tiles are small, so that one
+// small system fills the GPU (2,000 atoms: 63 tiles; 315 KB of rows at degree 24), and a batch of 100,000
+// would ask for 31 GB of rows at once; in passes of moments and finalisation, one behind the other, they
+// reuse the same rows.  The float path's tiles are larger, its rows fewer: always one pass.
+constexpr size_t kPassDoubles = size_t(1) << 27;
+
 struct Plan {
   std::vector<MomJob> jobs;
   std::vector<MomGroup> groups;    // (job, chunk) groups, largest tiles first; expanded on the device
   int n_tiles = 0;
-  // FP64 (one launch per degree): the tiles of L are [tile_begin[L], tile_begin[L+1]); mixed
-  // (one launch per chunk plan over all degrees): the tiles of plan p are
-  // [tile_begin[p - 1], tile_begin[p])
-  int tile_begin[kLmaxMax + 2] = {};
+  // A pass: jobs [job0, job0 + n_jobs), moment launches and a finalisation.  FP64 (one launch per degree):
+  // the tiles of L are [tile_begin[L], tile_begin[L+1]); mixed (one launch per chunk plan over all
+  // degrees): the tiles of plan p are [tile_begin[p - 1], tile_begin[p])
+  struct Pass {
+    int job0, n_jobs;
+    int tile_begin[kLmaxMax + 2];
+  };
+  std::vector<Pass> passes;
+  size_t part_doubles = 0;  // partial rows, of the pass that has most
   int n_tile_ids = 0;
   struct Group {
     int job, chunk;
@@ -291,7 +302,26 @@ void plan_job(tcm_ctx* c, int precision, MomJob& j, int& next_id) {
 }
 
 
-// The (job, chunk) groups in decreasing order of their tiles' cost (largest first, so the
+// Cuts the jobs into passes and places their partial rows.
+void plan_passes(int precision, Plan& P) {
+  P.passes.clear();
+  P.part_doubles = 0;
+  size_t at = 0;
+  for (int ji = 0; ji < (int)P.jobs.size(); ++ji) {
+    MomJob& j = P.jobs[ji];
+    const size_t need = (size_t)moments_nchunks(j.plan, j.L) * j.tiles_per_chunk * plan_row(j.plan, j.L);
+    if (ji == 0 || (precision == TCM_FP64 && at + need > kPassDoubles)) {
+      P.passes.push_back(Plan::Pass{ji, 0, {}});
+      at = 0;
+    }
+    ++P.passes.back().n_jobs;
+    j.part = (long long)at;
+    at += need;
+    P.part_doubles = std::max(P.part_doubles, at);
+  }
+}
+
+// The (job, chunk) groups of each pass in decreasing order of their tiles' cost (largest first, so the
 // persistent warps finish together).  FP64: grouped by degree (one launch per degree); mixed:
 // grouped by chunk plan (one launch per plan present, usually one), one order over all degrees.  The tiles themselves are written on the device
 // (k_expand_tiles), so the host work is O(groups log groups).
@@ -303,60 +333,63 @@ void build_tiles(int precision, Plan& P) {
   using Group = Plan::Group;
   std::vector<Group>& g = P.sort_groups;
   std::vector<uint32_t>& key = P.sort_key;
-  g.clear();
-  key.clear();
   const bool by_degree = precision == TCM_FP64;
-  for (int ji = 0; ji < (int)P.jobs.size(); ++ji) {
-    const MomJob& j = P.jobs[ji];
-    const int nch = moments_nchunks(j.plan, j.L);
-    const double* cc = moments_chunk_costs(j.plan, j.L);
-    for (int ch = 0; ch < nch; ++ch) {
-      const double cost = cc[ch] * (double)j.atoms_per_tile;
-      const uint32_t cq = (uint32_t)std::min(cost, 134217727.0);  // 27 bits
-      key.push_back(((uint32_t)(by_degree ? j.L : j.plan - 1) << 27) | (134217727u - cq));
-      g.push_back(Group{ji, ch});
-    }
-  }
-  const size_t n = key.size();
-  const bool few = n <= 64;  // an insertion sort beats the radix sort's histograms
-  std::vector<uint32_t>&order = P.sort_order, &k2 = P.sort_key2, &o2 = P.sort_order2;
-  order.resize(n);
-  k2.resize(n);
-  o2.resize(n);
-  for (size_t i = 0; i < n; ++i) order[i] = (uint32_t)i;
-  for (size_t i = 1; few && i < n; ++i) {
-    const uint32_t o = order[i];
-    size_t j = i;
-    for (; j > 0 && key[order[j - 1]] > key[o]; --j) order[j] = order[j - 1];
-    order[j] = o;
-  }
-  for (int shift = 0; !few && shift < 32; shift += 11) {
-    uint32_t count[2049] = {};
-    for (size_t i = 0; i < n; ++i) ++count[((key[i] >> shift) & 2047u) + 1];
-    for (int b = 0; b < 2048; ++b) count[b + 1] += count[b];
-    for (size_t i = 0; i < n; ++i) {
-      const uint32_t d = (key[i] >> shift) & 2047u;
-      k2[count[d]] = key[i];
-      o2[count[d]++] = order[i];
-    }
-    key.swap(k2);
-    order.swap(o2);
-  }
+  plan_passes(precision, P);
   P.groups.clear();
-  P.groups.reserve(n);
   int first = 0;
-  size_t gi = 0;
-  for (int L = 0; L <= kLmaxMax; ++L) {
-    P.tile_begin[L] = first;
-    for (; gi < n; ++gi) {
-      const Group& gr = g[order[gi]];
-      if ((by_degree ? P.jobs[gr.job].L : P.jobs[gr.job].plan - 1) != L) break;
-      const int nt = P.jobs[gr.job].tiles_per_chunk;
-      P.groups.push_back(MomGroup{gr.job, gr.chunk, nt, first});
-      first += nt;
+  for (Plan::Pass& pass : P.passes) {
+    g.clear();
+    key.clear();
+    for (int ji = pass.job0; ji < pass.job0 + pass.n_jobs; ++ji) {
+      const MomJob& j = P.jobs[ji];
+      const int nch = moments_nchunks(j.plan, j.L);
+      const double* cc = moments_chunk_costs(j.plan, j.L);
+      for (int ch = 0; ch < nch; ++ch) {
+        const double cost = cc[ch] * (double)j.atoms_per_tile;
+        const uint32_t cq = (uint32_t)std::min(cost, 134217727.0);  // 27 bits
+        key.push_back(((uint32_t)(by_degree ? j.L : j.plan - 1) << 27) | (134217727u - cq));
+        g.push_back(Group{ji, ch});
+      }
     }
+    const size_t n = key.size();
+    const bool few = n <= 64;  // an insertion sort beats the radix sort's histograms
+    std::vector<uint32_t>&order = P.sort_order, &k2 = P.sort_key2, &o2 = P.sort_order2;
+    order.resize(n);
+    k2.resize(n);
+    o2.resize(n);
+    for (size_t i = 0; i < n; ++i) order[i] = (uint32_t)i;
+    for (size_t i = 1; few && i < n; ++i) {
+      const uint32_t o = order[i];
+      size_t j = i;
+      for (; j > 0 && key[order[j - 1]] > key[o]; --j) order[j] = order[j - 1];
+      order[j] = o;
+    }
+    for (int shift = 0; !few && shift < 32; shift += 11) {
+      uint32_t count[2049] = {};
+      for (size_t i = 0; i < n; ++i) ++count[((key[i] >> shift) & 2047u) + 1];
+      for (int b = 0; b < 2048; ++b) count[b + 1] += count[b];
+      for (size_t i = 0; i < n; ++i) {
+        const uint32_t d = (key[i] >> shift) & 2047u;
+        k2[count[d]] = key[i];
+        o2[count[d]++] = order[i];
+      }
+      key.swap(k2);
+      order.swap(o2);
+    }
+    P.groups.reserve(P.groups.size() + n);
+    size_t gi = 0;
+    for (int L = 0; L <= kLmaxMax; ++L) {
+      pass.tile_begin[L] = first;
+      for (; gi < n; ++gi) {
+        const Group& gr = g[order[gi]];
+        if ((by_degree ? P.jobs[gr.job].L : P.jobs[gr.job].plan - 1) != L) break;
+        const int nt = P.jobs[gr.job].tiles_per_chunk;
+        P.groups.push_back(MomGroup{gr.job, gr.chunk, nt, first});
+        first += nt;
+      }
+    }
+    pass.tile_begin[kLmaxMax + 1] = first;
   }
-  P.tile_begin[kLmaxMax + 1] = first;
   P.n_tiles = first;
 }
 
@@ -365,18 +398,20 @@ void build_tiles(int precision, Plan& P) {
 int moment_launches(int precision, const Plan& P) {
   const int nb = precision == TCM_FP64 ? kLmaxMax + 1 : kNumPlans - 1;
   int n = 0;
-  for (int k = 0; k < nb; ++k) n += P.tile_begin[k + 1] > P.tile_begin[k];
+  for (const Plan::Pass& pass : P.passes)
+    for (int k = 0; k < nb; ++k) n += pass.tile_begin[k + 1] > pass.tile_begin[k];
   return n;
 }
 
-// CTAs per job of the finalisation.
-int split_of(const Plan& P) {
+// CTAs per job of a pass's finalisation.
+int split_of(const Plan& P, const Plan::Pass& pass) {
   int max_tiles = 0, max_slots = 0;
-  for (const MomJob& j : P.jobs) {
+  for (int ji = pass.job0; ji < pass.job0 + pass.n_jobs; ++ji) {
+    const MomJob& j = P.jobs[ji];
     max_tiles = std::max(max_tiles, j.tiles_per_chunk);
     max_slots = std::max(max_slots, moments_nchunks(j.plan, j.L) * plan_slots(j.plan, j.L));
   }
-  return finalize_split((int)P.jobs.size(), max_tiles, max_slots);
+  return finalize_split(pass.n_jobs, max_tiles, max_slots);
 }
 
 // Most columns in a chunk of the jobs under one float plan (the column kernel's grid).
@@ -390,10 +425,9 @@ int max_cols_of(const Plan& P, int plan) {
 // Queue the moment pass (step a2/a3) for every job of the plan.
 // The moment kernels' work counters and exit tickets (counters[L], counters[32 + L]) are zero
 // on entry and left zero by every launch, so they are cleared once, when allocated.
-int ensure_moment_buffers(tcm_ctx* c, int precision, const Plan& P, bool tiles_on_host) {
+int ensure_moment_buffers(tcm_ctx* c, const Plan& P, bool tiles_on_host) {
   if (P.jobs.empty()) return TCM_OK;
-  TRY(dev_ensure(c, c->partials, (size_t)std::max(P.n_tile_ids, 1) * plan_row(precision == TCM_FP64 ? 0 : 1) *
-                                     sizeof(double)));
+  TRY(dev_ensure(c, c->partials, std::max<size_t>(P.part_doubles, 1) * sizeof(double)));
   if (!tiles_on_host) TRY(dev_ensure(c, c->tiles, (size_t)std::max(P.n_tiles, 1) * sizeof(MomTile)));
   void* before = c->counters.p;
   TRY(dev_ensure(c, c->counters, 64 * sizeof(int)));
@@ -408,17 +442,16 @@ int ensure_moment_buffers(tcm_ctx* c, int precision, const Plan& P, bool tiles_o
 // chunk plan p over all degrees.
 constexpr int kAnyCounter = kLmaxMax;  // + plan (1 or 2)
 
-int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, const MomTile* tiles,
-                const SysGeom* d_geoms, cudaStream_t st) {
-  if (P.jobs.empty()) return TCM_OK;
+int run_pass(tcm_ctx* c, int precision, const Plan& P, const Plan::Pass& pass, const MomJob* d_jobs, const MomTile* tiles,
+             const SysGeom* d_geoms, cudaStream_t st) {
   int* counters = static_cast<int*>(c->counters.p);
   double* parts = static_cast<double*>(c->partials.p);
   if (precision == TCM_FP64) {
     int ngroups = 0;
-    for (int L = 0; L <= kLmaxMax; ++L) ngroups += P.tile_begin[L + 1] > P.tile_begin[L];
+    for (int L = 0; L <= kLmaxMax; ++L) ngroups += pass.tile_begin[L + 1] > pass.tile_begin[L];
     PhaseScope ps(c, TCM_PHASE_MOMENTS, ngroups);
     for (int L = 0; L <= kLmaxMax; ++L) {
-      const int b = P.tile_begin[L], e = P.tile_begin[L + 1];
+      const int b = pass.tile_begin[L], e = pass.tile_begin[L + 1];
       if (e == b) continue;
       const int grid = std::min(e - b, c->ctas_per_sm[0][L] * c->num_sms);  // a CTA per tile
       TRY_LAUNCH(launch_moments(0, L, d_jobs, tiles + b, e - b, counters + L, d_geoms, parts, grid, st));
@@ -426,7 +459,7 @@ int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, 
   } else if (P.n_tiles > 0) {
     PhaseScope ps(c, TCM_PHASE_MOMENTS, moment_launches(precision, P));
     for (int p = 1; p < kNumPlans; ++p) {
-      const int b = P.tile_begin[p - 1], e = P.tile_begin[p];
+      const int b = pass.tile_begin[p - 1], e = pass.tile_begin[p];
       if (e == b) continue;
       if (moments_use_cols(P.n_tiles, c->num_sms)) {
         TRY_LAUNCH(launch_moments_cols(d_jobs, tiles + b, e - b, max_cols_of(P, p), d_geoms, parts, st));
@@ -443,9 +476,17 @@ int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, 
   }
   {
     PhaseScope ps(c, TCM_PHASE_FINALIZE, 1);
-    TRY_LAUNCH(launch_finalize(d_jobs, (int)P.jobs.size(), parts, d_geoms, c->d_imap, c->d_fmap, c->d_imap_off,
-                               static_cast<double*>(c->gpart.p), split_of(P), st));
+    TRY_LAUNCH(launch_finalize(d_jobs + pass.job0, pass.n_jobs, parts, d_geoms, c->d_imap, c->d_fmap, c->d_imap_off,
+                               static_cast<double*>(c->gpart.p), split_of(P, pass), st));
   }
+  return TCM_OK;
+}
+
+// (A pass writes its rows only once the finalisation before it has read them: every moment kernel waits for
+// the launch before it first.)
+int run_moments(tcm_ctx* c, int precision, const Plan& P, const MomJob* d_jobs, const MomTile* tiles,
+                const SysGeom* d_geoms, cudaStream_t st) {
+  for (const Plan::Pass& pass : P.passes) TRY(run_pass(c, precision, P, pass, d_jobs, tiles, d_geoms, st));
   return TCM_OK;
 }
 
@@ -895,7 +936,7 @@ int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, i
   const size_t o_geo = pk.add(geoms), o_job = pk.add(P.jobs), o_tile = pk.add(P.groups), o_sj = pk.add(S.jobs);
   Lists T;
   T.plan(&P, S, pk);
-  TRY(ensure_moment_buffers(c, precision, P, T.on_host));
+  TRY(ensure_moment_buffers(c, P, T.on_host));
   TRY(ensure_sys_buffers(c, S, T.on_host));
   char* base = nullptr;
   TRY(upload(c, pk, &base));
@@ -1286,7 +1327,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   // every buffer the launches touch is sized before anything is queued (no reallocation
   // may happen while a graph is being captured)
   TRY(ensure_sys_buffers(c, S, T.on_host));
-  TRY(ensure_moment_buffers(c, precision, P, T.on_host));
+  TRY(ensure_moment_buffers(c, P, T.on_host));
   char* base = nullptr;
   TRY(upload(c, pk, &base, in_place,
              on_device ? (size_t)n_items * sizeof(PairDesc) + (size_t)n_rot * sizeof(EulerZYZ) : 0));
@@ -1319,7 +1360,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   // buffers as the captured one (only the uploaded descriptor contents differ).
   const bool cols = precision == TCM_MIXED && moments_use_cols(P.n_tiles, c->num_sms);
   std::vector<long long>& key = B.key;
-  key = {precision, split_of(P), cols ? max_cols_of(P, 1) : 0, cols ? max_cols_of(P, 2) : 0, G != nullptr, S.n.one,
+  key = {precision, (long long)P.passes.size(), cols ? max_cols_of(P, 1) : 0, cols ? max_cols_of(P, 2) : 0, G != nullptr, S.n.one,
          S.n.cluster, S.n.tiles1, S.n.tiles2, (long long)S.jobs.size(), (long long)T.o_mom, (long long)T.o_sys, T.on_host,
          (long long)P.jobs.size(), P.n_tile_ids, (long long)n_items, n_rot, Lmax_items, (long long)o_geo, (long long)o_job,
          (long long)o_tile, (long long)o_sj, (long long)o_it, (long long)o_rot, (long long)o_out,
@@ -1328,7 +1369,11 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
          (long long)(uintptr_t)c->gpart.p, (long long)(uintptr_t)c->systk.p, (long long)(uintptr_t)c->partials.p,
          (long long)(uintptr_t)c->counters.p, (long long)P.groups.size(), (long long)P.n_tiles,
          (long long)(uintptr_t)c->tiles.p, (long long)c->cfg_gen};
-  for (int L = 0; L <= kLmaxMax + 1; ++L) key.push_back(P.tile_begin[L]);
+  for (const Plan::Pass& pass : P.passes) {
+    key.push_back(pass.job0);
+    key.push_back(split_of(P, pass));
+    key.insert(key.end(), pass.tile_begin, pass.tile_begin + kLmaxMax + 2);
+  }
   if (!c->gexec || key != c->gkey) {
     // by default capture only a shape seen twice in a row: a stream of changing shapes
     // (continuous batching) launches directly instead of paying a capture per call
@@ -1365,7 +1410,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
   ++c->graph_launches;
   c->launches[TCM_PHASE_GEOM] += sys_launches(S.n) + !T.on_host + on_device;
   c->launches[TCM_PHASE_MOMENTS] += moment_launches(precision, P);
-  c->launches[TCM_PHASE_FINALIZE] += !P.jobs.empty();
+  c->launches[TCM_PHASE_FINALIZE] += (int64_t)P.passes.size();
   c->launches[TCM_PHASE_CONTRACT] += 1;
   return TCM_OK;
 }

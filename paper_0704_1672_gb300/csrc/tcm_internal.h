@@ -38,20 +38,20 @@ constexpr int kThreads = 128;  // threads per moment CTA (4 warps)
 #define TCM_MOMENT_CTAS_PER_SM 2
 #endif
 constexpr int kKmaxF32 = TCM_KMAX_F32;
-constexpr int kRowF64 = (kLmaxMax + 1) * (kLmaxMax + 1);  // partial row of the double kernel: every component
+constexpr int kRowF64 = (kLmaxMax + 1) * (kLmaxMax + 1);  // the double kernel's longest partial row: every component
 
 // Chunk plans ("plans" below): the split of the (L+1)^2 accumulators of degree L into column
 // chunks of at most kmax.  Plan 0 is the double kernel's (one chunk: it keeps every component of a
 // tile); the float kernel is built for two budgets, plan 1 (kKmaxF32 accumulators per lane, 2 CTAs per SM) and plan 2
 // (kKmaxF32Small, fewer accumulators and registers, 3 CTAs per SM), chosen per degree
 // (tcm_ctx_set_chunking_l, the autotuner).  Partial rows keep the largest budget's stride in
-// every plan.
+// both float plans; a row of the double kernel holds its degree's components.
 constexpr int kKmaxF32Small = 96;
 constexpr int kNumPlans = 3;
 __host__ __device__ constexpr int plan_kmax(int plan) {
   return plan == 0 ? kRowF64 : (plan == 1 ? kKmaxF32 : kKmaxF32Small);
 }
-__host__ __device__ constexpr int plan_row(int plan) { return plan == 0 ? kRowF64 : kKmaxF32; }
+__host__ __device__ constexpr int plan_row(int plan, int L) { return plan == 0 ? (L + 1) * (L + 1) : kKmaxF32; }
 // Slots of one chunk's partial row that degree L uses under a plan (the last chunk's may be fewer).
 __host__ __device__ constexpr int plan_slots(int plan, int L) { return plan == 0 ? (L + 1) * (L + 1) : plan_kmax(plan); }
 // CTAs per SM a float moment kernel of budget kmax is compiled for (its register limit).
@@ -160,6 +160,7 @@ struct MomJob {    // one moment set: a system at one Lmax under one rotation
   int tiles_per_chunk;
   int atoms_per_tile;
   int tile_base;   // id of the job's first tile; tile id = base + chunk * tpc + t
+  long long part;  // offset (doubles) of its partial rows: row chunk * tpc + t, plan_row doubles each
   double rot[9];   // row-major, identity when unrotated
   double* out;     // packed moments, (L+1)^2 doubles
   int low_base;    // mixed precision: the row of the system-pass partials holding the system's
@@ -173,7 +174,7 @@ struct MomTile {   // one tile of moment work
   int job;
   int chunk;
   int t;           // tile index inside the chunk
-  int id;          // global tile id (row of the partials buffer)
+  int id;          // global tile id (float plans: row of the partials buffer)
 };
 
 struct MomGroup {  // the tiles of one (job, chunk), written to the tile list on the device
@@ -306,7 +307,7 @@ int sys_tile_atoms(long long n);
 // Step a3: one CTA per job, or n_split CTAs over the job's slots.  imap + imap_off[plan (kLmaxMax + 2)
 // + L] lists, per (chunk, slot) of degree L under the job's plan, the packed component it holds (-1
 // for none), nch x plan_slots(plan, L) entries; fmap beside it holds that component's F_lm with the sign of the
-// kernels' H variables.  Partial rows are plan_row(plan) doubles apart.
+// kernels' H variables.  A job's partial rows are plan_row doubles apart, from MomJob.part.
 // Jobs with low_tiles != 0 take their degrees l <= min(kLowLmax, L) from the low-degree sums of
 // their system (row low_base of the system-pass partials syspart) rotated by the job's rotation.
 int launch_finalize(const MomJob* jobs, int n_jobs, const double* partials, const SysGeom* geoms,

@@ -147,7 +147,7 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
       plan == 0 ? 32LL * std::max<long long>(f64_rows(s->n), (s->n + 32 * kNaTilesF64 - 1) / (32 * kNaTilesF64))
                 : kNaTileAtoms;
   const int tpc = (int)std::max<long long>(1, (s->n + tile_atoms - 1) / tile_atoms);
-  if (nch * tpc > kNaMaxTiles || (long long)nch * tpc * plan_row(plan) > kNaPartialDoubles)
+  if (nch * tpc > kNaMaxTiles || (long long)nch * tpc * plan_row(plan, lmax) > kNaPartialDoubles)
     return na_err(TCM_EINVAL, "tcm_moments_noalloc: request exceeds the fixed scratch");
   MomJob job{};
   job.xyzq = s->xyzq;
@@ -158,6 +158,7 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   job.tiles_per_chunk = tpc;
   job.atoms_per_tile = (int)((s->n + tpc - 1) / tpc);
   job.tile_base = 0;
+  job.part = 0;
   job.plan = plan;
   for (int k = 0; k < 9; ++k) job.rot[k] = rot ? rot[k] : ((k % 4 == 0) ? 1.0 : 0.0);
   job.out = q_out;
