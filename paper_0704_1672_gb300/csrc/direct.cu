@@ -15,19 +15,25 @@
 // Fixed point, for separated systems (r_min = R - a_A - a_B > 0, D = R + a_A + a_B):
 //   positions in units of 1/f, f the power of two with 2^60 <= D f < 2^61, as two signed 31-bit
 //   limbs X = 2^31 h + l; differences of limbs need no carries:
-//     T = sum dh^2 + 2^-30 sum dh dl  =  r^2 f^2 / 2^62      (dl^2 < 2^-60 D^2 enters by its mean)
+//     T = sum dh^2 + 2^-30 sum dh dl  =  r^2 f^2 / 2^62      (the three dl^2, below one unit each, enter by
+//                                                              their mean)
 //   1/r from the float reciprocal square root of T, as the integer Y = 2^54 / sqrt(T), and one
 //   third-order correction: with p = T Y^2 / 2^32 mod 2^64 = -2^76 e (the residual e of
 //   Y, |e| < 2^-21.1 from the bounds of rsqrt.approx and the roundings of its argument and of Y, is all that the modulus leaves of the product),
-//     y = 2^32 Y (1 + e/2 + 3/8 e^2)  =  2^117 / (f r),   good to about 2^-54;
+//     y = 2^32 Y (1 + e/2 + 3/8 e^2)  =  2^117 / (f r),   good to about 2^-54 of 1/sqrt(T);
 //   charges as 53-bit integers on the scale of the range's largest, and three integer sums of limb
-//   products, which are exact.  Errors against 64-bit positions: T to about one unit, 2^-60 D^2
-//   (the double loop rounds b' to 2^-53 R); the sum itself rounds only when it leaves the loop.
+//   products, which are exact; the sum itself rounds only when it leaves the loop.  Errors against 64-bit
+//   positions: T to 0.42 units rms, 3 at most (one unit is 2^-60 to 2^-58 D^2), so 1/r to 0.21 / T rms;
+//   the double loop rounds b' to 2^-53 of itself, so 1/r to 2^-53 R / r.  The closest pairs decide.  With all
+//   atoms on the facing surfaces, rms of 1/r in fixed point and in double (against 113-bit arithmetic):
+//   7.4e-16 and 3.8e-16 at r_min f = 2^55 (all that Y needs), 2.7e-16 and 2.2e-16 at 2^56, 1.5e-16 and 1.5e-16
+//   at 2^57, and sums of such pairs 1.7e-17 and 1.8e-17 of their magnitude.  From there on fixed point
+//   is the more exact, so the limit stands at 2^57.
 // Measured (2,587 x 3,260 atoms, 256 placements): 47.9 ms in double, 5.37 ms in fixed point; error
 // against 64-bit torch 4.0e-14 before, 1.3e-14 now (net-zero charges: of the cancelled sum).  Two atoms
 // of A per thread were slower (116 cycles a pair at 128 registers); so were the same steps left to the
 // compiler as 64-bit expressions (125: it spends the multiplier on register moves).
-// The bound r_min f >= 2^55 (r_min / D above 1/64 to 1/32) keeps Y below 2^31.
+// The bound r_min f >= 2^57 (r_min / D above 1/16 to 1/8) keeps T above 2^52 and Y below 2^28.
 #include <cuda_runtime.h>
 
 #include "contract.h"
@@ -190,7 +196,7 @@ __device__ __forceinline__ Fixed fixed_scales(const Place& g, double aA, double 
   s.rB2 = aB * aB;
   s.ok = D > 0.0 && e > -400 && e < 400;
   s.f = pow2(s.ok ? 61 - e : 0);
-  s.ok = s.ok && (R - aA - aB) * s.f >= 36028797018963968.0;  // 2^55
+  s.ok = s.ok && (R - aA - aB) * s.f >= 0x1p57;
   return s;
 }
 
