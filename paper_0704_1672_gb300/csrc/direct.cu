@@ -97,6 +97,8 @@ __device__ __forceinline__ double load_q(const void* p, int dtype, long long i) 
 }
 
 __device__ __forceinline__ int exponent(double v) { return (int)((__double2hiint(v) >> 20) & 0x7ff) - 1022; }
+constexpr int kNoCharge = -1022;  // of a range without charge
+__device__ __forceinline__ int charge_exponent(double q) { return q == 0.0 ? kNoCharge : max(exponent(q), kNoCharge + 1); }
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
 // The item's transform: centres, rotation, separation.
@@ -242,14 +244,15 @@ __global__ void __launch_bounds__(kDirectThreads, 4)
   bool fixed = false;
   if (!__syncthreads_or(bad)) {
     // the range's largest charge sets the scale of the charges; every staged atom lies within the radius
-    int qe = -1022;
-    for (long long j = j0 + t; j < j1; j += kDirectThreads) qe = max(qe, exponent(load_q(b, dtb, j)));
+    int qe = kNoCharge;
+    for (long long j = j0 + t; j < j1; j += kDirectThreads) qe = max(qe, charge_exponent(load_q(b, dtb, j)));
     qe = __reduce_max_sync(0xffffffffu, qe);
     if ((t & 31) == 0) atomicMax(&s_exp, qe + 1022);
     __syncthreads();
     qe = s_exp - 1022;
-    fixed = qe < 900;  // (not finite: 1025)
-    if (qe < -800) qe = -800;
+    // (not finite: 1025); under 2^-500 the scale of the sum would leave the normal numbers
+    fixed = qe < 900 && (qe >= -500 || qe == kNoCharge);
+    if (qe == kNoCharge) qe = 0;
     const double gq = pow2(26 - qe);  // |q| gq < 2^26
     int ah[3], al[3];
 #pragma unroll
