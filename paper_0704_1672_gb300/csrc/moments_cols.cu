@@ -1,4 +1,5 @@
-// Float moment kernel for calls with little work: the lane sums of moments_kernel.cuh, bit for bit,
+// Float moment kernel for calls with little work: the lane sums of moments_kernel.cuh, bit for bit (but for
+// the degrees l <= 2, which come from the system pass: nothing reads what either kernel leaves there),
 // with one column m per warp instead of a chunk of columns.
 //
 // A warp tile of 64 atoms per lane and a chunk of up to 160 accumulators keeps its warp busy for about
@@ -197,8 +198,11 @@ __global__ void __launch_bounds__(kColThreads)
 
 }  // namespace
 
-// The column kernel's warps finish a tile in about 20 us where the chunk kernel's take 50 (degree 20),
-// at twice the instructions: taken while the chunk kernel would have no more than one warp per SM.
+// The column kernel's warps finish a tile sooner at twice the instructions: taken while the chunk kernel
+// would have no more than one warp per SM.  Moment pass of one system of 10, 30, 60, 100, 130 and 152 tiles, by
+// columns and by chunks: 20, 20, 22, 24, 28, 27 and 36 us throughout at degree 20; 16, 16, 18, 18, 22, 22 and 22 to
+// 24 at degree 8; 16 to 18 and 18 to 20 at degree 4; 22 to 28 and 34 at degree 24; a scan of 129 tiles at degree 8
+// 18 and 22, of 102 at degree 16 24 and 32: no slower anywhere up to the line.
 bool moments_use_cols(int n_tiles, int num_sms) { return n_tiles <= num_sms; }
 
 // Largest number of columns in a chunk of degree L.

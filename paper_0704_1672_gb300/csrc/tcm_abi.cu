@@ -553,14 +553,17 @@ void plan_sys(const tcm_system* systems, int n_systems, const std::vector<char>&
     }
 }
 
-// Mixed path: every computed moment job takes its degrees l <= 2 from its system's low sums.
-void link_low(const SysPlan& S, Plan& P) {
+// Mixed path: every computed moment job takes its degrees l <= 2 from its system's low sums (the float
+// kernels have no values of their own for them).
+int link_low(const SysPlan& S, Plan& P) {
   for (MomJob& j : P.jobs) {
+    if (j.plan == 0) continue;
     const int si = S.of_system[j.geom];
-    if (si < 0 || !S.jobs[si].need_low) continue;
+    if (si < 0 || !S.jobs[si].need_low) return set_err(TCM_ECUDA, "internal: a float moment job without its low-degree sums");
     j.low_base = S.jobs[si].sum_row;
     j.low_tiles = 1;
   }
+  return TCM_OK;
 }
 
 // Partial rows and tickets of the system pass; the tickets are zeroed when allocated and every
@@ -930,7 +933,7 @@ int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, i
   std::vector<char> used(1, 1), low(1, precision == TCM_MIXED ? 1 : 0);
   SysPlan S;
   plan_sys(s, 1, used, low, S);
-  link_low(S, P);
+  TRY(link_low(S, P));
   std::vector<SysGeom> geoms{host_geom(*s)};
   Packer pk;
   const size_t o_geo = pk.add(geoms), o_job = pk.add(P.jobs), o_tile = pk.add(P.groups), o_sj = pk.add(S.jobs);
@@ -1274,7 +1277,7 @@ int energy_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t 
     for (const MomJob& j : P.jobs) B.low[j.geom] = 1;
   SysPlan& S = B.S;
   plan_sys(systems, n_systems, B.used, B.low, S);
-  link_low(S, P);
+  TRY(link_low(S, P));
   const int n_computed = (int)P.jobs.size();  // cached sides follow them in the descriptor array (not finalised)
   const int n_rot = (int)(B.rotB.size() / 9);
   B.geoms.resize(std::max(n_systems, 1));

@@ -164,8 +164,8 @@ struct MomJob {    // one moment set: a system at one Lmax under one rotation
   double rot[9];   // row-major, identity when unrotated
   double* out;     // packed moments, (L+1)^2 doubles
   int low_base;    // mixed precision: the row of the system-pass partials holding the system's
-  int low_tiles;   // low-degree sums (SysJob.sum_row) when low_tiles != 0; 0 = the degrees l <= 2
-                   // keep the float kernel's values
+  int low_tiles;   // low-degree sums (SysJob.sum_row), low_tiles = 1: every job of a float plan, whose
+                   // kernels leave the degrees l <= 2 to them; 0: double plan
   int plan;        // chunk plan of its moment tiles (0: double kernels; 1, 2: float budgets)
   int pad_;
 };
