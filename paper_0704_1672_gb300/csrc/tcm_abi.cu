@@ -8,6 +8,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <new>
 #include <vector>
 
@@ -90,6 +91,9 @@ struct Packer {
     return off;
   }
 };
+
+// What the host arrays of a call throw stays behind the C entry.
+int no_host_memory(const char* what) { return set_err(TCM_ENOMEM, "%s: host allocation failed", what); }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -876,7 +880,7 @@ int tcm_ctx_read_profile(tcm_ctx_t c, double* ms, int64_t* launches) {
   return TCM_OK;
 }
 
-int tcm_prepare(tcm_ctx_t c, tcm_system* s) {
+int tcm_prepare(tcm_ctx_t c, tcm_system* s) try {
   TRY(check_ctx(c));
   TRY(check_system(s, "tcm_prepare"));
   if (geom_known(*s)) return TCM_OK;
@@ -903,9 +907,11 @@ int tcm_prepare(tcm_ctx_t c, tcm_system* s) {
   s->has_center = 1;
   s->radius = g->a;
   return TCM_OK;
+} catch (const std::exception&) {
+  return no_host_memory("tcm_prepare");
 }
 
-int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, int precision, tcm_moments_t* out) {
+int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, int precision, tcm_moments_t* out) try {
   TRY(check_ctx(c));
   TRY(check_system(s, "tcm_moments"));
   if (!out || !out->q) return set_err(TCM_EINVAL, "tcm_moments: null output");
@@ -962,9 +968,11 @@ int tcm_moments(tcm_ctx_t c, const tcm_system* s, const double* rot, int lmax, i
     out->radius = s->radius;
   }
   return TCM_OK;
+} catch (const std::exception&) {
+  return no_host_memory("tcm_moments");
 }
 
-int tcm_energy(tcm_ctx_t c, const tcm_moments_t* A, const tcm_moments_t* B, const double* R0, int lmax, double* E) {
+int tcm_energy(tcm_ctx_t c, const tcm_moments_t* A, const tcm_moments_t* B, const double* R0, int lmax, double* E) try {
   TRY(check_ctx(c));
   if (!A || !B || !R0 || !E || !A->q || !B->q) return set_err(TCM_EINVAL, "tcm_energy: null argument");
   if (lmax < 0 || lmax > c->lmax_cap || lmax > A->lmax || lmax > B->lmax)
@@ -1006,9 +1014,11 @@ int tcm_energy(tcm_ctx_t c, const tcm_moments_t* A, const tcm_moments_t* B, cons
   TRY_CUDA(cudaStreamSynchronize(c->stream));
   *E = *static_cast<const double*>(c->pinned_small);
   return TCM_OK;
+} catch (const std::exception&) {
+  return no_host_memory("tcm_energy");
 }
 
-int tcm_rotate_moments(tcm_ctx_t c, int64_t n, const tcm_moments_t* in, const double* rot, tcm_moments_t* out) {
+int tcm_rotate_moments(tcm_ctx_t c, int64_t n, const tcm_moments_t* in, const double* rot, tcm_moments_t* out) try {
   TRY(check_ctx(c));
   if (n < 0) return set_err(TCM_EINVAL, "tcm_rotate_moments: negative count");
   if (n == 0) return TCM_OK;
@@ -1038,6 +1048,8 @@ int tcm_rotate_moments(tcm_ctx_t c, int64_t n, const tcm_moments_t* in, const do
   PhaseScope ps(c, TCM_PHASE_CONTRACT, 1);
   TRY_LAUNCH(launch_rotate_moments(reinterpret_cast<RotDesc*>(base + o_set), (int)n, Lmax, c->d_ctab->dpi2, c->stream));
   return TCM_OK;
+} catch (const std::exception&) {
+  return no_host_memory("tcm_rotate_moments");
 }
 
 int tcm_ctx_set_rotate_cached(tcm_ctx_t c, int enable) {
@@ -1059,8 +1071,8 @@ int timed_batch(tcm_ctx_t c, int n_systems, const tcm_system* systems, int64_t n
   int rc;
   try {
     rc = energy_batch(c, n_systems, systems, n_items, items, precision, E, status, G);
-  } catch (const std::bad_alloc&) {
-    rc = set_err(TCM_ENOMEM, "tcm_energy_batch: host allocation failed");
+  } catch (const std::exception&) {
+    rc = no_host_memory("tcm_energy_batch");
   }
   if (c && c->prof) c->host_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   return rc;
@@ -1461,7 +1473,7 @@ int direct_items(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t 
 }
 }  // namespace
 
-int tcm_direct(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, const double* rotB, const double* R0, double* E) {
+int tcm_direct(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, const double* rotB, const double* R0, double* E) try {
   TRY(check_ctx(c));
   TRY(check_system(A, "tcm_direct A"));
   TRY(check_system(B, "tcm_direct B"));
@@ -1473,10 +1485,12 @@ int tcm_direct(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, const doub
   TRY_CUDA(cudaStreamSynchronize(c->stream));
   *E = *static_cast<const double*>(c->pinned_small);
   return TCM_OK;
+} catch (const std::exception&) {
+  return no_host_memory("tcm_direct");
 }
 
 int tcm_direct_batch(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int64_t n_items, const double* rotB,
-                     const double* R0, double* E) {
+                     const double* R0, double* E) try {
   TRY(check_ctx(c));
   TRY(check_system(A, "tcm_direct_batch A"));
   TRY(check_system(B, "tcm_direct_batch B"));
@@ -1487,6 +1501,8 @@ int tcm_direct_batch(tcm_ctx_t c, const tcm_system* A, const tcm_system* B, int6
   if ((A->n + 255) / 256 * n_items > (1LL << 34))
     return set_err(TCM_EINVAL, "tcm_direct_batch: A's blocks x items exceeds the partial-sum buffer limit");
   return direct_items(c, A, B, n_items, rotB, R0, E);
+} catch (const std::exception&) {
+  return no_host_memory("tcm_direct_batch");
 }
 
 }  // extern "C"

@@ -18,6 +18,7 @@
 
 #include <cmath>
 #include <cstring>
+#include <exception>
 #include <mutex>
 #include <vector>
 
@@ -136,7 +137,12 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
     return na_err(TCM_ECUDA, "tcm_moments_noalloc: no usable CUDA device");
   char* base = nullptr;
-  int rc = setup_device(dev, &base);
+  int rc;
+  try {
+    rc = setup_device(dev, &base);
+  } catch (const std::exception&) {
+    return na_err(TCM_ENOMEM, "tcm_moments_noalloc: host allocation failed");
+  }
   if (rc != TCM_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
