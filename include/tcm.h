@@ -280,7 +280,7 @@ int tcm_direct(tcm_ctx_t ctx, const tcm_system* A, const tcm_system* B, const do
  * IV): for item k, B rotated by rotB + 9 k (host row-major 3x3 array per item, or NULL for
  * none) about its centre, with its centre at A's centre plus R0 + 3 k (host).  E: device,
  * n_items doubles.  Fixed-order sums, split by the atom counts alone; for
- * systems separated by more than a sixteenth to an eighth of their common extent |R0| + a_A + a_B the
+ * systems separated by more than a thirty-second to a sixteenth of their common extent |R0| + a_A + a_B the
  * pairs are summed in 64-bit fixed point (an error no larger than that of double arithmetic), otherwise
  * in double.  Asynchronous on the context stream. */
 int tcm_direct_batch(tcm_ctx_t ctx, const tcm_system* A, const tcm_system* B, int64_t n_items,

@@ -13,27 +13,28 @@
 //   values that fixed point cannot hold (not finite, or outside the radii), and for extreme scales.
 //
 // Fixed point, for separated systems (r_min = R - a_A - a_B > 0, D = R + a_A + a_B):
-//   positions in units of 1/f, f the power of two with 2^60 <= D f < 2^61, as two signed 31-bit
+//   positions in units of 1/f, f the power of two with 2^61 <= D f < 2^62, as two signed 31-bit
 //   limbs X = 2^31 h + l; differences of limbs need no carries:
 //     T = sum dh^2 + 2^-30 sum dh dl  =  r^2 f^2 / 2^62      (the three dl^2, below one unit each, enter by
 //                                                              their mean)
-//   1/r from the float reciprocal square root of T, as the integer Y = 2^54 / sqrt(T), and one
-//   third-order correction: with p = T Y^2 / 2^32 mod 2^64 = -2^76 e (the residual e of
+//   1/r from the float reciprocal square root of T, as the integer Y = 2^55 / sqrt(T), and one
+//   third-order correction: with p = T Y^2 / 2^32 mod 2^64 = -2^78 e (the residual e of
 //   Y, |e| < 2^-21.1 from the bounds of rsqrt.approx and the roundings of its argument and of Y, is all that the modulus leaves of the product),
-//     y = 2^32 Y (1 + e/2 + 3/8 e^2)  =  2^117 / (f r),   good to about 2^-54 of 1/sqrt(T);
+//     y = 2^32 Y (1 + e/2 + 3/8 e^2)  =  2^118 / (f r),   good to about 2^-54 of 1/sqrt(T);
 //   charges as 53-bit integers on the scale of the range's largest, and three integer sums of limb
 //   products, which are exact; the sum itself rounds only when it leaves the loop.  Errors against 64-bit
-//   positions: T to 0.42 units rms, 3 at most (one unit is 2^-60 to 2^-58 D^2), so 1/r to 0.21 / T rms;
-//   the double loop rounds b' to 2^-53 of itself, so 1/r to 2^-53 R / r.  The closest pairs decide.  With all
-//   atoms on the facing surfaces, rms of 1/r in fixed point and in double (against 113-bit arithmetic):
-//   7.4e-16 and 3.8e-16 at r_min f = 2^55 (all that Y needs), 2.7e-16 and 2.2e-16 at 2^56, 1.5e-16 and 1.5e-16
-//   at 2^57, and sums of such pairs 1.7e-17 and 1.8e-17 of their magnitude.  From there on fixed point
-//   is the more exact, so the limit stands at 2^57.
+//   positions: T to 0.42 units rms, 3 at most (one unit is 2^-62 to 2^-60 D^2), so 1/r to 0.21 / T rms;
+//   the double loop rounds b' to 2^-53 of itself, so 1/r to 2^-53 |b'| / r.  The closest pairs decide.  With
+//   all charges on the facing surfaces, rms of 1/r in fixed point and in double (against 113-bit arithmetic):
+//   9.4e-16 and 7.0e-16 at r_min f = 2^55 and D / r_min = 62, 4.3e-16 and 3.9e-16 at 2^56 and 36, 2.7e-16 and
+//   2.7e-16 at 2^57 and 24, and sums of such pairs 2.3e-17 and 2.4e-17 of their magnitude.  From there on
+//   fixed point is the more exact, so the limit stands at 2^57.
 // Measured (2,587 x 3,260 atoms, 256 placements): 47.9 ms in double, 5.37 ms in fixed point; error
 // against 64-bit torch 4.0e-14 before, 1.3e-14 now (net-zero charges: of the cancelled sum).  Two atoms
 // of A per thread were slower (116 cycles a pair at 128 registers); so were the same steps left to the
 // compiler as 64-bit expressions (125: it spends the multiplier on register moves).
-// The bound r_min f >= 2^57 (r_min / D above 1/16 to 1/8) keeps T above 2^52 and Y below 2^28.
+// Bounds: r_min f >= 2^57 (r_min / D above 1/32 to 1/16) keeps T above 2^52 and Y below 2^29, D f < 2^62 (with
+// room for the limbs' rounding) dh below 2^31 and Y above 2^24.
 #include <cuda_runtime.h>
 
 #include "contract.h"
@@ -122,7 +123,7 @@ __device__ __forceinline__ void split31(double x, double f, int& h, int& l) {
 __device__ __forceinline__ long long madw(int a, int b, long long c) {
   return (long long)a * (long long)b + c;
 }
-// 2^117 / (f r) of one pair (see the head of the file).
+// 2^118 / (f r) of one pair (see the head of the file).
 __device__ __forceinline__ int2 inv_r(const int* ah, const int* al, const int4 bh, const int4 bl) {
   const int h0 = bh.x - ah[0], h1 = bh.y - ah[1], h2 = bh.z - ah[2];
   const int l0 = bl.x - al[0], l1 = bl.y - al[1], l2 = bl.z - al[2];
@@ -138,10 +139,10 @@ __device__ __forceinline__ int2 inv_r(const int* ah, const int* al, const int4 b
       : "l"(s), "l"(c));
   float y0;  // within 2^-22.9
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(fmaf((float)Th, 4294967296.0f, (float)Tl)));
-  const int Y = __float2int_rn(y0 * 18014398509481984.0f);  // 2^54
+  const int Y = __float2int_rn(y0 * 36028797018963968.0f);  // 2^55
   const unsigned long long U = (unsigned long long)(unsigned)Y * (unsigned)Y;
   const unsigned Uh = (unsigned)(U >> 32), Ul = (unsigned)U;
-  // p = T U / 2^32 mod 2^64 (its multiple of 2^76 drops out), |p| < 2^55; the product of the low
+  // p = T U / 2^32 mod 2^64 (its multiple of 2^78 drops out), |p| < 2^57; the product of the low
   // words by their upper halves
   const unsigned long long w = (unsigned long long)Tl * Uh + (unsigned long long)Th * Ul;
   unsigned pl, ph;
@@ -150,8 +151,8 @@ __device__ __forceinline__ int2 inv_r(const int* ah, const int* al, const int4 b
       : "=r"(pl), "=r"(ph)
       : "l"(w), "r"((Tl >> 16) * (Ul >> 16)), "r"(Th), "r"(Uh));
   const float t = (float)(int)ph;
-  // p / 2^24 with the second-order term, 3/8 e^2 2^53
-  const int q = (int)__funnelshift_r(pl, ph, 24) - __float2int_rn(t * t * (0.375f / 34359738368.0f));
+  // p / 2^26 with the second-order term, 3/8 e^2 2^53
+  const int q = (int)__funnelshift_r(pl, ph, 26) - __float2int_rn(t * t * (0.375f / 549755813888.0f));
   const long long M = (long long)Y * q;
   int lo, hi;
   asm("sub.cc.u32 %0, 0, %2;\n\tsubc.u32 %1, %3, %4;"  // 2^32 Y - (M >> 21)
@@ -192,12 +193,12 @@ __device__ __forceinline__ Fixed fixed_scales(const Place& g, double aA, double 
   const double R = sqrt(g.R0[0] * g.R0[0] + g.R0[1] * g.R0[1] + g.R0[2] * g.R0[2]);
   aA *= 1.0 + 1e-9;  // room for the rounding of the rotated offsets
   aB *= 1.0 + 1e-9;
-  const double D = R + aA + aB;
+  const double D = (R + aA + aB) * (1.0 + 1e-9);  // (and for the limbs)
   const int e = exponent(D);  // D < 2^e
   s.rA2 = aA * aA;
   s.rB2 = aB * aB;
   s.ok = D > 0.0 && e > -400 && e < 400;
-  s.f = pow2(s.ok ? 61 - e : 0);
+  s.f = pow2(s.ok ? 62 - e : 0);
   s.ok = s.ok && (R - aA - aB) * s.f >= 0x1p57;
   return s;
 }
@@ -292,8 +293,8 @@ __global__ void __launch_bounds__(kDirectThreads, 4)
       }
     }
     if (fixed) {
-      // q / r = 2^-117 f y / (2^27 gq) q's integer; FixSum::value leaves a weight of 2^32
-      const double scale = fs.f * pow2(-117 - 27 + 32) * pow2(qe - 26);
+      // q / r = 2^-118 f y / (2^27 gq) q's integer; FixSum::value leaves a weight of 2^32
+      const double scale = fs.f * pow2(-118 - 27 + 32) * pow2(qe - 26);
       acc = sum.value(scale);
     }
   }

@@ -5,8 +5,8 @@ Double arithmetic rounds B's placed position b' to 2^-53 of its components, and 
   rms over many directions, in units of 2^-53 |b'| / r: sqrt(3/5 x 0.54 / 3) = 0.33 (the mean of the fourth
   powers of a direction's components, of the squared unit in the last place, and of a uniform error), 0.34
   with the other roundings where |b'| / r is about 12; 0.40 leaves three standard errors and a margin.
-The rms is taken over the gaps next to the fixed-point form's own limit, (R + a_A + a_B) / gap from 16
-to 64, where an error of that form would show first."""
+The rms is taken over narrow gaps, 2^-6 to 2^-4 of the common extent D = R + a_A + a_B, where an error of the
+fixed-point form would show first."""
 import numpy as np
 import pytest
 import torch
@@ -38,8 +38,8 @@ def test_facing_charges():
             placed = (np.sqrt((b * b).sum(1)) / r).astype(np.float64)
             worst = max(worst, float((err / (placed + 6.0)).max()))
             D = 2.0 * (aA + aB) + gap
-            at = np.log2(gap / D) + np.log2(D) % 1.0 + 60.0  # log2 of gap f (csrc/direct.cu)
-            near.append((err / placed)[(at >= 55.0) & (at < 56.0)])
+            at = np.log2(gap / D) + np.log2(D) % 1.0  # log2 of the gap's share, D rounded down to a power of two
+            near.append((err / placed)[(at >= -5.0) & (at < -4.0)])
     near = np.concatenate(near)
     rms = float(np.sqrt(np.mean(near ** 2)))
     print(f"worst {worst:.3f} of the bound; rms {rms:.3f} over {len(near)} pairs")
