@@ -7,7 +7,7 @@ caller's own batch.
 For every degree present in the batch, the items of that degree (at most ``max_items_per_l`` of
 them) form a sub-batch; each candidate setting (atoms per lane, CTAs per SM, kmax) is applied
 with ``tcm_ctx_set_tiling_l`` and ``tcm_ctx_set_chunking_l``, the sub-batch is run once untimed
-and ``reps`` times timed, and the median time of the moment phase (the library's CUDA-event
+and ``reps`` times timed, and the shortest time of the moment phase (the library's CUDA-event
 phase profile: the moment kernels of that degree, nothing else) is kept.  The fastest candidate
 (when the sub-batch is a sample of the degree's items: among those within 1 % of it, the one
 with the largest warp tiles; ``choose``) is applied to the context and returned.  Results can be saved to a JSON file keyed by device
@@ -66,7 +66,7 @@ def set_setting(ctx, precision, L, setting):
 class TuneResult:
     precision: int
     best: dict = field(default_factory=dict)     # L -> (atoms_per_lane, ctas_per_sm, kmax)
-    timings: dict = field(default_factory=dict)  # L -> {(atoms_per_lane, ctas_per_sm, kmax): median ms}
+    timings: dict = field(default_factory=dict)  # L -> {(atoms_per_lane, ctas_per_sm, kmax): ms}
 
     def to_json(self):
         return {"precision": int(self.precision),
@@ -84,7 +84,7 @@ class TuneResult:
 
 
 def choose(timings: dict, tol=0.01):
-    """Among the candidates within ``tol`` (relative) of the smallest median time, the one with
+    """Among the candidates within ``tol`` (relative) of the smallest time, the one with
     the largest warp tiles (atoms per lane; ties: the first in candidate order).  Larger tiles
     mean fewer partial rows for the finalisation to read, which a sampled sub-batch
     under-represents: on the large assembly 256 and 512 atoms per lane time within 0.1 % on 512
@@ -113,7 +113,9 @@ def degree_groups(lmax, max_items_per_l):
 
 
 def moment_phase_ms(ctx, run, reps):
-    """Median over reps of the moment-phase time of run() (one untimed call first)."""
+    """Shortest of reps moment-phase times of run() (one untimed call first).  What disturbs a timing only
+    lengthens it, and with the two repetitions that a large batch is given a median would be their
+    mean: one slow run took a degree off a setting that is 2 to 3 % ahead of the next."""
     run()
     ctx.tcm_ctx_set_profiling(True)
     ctx.tcm_ctx_read_profile()
@@ -123,7 +125,7 @@ def moment_phase_ms(ctx, run, reps):
         ms, _ = ctx.tcm_ctx_read_profile()
         times.append(ms["moments"])
     ctx.tcm_ctx_set_profiling(False)
-    return float(np.median(times))
+    return float(np.min(times))
 
 
 def tune(ctx, systems, a, b, lmax, R0, rotB=None, precision=None, atoms_per_lane=DEFAULT_ATOMS_PER_LANE,
