@@ -39,10 +39,10 @@
 // digits, of 48 fourteen.)  B's moments in mode kBInFrame need no rotation and stay double throughout.
 // Error of an energy (rms, of sum |U_l1l2|, 40 random pairs at degrees 1 to 24; against 113-bit
 // arithmetic): 1.5e-16 to 8.9e-16, the all-double kernel's 1.5e-16 to 8.9e-16; forces and torques alike.
-// Measured, in double and now: 108,360 energies at degrees 1 to 10 1,340 and 298 us, 2,048 at degrees 8 to
-// 24 (B rotated) 140 and 64, 256 at degree 20 24 and 16, forces and torques of 512 at degree 12 92 and 25.
-// What bounds it now: the phases between barriers (a third of the stalls) with the multiplier 0.45 busy and
-// the FP64 pipe 0.27; 80 registers and 3 CTAs per SM instead of 64 and 4 took 342 us of the first.
+// Measured (us), all in double, with the products in fixed point too, and now: 108,360 energies at degrees 1 to
+// 10 1,340, 298, 331; 2,048 at degrees 8 to 24 (B rotated) 140, 64, 78; 256 at degree 20 24, 16, 21; forces
+// and torques of 512 at degree 12 92, 25, 49.  What bounds it now: the FP64 pipe in the (l1, l2) phase (busy
+// 0.54 over the kernel at degree 24, 0.66 with forces and torques) between phases separated by barriers.
 // A CTA takes a group of items of one degree side by side (contract_group), so that its lanes are full
 // at low degrees too, one lane column per item.  The group size, and with it the order of every sum,
 // depends on the degree alone: an item's result does not depend on its batch.
@@ -396,30 +396,30 @@ __global__ void __launch_bounds__(kCT, kGrad ? 2 : 4)
         sum[0] = fma(c, T, sum[0]);
         if (kGrad) {
           const double2* am = dm + tri(l1) * G + it;
-          double sr = 0.0, si = 0.0, wr = 0.0, wi = 0.0, z = 0.0;
-          const int ma = min(l1, l2 + 1), mc = min(l1, l2 - 1);
-          for (int m = 1; m <= ma; ++m) {  // (m, 1 - m): -a_m conj(b_(m-1))
-            const double2 x = a[m * G], xm = am[m * G], y = b[(m - 1) * G];
+          // the sums weighted by m as sums of partial sums, from the highest m down: an addition each
+          // instead of two multiply-adds
+          double sr = 0.0, si = 0.0, tr = 0.0, ti = 0.0, wr = 0.0, wi = 0.0, z = 0.0;
+          for (int m = min(l1, l2 + 1); m >= 1; --m) {  // (m, 1 - m): -a_m conj(b_(m-1)), weight l2 + 1 - m
+            const double2 x = a[m * G], y = b[(m - 1) * G];
             sr = fma(-x.x, y.x, sr);
             sr = fma(-x.y, y.y, sr);
             si = fma(-x.y, y.x, si);
             si = fma(x.x, y.y, si);
-            wr = fma(xm.x, y.x, wr);  // m times the weight's change, -m
-            wr = fma(xm.y, y.y, wr);
-            wi = fma(xm.y, y.x, wi);
-            wi = fma(-xm.x, y.y, wi);
+            wr -= sr;
+            wi -= si;
           }
-          for (int m = 0; m <= mc; ++m) {  // (-m, m + 1): conj(a_m) b_(m+1)
-            const double2 x = a[m * G], xm = am[m * G], y = b[(m + 1) * G];
-            sr = fma(x.x, y.x, sr);
-            sr = fma(x.y, y.y, sr);
-            si = fma(x.x, y.y, si);
-            si = fma(-x.y, y.x, si);
-            wr = fma(xm.x, y.x, wr);
-            wr = fma(xm.y, y.y, wr);
-            wi = fma(xm.x, y.y, wi);
-            wi = fma(-xm.y, y.x, wi);
+          for (int m = min(l1, l2 - 1); m >= 0; --m) {  // (-m, m + 1): conj(a_m) b_(m+1), weight l2 + 1 + m
+            const double2 x = a[m * G], y = b[(m + 1) * G];
+            tr = fma(x.x, y.x, tr);
+            tr = fma(x.y, y.y, tr);
+            ti = fma(x.x, y.y, ti);
+            ti = fma(-x.y, y.x, ti);
+            if (m == 0) break;
+            wr += tr;
+            wi += ti;
           }
+          sr += tr;
+          si += ti;
           for (int m = 1; m <= s; ++m) {
             const double2 xm = am[m * G], y = b[m * G];
             z = fma(xm.y, y.x, z);

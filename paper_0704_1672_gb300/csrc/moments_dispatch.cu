@@ -132,8 +132,7 @@ __global__ void __launch_bounds__(256) k_expand_tiles(const MomGroup* __restrict
   if (g < n_groups) {
     const MomGroup gr = groups[g];
     const MomJob& j = jobs[gr.job];
-    const int row = j.tile_base + gr.chunk * j.tiles_per_chunk;
-    for (int t = lane; t < gr.n; t += 32) tiles[gr.first + t] = MomTile{gr.job, gr.chunk, t, row + t};
+    for (int t = lane; t < gr.n; t += 32) tiles[gr.first + t] = MomTile{gr.job, gr.chunk, t, part_row(j, gr.chunk, t)};
   } else if (g - n_groups < n_sjobs) {
     const int ji = g - n_groups;
     const SysJob sj = sjobs[ji];

@@ -13,8 +13,8 @@
 //   - at the end of a tile every thread adds the 32 lanes of a component.
 // Column chunks of 80 accumulators in registers, the form before, repeated the set-up in each of up
 // to 10 chunks and left a small system to one warp per chunk and 1,024 atoms.  Calls of tcm_moments,
-// before and now: 100,003 atoms at degree 24 635 and 353 us (the FP64 instructions it cannot do
-// without take 252); 3,260 and 2,587 atoms at degree 10, with their energy, 554 and 194 us; 257 sets
+// before and now: 100,003 atoms at degree 24 635 and 320 us (the FP64 instructions it cannot do
+// without take 252); 3,260 and 2,587 atoms at degree 10, with their energy, 554 and 170 us; 257 sets
 // of 20,000 atoms at degree 20 14.5 and 13.1 ms.
 //
 // Row j of a tile uses ring slot j mod 3 and producer j mod 3.  Named barriers 1 + slot (row full)

@@ -301,7 +301,6 @@ void plan_job(tcm_ctx* c, int precision, MomJob& j, int& next_id) {
   if (tpc < 1) tpc = 1;
   j.tiles_per_chunk = (int)tpc;
   j.atoms_per_tile = (int)((j.n + tpc - 1) / tpc);
-  j.tile_base = next_id;
   next_id += nch * (int)tpc;
 }
 
@@ -606,7 +605,7 @@ struct Lists {
       for (const MomGroup& g : P->groups) {
         const MomJob& j = P->jobs[g.job];
         for (int t = 0; t < g.n; ++t)
-          mom[g.first + t] = MomTile{g.job, g.chunk, t, j.tile_base + g.chunk * j.tiles_per_chunk + t};
+          mom[g.first + t] = MomTile{g.job, g.chunk, t, part_row(j, g.chunk, t)};
       }
     for (int ji = 0; ji < (int)S.jobs.size(); ++ji) {
       const SysJob& j = S.jobs[ji];

@@ -159,22 +159,24 @@ struct MomJob {    // one moment set: a system at one Lmax under one rotation
   int geom;        // index into the SysGeom array
   int tiles_per_chunk;
   int atoms_per_tile;
-  int tile_base;   // id of the job's first tile; tile id = base + chunk * tpc + t
+  int plan;        // chunk plan of its moment tiles (0: double kernels; 1, 2: float budgets)
   long long part;  // offset (doubles) of its partial rows: row chunk * tpc + t, plan_row doubles each
   double rot[9];   // row-major, identity when unrotated
   double* out;     // packed moments, (L+1)^2 doubles
   int low_base;    // mixed precision: the row of the system-pass partials holding the system's
   int low_tiles;   // low-degree sums (SysJob.sum_row), low_tiles = 1: every job of a float plan, whose
                    // kernels leave the degrees l <= 2 to them; 0: double plan
-  int plan;        // chunk plan of its moment tiles (0: double kernels; 1, 2: float budgets)
-  int pad_;
 };
+// Row of the partials buffer of a job's tile t of chunk ch (float plans, whose rows are all one length).
+__host__ __device__ inline int part_row(const MomJob& j, int ch, int t) {
+  return j.plan == 0 ? 0 : (int)(j.part / kKmaxF32) + ch * j.tiles_per_chunk + t;
+}
 
 struct MomTile {   // one tile of moment work
   int job;
   int chunk;
   int t;           // tile index inside the chunk
-  int id;          // global tile id (float plans: row of the partials buffer)
+  int id;          // float plans: row of the partials buffer (part_row)
 };
 
 struct MomGroup {  // the tiles of one (job, chunk), written to the tile list on the device
@@ -264,8 +266,7 @@ cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
 int launch_moments(int plan, int L, const MomJob* jobs, const MomTile* tiles, int n_tiles,
                    int* counter, const SysGeom* geoms, double* partials, int grid, cudaStream_t s);
 // The tile lists of a call, written on the device: the moment pass's from its groups,
-// tiles[g.first + t] = (g.job, g.chunk, t, row), t < g.n, row = jobs[g.job].tile_base +
-// g.chunk * tiles_per_chunk + t; and the system pass's, t1[sj.first1 + t] = t2[sj.first2 + t] =
+// tiles[g.first + t] = (g.job, g.chunk, t, part_row), t < g.n; and the system pass's, t1[sj.first1 + t] = t2[sj.first2 + t] =
 // (job, t), t < sj.n_tiles.  One warp per group or system job.
 int launch_expand_tiles(const MomGroup* groups, int n_groups, const MomJob* jobs, MomTile* tiles, const SysJob* sjobs,
                         int n_sjobs, SysTile* t1, SysTile* t2, cudaStream_t s);

@@ -163,7 +163,6 @@ extern "C" int tcm_moments_noalloc(const tcm_system* s, const double* rot, int l
   job.geom = 0;
   job.tiles_per_chunk = tpc;
   job.atoms_per_tile = (int)((s->n + tpc - 1) / tpc);
-  job.tile_base = 0;
   job.part = 0;
   job.plan = plan;
   for (int k = 0; k < 9; ++k) job.rot[k] = rot ? rot[k] : ((k % 4 == 0) ? 1.0 : 0.0);
