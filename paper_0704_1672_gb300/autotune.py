@@ -9,8 +9,9 @@ them) form a sub-batch; each candidate setting (atoms per lane, CTAs per SM, kma
 with ``tcm_ctx_set_tiling_l`` and ``tcm_ctx_set_chunking_l``, the sub-batch is run once untimed
 and ``reps`` times timed, and the shortest time of the moment phase (the library's CUDA-event
 phase profile: the moment kernels of that degree, nothing else) is kept.  The fastest candidate
-(when the sub-batch is a sample of the degree's items: among those within 1 % of it, the one
-with the largest warp tiles; ``choose``) is applied to the context and returned.  Results can be saved to a JSON file keyed by device
+(when the sub-batch is a sample of the degree's items: the setting in force if it is within 2 % of
+that, else, among those within 1 %, the one with the largest warp tiles; ``choose``) is applied to the
+context and returned.  Results can be saved to a JSON file keyed by device
 name, library build and precision, and loaded into a later context.
 
 The tiling and the chunking change only the order in which atom contributions are summed, so
@@ -29,6 +30,10 @@ DEFAULT_ATOMS_PER_LANE = (16, 32, 48, 64, 96, 128, 256)
 DEFAULT_CTAS_PER_SM = (1, 2, 3)
 DEFAULT_KMAX = (160, 96)  # the mixed path's chunk budgets (tcm_ctx_set_chunking_l)
 FP64_KMAX = 80            # the double kernels' budget (fixed)
+# A sampled degree keeps the setting in force when that is within 2 % of the fastest: a sample does not tell
+# settings apart more finely (uneven batch, degree 16: 64 atoms per lane lead 96 by 1 to 3 %, or not at
+# all, from process to process), and the order of summation, with it the rounding, should not depend on that.
+STAY = 1.02
 
 
 def ctas_limit(precision, kmax):
@@ -158,6 +163,8 @@ def tune(ctx, systems, a, b, lmax, R0, rotB=None, precision=None, atoms_per_lane
         # larger tiles save: then prefer them within 1 %; the whole batch is timed as it is
         subsampled = len(idx) < int(np.count_nonzero(lmax == L))
         best = choose(t, tol=0.01 if subsampled else 0.0) or default
+        if subsampled and t.get(default, np.inf) <= STAY * min(t.values()):
+            best = default
         set_setting(ctx, precision, L, best)
         res.best[L] = best
         res.timings[L] = t
