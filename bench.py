@@ -73,16 +73,22 @@ def moment_instr_per_atom(L):
 
 
 def contract_imads(L, rotated_b=False):
-    """Algorithmic 32 x 32 + 64 bit multiply-adds (IMAD.WIDE, three per fixed-point product) of one
-    energy in k_contract: per (l, m >= 0) entry of A the input and beta phases (4 products each) and
-    the hat factor (2), of B the hat factor, or the same as A when its moments are rotated in the
-    kernel (and 4 more for the output phase); the two products through d^l(pi/2) (2 sum_l (l+1)^2 per
-    rotated side); the z-axis contraction (sum over (l1, l2) of 1 + 2 min(l1, l2))."""
+    """Algorithmic 32 x 32 + 64 bit multiply-adds (IMAD.WIDE, three per fixed-point product) of the
+    rotations of one energy in k_contract: per (l, m >= 0) entry of A the input and beta phases (4
+    products each) and the two products through d^l(pi/2) (2 sum_l (l+1)^2); the same for B when its
+    moments are rotated in the kernel, and 4 more per entry for the output phase."""
     T = (L + 1) * (L + 2) // 2
     S2 = (L + 1) * (L + 2) * (2 * L + 3) // 6
-    Z = sum(1 + 2 * min(a, b) for a in range(L + 1) for b in range(L + 1))
-    side = 10 * T + 2 * S2
-    return 3 * (side + (side + 4 * T if rotated_b else 2 * T) + Z)
+    side = 8 * T + 2 * S2
+    return 3 * (side + (side + 4 * T if rotated_b else 0))
+
+
+def contract_fp64(L, rotated_b=False):
+    """Algorithmic FP64 instructions of one energy in k_contract: per (l, m >= 0) entry of a rotated
+    side two conversions and two products by the entry's factor (B's entries in the frame: the products
+    alone); per (l1, l2) the 2 min(l1, l2) + 1 multiply-adds of the components and their weight (2)."""
+    T = (L + 1) * (L + 2) // 2
+    return 4 * T + (4 if rotated_b else 2) * T + sum(3 + 2 * min(a, b) for a in range(L + 1) for b in range(L + 1))
 
 
 def measured_peaks():
@@ -394,7 +400,6 @@ def run_ours(args, rank, world, dist):
     smx = sm_max_mhz()
     peak_fp32 = n_sm * FP32_LANES_PER_SM * smx * 1e6 / 1e12      # T lane-instr/s
     peak_fp64 = n_sm * FP64_PER_SM_CLK * smx * 1e6 / 1e9         # G FP64 op/s
-    peak_imad = n_sm * IMAD_PER_SM_CLK * smx * 1e6 / 1e9         # G IMAD.WIDE lane-op/s
     prec = tcm.TCM_MIXED if args.precision == "mixed" else tcm.TCM_FP64
     stream = torch.cuda.current_stream()
     timer = Timer(torch, stream)
@@ -467,12 +472,12 @@ def run_ours(args, rank, world, dist):
                 "peak_source": f"{n_sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x {smx:.0f} MHz (max SM clock of measured)",
                 "algorithmic_instr_per_atom": moment_instr_per_atom(L), "launch_ms": mom_launch_ms}
     con_launch_ms = phase_ms["contract"] / max(1, launches["contract"])
-    con_ops = k * contract_imads(L)
-    con_rate = con_ops / (con_launch_ms * 1e-3) / 1e9
-    contract_roofline = {"bound": "int", "kernel": "k_contract<false>", "achieved": con_rate, "peak": peak_imad,
-                         "unit": "G IMAD.WIDE lane-op/s", "frac": con_rate / peak_imad,
+    con_rate = k * contract_fp64(L) / (con_launch_ms * 1e-3) / 1e9
+    contract_roofline = {"bound": "fp64", "kernel": "k_contract<false>", "achieved": con_rate, "peak": peak_fp64,
+                         "unit": "G FP64 instr/s", "frac": con_rate / peak_fp64,
+                         "algorithmic_fp64_per_energy": contract_fp64(L),
                          "algorithmic_imads_per_energy": contract_imads(L), "launch_ms": con_launch_ms,
-                         "peak_source": f"{n_sm} SMs x {IMAD_PER_SM_CLK} per clk x {smx:.0f} MHz"}
+                         "peak_source": f"{n_sm} SMs x {FP64_PER_SM_CLK} per clk x {smx:.0f} MHz"}
 
     # the same steps with the library's default launch mode (phase events off: a replayed CUDA graph)
     g_ms = timer.run(step, min(args.steps, 10), 3)
@@ -626,8 +631,7 @@ def bench_config2(torch, tcm, synth, autotune, timer, stream, prec, peak_fp32, p
     instr = atoms * moment_instr_per_atom(L) / max(1.0, la["moments"] / n)
     ach = instr / (mom_launch_ms * 1e-3) / 1e12
     con_launch_ms = ph["contract"] / max(1, la["contract"])
-    con = k * contract_imads(L) / (con_launch_ms * 1e-3) / 1e9
-    peak_imad = n_sm * IMAD_PER_SM_CLK * smx * 1e6 / 1e9
+    con = k * contract_fp64(L) / (con_launch_ms * 1e-3) / 1e9
     g_ms = timer.run(step, steps, 3)
     out = {"workload": "protein-like PES scan: 2 x 20000 random-walk atoms (r=30 A, N(0,0.3) net-zero), 256 "
                        "orientations of B, |R0| in [70,150] A, Lmax=20",
@@ -639,8 +643,9 @@ def bench_config2(torch, tcm, synth, autotune, timer, stream, prec, peak_fp32, p
            "roofline": {"bound": "alu", "kernel": f"k_moments<float,{L}>", "achieved": ach, "peak": peak_fp32,
                         "unit": "T FP32-pipe lane-instr/s", "frac": ach / peak_fp32, "launch_ms": mom_launch_ms,
                         "traffic": captured_traffic("k_moments_pes_scan_L20.md", ["moments_kernel.cuh", "tcm_internal.h"])},
-           "contract_roofline": {"bound": "int", "achieved": con, "peak": peak_imad, "unit": "G IMAD.WIDE lane-op/s",
-                                 "frac": con / peak_imad, "launch_ms": con_launch_ms,
+           "contract_roofline": {"bound": "fp64", "achieved": con, "peak": peak_fp64, "unit": "G FP64 instr/s",
+                                 "frac": con / peak_fp64, "launch_ms": con_launch_ms,
+                                 "algorithmic_fp64_per_energy": contract_fp64(L),
                                  "algorithmic_imads_per_energy": contract_imads(L)},
            "tiling": ({"atoms_per_lane": tuned.best[L][0], "ctas_per_sm": tuned.best[L][1], "kmax": tuned.best[L][2],
                        "chunks": ctx.tcm_ctx_get_chunking_l(L)[1]} if tuned else (fixed or "default"))}

@@ -40,9 +40,9 @@
 // Error of an energy (rms, of sum |U_l1l2|, 40 random pairs at degrees 1 to 24; against 113-bit
 // arithmetic): 1.5e-16 to 8.9e-16, the all-double kernel's 1.5e-16 to 8.9e-16; forces and torques alike.
 // Measured (us), all in double, with the products in fixed point too, and now: 108,360 energies at degrees 1 to
-// 10 1,340, 298, 331; 2,048 at degrees 8 to 24 (B rotated) 140, 64, 78; 256 at degree 20 24, 16, 21; forces
-// and torques of 512 at degree 12 92, 25, 49.  What bounds it now: the FP64 pipe in the (l1, l2) phase (busy
-// 0.54 over the kernel at degree 24, 0.66 with forces and torques) between phases separated by barriers.
+// 10 1,340, 298, 328; 2,048 at degrees 8 to 24 (B rotated) 140, 64, 76; 256 at degree 20 24, 16, 20; forces
+// and torques of 512 at degree 12 92, 25, 42 (49 with products by m instead of partial sums).  What bounds it now: the
+// FP64 pipe in the (l1, l2) phase (busy 0.54 over the kernel at degree 24) between phases separated by barriers.
 // A CTA takes a group of items of one degree side by side (contract_group), so that its lanes are full
 // at low degrees too, one lane column per item.  The group size, and with it the order of every sum,
 // depends on the degree alone: an item's result does not depend on its batch.
