@@ -245,7 +245,8 @@ int tcm_ctx_set_rotate_cached(tcm_ctx_t ctx, int enable);
  * two-center energy at R0.  Moment sets shared by several items (same system, lmax
  * and no rotation) are computed once.  Systems without a centre or radius get them
  * on the device (step a1) without a host round trip.
- *   E:      device, n_items doubles (NaN for an item that does not converge)
+ *   E:      device, n_items doubles (NaN for an item that does not converge, and, above degree 0, for one
+ *           whose rotation or separation is not finite)
  *   status: device, n_items int32 (TCM_OK or TCM_ENOTCONV), or NULL
  * Systems that carry a moment cache (tcm_system.moments) reuse it for their unrotated sides
  * (and for rotated sides too under tcm_ctx_set_rotate_cached).
